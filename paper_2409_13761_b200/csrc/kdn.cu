@@ -748,12 +748,13 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
                 op.rope = n_rope++;
             }
             tp.inline_ops[i] = op;
+            tp.layout[i] = td_layout(pool.L, row_elems, op.T, op.codec);
+            if (td_words(op.codec) > tp.words) tp.words = td_words(op.codec);
             const int g = (op.T + 63) / 64;
             if (g > max_groups) max_groups = g;
             if (op.nl > max_layers) max_layers = op.nl;
         }
         if (max_groups == 0 || max_layers == 0) continue;
-        tp.ops = nullptr;
         tp.n_ops = m;
         tp.k_layers = pool.d_k;
         tp.v_layers = pool.d_v;
@@ -764,6 +765,12 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
         tp.row_elems = row_elems;
         tp.cols = cols;
         tp.n_split = n_split;
+        while ((1u << tp.split_shift) < n_split) ++tp.split_shift;
+        tp.word_row = cols * 4u;
+        tp.one = 1;
+        tp.minus_two = -2;
+        tp.bs_shift = -1;
+        for (int b = 0; b < 31; ++b) if (pool.bs == 1 << b) tp.bs_shift = b;
         tp.status = ctx->d_status;
         const dim3 grid((unsigned)max_groups * n_split, (unsigned)max_layers * 2u, (unsigned)m);
         int per_sm = 0;
@@ -782,7 +789,7 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
             KDN_CUDA(cudaGetLastError());
             ctx->launches += 3;
         } else {
-            const size_t smem = td_decode_smem_bytes(cols);
+            const size_t smem = td_decode_smem_bytes(cols, tp.words);
             if (smem > smem_limit) return KDN_E_UNSUPPORTED;
             RingSlot *slot = nullptr;
             if (n_rope) {
@@ -797,14 +804,15 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
                 tp.rope = slot->d_table;
             }
             kdn_status r = KDN_OK;
+            const unsigned dec_threads = (cols / 2u + 31u) & ~31u;       // a thread decodes two channels
 #define KDN_TD_DECODE(COMPOSE, COLS)                                                                        \
             {                                                                                               \
-                r = ctx->env.resident(kdn_td_decode_kernel<COMPOSE, COLS>, (int)threads, smem, &per_sm);    \
+                r = ctx->env.resident(kdn_td_decode_kernel<COMPOSE, COLS>, (int)dec_threads, smem, &per_sm); \
                 if (r != KDN_OK) return r;                                                                  \
                 if (per_sm < 1) return KDN_E_UNSUPPORTED;                                                   \
-                kdn_td_decode_kernel<COMPOSE, COLS><<<grid, threads, smem, stream>>>(tp);                   \
+                kdn_td_decode_kernel<COMPOSE, COLS><<<grid, dec_threads, smem, stream>>>(tp);               \
             }
-            if (cols == kTdCols && threads == kTdCols) {
+            if (cols == kTdCols) {
                 if (OP == OP_COMPOSE) KDN_TD_DECODE(true, kTdCols) else KDN_TD_DECODE(false, kTdCols)
             } else {
                 if (OP == OP_COMPOSE) KDN_TD_DECODE(true, 0) else KDN_TD_DECODE(false, 0)

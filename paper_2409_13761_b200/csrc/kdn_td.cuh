@@ -8,9 +8,9 @@
 //   store    plan   (kdn_td_plan_kernel):   quantise, pick (mode, k) per channel, write scales / lens / params
 //            scan   (kdn_td_scan_kernel):   segment sizes -> seg_off (one CTA per op)
 //            encode (kdn_td_encode_kernel): quantise again, write every sub-stream at its final place
-//   retrieve / compose (kdn_td_decode_kernel): bulk-copy the slice's bytes into shared memory, one thread per
-//            channel undoes Rice, zigzag and the delta into a code tile, which the ordinary per-channel decoder or
-//            key rotation turns into bf16 rows that bulk copies scatter to the pool blocks.
+//   retrieve / compose (kdn_td_decode_kernel): bulk-copy the slice's bytes into shared memory; a thread undoes Rice,
+//            zigzag and the delta of two channels, scales (and rotates) the values and writes them into bf16 rows that
+//            128-bit stores scatter to the pool blocks.
 // The store reads the pool twice instead of keeping codes in scratch memory: no kernel here uses memory beyond the
 // pool and the chunk.  Every wait is bounded as in the tile pipeline.
 #pragma once
@@ -18,24 +18,6 @@
 #include "kdn_kernels.cuh"
 
 namespace kdn {
-
-struct TdLaunch {
-    const DevOp *ops;         // device array, or nullptr: inline_ops
-    int n_ops;
-    void *const *k_layers;
-    void *const *v_layers;
-    long long n_blocks;
-    int bs;
-    int D;
-    int L;                    // layers of the pool = layers of every chunk
-    unsigned row_elems;
-    unsigned cols;            // channels per CTA
-    unsigned n_split;         // row_elems / cols
-    const float2 *rope;
-    int *status;
-    unsigned long long wait_limit_ns;   // a wait for a slice's bytes gives up after this long
-    DevOp inline_ops[kInlineOps];
-};
 
 __host__ __device__ inline int td_qmax(int codec) { return codec == 5 ? 127 : 7; }
 __host__ __device__ inline int td_raw_bits(int codec) { return codec == 5 ? 9 : 5; }
@@ -58,6 +40,29 @@ __host__ __device__ inline TdLayout td_layout(int L, unsigned row_elems, int T, 
     return t;
 }
 
+struct TdLaunch {
+    int n_ops;
+    void *const *k_layers;
+    void *const *v_layers;
+    long long n_blocks;
+    int bs;
+    int D;
+    int L;                    // layers of the pool = layers of every chunk
+    unsigned row_elems;
+    unsigned cols;            // channels per CTA
+    unsigned n_split;         // row_elems / cols, a power of two
+    unsigned split_shift;     // log2(n_split)
+    unsigned words;           // decode: 32-bit words kept per sub-stream (the longest of the launch's codecs, and one more)
+    int bs_shift;             // log2(bs), -1 where bs is not a power of two
+    int one, minus_two;       // 1 and -2 as launch parameters: see TdStream
+    unsigned word_row;        // decode: bytes of one row of interleaved words (4 * cols), for the same reason
+    const float2 *rope;
+    int *status;
+    unsigned long long wait_limit_ns;   // a wait for a slice's bytes gives up after this long
+    TdLayout layout[kInlineOps];        // of each op's chunk
+    DevOp inline_ops[kInlineOps];
+};
+
 // Shared memory of the store kernels: token rows, slice maxima, reciprocals, the stream staging area (encode only),
 // small per-warp scratch, barrier.
 // (the plan kernel keeps two tables of code-word lengths in place of the staging area, each replicated so that the
@@ -72,19 +77,22 @@ __host__ __device__ inline size_t td_store_smem_bytes(unsigned cols, bool encode
     return (size_t)64 * cols * 2u + (size_t)kKcSlices * cols * 2u + (size_t)cols * 4u +
            (encode ? (size_t)cols * 72u + 32u + kTdStageSlack : (size_t)kTdCostBytes) + 256u + 16u;
 }
-// Shared memory of the decode kernel: the slice's stream bytes as they lie in the chunk, the same sub-streams
-// interleaved word by word (so that the 32 lanes of a warp read 32 different banks), codes, scales, offsets, barrier.
-// The bf16 rows reuse the two stream areas once the codes are complete.
-constexpr unsigned kTdWords = 19;                           // 32-bit words per interleaved sub-stream: 72 bytes, and the word after
-__host__ __device__ inline size_t td_decode_packed_bytes(unsigned cols) { return ((size_t)cols * 72u + 128u + 127u) & ~(size_t)127u; }
-__host__ __device__ inline size_t td_decode_front_bytes(unsigned cols)
+// Shared memory of the decode kernel: the sub-streams interleaved word by word (so that the 32 lanes of a warp, each
+// somewhere else in its stream, read 32 different banks), half of the group's bf16 rows, the sub-streams' offsets, the
+// rows' addresses.  The slice's stream bytes as they lie in the chunk share the rows' place: they are interleaved before
+// the first row is written.  The interleaved words come first: a damaged stream may look a few rows past them, which is
+// then still inside the CTA's memory, and garbage either way.
+constexpr unsigned kTdHalf = 32;                            // rows between two write-outs
+__host__ __device__ inline unsigned td_words(int codec) { return td_max_len(codec) / 4u + 1u; }   // the longest sub-stream, and the word after
+__host__ __device__ inline size_t td_decode_words_bytes(unsigned cols, unsigned words) { return (size_t)words * cols * 4u; }
+__host__ __device__ inline size_t td_decode_rows_bytes(unsigned cols, unsigned words)
 {
-    const size_t a = (size_t)64 * cols * 2u, s = td_decode_packed_bytes(cols) + (size_t)kTdWords * cols * 4u;
+    const size_t a = (size_t)kTdHalf * cols * 2u, s = ((size_t)cols * (words - 1u) * 4u + 256u + 127u) & ~(size_t)127u;
     return a > s ? a : s;
 }
-__host__ __device__ inline size_t td_decode_smem_bytes(unsigned cols)
+__host__ __device__ inline size_t td_decode_smem_bytes(unsigned cols, unsigned words)
 {
-    return td_decode_front_bytes(cols) + (size_t)64 * cols + (size_t)cols * 4u + 256u + 16u;
+    return td_decode_words_bytes(cols, words) + td_decode_rows_bytes(cols, words) + (size_t)cols * 4u + 64u * 8u + 256u + 16u;
 }
 
 // Bits of one Rice code word.
@@ -245,10 +253,9 @@ struct TdSlice {              // what a CTA of the store and decode kernels work
 __device__ __forceinline__ TdSlice td_slice(const TdLaunch &P)
 {
     TdSlice s;
-    const DevOp *ops = P.ops ? P.ops : P.inline_ops;
-    s.op = ops[blockIdx.z];
-    s.g = blockIdx.x / P.n_split;
-    s.part = blockIdx.x - s.g * P.n_split;
+    s.op = P.inline_ops[blockIdx.z];
+    s.g = blockIdx.x >> P.split_shift;
+    s.part = blockIdx.x & (P.n_split - 1u);
     s.plane = blockIdx.y;                                      // index into the op's layer range: li * 2 + kv
     s.li = s.plane >> 1;
     s.kv = s.plane & 1u;
@@ -400,8 +407,7 @@ __global__ void __launch_bounds__(512) kdn_td_plan_kernel(const __grid_constant_
 __global__ void __launch_bounds__(256) kdn_td_scan_kernel(const __grid_constant__ TdLaunch P)
 {
     __shared__ unsigned long long part[256];
-    const DevOp *ops = P.ops ? P.ops : P.inline_ops;
-    const DevOp op = ops[blockIdx.x];
+    const DevOp op = P.inline_ops[blockIdx.x];
     if (op.codec < 5 || op.T <= 0) return;
     const unsigned RE = P.row_elems;
     const TdLayout lay = td_layout(P.L, RE, op.T, op.codec);
@@ -561,11 +567,136 @@ __global__ void __launch_bounds__(512) kdn_td_encode_kernel(const __grid_constan
 
 // ----------------------------------------------------------------------------------- retrieve / compose --
 
+// One sub-stream on its way through the decoder.  Everything is kept in the form that takes the fewest operations of the
+// pipe that shifts, compares and logic share (it issues every other cycle and is what bounds this kernel):
+//  * the words hold the complement of the stream, so the ones of the unary part are leading zeros.  With h the next 32
+//    bits, n = clz(h), z = (h << n) >> (31 - k) = 2^(k+1) - 1 - rem, and v = z - n 2^k = c - u with c = 2^(k+1) - 1, the
+//    symbol u never appears itself;
+//  * 2 e (e = the signed code or code difference) is u for even u and -(u + 1) for odd u, i.e. with s = v & 1
+//    2 e = s (2 c + 1 - 2 v) + v - c - 1: multiply-adds, which run on the other integer pipe (their small constant factors
+//    arrive as launch parameters: known ones would be turned back into shifts and adds);
+//  * the running code is kept as the bits of the fp32 number 2^22 + 512 + q, whose unit in the last place is 1/2: adding
+//    2 e to the bits adds e to the number, and one subtraction gives q exactly.
+struct TdStream {
+    uint32_t col;          // shared address of word 0 of the sub-stream
+    unsigned bp;           // bits consumed
+    unsigned k1, sh;       // k + 1, 31 - k
+    int kneg;              // -2^k
+    int c21;               // 2 c + 1
+    int d, c2;             // next = acc * d + c2 + ...: d = 1 in delta mode, else 0 and c2 holds the fresh start
+    int acc;
+};
+constexpr int kTdCodeBits = 0x4A800000 + 1024;             // 2^22 + 512 as fp32 bits
+constexpr float kTdCodeZero = 4194304.0f + 512.0f;
 
+__device__ __forceinline__ void td_stream_init(TdStream &s, uint32_t col, unsigned param)
+{
+    const unsigned k = param & 7u;
+    const int c = (int)((2u << k) - 1u);
+    s.col = col;
+    s.bp = 0u;
+    s.k1 = k + 1u;
+    s.sh = 31u - k;
+    s.kneg = -(int)(1u << k);
+    s.c21 = 2 * c + 1;
+    s.d = (param & 8u) ? 1 : 0;
+    s.c2 = -(c + 1) + ((param & 8u) ? 0 : kTdCodeBits);
+    s.acc = kTdCodeBits;
+}
+// (PTX shifts by 32 and more give 0: a window of ones only)
+__device__ __forceinline__ uint32_t td_shl(uint32_t x, unsigned n)
+{
+    uint32_t r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(n));
+    return r;
+}
+template <unsigned kCols>
+__device__ __forceinline__ uint32_t td_window(const TdStream &s, unsigned row_b)
+{
+    const uint32_t a = (s.bp >> 5) * row_b + s.col;
+    uint32_t w0, w1;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w0) : "r"(a));
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w1) : "r"(a + (kCols ? kCols * 4u : row_b)));
+    return __funnelshift_l(w1, w0, s.bp);
+}
+// The next symbol out of the window h, taken not to be an escape; returns the length of its unary part (15 and more: it was one)
+// and, in len, the length of the code word.
+__device__ __forceinline__ unsigned td_symbol(const TdLaunch &P, TdStream &s, uint32_t h, unsigned &len)
+{
+    unsigned n;
+    asm("bfind.shiftamt.u32 %0, %1;" : "=r"(n) : "r"(h));
+    const int z = (int)(td_shl(h, n) >> s.sh);
+    const int v = (int)n * s.kneg + z;
+    len = n + s.k1;
+    s.bp += len;
+    const int a = v * P.minus_two + s.c21;
+    const int r = v * P.one + (s.acc * s.d + s.c2);
+    s.acc = (v & 1) * a + r;
+    return n;
+}
+// The same with escapes.
+__device__ __forceinline__ void td_symbol_any(const TdLaunch &P, TdStream &s, uint32_t h, unsigned raw_bits)
+{
+    if ((h >> 17) != 0u) {                                  // fewer than fifteen ones
+        unsigned len;
+        td_symbol(P, s, h, len);
+        return;
+    }
+    const int u = (int)((~h << 15) >> (32u - raw_bits));
+    s.bp += 15u + raw_bits;
+    s.acc = (u ^ -(u & 1)) + (s.d ? s.acc : kTdCodeBits);
+}
+
+constexpr unsigned kTdStep = 4;                             // symbols of a stream between two looks for escapes
+// kTdStep symbols of two streams side by side, kWin of them out of one 32-bit window (code words of 4-bit codes are short:
+// four in a window; of 8-bit codes: two).  Taken to be no escapes and to fit their windows; where that was wrong, once more
+// with care.  (8B shape, 32 chunks of 512 tokens, 4-bit codes: a window a symbol 965 us, two 908, four 867.)
+template <unsigned kCols, unsigned kWin>
+__device__ __forceinline__ void td_step(const TdLaunch &P, TdStream &x, TdStream &y, unsigned row_b, unsigned max_bits, unsigned raw_bits,
+                                        int (&vx)[kTdStep], int (&vy)[kTdStep])
+{
+    x.bp = x.bp < max_bits ? x.bp : max_bits;               // (a damaged stream cannot run off the area)
+    y.bp = y.bp < max_bits ? y.bp : max_bits;
+    const unsigned bp_x = x.bp, bp_y = y.bp;
+    const int acc_x = x.acc, acc_y = y.acc;
+    unsigned longest = 0, most = 0;
+#pragma unroll
+    for (unsigned i = 0; i < kTdStep; i += kWin) {
+        uint32_t hx = td_window<kCols>(x, row_b), hy = td_window<kCols>(y, row_b);
+        const unsigned from_x = x.bp, from_y = y.bp;
+#pragma unroll
+        for (unsigned j = 0; j < kWin; ++j) {
+            unsigned lx, ly;
+            const unsigned nx = td_symbol(P, x, hx, lx), ny = td_symbol(P, y, hy, ly);
+            longest = max(longest, max(nx, ny));
+            hx = td_shl(hx, lx);
+            hy = td_shl(hy, ly);
+            vx[i + j] = x.acc; vy[i + j] = y.acc;
+        }
+        most = max(most, max(x.bp - from_x, y.bp - from_y));
+    }
+    if (__builtin_expect(longest >= 15u || most > 32u, 0)) {
+        x.bp = bp_x; y.bp = bp_y; x.acc = acc_x; y.acc = acc_y;
+#pragma unroll
+        for (unsigned i = 0; i < kTdStep; ++i) {
+            td_symbol_any(P, x, td_window<kCols>(x, row_b), raw_bits);
+            td_symbol_any(P, y, td_window<kCols>(y, row_b), raw_bits);
+            vx[i] = x.acc; vy[i] = y.acc;
+        }
+    }
+}
+
+// Bound by the integer pipes (8B shape, 4-bit codes: ALU pipe about 70 %, issue slots 80 %, DRAM 30 %); what was done
+// about it is at TdStream and td_step.  A thread decodes two channels side by side -- neighbours, whose bf16 values make one
+// word, or, where keys are re-rotated, the two channels of a rotation pair -- so that one stream's chain of dependent
+// operations hides the other's, and writes finished values into the rows: no pass over codes.  Half of the rows at a time
+// keeps a CTA of 64 threads at 16 KiB of shared memory, fourteen (8-bit codes: ten) to an SM.  The rows leave with 128-bit
+// stores, sixteen lanes to a 256-byte piece of a token row.  8B shape, 32 chunks of 512 tokens, 4-bit codes: 1727 -> 867 us
+// against one thread per channel, a code tile and a separate pass that multiplied.
 // kCols: channels per CTA when known at compile time (the usual slice; every stride in the decoding loop is then an
 // immediate), 0: taken from the launch record.
 template <bool kCompose, unsigned kCols>
-__global__ void __launch_bounds__(kCols ? kCols : 512) kdn_td_decode_kernel(const __grid_constant__ TdLaunch P)
+__global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 14 : 1) kdn_td_decode_kernel(const __grid_constant__ TdLaunch P)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const TdSlice s = td_slice(P);
@@ -573,16 +704,17 @@ __global__ void __launch_bounds__(kCols ? kCols : 512) kdn_td_decode_kernel(cons
     const unsigned C = kCols ? kCols : P.cols, RE = P.row_elems;
     const int codec = s.op.codec;
     const unsigned raw_bits = (unsigned)td_raw_bits(codec);
+    const unsigned nthreads = kCols ? kCols / 2u : blockDim.x, nwarps = nthreads >> 5;
 
-    unsigned char *A = smem_raw;                                         // bf16 rows; first the slice's stream bytes ...
-    uint32_t *I = reinterpret_cast<uint32_t *>(A + td_decode_packed_bytes(C));   // ... and the interleaved sub-streams [word][C]
-    unsigned char *B = A + td_decode_front_bytes(C);                     // codes [n_tok][C]
-    float *Sc = reinterpret_cast<float *>(B + (size_t)64 * C);           // scales [C]
-    unsigned *scratch = reinterpret_cast<unsigned *>(Sc + C);            // 64 words
+    uint32_t *I = reinterpret_cast<uint32_t *>(smem_raw);                // interleaved sub-streams [word][C]
+    unsigned char *A = smem_raw + td_decode_words_bytes(C, P.words);     // the slice's stream bytes, then bf16 rows [kTdHalf][C]
+    unsigned *offs = reinterpret_cast<unsigned *>(A + td_decode_rows_bytes(C, P.words));   // where each channel's sub-stream starts
+    unsigned long long *rows = reinterpret_cast<unsigned long long *>(offs + C);     // pool address of each token row's slice, 0: not written
+    unsigned *scratch = reinterpret_cast<unsigned *>(rows + 64);         // 64 words
     unsigned long long *bar_mem = reinterpret_cast<unsigned long long *>(reinterpret_cast<unsigned char *>(scratch) + 256u);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bar_mem + 1);
     const uint32_t bar = smem_u32(bar_mem);
-    const unsigned tid = threadIdx.x;
+    const unsigned tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     if (tid == 0) {
         mbar_init(bar, 1u);
         *abort_flag = 0;
@@ -592,20 +724,35 @@ __global__ void __launch_bounds__(kCols ? kCols : 512) kdn_td_decode_kernel(cons
     // a select-list (compose): which of its entries fall into this group?  Two threads look; none: nothing to do here
     const bool selecting = kCompose && s.op.list_mode == 2;
     if (selecting && tid < 2u) scratch[40u + tid] = td_lower_bound(s.op.list, (unsigned)s.op.n_list, ((long long)s.g + tid) << 6);
-    const TdLayout lay = td_layout(P.L, RE, s.op.T, codec);
+    const TdLayout &lay = P.layout[blockIdx.z];
     const unsigned long long row = (unsigned long long)s.seg * RE;
     const unsigned char *lens = s.op.data + lay.lens + row;
+    const bool act = 2u * tid < C;
+    // bytes of the channels before the slice (16 lengths a load: the table's rows and c0 are multiples of 16), and of the
+    // slice's own channels, two a thread
     unsigned before = 0;
-    for (unsigned c = tid; c < s.c0; c += blockDim.x) before += lens[c];
-    unsigned total_before, total_slice;
-    td_block_scan(before, scratch, &total_before);                        // (its barriers also publish the mbarrier and the two indices)
+    for (unsigned i = tid; i < (s.c0 >> 4); i += nthreads) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(lens + 16u * i);
+        before = __dp4a(v.x, 0x01010101u, before); before = __dp4a(v.y, 0x01010101u, before);
+        before = __dp4a(v.z, 0x01010101u, before); before = __dp4a(v.w, 0x01010101u, before);
+    }
+    const unsigned pair = act ? *reinterpret_cast<const unsigned short *>(lens + s.c0 + 2u * tid) : 0u;
+    const unsigned both = (pair & 0xffu) + (pair >> 8);
+    unsigned inc = both;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned o = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= (unsigned)d) inc += o;
+    }
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 31u) { scratch[warp] = inc; scratch[16u + warp] = before; }
+    __syncthreads();                                                      // (also publishes the mbarrier and the two indices)
     if (selecting && scratch[40] >= scratch[41]) return;                  // every thread alike, and no copy has been started
-    const unsigned my_len = tid < C ? lens[s.c0 + tid] : 0u;               // blockDim.x >= C
-    const unsigned my_off = td_block_scan(my_len, scratch, &total_slice);
-    unsigned param = 0;
-    if (tid < C) {
-        param = s.op.data[lay.params + row + s.c0 + tid];
-        Sc[tid] = reinterpret_cast<const float *>(s.op.data + lay.scales)[row + s.c0 + tid];
+    unsigned total_before = 0, total_slice = 0, my_off = inc - both;
+    for (unsigned w = 0; w < nwarps; ++w) {
+        if (w == warp) my_off += total_slice;
+        total_slice += scratch[w];
+        total_before += scratch[16u + w];
     }
     const unsigned long long seg_begin = reinterpret_cast<const unsigned long long *>(s.op.data)[s.seg];
     const unsigned long long src = seg_begin + total_before;
@@ -616,7 +763,7 @@ __global__ void __launch_bounds__(kCols ? kCols : 512) kdn_td_decode_kernel(cons
     // its capacity, or what a staging slab holds of it)
     const unsigned long long exist = (unsigned long long)(s.op.scales - s.op.data);
     const unsigned long long have = exist < lay.capacity ? exist : lay.capacity;
-    const bool sane = total_slice <= C * td_max_len(codec) && src >= lay.streams && src - shift + bytes_al <= have;
+    const bool sane = total_slice <= C * td_max_len(codec) && src >= lay.streams && src <= have && src - shift + bytes_al <= have;
     if (tid == 0) {
         if (!sane) {
             atomicCAS(P.status, 0, kStatusRange);
@@ -630,139 +777,151 @@ __global__ void __launch_bounds__(kCols ? kCols : 512) kdn_td_decode_kernel(cons
             mbar_arrive(bar);
         }
     }
-    __syncthreads();
-    if (*abort_flag) return;
+    // while the bytes are on their way: the thread's two channels, and where the rows go
+    const bool rotating = kCompose && s.kv == 0u && s.op.rope >= 0;
+    const unsigned half = (unsigned)P.D >> 1;
+    const unsigned head = rotating ? tid / half : 0u;
+    const unsigned ca = rotating ? head * (unsigned)P.D + (tid - head * half) : 2u * tid;   // first channel, inside the slice
+    const unsigned cb = rotating ? ca + half : ca + 1u;
+    unsigned param_a = 0, param_b = 0;
+    float sc_a = 0.0f, sc_b = 0.0f;
+    if (act) {
+        const unsigned char *params = s.op.data + lay.params + row + s.c0;
+        const float *scales = reinterpret_cast<const float *>(s.op.data + lay.scales) + row + s.c0;
+        param_a = params[ca]; param_b = params[cb];
+        sc_a = scales[ca]; sc_b = scales[cb];
+        offs[2u * tid] = my_off | ((pair & 0xffu) << 24);                 // (a slice holds fewer than 2^24 bytes)
+        offs[2u * tid + 1u] = (my_off + (pair & 0xffu)) | ((pair >> 8) << 24);
+    }
+    {
+        unsigned char *base = reinterpret_cast<unsigned char *>((s.kv ? P.v_layers : P.k_layers)[s.op.l0 + (int)s.li]);
+        if (selecting) {
+            for (unsigned r = tid; r < 64u; r += nthreads) rows[r] = 0ull;
+            __syncthreads();
+        }
+        // the rows of the group, or its listed ones
+        const unsigned first = selecting ? scratch[40] : 0u, last = selecting ? scratch[41] : s.n_tok;
+        for (unsigned i = first + tid; i < last; i += nthreads) {
+            bool bad = false;
+            unsigned r = i;
+            if (selecting) {
+                const long long c = (long long)__ldg(s.op.list + i) - ((long long)s.g << 6);
+                bad = c < 0 || c >= (long long)s.n_tok;                   // (a list that is not increasing)
+                r = (unsigned)c;
+            }
+            if (!bad) {
+                const long long pos = group_row_pos(s.op, s.g, r);
+                bad = pos < 0;
+                if (!bad) {
+                    const long long blk = P.bs_shift >= 0 ? pos >> P.bs_shift : pos / P.bs;
+                    const long long id = __ldg(s.op.table + blk);
+                    bad = id < 0 || id >= P.n_blocks;
+                    if (!bad) rows[r] = (unsigned long long)(base + ((unsigned long long)(id * P.bs + (pos - blk * P.bs)) * RE + s.c0) * 2ull);
+                }
+            }
+            if (bad) {
+                atomicCAS(P.status, 0, kStatusRange);
+                *abort_flag = 2;                                          // nothing of this slice is written
+            }
+        }
+    }
     const bool landed = mbar_wait(bar, 0u, abort_flag, P.wait_limit_ns);
-    if (!__syncthreads_and(landed)) {
-        if (tid == 0) {
-            atomicCAS(P.status, 0, kStatusTimeout);
+    if (!__syncthreads_and(landed)) {                                     // all threads leave together
+        if (tid == 0 && sane) {
+            if (*abort_flag != 2) atomicCAS(P.status, 0, kStatusTimeout);
+            // the CTA does not leave while a copy into its shared memory is in flight
             const unsigned long long t0 = global_timer_ns();
             while (!mbar_try_wait(bar, 0u))
                 if (global_timer_ns() - t0 > kWaitLimitNs) break;
         }
         return;
     }
-    // one thread per channel: Rice, zigzag, delta -> codes
-    if (tid < C) {
-        const unsigned k = param & 7u;
-        // the sub-stream, as big-endian words, into column tid of the interleaved area: word j of every channel sits in
-        // one row, so a warp's loads below never meet in a bank wherever each lane is in its stream
-        {
-            const uint32_t addr = smem_u32(A) + shift + my_off;
-            const uint32_t al = addr & ~3u;
-            const unsigned sh8 = (addr & 3u) * 8u;
-            // (a length no sub-stream can have means a damaged chunk: reported, and clamped so that nothing leaves the area)
-            if (my_len > td_max_len(codec)) atomicCAS(P.status, 0, kStatusRange);
-            const unsigned len_c = my_len < td_max_len(codec) ? my_len : td_max_len(codec);
-            const unsigned nw = ((len_c + 3u) >> 2) + 1u;                 // the window below looks one word past the last bit
-            uint32_t x0, x1;
-            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(x0) : "r"(al));
-            for (unsigned j = 0; j < nw; ++j) {
-                asm volatile("ld.shared.u32 %0, [%1];" : "=r"(x1) : "r"(al + 4u * (j + 1u)));
-                I[(size_t)j * C + tid] = td_be(__funnelshift_r(x0, x1, sh8));
-                x0 = x1;
-            }
+    if (*abort_flag) return;
+    TdStream x, y;
+    if (act) {
+        // the sub-streams, as complemented big-endian words, into two columns of the interleaved area (the first streams
+        // of all threads, then the second ones): word j of every channel sits in one row, so a warp's loads below never
+        // meet in a bank wherever each lane is in its stream
+        const unsigned oa = offs[ca], ob = offs[cb];
+        unsigned len_a = oa >> 24, len_b = ob >> 24;
+        // (a length no sub-stream can have means a damaged chunk: reported, and clamped so that nothing leaves the area)
+        if (len_a > td_max_len(codec) || len_b > td_max_len(codec)) atomicCAS(P.status, 0, kStatusRange);
+        len_a = len_a < td_max_len(codec) ? len_a : td_max_len(codec);
+        len_b = len_b < td_max_len(codec) ? len_b : td_max_len(codec);
+        const uint32_t addr_a = smem_u32(A) + shift + (oa & 0xffffffu), addr_b = smem_u32(A) + shift + (ob & 0xffffffu);
+        const uint32_t al_a = addr_a & ~3u, al_b = addr_b & ~3u;
+        const uint32_t sel_a = 0x0123u + (addr_a & 3u) * 0x1111u, sel_b = 0x0123u + (addr_b & 3u) * 0x1111u;   // realign and swap bytes
+        const unsigned nw = (((len_a > len_b ? len_a : len_b) + 3u) >> 2) + 1u;     // the window looks one word past the last bit
+        uint32_t a0, a1, b0, b1;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(a0) : "r"(al_a));
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(b0) : "r"(al_b));
+        uint32_t *col_a = I + tid, *col_b = I + (C >> 1) + tid;
+#pragma unroll 2
+        for (unsigned j = 0; j < nw; ++j) {
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(a1) : "r"(al_a + 4u * (j + 1u)));
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(b1) : "r"(al_b + 4u * (j + 1u)));
+            col_a[(size_t)j * C] = ~__byte_perm(a0, a1, sel_a);
+            col_b[(size_t)j * C] = ~__byte_perm(b0, b1, sel_b);
+            a0 = a1; b0 = b1;
         }
-        // 32-bit shared addresses throughout: column tid of the interleaved words, column tid of the code tile
-        const uint32_t col = smem_u32(I) + tid * 4u, row_b = C * 4u;
-        uint32_t out = smem_u32(B) + tid;
-        const unsigned k1 = k + 1u, kpow = 1u << k, krem = 32u - k;
-        const bool delta = (param & 8u) != 0u;
-        unsigned bp = 0;                                                  // bits consumed so far
-        int prev = 0;
-#pragma unroll 4
-        for (unsigned t = 0; t < s.n_tok; ++t) {
-            const unsigned wi = (bp >> 5) < kTdWords - 2u ? (bp >> 5) : kTdWords - 2u;   // a damaged stream cannot run off the area
-            const uint32_t a = col + wi * row_b;
-            uint32_t w0, w1;
-            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w0) : "r"(a));
-            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w1) : "r"(a + row_b));
-            const uint32_t hi = __funnelshift_l(w1, w0, bp);             // the next 32 bits of the stream
-            const unsigned ones = (unsigned)__clz((int)~hi);
-            // quo ones, a zero, k bits: the k bits are the top of hi << (ones + 1); a shift by 32 (k = 0) gives 0 in PTX
-            unsigned rem;
-            asm("shr.b32 %0, %1, %2;" : "=r"(rem) : "r"(hi << (ones + 1u)), "r"(krem));
-            unsigned u = ones * kpow + rem;
-            unsigned len = ones + k1;
-            if (__builtin_expect(ones >= 15u, 0)) { u = (hi << 15) >> (32u - raw_bits); len = 15u + raw_bits; }   // the escape: rare
-            bp += len;
-            int sgn;
-            asm("bfe.s32 %0, %1, 0, 1;" : "=r"(sgn) : "r"(u));           // -(u & 1)
-            int q = (int)(u >> 1) ^ sgn;
-            if (delta) q += prev;
-            prev = q;
-            asm volatile("st.shared.u8 [%0], %1;" :: "r"(out), "r"(q) : "memory");
-            out += C;
-        }
+        td_stream_init(x, smem_u32(col_a), param_a);
+        td_stream_init(y, smem_u32(col_b), param_b);
     }
-    __syncthreads();                                                      // codes complete, stream bytes no longer read
-    const unsigned n = s.n_tok * C;
-    if (kCompose && s.kv == 0u && s.op.rope >= 0) {
-        RotCoef rc;
-        rc.rope = -1; rc.col = 0xffffffffu;
-        rotate_tile<1, true>(A, B, Sc, n, (unsigned)P.D, P.rope, s.op.rope, rc, (int)tid, blockDim.x, C);
-    } else {
-        dequantise_kc_tile<false, !kCompose>(B, Sc, A, n, C, (int)tid, blockDim.x);
+    __syncthreads();                                                      // stream bytes no longer read: the rows may be written
+    const unsigned row_b = P.word_row, max_bits = (P.words - 1u) * 32u;   // a sub-stream's last symbol starts before that bit
+    const bool short_codes = codec == 6;
+    const f32x2 sc2 = pack2(sc_a, sc_b), zero2 = pack2(-kTdCodeZero, -kTdCodeZero);
+    f32x2 cc = 0ull, ss = 0ull;
+    if (rotating && act) {
+        const float2 cs = __ldg(P.rope + (size_t)s.op.rope * half + (tid - head * half));
+        cc = pack2(cs.x, cs.x);
+        ss = pack2(-cs.y, cs.y);
     }
-    fence_async_smem();
-    __syncthreads();
-    // rows -> pool blocks
-    if (tid < 32) {
-        unsigned char *base = reinterpret_cast<unsigned char *>((s.kv ? P.v_layers : P.k_layers)[s.op.l0 + (int)s.li]);
-        long long id[2] = { 0, 0 }, pos[2] = { 0, 0 };
-        unsigned row_t[2] = { tid, tid + 32u };                       // which row of the group lane k writes (64: none)
-        bool bad = false;
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            if (selecting) {
-                // the group's listed tokens, at most 64 of them: lane k takes entry first + tid + 32 k (the two indices
-                // still sit where the search left them: the scans use the words below)
-                const unsigned idx = scratch[40] + tid + 32u * (unsigned)k;
-                row_t[k] = 64u;
-                if (idx < scratch[41]) {
-                    const long long c = (long long)__ldg(s.op.list + idx) - ((long long)s.g << 6);
-                    if (c < 0 || c >= (long long)s.n_tok) bad = true;      // (a list that is not increasing)
-                    else row_t[k] = (unsigned)c;
-                }
-            } else if (row_t[k] >= s.n_tok) {
-                row_t[k] = 64u;
-            }
-            if (row_t[k] < 64u) {
-                pos[k] = group_row_pos(s.op, s.g, row_t[k]);
-                if (pos[k] < 0) { bad = true; continue; }
-                id[k] = __ldg(s.op.table + pos[k] / P.bs);
-                if (id[k] < 0 || id[k] >= P.n_blocks) bad = true;
-            }
-        }
-        if (__any_sync(0xffffffffu, bad)) {
-            if (tid == 0) atomicCAS(P.status, 0, kStatusRange);        // nothing of this slice is written
+    const uint32_t out = smem_u32(A) + ca * 2u;
+    auto put = [&](unsigned t, int acc_x, int acc_y) {
+        const f32x2 val = mul2(add2(pack2(__int_as_float(acc_x), __int_as_float(acc_y)), zero2), sc2);
+        const uint32_t o = out + t * (C * 2u);
+        if (kCompose && rotating) {
+            float u, w;
+            unpack2(val, u, w);
+            const uint32_t r = pack_bf16x2(fma2(val, cc, mul2(pack2(w, u), ss)));         // u cos - w sin, w cos + u sin
+            asm volatile("st.shared.u16 [%0], %1;" :: "r"(o), "h"((unsigned short)r) : "memory");
+            asm volatile("st.shared.u16 [%0], %1;" :: "r"(o + half * 2u), "h"((unsigned short)(r >> 16)) : "memory");
         } else {
-            if (P.n_split == 1u && s.op.list_mode == 0) {
-                if (tid == 0) {
-                    const long long first_block = (s.op.off + (long long)(s.g << 6)) / P.bs;
-                    for (unsigned t = 0; t < s.n_tok; t += (unsigned)P.bs) {
-                        const unsigned k = s.n_tok - t < (unsigned)P.bs ? s.n_tok - t : (unsigned)P.bs;
-                        const long long b = __ldg(s.op.table + first_block + t / (unsigned)P.bs);
-                        unsigned char *d = base + (unsigned long long)b * P.bs * RE * 2ull;
-                        const unsigned bytes = k * RE * 2u;
-                        for (unsigned o = 0; o < bytes; o += 32768u)
-                            bulk_s2g(d + o, smem_u32(A + (size_t)t * RE * 2u + o), bytes - o < 32768u ? bytes - o : 32768u);
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    const unsigned t = row_t[k];
-                    if (t < 64u) {
-                        const unsigned slot = (unsigned)(pos[k] % P.bs);
-                        unsigned char *d = base + (((unsigned long long)id[k] * P.bs + slot) * RE + s.c0) * 2ull;
-                        bulk_s2g(d, smem_u32(A + (size_t)t * C * 2u), C * 2u);
-                    }
-                }
-            }
-            bulk_commit();
-            bulk_wait_all();
+            asm volatile("st.shared.u32 [%0], %1;" :: "r"(o), "r"(pack_bf16x2(val)) : "memory");
         }
+    };
+    const unsigned vecs = C >> 3;                                          // 16-byte vectors per row
+#pragma unroll 1
+    for (unsigned t0 = 0; t0 < s.n_tok; t0 += kTdHalf) {
+        const unsigned nt = s.n_tok - t0 < kTdHalf ? s.n_tok - t0 : kTdHalf;
+        if (act) {
+            unsigned t = 0;
+#pragma unroll 1
+            for (; t + kTdStep <= nt; t += kTdStep) {
+                int vx[kTdStep], vy[kTdStep];
+                if (short_codes) td_step<kCols, 4>(P, x, y, row_b, max_bits, raw_bits, vx, vy);
+                else td_step<kCols, 2>(P, x, y, row_b, max_bits, raw_bits, vx, vy);
+#pragma unroll
+                for (unsigned i = 0; i < kTdStep; ++i) put(t + i, vx[i], vy[i]);
+            }
+#pragma unroll 1
+            for (; t < nt; ++t) {
+                x.bp = x.bp < max_bits ? x.bp : max_bits;
+                y.bp = y.bp < max_bits ? y.bp : max_bits;
+                td_symbol_any(P, x, td_window<kCols>(x, row_b), raw_bits);
+                td_symbol_any(P, y, td_window<kCols>(y, row_b), raw_bits);
+                put(t, x.acc, y.acc);
+            }
+        }
+        __syncthreads();
+        // rows -> pool blocks
+        for (unsigned v = tid; v < nt * vecs; v += nthreads) {
+            const unsigned t = v / vecs, c = v - t * vecs;
+            const unsigned long long d = rows[t0 + t];
+            if (d) *reinterpret_cast<uint4 *>(d + 16ull * c) = lds128(A + (size_t)v * 16u);
+        }
+        __syncthreads();
     }
 }
 

@@ -109,6 +109,42 @@ def test_store_retrieve_compose_against_the_oracle(shape, codec, rho):
         dev.close()
 
 
+@pytest.mark.parametrize("T", [1, 3, 4, 5, 31, 32, 33, 35, 36, 63, 64, 65, 97])
+@pytest.mark.parametrize("codec", [TD8, TD4], ids=["int8td", "int4td"])
+@pytest.mark.parametrize("shape", [SHAPES[0], SHAPES[3].with_(block_size=16)], ids=["slice128", "slice64"])
+def test_group_tails_and_escapes_at_every_place(shape, codec, T):
+    """The decoder takes four symbols at a time, several out of one 32-bit window, and half of a group's rows at a time:
+    lengths around those steps, channels whose escapes (rare large codes among zeros) sit at every phase of a step, and
+    channels whose code words straddle windows.  Bit-exact."""
+    bs = shape.block_size
+    rng = np.random.default_rng(1000 + T)
+    perm = rng.permutation(shape.n_blocks).astype(np.int32)
+    nb = -(-T // bs)
+    pool = make_pool_np(shape, perm[:nb], 0, nb * bs, 0.9, seed=T)
+    t = np.arange(nb * bs)
+    for c in range(8, 40):
+        x = np.zeros(nb * bs, dtype=np.float32)
+        x[(t + c) % (7 + c % 5) == 0] = 2.0 * (1 - 2 * (c & 1))              # escapes at every phase of a step
+        x[(t * 5 + c) % 11 == 0] += 0.07 * (c % 7)                           # among small codes, so that k stays small
+        pool[0, c & 1, perm[t // bs], t % bs, 0, c] = bf16_bits(x)
+    dev = Device(shape, pool_np=pool)
+    try:
+        want = oracle.store(pool, perm[:nb], 0, T, codec)
+        used = oracle.td_used_bytes(want, shape.n_layers, shape.n_kv_heads, shape.head_dim, T, codec)
+        buf = dev.chunk_buf(T, codec)
+        dev.store([dev.op(dev.table(perm[:nb]), 0, buf, T, codec)])
+        assert dev.sync() == 0
+        got = to_np(buf)
+        assert np.array_equal(got[:used], want[:used]) and np.all(got[used:] == 0xA5)
+        dev.retrieve([dev.op(dev.table(perm[nb:2 * nb]), 0, buf, T, codec)])
+        assert dev.sync() == 0
+        ref = pool.copy()
+        oracle.retrieve(ref, perm[nb:2 * nb], 0, T, codec, want)
+        assert np.array_equal(dev.pool_np(), ref)
+    finally:
+        dev.close()
+
+
 def test_mixed_batch_and_many_ops():
     """One call carrying token-delta chunks of both widths next to raw and int8 chunks, more ops than one launch holds."""
     shape = synth.TOY.with_(n_layers=2, n_kv_heads=2, head_dim=64, block_size=16, n_blocks=512)
