@@ -768,6 +768,8 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
         while ((1u << tp.split_shift) < n_split) ++tp.split_shift;
         tp.word_row = cols * 4u;
         tp.one = 1;
+        tp.fone = 1.0f;
+        for (unsigned i = 0; i < 12u; ++i) tp.pow2[i] = 1u << i;
         tp.minus_two = -2;
         tp.bs_shift = -1;
         for (int b = 0; b < 31; ++b) if (pool.bs == 1 << b) tp.bs_shift = b;
@@ -775,15 +777,16 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
         const dim3 grid((unsigned)max_groups * n_split, (unsigned)max_layers * 2u, (unsigned)m);
         int per_sm = 0;
         if (OP == OP_STORE) {
-            const size_t smem_plan = td_store_smem_bytes(cols, false), smem_enc = td_store_smem_bytes(cols, true);
+            const size_t smem_enc = td_encode_smem_bytes(cols);
             if (smem_enc > smem_limit) return KDN_E_UNSUPPORTED;
-            kdn_status r = ctx->env.resident(kdn_td_plan_kernel, (int)threads, smem_plan, &per_sm);
-            if (r == KDN_OK && per_sm >= 1) r = ctx->env.resident(kdn_td_encode_kernel, (int)threads, smem_enc, &per_sm);
+            kdn_status r = ctx->env.resident(kdn_td_encode_kernel, (int)threads, smem_enc, &per_sm);
             if (r != KDN_OK) return r;
             if (per_sm < 1) return KDN_E_UNSUPPORTED;
-            kdn_td_plan_kernel<<<grid, threads, smem_plan, stream>>>(tp);
+            const unsigned plan_threads = (cols + 31u) & ~31u;           // a warp takes 32 channels
+            if (plan_threads == 128u) kdn_td_plan_kernel<128><<<grid, 128, 0, stream>>>(tp);
+            else kdn_td_plan_kernel<512><<<grid, plan_threads, 0, stream>>>(tp);
             KDN_CUDA(cudaGetLastError());
-            kdn_td_scan_kernel<<<(unsigned)m, 256, 0, stream>>>(tp);
+            kdn_td_scan_kernel<<<(unsigned)m, kTdScanThreads, 0, stream>>>(tp);
             KDN_CUDA(cudaGetLastError());
             kdn_td_encode_kernel<<<grid, threads, smem_enc, stream>>>(tp);
             KDN_CUDA(cudaGetLastError());

@@ -5,7 +5,7 @@
 // Every (layer, K|V, 64-token group) is a SEGMENT of row_elems channels; a channel's n <= 64 codes are one
 // SUB-STREAM: zigzag of the codes (mode 0) or of their token-to-token differences (mode 1), Rice-coded with a
 // parameter k, bits filling bytes from the top.  A CTA works on one slice of `cols` channels of one segment:
-//   store    plan   (kdn_td_plan_kernel):   quantise, pick (mode, k) per channel, write scales / lens / params
+//   store    plan   (kdn_td_plan_kernel):   quantise, pick (mode, k) per channel from bit planes, write scales / lens / params
 //            scan   (kdn_td_scan_kernel):   segment sizes -> seg_off (one CTA per op)
 //            encode (kdn_td_encode_kernel): quantise again, write every sub-stream at its final place
 //   retrieve / compose (kdn_td_decode_kernel): bulk-copy the slice's bytes into shared memory; a thread undoes Rice,
@@ -55,6 +55,8 @@ struct TdLaunch {
     unsigned words;           // decode: 32-bit words kept per sub-stream (the longest of the launch's codecs, and one more)
     int bs_shift;             // log2(bs), -1 where bs is not a power of two
     int one, minus_two;       // 1 and -2 as launch parameters: see TdStream
+    float fone;               // 1.0f (see Launch::one)
+    unsigned pow2[12];        // 1 << i: multiply-adds by these stay on the multiplier's pipe (as literals they become shifts)
     unsigned word_row;        // decode: bytes of one row of interleaved words (4 * cols), for the same reason
     const float2 *rope;
     int *status;
@@ -63,19 +65,14 @@ struct TdLaunch {
     DevOp inline_ops[kInlineOps];
 };
 
-// Shared memory of the store kernels: token rows, slice maxima, reciprocals, the stream staging area (encode only),
-// small per-warp scratch, barrier.
-// (the plan kernel keeps two tables of code-word lengths in place of the staging area, each replicated so that the
-// lanes of a warp never meet in a bank: 64 entries x 32 copies x 4 bytes and 64 entries x 16 copies x 8 bytes)
+// Shared memory of the encoder: token rows, slice maxima, reciprocals, the stream staging area, small per-warp scratch, barrier.
 // Behind the encoder's staging area: room for the longest thing a channel could write from the last planned byte on (64
 // symbols of 24 bits), so that a sub-stream that came out longer than planned -- the pool changed under the store --
 // garbles the chunk's bytes, which the caller has then forfeited, but never leaves the area.
 constexpr unsigned kTdStageSlack = 256u;
-constexpr unsigned kTdCostBytes = 64u * 32u * 4u + 64u * 16u * 8u + 64u * 4u + 64u * 8u;   // the copies, and one set of entries to copy from
-__host__ __device__ inline size_t td_store_smem_bytes(unsigned cols, bool encode)
+__host__ __device__ inline size_t td_encode_smem_bytes(unsigned cols)
 {
-    return (size_t)64 * cols * 2u + (size_t)kKcSlices * cols * 2u + (size_t)cols * 4u +
-           (encode ? (size_t)cols * 72u + 32u + kTdStageSlack : (size_t)kTdCostBytes) + 256u + 16u;
+    return (size_t)64 * cols * 2u + (size_t)kKcSlices * cols * 2u + (size_t)cols * 4u + (size_t)cols * 72u + 32u + kTdStageSlack + 256u + 16u;
 }
 // Shared memory of the decode kernel: the sub-streams interleaved word by word (so that the 32 lanes of a warp, each
 // somewhere else in its stream, read 32 different banks), half of the group's bf16 rows, the sub-streams' offsets, the
@@ -95,12 +92,6 @@ __host__ __device__ inline size_t td_decode_smem_bytes(unsigned cols, unsigned w
     return td_decode_words_bytes(cols, words) + td_decode_rows_bytes(cols, words) + (size_t)cols * 4u + 64u * 8u + 256u + 16u;
 }
 
-// Bits of one Rice code word.
-__device__ __forceinline__ unsigned td_cost(unsigned u, unsigned k, unsigned esc_bits)
-{
-    const unsigned quo = u >> k;
-    return quo < 15u ? quo + 1u + k : esc_bits;
-}
 __device__ __forceinline__ unsigned td_zigzag(int e) { return ((unsigned)e << 1) ^ (unsigned)(e >> 31); }   // 2e, or -2e - 1 for e < 0
 
 // Big-endian view of a little-endian word: the stream's first byte in the top bits.
@@ -268,181 +259,304 @@ __device__ __forceinline__ TdSlice td_slice(const TdLaunch &P)
     return s;
 }
 
+// Pool addresses of the slice in the token rows of the group, row t at rows[t + t / 32] (0 for rows past the chunk's end).  All
+// threads of the block call this; true when one of the thread's rows lies outside the pool or the table.
+__device__ __forceinline__ bool td_row_addresses(const TdLaunch &P, const TdSlice &s, unsigned long long *rows)
+{
+    const unsigned char *base = reinterpret_cast<const unsigned char *>((s.kv ? P.v_layers : P.k_layers)[s.op.l0 + (int)s.li]);
+    bool bad = false;
+    for (unsigned t = threadIdx.x; t < 64u; t += blockDim.x) {
+        unsigned long long a = 0ull;
+        if (t < s.n_tok) {
+            const long long pos = group_row_pos(s.op, s.g, t);
+            long long id = -1;
+            const long long blk = P.bs_shift >= 0 ? pos >> P.bs_shift : pos / P.bs;
+            if (pos >= 0) id = __ldg(s.op.table + blk);
+            if (id < 0 || id >= P.n_blocks) bad = true;
+            else a = (unsigned long long)(base + ((unsigned long long)(id * P.bs + (pos - blk * P.bs)) * P.row_elems + s.c0) * 2ull);
+        }
+        rows[t + (t >> 5)] = a;
+    }
+    return bad;
+}
+
 // ------------------------------------------------------------------------------------------ store: plan --
 
-__global__ void __launch_bounds__(512) kdn_td_plan_kernel(const __grid_constant__ TdLaunch P)
+// The planner works on bit planes: plane i of a channel's 32 tokens is one 32-bit word, bit t of it bit i of token t's
+// code, so one logic operation handles 32 symbols and counting is popc.
+//
+// From codes to planes.  A thread holds two neighbouring channels of 32 tokens; their codes, biased to be positive, are
+// gathered in the floating-point pipe (see gather2), a word of four tokens t, t + 8, t + 16, t + 24 (8-bit codes) or of eight
+// tokens t, t + 4, .. (4-bit codes).  Transposing 8 x 8 (4 x 4) bits inside every byte (nibble) lane across the eight (four)
+// words then leaves the planes in the tokens' own order.
+template <int kN> __device__ __forceinline__ void td_transpose(const TdLaunch &P, uint32_t (&w)[kN])
 {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    const TdSlice s = td_slice(P);
-    if (!s.valid) return;
-    const unsigned C = P.cols, RE = P.row_elems;
-    const int codec = s.op.codec;
-    const float qmax = (float)td_qmax(codec);
-    const unsigned esc_bits = 15u + (unsigned)td_raw_bits(codec);
+#pragma unroll
+    for (int d = kN / 2; d >= 1; d >>= 1) {
+        const uint32_t m = d == 4 ? 0x0f0f0f0fu : d == 2 ? 0x33333333u : 0x55555555u;
+#pragma unroll
+        for (int j = 0; j < kN; ++j) {
+            if (j & d) continue;
+            const uint32_t a = w[j], b = w[j + d];
+            w[j] = (a & m) | ((b * P.pow2[d]) & ~m);
+            w[j + d] = ((a >> d) & m) | (b & ~m);
+        }
+    }
+}
 
-    unsigned char *X = smem_raw;
-    unsigned char *pmax = X + (size_t)64 * C * 2u;
-    float *inv = reinterpret_cast<float *>(pmax + (size_t)kKcSlices * C * 2u);
-    // code-word lengths as 8-bit fields.  lo[min(u, 60)][lane]: k = 0, 1, 2 (from u = 60 on all three are the escape);
-    // hi[u >> 3][lane / 2]: k = 3 .. 7 (their quotients are functions of u >> 3).  One copy per lane / pair of lanes.
-    uint32_t *lo_tab = reinterpret_cast<uint32_t *>(reinterpret_cast<unsigned char *>(inv) + (size_t)C * 4u);
-    uint2 *hi_tab = reinterpret_cast<uint2 *>(lo_tab + 64u * 32u);
-    unsigned long long *bar_mem = reinterpret_cast<unsigned long long *>(reinterpret_cast<unsigned char *>(lo_tab) + (size_t)kTdCostBytes + 256u);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(bar_mem + 1);
-    const uint32_t bar = smem_u32(bar_mem);
-    const unsigned tid = threadIdx.x;
-    if (tid == 0) {
-        mbar_init(bar, 1u);
-        *abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        fence_async_smem();
-    }
-    __syncthreads();
-    if (tid < 32) {
-        const unsigned char *base = reinterpret_cast<const unsigned char *>((s.kv ? P.v_layers : P.k_layers)[s.op.l0 + (int)s.li]);
-        if (!td_load_slice(X, bar, base, s.op, s.g, s.n_tok, P.bs, P.n_blocks, RE, C, s.c0,
-                           P.n_split == 1u, P.status) && tid == 0)
-            *abort_flag = 1;
-    }
-    // while the rows are on their way: fill the tables -- every entry is worked out once, then copied
-    {
-        uint32_t *lo_one = reinterpret_cast<uint32_t *>(hi_tab + 64u * 16u);
-        uint2 *hi_one = reinterpret_cast<uint2 *>(lo_one + 64u);
-        for (unsigned i = tid; i < 128u; i += blockDim.x) {
-            if (i < 64u) {
-                lo_one[i] = td_cost(i, 0u, esc_bits) | (td_cost(i, 1u, esc_bits) << 8) | (td_cost(i, 2u, esc_bits) << 16);
+// `sum` plus the sum over 64 symbols of what a code word takes beyond its k + 1 bits, times 16: min(u >> k, ...) for the unary part, or
+// kEsc - 1 - k for an escape (u >> k >= 15).  lo and hi are the planes of u for tokens 0-31 and 32-63; the two halves' numbers are added
+// plane by plane first, which leaves one count per plane of the sum: popc runs at an eighth of the rate of the logic.
+template <int kPlanes, int kMax, int kEsc, int kK>
+__device__ __forceinline__ unsigned td_plan_sum(const TdLaunch &P, unsigned sum, const uint32_t (&lo)[kPlanes], const uint32_t (&hi)[kPlanes])
+{
+    constexpr bool kEscapes = (kMax >> kK) >= 15;
+    constexpr int kBits = kEscapes ? 5 : kPlanes - kK;
+    if constexpr (kBits <= 0) {
+        return sum;
+    } else {
+        uint32_t x[2][kBits];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t (&b)[kPlanes] = h ? hi : lo;
+            if constexpr (kEscapes) {
+                constexpr int v = kEsc - 1 - kK;
+                static_assert(v >= 16 && v < 32, "the planes of an escape's cost");
+                uint32_t over = 0u;                          // bits above the four that a short quotient has
+#pragma unroll
+                for (int i = kK + 4; i < kPlanes; ++i) over |= b[i];
+                const uint32_t esc = (b[kK] & b[kK + 1] & b[kK + 2] & b[kK + 3]) | over;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) x[h][i] = ((v >> i) & 1) ? b[kK + i] | esc : b[kK + i] & ~esc;
+                x[h][4] = esc;
             } else {
-                const unsigned u = (i - 64u) << 3;
-                hi_one[i - 64u] = make_uint2(td_cost(u, 3u, esc_bits) | (td_cost(u, 4u, esc_bits) << 8) | (td_cost(u, 5u, esc_bits) << 16) |
-                                             (td_cost(u, 6u, esc_bits) << 24), td_cost(u, 7u, esc_bits));
+#pragma unroll
+                for (int i = 0; i < kBits; ++i) x[h][i] = b[kK + i];
             }
         }
-        __syncthreads();
-        for (unsigned i = tid; i < 64u * 32u; i += blockDim.x) lo_tab[i] = lo_one[i >> 5];
-        for (unsigned i = tid; i < 64u * 16u; i += blockDim.x) hi_tab[i] = hi_one[i >> 4];
+        uint32_t carry = 0u;
+#pragma unroll
+        for (int i = 0; i < kBits; ++i) {
+            const uint32_t p = x[0][i], q = x[1][i];
+            sum += (unsigned)__popc(p ^ q ^ carry) * P.pow2[4 + i];
+            carry = (p & q) | (carry & (p | q));
+        }
+        return sum + (unsigned)__popc(carry) * P.pow2[4 + kBits];
     }
-    __syncthreads();
-    const TdLayout lay = td_layout(P.L, RE, s.op.T, codec);
+}
+// The smallest (bits * 16 + mode * 8 + k) over the parameters of one mode, and `best`, for n symbols.  From the large k down, and no
+// further than can pay: a code word of a smaller k takes at least 1 + 2 (u >> k) bits, or kEsc, so with V the sum that
+// td_plan_sum adds up at k every smaller k needs n + V * 34 / 32 bits or more (an escape counts kEsc - 1 - k <= 21 in V where k >= 2).
+// Where all of a warp's channels have something better already, the rest is left out: on uncorrelated input k = 0 .. 2, a fifth
+// of the logic.
+template <int kMode, int kPlanes, int kMax, int kEsc>
+__device__ __forceinline__ unsigned td_plan_mode(const TdLaunch &P, unsigned best, const uint32_t (&lo)[kPlanes], const uint32_t (&hi)[kPlanes],
+                                                 unsigned n, bool act)
+{
+    const unsigned n16 = n * 16u;
+    unsigned v;
+#define KDN_TD_K(K)                                                                          \
+    v = td_plan_sum<kPlanes, kMax, kEsc, K>(P, 0u, lo, hi);                                  \
+    best = min(best, v + n16 * (K + 1u) + (kMode * 8u + K));
+#define KDN_TD_ENOUGH (!__any_sync(0xffffffffu, act && n16 + v + (v >> 4) <= best + 15u))
+    KDN_TD_K(7) KDN_TD_K(6) KDN_TD_K(5) KDN_TD_K(4) KDN_TD_K(3)
+    if (kMax > 128 && KDN_TD_ENOUGH) return best;
+    KDN_TD_K(2)
+    if (kMax > 128 && KDN_TD_ENOUGH) return best;
+    KDN_TD_K(1) KDN_TD_K(0)
+#undef KDN_TD_ENOUGH
+#undef KDN_TD_K
+    return best;
+}
+
+// Two channels of 32 tokens (x: bf16 pairs) -> bits * 16 + parameters of the one channel this thread answers for (lane 16 + l
+// has tokens 32-63 of the channels lane l has 0-31 of; lane l answers for the first of the two).  n: tokens of the group.
+// kFull: n = 64, known when the code is made.
+template <bool kInt4, bool kFull>
+__device__ __forceinline__ unsigned td_plan_channel(const TdLaunch &P, const uint32_t (&x)[32], float inv_a, float inv_b, unsigned n, bool act)
+{
+    constexpr int kW = kInt4 ? 4 : 8;                       // words per channel before, planes after transposing
+    const f32x2 inv2 = pack2(inv_a, inv_b), one2 = pack2(P.fone, P.fone);
+    const float magic = 12582912.0f + (kInt4 ? 8.0f : 128.0f);
+    const f32x2 magic2 = pack2(magic, magic), minus_m2 = pack2(-12582912.0f, -12582912.0f);
+    auto code = [&](int t) { return add2_unfused(mul2(bf16x2_widen(x[t]), inv2), magic2, one2); };      // 1.5 * 2^23 + bias + code
+    uint32_t wa[kW], wb[kW];
+#pragma unroll
+    for (int j = 0; j < kW; ++j) {
+        f32x2 g[2];
+        if (kInt4) {
+            const f32x2 k16 = pack2(16.0f, 16.0f), k256 = pack2(256.0f, 256.0f), k4096 = pack2(4096.0f, 4096.0f);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                g[h] = gather2(code(j + 16 * h), code(j + 16 * h + 4), minus_m2, k16);
+                g[h] = gather2(g[h], code(j + 16 * h + 8), minus_m2, k256);
+                g[h] = gather2(g[h], code(j + 16 * h + 12), minus_m2, k4096);
+            }
+        } else {
+            const f32x2 k256 = pack2(256.0f, 256.0f);
+            g[0] = gather2(code(j), code(j + 8), minus_m2, k256);
+            g[1] = gather2(code(j + 16), code(j + 24), minus_m2, k256);
+        }
+        uint32_t a0, b0, a1, b1;
+        unpack2_bits(g[0], a0, b0);
+        unpack2_bits(g[1], a1, b1);
+        wa[j] = __byte_perm(a0, a1, 0x5410);
+        wb[j] = __byte_perm(b0, b1, 0x5410);
+    }
+    td_transpose<kW>(P, wa);
+    td_transpose<kW>(P, wb);
+    // each of the two lanes that share a pair of channels takes one of them over whole
+    const bool upper = (threadIdx.x & 16u) != 0u;
+    uint32_t lo[kW], hi[kW];
+#pragma unroll
+    for (int i = 0; i < kW; ++i) {
+        const uint32_t got = __shfl_xor_sync(0xffffffffu, upper ? wa[i] : wb[i], 16);
+        lo[i] = upper ? got : wa[i];
+        hi[i] = upper ? wb[i] : got;
+    }
+    // mode 0: the biased code's top plane is the complement of the sign; u = 2 q or 2 ~q + 1
+    unsigned best;
+    {
+        uint32_t ul[kW], uh[kW];
+        ul[0] = ~lo[kW - 1]; uh[0] = ~hi[kW - 1];
+#pragma unroll
+        for (int i = 1; i < kW; ++i) { ul[i] = lo[i - 1] ^ ul[0]; uh[i] = hi[i - 1] ^ uh[0]; }
+        best = td_plan_mode<0, kW, kInt4 ? 14 : 254, kInt4 ? 20 : 24>(P, 0xffffffffu, ul, uh, n, act);
+    }
+    // mode 1: e = code - code of the token before (the bias falls out; before the first token stands the bias itself)
+    {
+        uint32_t dl[kW + 1], dh[kW + 1];
+        const uint32_t vl = n >= 32u ? 0xffffffffu : (1u << n) - 1u, vh = n >= 64u ? 0xffffffffu : n > 32u ? (1u << (n - 32u)) - 1u : 0u;
+        uint32_t bl = 0u, bh = 0u;                           // borrows
+#pragma unroll
+        for (int i = 0; i < kW; ++i) {
+            uint32_t pl = lo[i] * P.pow2[1] + (i == kW - 1 ? 1u : 0u), ph = __funnelshift_l(lo[i], hi[i], 1);
+            if (!kFull) {                                   // tokens that are not there: no difference
+                pl = (pl & vl) | (lo[i] & ~vl);
+                ph = (ph & vh) | (hi[i] & ~vh);
+            }
+            dl[i + 1] = lo[i] ^ pl ^ bl;
+            dh[i + 1] = hi[i] ^ ph ^ bh;
+            bl = (~lo[i] & pl) | (bl & (~lo[i] | pl));
+            bh = (~hi[i] & ph) | (bh & (~hi[i] | ph));
+        }
+        dl[0] = bl; dh[0] = bh;                              // the last borrow is the sign
+#pragma unroll
+        for (int i = 1; i <= kW; ++i) { dl[i] ^= bl; dh[i] ^= bh; }
+        best = td_plan_mode<1, kW + 1, kInt4 ? 28 : 508, kInt4 ? 20 : 24>(P, best, dl, dh, n, act);
+    }
+    return best;
+}
+
+// A warp takes 32 channels: lanes l and l + 16 hold the same two channels, tokens 0-31 and 32-63, straight from the pool in
+// registers (no shared tile: every value is used once, and a thread has 32 loads in flight).  Bound by the pipe of logic and shifts
+// (two thirds busy).  8B shape, 16 chunks of 512 tokens, 8-bit codes: 1100 us with a table of code-word lengths looked up per
+// symbol, 345 us this way; 4-bit codes 1080 -> 230 us.  Seven CTAs of 128 threads an SM (72 registers): 345 us, eight 365.
+// kThreads: 128 is the usual slice of 128 channels, 512 stands for any other.
+template <unsigned kThreads>
+__global__ void __launch_bounds__(kThreads, kThreads == 128u ? 7 : 1) kdn_td_plan_kernel(const __grid_constant__ TdLaunch P)
+{
+    __shared__ unsigned long long rows[66];                 // pool addresses of the group's token rows (0: past the chunk's end), ...
+    __shared__ unsigned warp_bytes[16];                     // ... row t at index t + t / 32: the two that a warp reads at once in different banks
+    const TdSlice s = td_slice(P);
+    if (!s.valid) return;
+    const unsigned C = P.cols, RE = P.row_elems, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const int codec = s.op.codec;
+    const TdLayout &lay = P.layout[blockIdx.z];
     const unsigned long long row = (unsigned long long)s.seg * RE + s.c0;
-    // a slice that is given up (a block id outside the pool, a wait that ran out) leaves lengths of zero behind: the scan
-    // and the encoder then see a consistent, if incomplete, chunk instead of whatever the buffer held before
-    auto give_up = [&]() {
-        for (unsigned ch = tid; ch < C; ch += blockDim.x) {
+    const bool bad = td_row_addresses(P, s, rows);
+    const unsigned half = lane >> 4, pair = warp * 16u + (lane & 15u), ch = 2u * pair + half;      // ch: the channel the thread answers for
+    const bool act = 2u * pair < C;                         // (C is a multiple of 16)
+    unsigned *slice_bytes = reinterpret_cast<unsigned *>(s.op.data + lay.streams) + (size_t)s.seg * P.n_split + s.part;
+    if (__syncthreads_or(bad)) {
+        // a slice that is given up leaves lengths of zero behind: the scan and the encoder then see a consistent, if
+        // incomplete, chunk instead of whatever the buffer held before
+        if (act) {
             s.op.data[lay.lens + row + ch] = 0;
             s.op.data[lay.params + row + ch] = 0;
         }
-    };
-    if (*abort_flag) { give_up(); return; }
-    const bool landed = mbar_wait(bar, 0u, abort_flag, P.wait_limit_ns);
-    if (!__syncthreads_and(landed)) {
         if (tid == 0) {
-            atomicCAS(P.status, 0, kStatusTimeout);
-            const unsigned long long t0 = global_timer_ns();
-            while (!mbar_try_wait(bar, 0u))
-                if (global_timer_ns() - t0 > kWaitLimitNs) break;
+            atomicCAS(P.status, 0, kStatusRange);
+            *slice_bytes = 0u;
         }
-        give_up();
         return;
     }
-    td_channel_scales(X, pmax, inv, reinterpret_cast<float *>(s.op.data + lay.scales) + row, s.n_tok, C, qmax);
-    // one thread per channel: the cost in bits of every (mode, k), then the first minimum.  Lengths are at most 24, so
-    // the 8-bit fields hold eight symbols' worth; after every eight symbols they are spread into 16-bit fields.
-    for (unsigned ch = tid; ch < C; ch += blockDim.x) {
-        const float iv = inv[ch];
-        const uint32_t *lo_l = lo_tab + (tid & 31u);
-        const uint2 *hi_l = hi_tab + ((tid & 31u) >> 1);
-        unsigned w02[2] = { 0u, 0u }, w1[2] = { 0u, 0u }, w35[2] = { 0u, 0u }, w46[2] = { 0u, 0u }, w7[2] = { 0u, 0u };
-        int prev = 0;
-        unsigned al[2], ah[2];
-        auto symbol = [&](unsigned t) {
-            const int q = td_code(*reinterpret_cast<const unsigned short *>(X + ((size_t)t * C + ch) * 2u), iv);
-            const unsigned u[2] = { td_zigzag(q), td_zigzag(q - prev) };        // at most 4 * 127 < 512
-            prev = q;
+    uint32_t x[32];
+    const unsigned long long *my_rows = rows + 33u * half;
+    const bool full = s.n_tok == 64u;
+    const unsigned n_mine = !act ? 0u : s.n_tok < 32u * half ? 0u : s.n_tok - 32u * half;
+    if (full && act) {
 #pragma unroll
-            for (int m = 0; m < 2; ++m) {
-                al[m] += lo_l[(u[m] < 60u ? u[m] : 60u) << 5];
-                const uint2 h = hi_l[(u[m] >> 3) << 4];
-                ah[m] += h.x;
-                w7[m] += h.y;
-            }
-        };
-        auto widen = [&]() {
+        for (int t = 0; t < 32; ++t) x[t] = __ldg(reinterpret_cast<const uint32_t *>(my_rows[t] + (unsigned long long)(2u * pair) * P.pow2[1]));
+    } else {
 #pragma unroll
-            for (int m = 0; m < 2; ++m) {
-                w02[m] += al[m] & 0x00ff00ffu; w1[m] += (al[m] >> 8) & 0x00ff00ffu;
-                w35[m] += ah[m] & 0x00ff00ffu; w46[m] += (ah[m] >> 8) & 0x00ff00ffu;
-            }
-        };
-        if (s.n_tok == 64u) {                                   // a full group: fixed trip counts, eight symbols unrolled
-#pragma unroll 1
-            for (unsigned t0 = 0; t0 < 64u; t0 += 8u) {
-                al[0] = al[1] = ah[0] = ah[1] = 0u;
+        for (int t = 0; t < 32; ++t) x[t] = (unsigned)t < n_mine ? __ldg(reinterpret_cast<const uint32_t *>(my_rows[t]) + pair) : 0u;
+    }
+    uint32_t m0 = maxabs_bf16x2(x[0], x[1]), m1 = maxabs_bf16x2(x[2], x[3]);
 #pragma unroll
-                for (unsigned k = 0; k < 8u; ++k) symbol(t0 + k);
-                widen();
-            }
-        } else {
-            for (unsigned t0 = 0; t0 < s.n_tok; t0 += 8u) {
-                al[0] = al[1] = ah[0] = ah[1] = 0u;
-                const unsigned t1 = t0 + 8u < s.n_tok ? t0 + 8u : s.n_tok;
-                for (unsigned t = t0; t < t1; ++t) symbol(t);
-                widen();
-            }
-        }
-        const unsigned b0[8] = { w02[0] & 0xffffu, w1[0] & 0xffffu, w02[0] >> 16, w35[0] & 0xffffu, w46[0] & 0xffffu, w35[0] >> 16, w46[0] >> 16, w7[0] };
-        const unsigned b1[8] = { w02[1] & 0xffffu, w1[1] & 0xffffu, w02[1] >> 16, w35[1] & 0xffffu, w46[1] & 0xffffu, w35[1] >> 16, w46[1] >> 16, w7[1] };
-        unsigned best = b0[0], param = 0u;
-#pragma unroll
-        for (int k = 1; k < 8; ++k) if (b0[k] < best) { best = b0[k]; param = (unsigned)k; }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) if (b1[k] < best) { best = b1[k]; param = 8u + (unsigned)k; }
-        s.op.data[lay.lens + row + ch] = (unsigned char)((best + 7u) >> 3);
-        s.op.data[lay.params + row + ch] = (unsigned char)param;
+    for (int t = 4; t < 32; t += 2) { m0 = maxabs_bf16x2(m0, x[t]); m1 = maxabs_bf16x2(m1, x[t + 1]); }
+    m0 = maxabs_bf16x2(m0, m1);
+    m0 = maxabs_bf16x2(m0, __shfl_xor_sync(0xffffffffu, m0, 16));
+    // scale and reciprocal of the thread's own channel, the other channel's reciprocal from its partner
+    const float qmax = (float)td_qmax(codec);
+    const float a = __uint_as_float(half ? m0 & 0x7fff0000u : (m0 & 0x7fffu) << 16);
+    const float sc = __fdiv_rn(a, qmax);
+    const bool ok = sc >= 1.17549435e-38f;                  // smallest normal fp32; false for NaN too
+    const float inv = ok ? __fdiv_rn(qmax, a) : 0.0f;
+    const float other = __shfl_xor_sync(0xffffffffu, inv, 16);
+    const float inv_a = half ? other : inv, inv_b = half ? inv : other;
+    unsigned best;
+    if (codec == 5) best = full ? td_plan_channel<false, true>(P, x, inv_a, inv_b, 64u, act) : td_plan_channel<false, false>(P, x, inv_a, inv_b, s.n_tok, act);
+    else best = full ? td_plan_channel<true, true>(P, x, inv_a, inv_b, 64u, act) : td_plan_channel<true, false>(P, x, inv_a, inv_b, s.n_tok, act);
+    const unsigned len = act ? (best + 7u * 16u) >> 7 : 0u;                   // bytes of the sub-stream
+    if (act) {
+        reinterpret_cast<float *>(s.op.data + lay.scales)[row + ch] = ok ? sc : 0.0f;
+        s.op.data[lay.lens + row + ch] = (unsigned char)len;
+        s.op.data[lay.params + row + ch] = (unsigned char)(best & 15u);
+    }
+    // The slice's bytes are left for the scan at the start of the streams, four bytes a slice: the encoder overwrites them, as
+    // every sub-stream takes at least a byte.
+    const unsigned sum = __reduce_add_sync(0xffffffffu, len);
+    if (lane == 0) warp_bytes[warp] = sum;
+    __syncthreads();
+    if (tid == 0) {
+        unsigned total = 0;
+        for (unsigned w = 0; w < (blockDim.x >> 5); ++w) total += warp_bytes[w];
+        *slice_bytes = total;
     }
 }
 
 // ------------------------------------------------------------------------------------------ store: scan --
 
-// One CTA per op: seg_off[s + 1] = seg_off[s] + the segment's sub-stream bytes rounded up to 16.
-__global__ void __launch_bounds__(256) kdn_td_scan_kernel(const __grid_constant__ TdLaunch P)
+// One CTA per op: seg_off[s + 1] = seg_off[s] + the segment's sub-stream bytes rounded up to 16, 1024 segments at a time.
+// Latency is all that counts here: 512 tokens at the 8B shape took 58 us when the lengths were added up here, and take 5 now
+// that the planner leaves one sum per slice.
+constexpr unsigned kTdScanThreads = 1024;
+__global__ void __launch_bounds__(kTdScanThreads) kdn_td_scan_kernel(const __grid_constant__ TdLaunch P)
 {
-    __shared__ unsigned long long part[256];
+    __shared__ unsigned scratch[33];
     const DevOp op = P.inline_ops[blockIdx.x];
     if (op.codec < 5 || op.T <= 0) return;
-    const unsigned RE = P.row_elems;
-    const TdLayout lay = td_layout(P.L, RE, op.T, op.codec);
+    const TdLayout &lay = P.layout[blockIdx.x];
     unsigned long long *seg_off = reinterpret_cast<unsigned long long *>(op.data);
-    const unsigned char *lens = op.data + lay.lens;
-    const unsigned tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    // phase 1: one warp per segment sums its row of lengths
-    for (unsigned long long sidx = warp; sidx < lay.S; sidx += 8u) {
-        const uint32_t *rowp = reinterpret_cast<const uint32_t *>(lens + sidx * RE);     // RE is a multiple of 64
-        unsigned sum = 0;
-        for (unsigned w = lane; w < (RE >> 2); w += 32u) {
-            const uint32_t v = rowp[w];
-            sum += (v & 0xffu) + ((v >> 8) & 0xffu) + ((v >> 16) & 0xffu) + (v >> 24);
-        }
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
-        if (lane == 0) seg_off[sidx + 1ull] = ((unsigned long long)sum + 15ull) & ~15ull;
-    }
-    __syncthreads();
-    // phase 2: running sum over the S sizes, each thread a contiguous range
-    const unsigned long long per = (lay.S + 255ull) / 256ull;
-    const unsigned long long a = (unsigned long long)tid * per, b = a + per < lay.S ? a + per : lay.S;
-    unsigned long long local = 0;
-    for (unsigned long long i = a; i < b; ++i) local += seg_off[i + 1ull];
-    part[tid] = local;
-    __syncthreads();
+    const unsigned *slice_bytes = reinterpret_cast<const unsigned *>(op.data + lay.streams);
+    const unsigned tid = threadIdx.x;
+    unsigned long long run = lay.streams;
     if (tid == 0) {
-        unsigned long long run = lay.streams;
-        for (int i = 0; i < 256; ++i) { const unsigned long long v = part[i]; part[i] = run; run += v; }
-        seg_off[0] = lay.streams;
+        seg_off[0] = run;
         if ((lay.S + 1ull) & 1ull) seg_off[lay.S + 1ull] = 0ull;             // the table is padded to 16 bytes with zeros
     }
-    __syncthreads();
-    unsigned long long run = part[tid];
-    for (unsigned long long i = a; i < b; ++i) { run += seg_off[i + 1ull]; seg_off[i + 1ull] = run; }
+    for (unsigned long long base = 0; base < lay.S; base += kTdScanThreads) {
+        const unsigned long long sidx = base + tid;
+        unsigned size = 0;
+        if (sidx < lay.S)
+            for (unsigned p = 0; p < P.n_split; ++p) size += slice_bytes[sidx * P.n_split + p];
+        size = (size + 15u) & ~15u;
+        unsigned total;
+        const unsigned before = td_block_scan(size, scratch, &total);
+        if (sidx < lay.S) seg_off[sidx + 1ull] = run + before + size;
+        run += total;
+    }
 }
 
 // ---------------------------------------------------------------------------------------- store: encode --
