@@ -728,10 +728,7 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
     unsigned n_split = 1;
     while (row_elems / n_split > kTdCols && row_elems % (n_split * 2u) == 0u && (row_elems / (n_split * 2u)) % unit == 0u) n_split *= 2u;
     const unsigned cols = row_elems / n_split;
-    if (cols % 16u || cols > 1024u) return KDN_E_UNSUPPORTED;
-    unsigned threads = (cols + 31u) & ~31u;                  // one thread per channel in the coding loops
-    if (threads < 64u) threads = 64u;
-    if (threads > 512u) return KDN_E_UNSUPPORTED;
+    if (cols % 16u || cols > 512u) return KDN_E_UNSUPPORTED;
     const size_t smem_limit = (size_t)ctx->env.smem_optin;
 
     for (int first = 0; first < n; first += kInlineOps) {
@@ -777,9 +774,11 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
         const dim3 grid((unsigned)max_groups * n_split, (unsigned)max_layers * 2u, (unsigned)m);
         int per_sm = 0;
         if (OP == OP_STORE) {
-            const size_t smem_enc = td_encode_smem_bytes(cols);
+            const size_t smem_enc = td_encode_smem_bytes(cols, tp.words);
             if (smem_enc > smem_limit) return KDN_E_UNSUPPORTED;
-            kdn_status r = ctx->env.resident(kdn_td_encode_kernel, (int)threads, smem_enc, &per_sm);
+            const unsigned enc_threads = (cols / 2u + 31u) & ~31u;       // a thread codes two channels
+            kdn_status r = cols == kTdCols ? ctx->env.resident(kdn_td_encode_kernel<kTdCols>, (int)enc_threads, smem_enc, &per_sm)
+                                           : ctx->env.resident(kdn_td_encode_kernel<0>, (int)enc_threads, smem_enc, &per_sm);
             if (r != KDN_OK) return r;
             if (per_sm < 1) return KDN_E_UNSUPPORTED;
             const unsigned plan_threads = (cols + 31u) & ~31u;           // a warp takes 32 channels
@@ -788,7 +787,8 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
             KDN_CUDA(cudaGetLastError());
             kdn_td_scan_kernel<<<(unsigned)m, kTdScanThreads, 0, stream>>>(tp);
             KDN_CUDA(cudaGetLastError());
-            kdn_td_encode_kernel<<<grid, threads, smem_enc, stream>>>(tp);
+            if (cols == kTdCols) kdn_td_encode_kernel<kTdCols><<<grid, enc_threads, smem_enc, stream>>>(tp);
+            else kdn_td_encode_kernel<0><<<grid, enc_threads, smem_enc, stream>>>(tp);
             KDN_CUDA(cudaGetLastError());
             ctx->launches += 3;
         } else {

@@ -65,15 +65,12 @@ struct TdLaunch {
     DevOp inline_ops[kInlineOps];
 };
 
-// Shared memory of the encoder: token rows, slice maxima, reciprocals, the stream staging area, small per-warp scratch, barrier.
+// Shared memory of the encoder: the rows' addresses, a little scratch, the stream staging area.
 // Behind the encoder's staging area: room for the longest thing a channel could write from the last planned byte on (64
-// symbols of 24 bits), so that a sub-stream that came out longer than planned -- the pool changed under the store --
+// appends, a word each, and the last word), so that a sub-stream that came out longer than planned -- the pool changed under the store --
 // garbles the chunk's bytes, which the caller has then forfeited, but never leaves the area.
-constexpr unsigned kTdStageSlack = 256u;
-__host__ __device__ inline size_t td_encode_smem_bytes(unsigned cols)
-{
-    return (size_t)64 * cols * 2u + (size_t)kKcSlices * cols * 2u + (size_t)cols * 4u + (size_t)cols * 72u + 32u + kTdStageSlack + 256u + 16u;
-}
+constexpr unsigned kTdStageSlack = 288u;
+constexpr unsigned kTdEncodeHead = 66u * 8u + 32u * 4u + 112u;      // a multiple of 128
 // Shared memory of the decode kernel: the sub-streams interleaved word by word (so that the 32 lanes of a warp, each
 // somewhere else in its stream, read 32 different banks), half of the group's bf16 rows, the sub-streams' offsets, the
 // rows' addresses.  The slice's stream bytes as they lie in the chunk share the rows' place: they are interleaved before
@@ -81,6 +78,10 @@ __host__ __device__ inline size_t td_encode_smem_bytes(unsigned cols)
 // then still inside the CTA's memory, and garbage either way.
 constexpr unsigned kTdHalf = 32;                            // rows between two write-outs
 __host__ __device__ inline unsigned td_words(int codec) { return td_max_len(codec) / 4u + 1u; }   // the longest sub-stream, and the word after
+__host__ __device__ inline size_t td_encode_smem_bytes(unsigned cols, unsigned words)
+{
+    return kTdEncodeHead + (size_t)cols * (words - 1u) * 4u + 32u + kTdStageSlack;
+}
 __host__ __device__ inline size_t td_decode_words_bytes(unsigned cols, unsigned words) { return (size_t)words * cols * 4u; }
 __host__ __device__ inline size_t td_decode_rows_bytes(unsigned cols, unsigned words)
 {
@@ -92,17 +93,8 @@ __host__ __device__ inline size_t td_decode_smem_bytes(unsigned cols, unsigned w
     return td_decode_words_bytes(cols, words) + td_decode_rows_bytes(cols, words) + (size_t)cols * 4u + 64u * 8u + 256u + 16u;
 }
 
-__device__ __forceinline__ unsigned td_zigzag(int e) { return ((unsigned)e << 1) ^ (unsigned)(e >> 31); }   // 2e, or -2e - 1 for e < 0
-
 // Big-endian view of a little-endian word: the stream's first byte in the top bits.
 __device__ __forceinline__ uint32_t td_be(uint32_t w) { return __byte_perm(w, 0u, 0x0123); }
-
-// round_half_even(x * inv) as the low byte of the sum with 1.5 * 2^23: two separately rounded fp32 operations.
-__device__ __forceinline__ int td_code(unsigned short x_bf16, float inv)
-{
-    const float p = __fmul_rn(__uint_as_float((uint32_t)x_bf16 << 16), inv);
-    return (int)(signed char)(__float_as_uint(__fadd_rn(p, 12582912.0f)) & 0xffu);
-}
 
 // Exclusive prefix sum of one value per thread over the block (blockDim.x a multiple of 32, at most 1024);
 // *total receives the sum.  `scratch` is 33 words of shared memory.
@@ -145,96 +137,6 @@ __device__ __forceinline__ unsigned td_lower_bound(const int32_t *list, unsigned
     return lo;
 }
 
-// Bring the slice [c0, c0 + C) of the n_tok token rows of one group (request positions pos0 ..) of a pool plane
-// into X[n_tok][C] with bulk copies counted on `bar`.  Warp 0 calls this; returns false (and records KDN_E_RANGE)
-// when a block id lies outside the pool, in which case nothing was issued.
-__device__ __forceinline__ bool td_load_slice(unsigned char *X, uint32_t bar, const unsigned char *base, const DevOp &op, unsigned g,
-                                              unsigned n_tok, int bs, long long n_blocks, unsigned RE,
-                                              unsigned C, unsigned c0, bool whole_row, int *status)
-{
-    const unsigned lane = threadIdx.x & 31u;
-    const int32_t *table = op.table;
-    long long id[2] = { 0, 0 }, pos[2] = { 0, 0 };
-    bool bad = false;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const unsigned t = lane + 32u * (unsigned)k;
-        if (t < n_tok) {
-            pos[k] = group_row_pos(op, g, t);
-            if (pos[k] < 0) { bad = true; continue; }
-            id[k] = __ldg(table + pos[k] / bs);
-            if (id[k] < 0 || id[k] >= n_blocks) bad = true;
-        }
-    }
-    if (__any_sync(0xffffffffu, bad)) {
-        if (lane == 0) atomicCAS(status, 0, kStatusRange);
-        return false;
-    }
-    if (lane == 0) mbar_arrive_expect_tx(bar, n_tok * C * 2u);
-    __syncwarp();
-    if (whole_row && op.list_mode == 0) {
-        // a block's tokens are contiguous in the pool: one copy per block (pieces <= 32 KiB); the host sees to it that
-        // the group starts at a block start
-        if (lane == 0) {
-            const long long first_block = (op.off + (long long)(g << 6)) / bs;
-            for (unsigned t = 0; t < n_tok; t += (unsigned)bs) {
-                const unsigned k = n_tok - t < (unsigned)bs ? n_tok - t : (unsigned)bs;
-                const long long b = __ldg(table + first_block + t / (unsigned)bs);
-                const unsigned char *src = base + (unsigned long long)b * bs * RE * 2ull;
-                const unsigned bytes = k * RE * 2u;
-                for (unsigned o = 0; o < bytes; o += 32768u)
-                    bulk_g2s(smem_u32(X + (size_t)t * RE * 2u + o), src + o, bytes - o < 32768u ? bytes - o : 32768u, bar);
-            }
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const unsigned t = lane + 32u * (unsigned)k;
-            if (t < n_tok) {
-                const unsigned slot = (unsigned)(pos[k] % bs);
-                const unsigned char *src = base + (((unsigned long long)id[k] * bs + slot) * RE + c0) * 2ull;
-                for (unsigned o = 0; o < C * 2u; o += 32768u)              // (a slice is at most 1024 channels: one piece)
-                    bulk_g2s(smem_u32(X + (size_t)t * C * 2u + o), src + o, C * 2u - o < 32768u ? C * 2u - o : 32768u, bar);
-            }
-        }
-    }
-    return true;
-}
-
-// Per-channel reciprocal (and scale) of the slice in X: largest magnitude over the group's tokens, then the two IEEE
-// divides of the codec.  All threads of the block call this; X must have landed.  g_scales may be nullptr.
-__device__ __forceinline__ void td_channel_scales(const unsigned char *X, unsigned char *pmax, float *inv, float *g_scales,
-                                                  unsigned n_tok, unsigned C, float qmax)
-{
-    const unsigned tid = threadIdx.x, nthreads = blockDim.x;
-    const unsigned octets = C >> 3, items = octets * kKcSlices;
-    for (unsigned it = tid; it < items; it += nthreads) {
-        const unsigned q = it / octets, o = it - q * octets;
-        const unsigned ta = q * kKcTok, tb = ta + kKcTok < n_tok ? ta + kKcTok : n_tok;
-        uint32_t m0 = 0u, m1 = 0u, m2 = 0u, m3 = 0u;
-        for (unsigned t = ta; t < tb; ++t) {
-            const uint4 x = lds128(X + ((size_t)t * C + (size_t)o * 8u) * 2u);
-            m0 = maxabs_bf16x2(m0, x.x); m1 = maxabs_bf16x2(m1, x.y);
-            m2 = maxabs_bf16x2(m2, x.z); m3 = maxabs_bf16x2(m3, x.w);
-        }
-        sts128(pmax + ((size_t)q * C + (size_t)o * 8u) * 2u, make_uint4(m0, m1, m2, m3));
-    }
-    __syncthreads();
-    for (unsigned ch = tid; ch < C; ch += nthreads) {
-        unsigned short mx = 0;
-        for (unsigned q = 0; q < kKcSlices; ++q) {
-            const unsigned short v = *reinterpret_cast<const unsigned short *>(pmax + ((size_t)q * C + ch) * 2u) & 0x7fffu;
-            mx = v > mx ? v : mx;                              // magnitudes of bf16 order like their bit patterns
-        }
-        const float a = __uint_as_float((uint32_t)mx << 16);
-        const float sc = __fdiv_rn(a, qmax);
-        const bool ok = sc >= 1.17549435e-38f;                 // smallest normal fp32; false for NaN too
-        if (g_scales) g_scales[ch] = ok ? sc : 0.0f;
-        inv[ch] = ok ? __fdiv_rn(qmax, a) : 0.0f;
-    }
-    __syncthreads();
-}
-
 struct TdSlice {              // what a CTA of the store and decode kernels works on
     DevOp op;
     unsigned g, part, plane, li, kv, n_tok, c0, seg;
@@ -257,6 +159,46 @@ __device__ __forceinline__ TdSlice td_slice(const TdLaunch &P)
     s.c0 = s.part * P.cols;
     s.seg = (unsigned)(((unsigned long long)(s.op.l0 + (int)s.li) * 2ull + s.kv) * s.G + s.g);
     return s;
+}
+
+// Where a slice's sub-streams lie: two channels a thread, 2 tid and 2 tid + 1 of the slice.  `scratch`: 32 words of shared memory.
+// All threads of the block call this (one barrier).
+struct TdOffsets {
+    unsigned pair;                // lengths of the thread's two sub-streams, one byte each (0 past the slice's end)
+    unsigned off;                 // byte offset of the first of them inside the slice
+    unsigned slice, before;       // bytes of the slice, and of the segment's slices before it
+};
+__device__ __forceinline__ TdOffsets td_offsets(const unsigned char *lens, unsigned c0, unsigned C, unsigned nthreads, unsigned *scratch)
+{
+    const unsigned tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, nwarps = nthreads >> 5;
+    TdOffsets o;
+    // channels before the slice: 16 lengths a load (the table's rows and c0 are multiples of 16)
+    unsigned before = 0;
+    for (unsigned i = tid; i < (c0 >> 4); i += nthreads) {
+        const uint4 v = *reinterpret_cast<const uint4 *>(lens + 16u * i);
+        before = __dp4a(v.x, 0x01010101u, before); before = __dp4a(v.y, 0x01010101u, before);
+        before = __dp4a(v.z, 0x01010101u, before); before = __dp4a(v.w, 0x01010101u, before);
+    }
+    o.pair = 2u * tid < C ? *reinterpret_cast<const unsigned short *>(lens + c0 + 2u * tid) : 0u;
+    const unsigned both = (o.pair & 0xffu) + (o.pair >> 8);
+    unsigned inc = both;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned v = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= (unsigned)d) inc += v;
+    }
+    before = __reduce_add_sync(0xffffffffu, before);
+    if (lane == 31u) { scratch[warp] = inc; scratch[16u + warp] = before; }
+    __syncthreads();
+    o.off = inc - both;
+    o.slice = 0u;
+    o.before = 0u;
+    for (unsigned w = 0; w < nwarps; ++w) {
+        if (w == warp) o.off += o.slice;
+        o.slice += scratch[w];
+        o.before += scratch[16u + w];
+    }
+    return o;
 }
 
 // Pool addresses of the slice in the token rows of the group, row t at rows[t + t / 32] (0 for rows past the chunk's end).  All
@@ -561,122 +503,231 @@ __global__ void __launch_bounds__(kTdScanThreads) kdn_td_scan_kernel(const __gri
 
 // ---------------------------------------------------------------------------------------- store: encode --
 
-__global__ void __launch_bounds__(512) kdn_td_encode_kernel(const __grid_constant__ TdLaunch P)
+// One sub-stream on its way out.  As in the decoder the bits are kept complemented, so that unary parts are zeros: a symbol u
+// is the number 2^(k+1) - 1 - (u mod 2^k) in (u >> k) + k + 1 bits.  u itself comes out of the floating-point pipe as
+// |2 e + 1/2| - 1/2 (2 e for e >= 0, else -2 e - 1), in the low bits of 2^23 + u.
+struct TdOut {
+    uint32_t acc;          // the bits not yet written, in the low (bits mod 32) bits; garbage above them
+    unsigned bits;         // bits so far, those of the first word that are not the sub-stream's own included
+    uint32_t wp;           // shared address of the word being filled
+    unsigned k, len0;      // Rice parameter; k + 1 - (bits of 2^23 >> k)
+    uint32_t kmask, kbit;  // 2^k - 1, 2^k
+    unsigned limit;        // k + 16: code words this long are escapes
+};
+constexpr unsigned kTdLoad = 8;                              // tokens loaded ahead
+constexpr uint32_t kTdUZero = 0x4B000000u;                   // bits of 2^23
+
+__device__ __forceinline__ void td_out_init(TdOut &o, uint32_t addr, unsigned param)
+{
+    o.k = param & 7u;
+    o.kbit = 1u << o.k;
+    o.kmask = o.kbit - 1u;
+    o.len0 = o.k + 1u - (kTdUZero >> o.k);
+    o.limit = o.k + 16u;
+    o.acc = 0u;
+    o.bits = (addr & 3u) * 8u;
+    o.wp = addr & ~3u;
+}
+// Append the low `len` bits of w (1 <= len <= 32, nothing above them).  A word that is full is OR-ed into the staging area: the
+// first and the last word of a sub-stream also hold bits of its neighbours.  (The shifts take their count modulo 32.)
+__device__ __forceinline__ void td_append(TdOut &o, uint32_t w, unsigned len)
+{
+    const uint32_t left = __funnelshift_l(0u, w, 0u - len);                 // left-aligned
+    const uint32_t word = __funnelshift_r(left, o.acc, o.bits);
+    const unsigned bits = o.bits + len;
+    o.acc = __funnelshift_r(left, o.acc, 0u - len);
+    // (predicated by hand: a branch around two instructions costs more than they do)
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p red.shared.or.b32 [%0], %1; @p add.u32 %0, %0, 4; }"
+                 : "+r"(o.wp) : "r"(word), "r"((o.bits ^ bits) & ~31u) : "memory");
+    o.bits = bits;
+}
+// One symbol, escapes included; ub: bits of 2^23 + u.
+__device__ __forceinline__ void td_append_any(TdOut &o, uint32_t ub, unsigned raw_bits)
+{
+    unsigned len = (ub >> o.k) + o.len0;
+    uint32_t z = (~ub & o.kmask) | o.kbit;
+    if (len >= o.limit) { len = 15u + raw_bits; z = ~ub & ((1u << raw_bits) - 1u); }
+    td_append(o, z, len);
+}
+// Four symbols of two sub-streams, kJoin of them joined before they are appended (4-bit codes: four, 8-bit codes: two).  Where
+// one is an escape, or the joined ones are longer than a word, one at a time.
+template <unsigned kN> struct TdJoin { static constexpr unsigned value = kN; };
+template <unsigned kJoin>
+__device__ __forceinline__ void td_append4(const TdLaunch &P, TdOut &x, TdOut &y, const uint32_t (&ux)[4], const uint32_t (&uy)[4], unsigned raw_bits)
+{
+    unsigned lx[4], ly[4];
+    uint32_t zx[4], zy[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        lx[i] = (ux[i] >> x.k) * P.pow2[0] + x.len0;
+        ly[i] = (uy[i] >> y.k) * P.pow2[0] + y.len0;
+        zx[i] = (~ux[i] & x.kmask) | x.kbit;
+        zy[i] = (~uy[i] & y.kmask) | y.kbit;
+    }
+    const unsigned mx = max(max(lx[0], lx[1]), max(lx[2], lx[3])), my = max(max(ly[0], ly[1]), max(ly[2], ly[3]));
+    unsigned jx[4], jy[4], longest = 0;                      // joined lengths
+#pragma unroll
+    for (int i = 0; i < 4; i += (int)kJoin) {
+        jx[i] = lx[i]; jy[i] = ly[i];
+#pragma unroll
+        for (int j = 1; j < (int)kJoin; ++j) {
+            zx[i] = (zx[i] << (lx[i + j] & 31u)) * P.pow2[0] + zx[i + j];
+            zy[i] = (zy[i] << (ly[i + j] & 31u)) * P.pow2[0] + zy[i + j];
+            jx[i] = jx[i] * P.pow2[0] + lx[i + j];
+            jy[i] = jy[i] * P.pow2[0] + ly[i + j];
+        }
+        longest = max(longest, max(jx[i], jy[i]));
+    }
+    if (__builtin_expect(mx >= x.limit || my >= y.limit || longest > 32u, 0)) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { lx[i] = ux[i]; ly[i] = uy[i]; }
+#pragma unroll 1
+        for (int i = 0; i < 4; ++i) {                        // (rolled up: instruction fetch is felt in this kernel)
+            td_append_any(x, lx[0], raw_bits);
+            td_append_any(y, ly[0], raw_bits);
+            lx[0] = lx[1]; lx[1] = lx[2]; lx[2] = lx[3];
+            ly[0] = ly[1]; ly[1] = ly[2]; ly[2] = ly[3];
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; i += (int)kJoin) {
+            td_append(x, zx[i], jx[i]);
+            td_append(y, zy[i], jy[i]);
+        }
+    }
+}
+// The end of a sub-stream: zero bits (ones, complemented) up to the byte, and the last word.
+__device__ __forceinline__ void td_out_finish(TdOut &o)
+{
+    const unsigned pad = (0u - o.bits) & 7u;
+    if (pad) td_append(o, (1u << pad) - 1u, pad);
+    if (o.bits & 31u) {
+        const uint32_t word = o.acc << (32u - (o.bits & 31u));
+        asm volatile("red.shared.or.b32 [%0], %1;" :: "r"(o.wp), "r"(word) : "memory");
+    }
+}
+
+// A thread quantises and codes two neighbouring channels side by side, token by token, straight from the pool: the planner's scale
+// says what the largest magnitude was (a bf16 number: scale * qmax rounded to bf16 is that number again), so there is no pass
+// for it and no tile.  The staging area holds the slice's bits complemented, as big-endian words.  Bound by instruction issue
+// (77 % of the slots).  8B shape, 16 chunks of 512 tokens: 1020 us for 8-bit codes with a tile, a pass over it for the magnitudes and
+// every symbol appended by itself, 540 us this way; 4-bit codes 1000 -> 490 us.  Fourteen CTAs of 64 threads an SM (72 registers) with
+// eight tokens loaded ahead; twelve or sixteen CTAs, four or sixteen tokens are 0-7 % slower.
+template <unsigned kCols>
+__global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 14 : 1) kdn_td_encode_kernel(const __grid_constant__ TdLaunch P)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const TdSlice s = td_slice(P);
     if (!s.valid) return;
-    const unsigned C = P.cols, RE = P.row_elems;
+    const unsigned C = kCols ? kCols : P.cols, RE = P.row_elems;
+    const unsigned nthreads = kCols ? kCols / 2u : blockDim.x, tid = threadIdx.x;
     const int codec = s.op.codec;
-    const float qmax = (float)td_qmax(codec);
     const unsigned raw_bits = (unsigned)td_raw_bits(codec);
-
-    unsigned char *X = smem_raw;
-    unsigned char *pmax = X + (size_t)64 * C * 2u;
-    float *inv = reinterpret_cast<float *>(pmax + (size_t)kKcSlices * C * 2u);
-    unsigned char *stage = reinterpret_cast<unsigned char *>(inv) + (size_t)C * 4u;          // C * 72 + 32 bytes
-    unsigned *scratch = reinterpret_cast<unsigned *>(stage + (size_t)C * 72u + 32u + kTdStageSlack);   // 64 words
-    unsigned long long *bar_mem = reinterpret_cast<unsigned long long *>(reinterpret_cast<unsigned char *>(scratch) + 256u);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(bar_mem + 1);
-    const uint32_t bar = smem_u32(bar_mem);
-    const unsigned tid = threadIdx.x;
-    if (tid == 0) {
-        mbar_init(bar, 1u);
-        *abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        fence_async_smem();
-    }
-    __syncthreads();
-    if (tid < 32) {
-        const unsigned char *base = reinterpret_cast<const unsigned char *>((s.kv ? P.v_layers : P.k_layers)[s.op.l0 + (int)s.li]);
-        if (!td_load_slice(X, bar, base, s.op, s.g, s.n_tok, P.bs, P.n_blocks, RE, C, s.c0,
-                           P.n_split == 1u, P.status) && tid == 0)
-            *abort_flag = 1;
-    }
-    // meanwhile: where the slice's bytes go.  Lengths of the channels before the slice, then of the slice itself.
-    const TdLayout lay = td_layout(P.L, RE, s.op.T, codec);
+    unsigned long long *rows = reinterpret_cast<unsigned long long *>(smem_raw);            // [66]
+    unsigned *scratch = reinterpret_cast<unsigned *>(rows + 66);                             // 32 words
+    unsigned char *stage = smem_raw + kTdEncodeHead;
+    const TdLayout &lay = P.layout[blockIdx.z];
     const unsigned long long row = (unsigned long long)s.seg * RE;
-    const unsigned char *lens = s.op.data + lay.lens + row;
-    unsigned before = 0;
-    for (unsigned c = tid; c < s.c0; c += blockDim.x) before += lens[c];
-    unsigned total_before, total_slice;
-    td_block_scan(before, scratch, &total_before);
-    const unsigned my_len = tid < C ? lens[s.c0 + tid] : 0u;                                 // blockDim.x >= C
-    const unsigned my_off = td_block_scan(my_len, scratch, &total_slice);
+    const bool act = 2u * tid < C;
+    const bool bad = td_row_addresses(P, s, rows);
+    const TdOffsets o = td_offsets(s.op.data + lay.lens + row, s.c0, C, nthreads, scratch);
     const unsigned long long seg_begin = reinterpret_cast<const unsigned long long *>(s.op.data)[s.seg];
-    unsigned char *dst = s.op.data + seg_begin + total_before;
+    unsigned char *dst = s.op.data + seg_begin + o.before;
     const unsigned shift = (unsigned)((unsigned long long)dst & 15ull);                      // staging mirrors the destination's alignment
     // the lengths are the planner's, but a planner CTA may have given up: nothing may leave the staging area or the chunk
     // (the capacity ends on a 16-byte boundary, so the padding of a segment's last slice fits whenever its bytes do)
-    const bool sane = total_slice <= C * td_max_len(codec) && seg_begin >= lay.streams &&
-                      seg_begin + total_before + total_slice <= lay.capacity;
-    if (tid == 0 && !sane) {
-        atomicCAS(P.status, 0, kStatusRange);
-        *abort_flag = 1;
-    }
-    __syncthreads();
-    if (*abort_flag) return;
-    const bool landed = mbar_wait(bar, 0u, abort_flag, P.wait_limit_ns);
-    if (!__syncthreads_and(landed)) {
-        if (tid == 0) {
-            atomicCAS(P.status, 0, kStatusTimeout);
-            const unsigned long long t0 = global_timer_ns();
-            while (!mbar_try_wait(bar, 0u))
-                if (global_timer_ns() - t0 > kWaitLimitNs) break;
-        }
+    const bool sane = o.slice <= C * td_max_len(codec) && seg_begin >= lay.streams && seg_begin + o.before + o.slice <= lay.capacity;
+    for (unsigned i = tid; i < (shift + (sane ? o.slice : 0u) + 31u) / 16u; i += nthreads) sts128(stage + (size_t)i * 16u, make_uint4(0u, 0u, 0u, 0u));
+    if (__syncthreads_or(bad || !sane)) {                                                     // (also publishes the zeros and the rows)
+        if (tid == 0) atomicCAS(P.status, 0, kStatusRange);
         return;
     }
-    // the staging area starts out as zeros: sub-streams are OR-ed into it a 32-bit word at a time, since the first and
-    // the last word of a sub-stream also hold bits of its neighbours
-    for (unsigned i = tid; i < (C * 72u + 32u) / 16u; i += blockDim.x) sts128(stage + (size_t)i * 16u, make_uint4(0u, 0u, 0u, 0u));
-    td_channel_scales(X, pmax, inv, nullptr, s.n_tok, C, qmax);                 // (its barriers also publish the zeros)
-    if (tid < C && my_len != 0u && my_len <= td_max_len(codec)) {       // (a length of zero: the planner gave this slice up)
-        const unsigned param = s.op.data[lay.params + row + s.c0 + tid];
-        const bool delta = (param & 8u) != 0u;
-        const unsigned k = param & 7u, kmask = (1u << k) - 1u, k1 = k + 1u;
-        const float iv = inv[tid];
-        const uint32_t addr = smem_u32(stage) + shift + my_off;          // first byte of the sub-stream
-        uint32_t wp = addr & ~3u;                                         // the word it starts in ...
-        unsigned nb = (addr & 3u) * 8u;                                   // ... after this many bits that are not its own
-        unsigned long long acc = 0;
-        int prev = 0;
-#pragma unroll 4
-        for (unsigned t = 0; t < s.n_tok; ++t) {
-            const int q = td_code(*reinterpret_cast<const unsigned short *>(X + ((size_t)t * C + tid) * 2u), iv);
-            const unsigned u = td_zigzag(delta ? q - prev : q);
-            prev = q;
-            const unsigned quo = u >> k;
-            unsigned w = (((1u << quo) - 1u) << k1) | (u & kmask), len = quo + k1;
-            if (__builtin_expect(quo >= 15u, 0)) { w = (0x7fffu << raw_bits) | u; len = 15u + raw_bits; }
-            acc = (acc << len) | w;
-            nb += len;
-            if (nb >= 32u) {                                              // a full word: bytes in stream order, first byte lowest
-                nb -= 32u;
-                const uint32_t word = td_be((uint32_t)(acc >> nb));
-                asm volatile("red.shared.or.b32 [%0], %1;" :: "r"(wp), "r"(word) : "memory");
-                wp += 4u;
+    const unsigned len_x = o.pair & 0xffu, len_y = o.pair >> 8;
+    // (a length of zero: the planner gave this slice up)
+    if (act && len_x != 0u && len_y != 0u && len_x <= td_max_len(codec) && len_y <= td_max_len(codec)) {
+        const unsigned long long at = row + s.c0 + 2u * tid;
+        const unsigned params = *reinterpret_cast<const unsigned short *>(s.op.data + lay.params + at);
+        const float2 sc = *reinterpret_cast<const float2 *>(s.op.data + lay.scales + 4ull * at);
+        const float qmax = (float)td_qmax(codec);
+        const float inv_x = sc.x != 0.0f ? __fdiv_rn(qmax, __bfloat162float(__float2bfloat16_rn(__fmul_rn(sc.x, qmax)))) : 0.0f;
+        const float inv_y = sc.y != 0.0f ? __fdiv_rn(qmax, __bfloat162float(__float2bfloat16_rn(__fmul_rn(sc.y, qmax)))) : 0.0f;
+        TdOut x, y;
+        td_out_init(x, smem_u32(stage) + shift + o.off, params & 0xffu);
+        td_out_init(y, smem_u32(stage) + shift + o.off + len_x, params >> 8);
+        // per token: m + code (m = 1.5 * 2^23), minus m or the token before (delta mode), all exact
+        const float m = 12582912.0f;
+        const f32x2 inv2 = pack2(inv_x, inv_y), m2 = pack2(m, m), one2 = pack2(P.fone, P.fone), two2 = pack2(2.0f, 2.0f), half2 = pack2(0.5f, 0.5f);
+        const bool dx = (params & 8u) != 0u, dy = (params & 0x800u) != 0u;
+        const f32x2 nd2 = pack2(dx ? -1.0f : 0.0f, dy ? -1.0f : 0.0f), nc2 = pack2(dx ? 0.0f : -m, dy ? 0.0f : -m);
+        f32x2 base = pack2(-m, -m);
+        auto symbol = [&](uint32_t v, uint32_t &a, uint32_t &b) {
+            const f32x2 r = add2_unfused(mul2(bf16x2_widen(v), inv2), m2, one2);
+            const f32x2 f = fma2(add2(r, base), two2, half2);
+            base = fma2(r, nd2, nc2);
+            float fa, fb;
+            unpack2(f, fa, fb);
+            a = __float_as_uint(__fadd_rn(fabsf(fa), 8388607.5f));
+            b = __float_as_uint(__fadd_rn(fabsf(fb), 8388607.5f));
+        };
+        // kTdLoad tokens at a time, the next ones already on their way
+        auto load = [&](unsigned t0, uint32_t (&v)[kTdLoad]) {
+            const unsigned long long *r = rows + t0 + (t0 >> 5);
+#pragma unroll
+            for (int i = 0; i < (int)kTdLoad; ++i) v[i] = __ldg(reinterpret_cast<const uint32_t *>(r[i] + (unsigned long long)(2u * tid) * P.pow2[1]));
+        };
+        auto code = [&](auto join) -> unsigned {
+            unsigned t0 = 0;
+            uint32_t v[kTdLoad], next[kTdLoad];
+            if (kTdLoad <= s.n_tok) load(0u, next);
+#pragma unroll 1
+            for (; t0 + kTdLoad <= s.n_tok; t0 += kTdLoad) {
+#pragma unroll
+                for (int i = 0; i < (int)kTdLoad; ++i) v[i] = next[i];
+                if (t0 + 2u * kTdLoad <= s.n_tok) load(t0 + kTdLoad, next);
+#pragma unroll
+                for (int i = 0; i < (int)kTdLoad; i += 4) {
+                    uint32_t ux[4], uy[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) symbol(v[i + j], ux[j], uy[j]);
+                    td_append4<decltype(join)::value>(P, x, y, ux, uy, raw_bits);
+                }
             }
+            return t0;
+        };
+        unsigned t0 = codec == 6 ? code(TdJoin<4>()) : code(TdJoin<2>());
+#pragma unroll 1
+        for (; t0 < s.n_tok; ++t0) {
+            uint32_t ux, uy;
+            symbol(__ldg(reinterpret_cast<const uint32_t *>(rows[t0 + (t0 >> 5)]) + tid), ux, uy);
+            td_append_any(x, ux, raw_bits);
+            td_append_any(y, uy, raw_bits);
         }
-        if (nb > 0u) {
-            const uint32_t word = td_be((uint32_t)(acc << (32u - nb)));
-            asm volatile("red.shared.or.b32 [%0], %1;" :: "r"(wp), "r"(word) : "memory");
-        }
+        td_out_finish(x);
+        td_out_finish(y);
     }
     // the last slice of a segment also writes the zero bytes that pad the segment to 16
     unsigned pad = 0;
     if (s.part == P.n_split - 1u) {
-        pad = (16u - ((shift + total_slice) & 15u)) & 15u;
-        if (tid < pad) stage[shift + total_slice + tid] = 0;
+        pad = (16u - ((shift + o.slice) & 15u)) & 15u;
+        if (tid < pad) {
+            const unsigned i = shift + o.slice + tid;
+            const uint32_t word = 0xff000000u >> (8u * (i & 3u));
+            asm volatile("red.shared.or.b32 [%0], %1;" :: "r"(smem_u32(stage) + (i & ~3u)), "r"(word) : "memory");
+        }
     }
     __syncthreads();
-    const unsigned n_out = total_slice + pad;
-    // staging -> chunk: bytes up to the first 16-byte boundary, 16-byte words, bytes after the last boundary
+    const unsigned n_out = o.slice + pad;
+    // staging -> chunk, words turned to little-endian and complemented: bytes up to the first 16-byte boundary, 16-byte vectors,
+    // bytes after the last boundary
     const unsigned head = shift ? (16u - shift < n_out ? 16u - shift : n_out) : 0u;
     const unsigned vecs = (n_out - head) >> 4, tail = (n_out - head) & 15u;
-    if (tid < head) dst[tid] = stage[shift + tid];
-    for (unsigned v = tid; v < vecs; v += blockDim.x)
-        *reinterpret_cast<uint4 *>(dst + head + (size_t)v * 16u) = lds128(stage + shift + head + (size_t)v * 16u);
-    if (tid < tail) dst[head + vecs * 16u + tid] = stage[shift + head + vecs * 16u + tid];
+    auto byte_at = [&](unsigned i) { return (unsigned char)~(*reinterpret_cast<const uint32_t *>(stage + (i & ~3u)) >> (24u - 8u * (i & 3u))); };
+    if (tid < head) dst[tid] = byte_at(shift + tid);
+    for (unsigned v = tid; v < vecs; v += nthreads) {
+        const uint4 w = lds128(stage + shift + head + (size_t)v * 16u);
+        *reinterpret_cast<uint4 *>(dst + head + (size_t)v * 16u) = make_uint4(~td_be(w.x), ~td_be(w.y), ~td_be(w.z), ~td_be(w.w));
+    }
+    if (tid < tail) dst[head + vecs * 16u + tid] = byte_at(shift + head + vecs * 16u + tid);
 }
 
 // ----------------------------------------------------------------------------------- retrieve / compose --
@@ -818,7 +869,7 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 14 : 1) kdn
     const unsigned C = kCols ? kCols : P.cols, RE = P.row_elems;
     const int codec = s.op.codec;
     const unsigned raw_bits = (unsigned)td_raw_bits(codec);
-    const unsigned nthreads = kCols ? kCols / 2u : blockDim.x, nwarps = nthreads >> 5;
+    const unsigned nthreads = kCols ? kCols / 2u : blockDim.x;
 
     uint32_t *I = reinterpret_cast<uint32_t *>(smem_raw);                // interleaved sub-streams [word][C]
     unsigned char *A = smem_raw + td_decode_words_bytes(C, P.words);     // the slice's stream bytes, then bf16 rows [kTdHalf][C]
@@ -828,7 +879,7 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 14 : 1) kdn
     unsigned long long *bar_mem = reinterpret_cast<unsigned long long *>(reinterpret_cast<unsigned char *>(scratch) + 256u);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(bar_mem + 1);
     const uint32_t bar = smem_u32(bar_mem);
-    const unsigned tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const unsigned tid = threadIdx.x;
     if (tid == 0) {
         mbar_init(bar, 1u);
         *abort_flag = 0;
@@ -842,32 +893,9 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 14 : 1) kdn
     const unsigned long long row = (unsigned long long)s.seg * RE;
     const unsigned char *lens = s.op.data + lay.lens + row;
     const bool act = 2u * tid < C;
-    // bytes of the channels before the slice (16 lengths a load: the table's rows and c0 are multiples of 16), and of the
-    // slice's own channels, two a thread
-    unsigned before = 0;
-    for (unsigned i = tid; i < (s.c0 >> 4); i += nthreads) {
-        const uint4 v = *reinterpret_cast<const uint4 *>(lens + 16u * i);
-        before = __dp4a(v.x, 0x01010101u, before); before = __dp4a(v.y, 0x01010101u, before);
-        before = __dp4a(v.z, 0x01010101u, before); before = __dp4a(v.w, 0x01010101u, before);
-    }
-    const unsigned pair = act ? *reinterpret_cast<const unsigned short *>(lens + s.c0 + 2u * tid) : 0u;
-    const unsigned both = (pair & 0xffu) + (pair >> 8);
-    unsigned inc = both;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const unsigned o = __shfl_up_sync(0xffffffffu, inc, d);
-        if (lane >= (unsigned)d) inc += o;
-    }
-    before = __reduce_add_sync(0xffffffffu, before);
-    if (lane == 31u) { scratch[warp] = inc; scratch[16u + warp] = before; }
-    __syncthreads();                                                      // (also publishes the mbarrier and the two indices)
+    const TdOffsets o = td_offsets(lens, s.c0, C, nthreads, scratch);     // (its barrier also publishes the mbarrier and the two indices)
     if (selecting && scratch[40] >= scratch[41]) return;                  // every thread alike, and no copy has been started
-    unsigned total_before = 0, total_slice = 0, my_off = inc - both;
-    for (unsigned w = 0; w < nwarps; ++w) {
-        if (w == warp) my_off += total_slice;
-        total_slice += scratch[w];
-        total_before += scratch[16u + w];
-    }
+    const unsigned total_before = o.before, total_slice = o.slice, my_off = o.off, pair = o.pair;
     const unsigned long long seg_begin = reinterpret_cast<const unsigned long long *>(s.op.data)[s.seg];
     const unsigned long long src = seg_begin + total_before;
     const unsigned shift = (unsigned)(((unsigned long long)s.op.data + src) & 15ull);
