@@ -4,6 +4,7 @@
 // delivery and blending modules).
 #include "kdn.h"
 #include "kdn_kernels.cuh"
+#include "kdn_rows.cuh"
 #include "kdn_td.cuh"
 
 #include <cerrno>
@@ -370,7 +371,7 @@ Shape default_shape(int OP, bool any_coded, bool any_rot)
 // Pipeline slots: at least lag + 2, a multiple of the compute groups (a slot must always belong to the
 // same group), and, unless the caller fixed the count, few enough for ctas_per_sm CTAs to share an SM.
 kdn_status fit_stages(int &stages, int groups, int lag, bool shrink, unsigned stage_bytes, int ctas_per_sm, size_t smem_limit,
-                      int rows_per_tile = 1, bool wide = false)
+                      int rows_per_tile = 1)
 {
     const int g = groups > 0 ? groups : 1;
     if (stages > kMaxStages) stages = kMaxStages;
@@ -379,32 +380,20 @@ kdn_status fit_stages(int &stages, int groups, int lag, bool shrink, unsigned st
     stages = stages / g * g;
     if (shrink)
         while (stages - g >= min_stages &&
-               smem_bytes(stages, stage_bytes, rows_per_tile, wide) * (size_t)ctas_per_sm > smem_limit - 1024u * (size_t)ctas_per_sm)
+               smem_bytes(stages, stage_bytes, rows_per_tile) * (size_t)ctas_per_sm > smem_limit - 1024u * (size_t)ctas_per_sm)
             stages -= g;
-    return smem_bytes(stages, stage_bytes, rows_per_tile, wide) > smem_limit ? KDN_E_UNSUPPORTED : KDN_OK;
+    return smem_bytes(stages, stage_bytes, rows_per_tile) > smem_limit ? KDN_E_UNSUPPORTED : KDN_OK;
 }
 
 // Launch the instantiation for (OP, compute groups, warps per group); groups = 0 is the pure-copy form.
 kdn_status launch_tiles(LaunchEnv &env, int OP, int groups, int gw, unsigned grid, size_t smem, cudaStream_t stream,
-                        const Launch &lp, bool overlap = false, bool wide = false)
+                        const Launch &lp, bool overlap = false)
 {
 #define KDN_CASE(G, W)                                                                                             \
     if (groups == G && (G == 0 || gw == W)) {                                                                      \
         if (OP == OP_STORE) return launch_kernel(env, kdn_store_kernel<G, W>, threads_for(G, W), grid, smem, stream, lp, overlap);      \
         if (OP == OP_RETRIEVE) return launch_kernel(env, kdn_retrieve_kernel<G, W>, threads_for(G, W), grid, smem, stream, lp, overlap); \
         return launch_kernel(env, kdn_compose_kernel<G, W>, threads_for(G, W), grid, smem, stream, lp, overlap);               \
-    }
-    if (wide) {
-        // tiles of up to 16 token rows: the kernels that keep the row indices in shared memory (store and retrieve, copy
-        // form and two single-warp groups)
-#define KDN_ROWS_CASE(G, W)                                                                                        \
-        if (groups == G && (G == 0 || gw == W)) {                                                                  \
-            if (OP == OP_STORE) return launch_kernel(env, kdn_store_rows_kernel<G, W>, threads_for(G, W), grid, smem, stream, lp, overlap);       \
-            if (OP == OP_RETRIEVE) return launch_kernel(env, kdn_retrieve_rows_kernel<G, W>, threads_for(G, W), grid, smem, stream, lp, overlap); \
-        }
-        KDN_ROWS_CASE(0, 4) KDN_ROWS_CASE(2, 1)
-#undef KDN_ROWS_CASE
-        return KDN_E_UNSUPPORTED;
     }
     KDN_CASE(0, 4) KDN_CASE(1, 4) KDN_CASE(2, 4) KDN_CASE(3, 4) KDN_CASE(4, 4) KDN_CASE(6, 4)
     KDN_CASE(2, 1) KDN_CASE(4, 1) KDN_CASE(8, 1)
@@ -426,6 +415,166 @@ kdn_status ensure_table(RingSlot *slot, int n_rope, int half)
     return KDN_OK;
 }
 
+// Key planes of the per-channel key codecs, store: one CTA per (64-token group, slice of channels, layer, op).  The ops' records are
+// inl[0 .. n) (kernel parameters) or at d_ops.
+kdn_status launch_key_planes(kdn_ctx *ctx, const Pool &pool, const DevOp *inl, const DevOp *d_ops, int n, int groups, int layers, cudaStream_t stream)
+{
+    const unsigned row_elems = (unsigned)pool.H * (unsigned)pool.D;
+    // channels per CTA: at most 256 (36 KiB of shared memory, six CTAs per SM), a multiple of eight that divides the row
+    unsigned n_split = 1;
+    while (row_elems / n_split > kKcCols && row_elems % (n_split * 2u * 8u) == 0u) n_split *= 2u;
+    const unsigned cols = row_elems / n_split;
+    const size_t kc_smem = kc_smem_bytes(cols);
+    if (kc_smem > (size_t)ctx->env.smem_optin) return KDN_E_UNSUPPORTED;
+    unsigned kc_threads = (cols / 8u + 7u) / 8u * 32u;       // a warp per 64 channels
+    if (kc_threads > 512u) kc_threads = 512u;
+    if (kc_threads < 64u) kc_threads = 64u;
+    KcLaunch kp{};
+    kp.one = 1.0f;
+    kp.wait_limit_ns = ctx->wait_limit_ns;
+    kp.cols = cols;
+    kp.n_split = n_split;
+    kp.ops = d_ops;
+    kp.n_ops = n;
+    kp.k_layers = pool.d_k;
+    kp.n_blocks = pool.nb;
+    kp.bs = pool.bs;
+    kp.row_elems = row_elems;
+    kp.status = ctx->d_status;
+    if (inl) std::memcpy(kp.inline_ops, inl, sizeof(DevOp) * (size_t)n);
+    int per_sm = 0;                                          // first sight of the kernel raises its shared-memory limit
+    kdn_status r = ctx->env.resident(kdn_store_kc_kernel, (int)kc_threads, kc_smem, &per_sm);
+    if (r != KDN_OK) return r;
+    if (per_sm < 1) return KDN_E_UNSUPPORTED;
+    kdn_store_kc_kernel<<<dim3((unsigned)groups * n_split, (unsigned)layers, (unsigned)n), kc_threads, kc_smem, stream>>>(kp);
+    KDN_CUDA(cudaGetLastError());
+    ctx->launches++;
+    return KDN_OK;
+}
+
+// Whether a launch goes to the kernels that move token rows one by one (kdn_rows.cuh): keep-lists over rows of up to 1024 elements --
+// the tile pipeline issues a copy a row -- and coded dense ops on pool blocks of 2 KiB or less, where a coding tile that stops at the
+// end of its block is far too small.  Half of the tokens kept, us in the tile pipeline / here (8B shape, 16 x 1024 tokens): two heads (rows of
+// 256) retrieve int8 114 / 79, int4 115 / 70, store int8 117 / 77, int4 117 / 66; one head raw (32 x 1024) 125 / 93; eight heads (rows of
+// 1024, 16 x 512) retrieve int8 146 / 144, int4 142 / 127, store int8 143 / 140, raw 172 / 171.  Only the retrieve of long rows with a scale per channel
+// (eight heads: 185 / 327) stays, since it would read the scales of every row anew.
+bool rows_apply(const kdn_ctx *ctx, const Pool &pool, int OP, bool any_coded, bool any_rot, bool any_list, bool any_kc, const HostOp *hops, int n)
+{
+    const unsigned row_elems = (unsigned)pool.H * (unsigned)pool.D;
+    const kdn_tuning &t = ctx->tuning;
+    // a caller-set launch shape is one of the tile pipeline
+    if (t.tile_bytes > 0 || t.stages > 0 || t.ctas_per_sm > 0 || t.compute_groups > 0 || t.store_lag > 0 || t.group_warps > 0) return false;
+    if ((OP != OP_STORE && OP != OP_RETRIEVE) || any_rot || row_elems % 16u) return false;
+    if (!any_list) return any_coded && !any_kc && (unsigned long long)pool.bs * row_elems * 2ull <= 2048ull;
+    for (int i = 0; i < n; ++i)
+        if (hops[i].op.list_mode != 1) return false;
+    return row_elems < 512u || (row_elems <= 1024u && !(any_kc && OP == OP_RETRIEVE));
+}
+
+kdn_status launch_rows(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops, int n, cudaStream_t stream)
+{
+    RowsLaunch lp{};
+    const bool inl = n <= kInlineOps;
+    RingSlot *slot = nullptr;
+    if (!inl) {
+        slot = &ctx->ring[ctx->ring_next++ % kRing];
+        if (slot->used) KDN_CUDA(cudaEventSynchronize(slot->done));
+    }
+    DevOp *h_ops = inl ? lp.inline_ops : slot->h_ops;
+    bool all_coded = true;
+    for (int i = 0; i < n; ++i) all_coded &= hops[i].op.codec != KDN_CODEC_RAW_BF16;
+    constexpr int kj = kRowsVectors;
+    const unsigned vec = OP == OP_STORE || all_coded ? 16u : 8u;
+    const unsigned vectors = OP == OP_STORE ? kj / 2u : kj;    // a thread
+    lp.row_elems = (unsigned)pool.H * (unsigned)pool.D;
+    lp.vpr = lp.row_elems / vec;
+    lp.unit = lp.row_elems < 2048u ? 2048u / lp.row_elems : 1u;
+    if (lp.unit > 16u) lp.unit = 16u;
+    lp.rows = vectors * kRowsThreads / lp.vpr;
+    if (lp.rows > kRowsPerCta) lp.rows = kRowsPerCta;
+    if (lp.rows > lp.unit) lp.rows = lp.rows / lp.unit * lp.unit;
+    lp.vpr_magic = lp.rows > 1u && lp.vpr > 1u ? 0xffffffffu / lp.vpr + 1u : 0u;
+    unsigned long long ctas = 0;                             // with one plane each
+    for (int i = 0; i < n; ++i) {
+        const unsigned rows = (unsigned)(hops[i].op.list_mode ? hops[i].op.n_list : hops[i].op.T);
+        ctas += (unsigned long long)((rows + lp.rows - 1u) / lp.rows) * (unsigned)hops[i].op.nl * 2ull;
+    }
+    // planes a CTA goes through: enough to pay for the look-ups and the pipeline's start, few enough to leave some waves of CTAs
+    lp.planes = 1u;
+    while (lp.planes < 16u && ctas / (lp.planes * 2u) >= 6ull * (unsigned)ctx->env.sm_count) lp.planes *= 2u;
+    int kc_layers = 0, kc_groups = 0;
+    unsigned long long tiles = 0;
+    for (int i = 0; i < n; ++i) {
+        DevOp op = hops[i].op;
+        op.tile_begin = (unsigned)tiles;
+        if (OP == OP_STORE && is_kc(op.codec)) {
+            op.kv_sel = 2;                                   // the key planes go through kdn_store_kc_kernel
+            if (op.nl > kc_layers) kc_layers = op.nl;
+            if ((op.T + 63) / 64 > kc_groups) kc_groups = (op.T + 63) / 64;
+        }
+        h_ops[i] = op;
+        const unsigned rows = (unsigned)(op.list_mode ? op.n_list : op.T), planes = (unsigned)op.nl * (op.kv_sel ? 1u : 2u);
+        tiles += (unsigned long long)((rows + lp.rows - 1u) / lp.rows) * ((planes + lp.planes - 1u) / lp.planes);
+        if (tiles > kMaxTilesPerLaunch) return KDN_E_UNSUPPORTED;
+    }
+    if (tiles == 0) return KDN_OK;
+    if (!inl) KDN_CUDA(cudaMemcpyAsync(slot->d_ops, slot->h_ops, sizeof(DevOp) * (size_t)n, cudaMemcpyHostToDevice, stream));
+    lp.ops = inl ? nullptr : slot->d_ops;
+    lp.n_ops = n;
+    lp.k_layers = pool.d_k;
+    lp.v_layers = pool.d_v;
+    lp.n_blocks = pool.nb;
+    lp.bs = pool.bs;
+    lp.bs_shift = -1;
+    for (int b = 0; b < 31; ++b) if (pool.bs == 1 << b) lp.bs_shift = b;
+    lp.status = ctx->d_status;
+    lp.one = 1.0f;
+    if (kc_groups > 0) {
+        kdn_status r = launch_key_planes(ctx, pool, inl ? lp.inline_ops : nullptr, lp.ops, n, kc_groups, kc_layers, stream);
+        if (r != KDN_OK) return r;
+    }
+    lp.wait_limit_ns = ctx->wait_limit_ns;
+    const size_t smem = rows_smem_bytes(kj);
+    auto go = [&](auto kernel) -> kdn_status {
+        int per_sm = 0;                                      // first sight of the kernel raises its shared-memory limit
+        kdn_status r = ctx->env.resident(kernel, (int)kRowsThreads, smem, &per_sm);
+        if (r != KDN_OK) return r;
+        if (per_sm < 1) return KDN_E_UNSUPPORTED;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)tiles);
+        cfg.blockDim = dim3(kRowsThreads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        KDN_CUDA(cudaLaunchKernelEx(&cfg, kernel, lp));
+        return KDN_OK;
+    };
+    const kdn_status launched = OP == OP_STORE ? go(kdn_store_rows_kernel<kj, 16>)
+                              : vec == 16u ? go(kdn_retrieve_rows_kernel<kj, 16>) : go(kdn_retrieve_rows_kernel<kj, 8>);
+    if (launched != KDN_OK) return launched;
+    ctx->launches++;
+    ctx->last = kdn_launch_info{};
+    ctx->last.op = OP;
+    ctx->last.compute_groups = kj;
+    ctx->last.group_warps = (int32_t)vec;
+    ctx->last.tile_bytes = (int32_t)(lp.unit * lp.row_elems * 2u);
+    ctx->last.grid = (int32_t)tiles;
+    ctx->last.n_tiles = (uint32_t)tiles;
+    ctx->last.stages = kRowsStages;
+    ctx->last.smem_bytes = (int32_t)smem;
+    ctx->last.rows_per_tile = (int32_t)lp.unit;
+    ctx->last.rows_kernel = 1;
+    if (slot) {
+        KDN_CUDA(cudaEventRecord(slot->done, stream));
+        slot->used = true;
+    }
+    return KDN_OK;
+}
+
 // Tile one batch of host ops (at most kMaxOpsPerLaunch, all on the device side) and launch it.
 kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops, int n, cudaStream_t stream)
 {
@@ -441,24 +590,7 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     }
     const bool compute = any_coded || any_rot;
     const unsigned row_elems = (unsigned)pool.H * (unsigned)pool.D;
-    // Pool blocks of 2 KiB or less (block_size 1 or 2 with whole rows, a few tokens of one KV head): a coding tile that stops
-    // at the end of its block is far too small.  Such launches run as keep-list launches over the implied list 0, 1, 2, ...
-    // (list_mode 3): a tile then takes several token rows, wherever their blocks are, and rows that are neighbours in the
-    // pool still share a copy (8B shape, block_size 1: int8 store / retrieve 3.5 / 3.7 -> 5.2 / 5.3 TB/s).
-    std::vector<HostOp> as_rows;
-    // (the kernels for tiles of many rows exist for the built-in shapes only: a caller-set shape keeps the ordinary kernels)
-    const bool own_shape = ctx->tuning.compute_groups > 0 || ctx->tuning.group_warps > 0;
-    if (any_coded && !any_rot && !any_list && !any_kc && (OP == OP_STORE || OP == OP_RETRIEVE) && ctx->tuning.tile_bytes <= 0 && !own_shape &&
-        (unsigned long long)pool.bs * row_elems * 2ull <= 2048ull && (unsigned long long)pool.nb * (unsigned)pool.bs < 0xffffffffull) {
-        as_rows.assign(hops, hops + n);
-        for (HostOp &h : as_rows) {
-            h.op.list_mode = 3;
-            h.op.n_list = h.op.T;
-            h.op.list = nullptr;
-        }
-        hops = as_rows.data();
-        any_list = all_list = true;
-    }
+    if (rows_apply(ctx, pool, OP, any_coded, any_rot, any_list, any_kc, hops, n)) return launch_rows(ctx, pool, OP, hops, n, stream);
 
     // tile size: whole 16-byte units; whole 64-element groups with int8 / int4; whole head rows with rotation
     unsigned unit = 8;
@@ -496,14 +628,14 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
         // the 8B shape (2 KiB rows), throughput grows with CTAs per SM up to 8 (copy form 3.0 -> 6.4 TB/s)
         tile_elems = row_elems;
         bool all_keep = true;
-        for (int i = 0; i < n; ++i) all_keep &= hops[i].op.list_mode == 1 || hops[i].op.list_mode == 3;
+        for (int i = 0; i < n; ++i) all_keep &= hops[i].op.list_mode == 1;
         int want_rows = ctx->tuning.tile_bytes > 0 ? ctx->tuning.tile_bytes / 2 / (int)row_elems : 2048 / (int)row_elems;
         if (kc_decode)                                     // a key tile must lie inside one 64-token group: a power of two
             while (want_rows & (want_rows - 1)) want_rows &= want_rows - 1;
-        if (own_shape && want_rows > kMaxRowsPerTile) want_rows = kMaxRowsPerTile;
+        if (want_rows > kMaxRowsPerTile) want_rows = kMaxRowsPerTile;
         if (!any_coded && !any_rot && all_keep && want_rows >= 2 && row_elems < 1024u && (unsigned long long)pool.nb * (unsigned)pool.bs < 0xffffffffull) {
             // copy form on rows shorter than 2 KiB (few KV heads per GPU): several rows per tile as well
-            rows_per_tile = want_rows > kWideRowsPerTile ? kWideRowsPerTile : want_rows;
+            rows_per_tile = want_rows;
             tile_elems = (unsigned)rows_per_tile * row_elems;
             def = Shape{ 0, 4, 8, 0, 1 };
         } else if (any_coded && !any_rot && all_keep && want_rows >= 2 && (unsigned long long)pool.nb * (unsigned)pool.bs < 0xffffffffull) {
@@ -511,7 +643,7 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
             // scales move with one copy each, and rows that are neighbours in the pool share a copy too.  From a sweep on
             // the 8B shape with half of the tokens kept: two 1024-element rows per tile, five CTAs per SM with two
             // single-warp groups each, one store in flight (int8 5.1 -> 5.9 TB/s, int4 4.0 -> 4.9)
-            rows_per_tile = want_rows > kWideRowsPerTile ? kWideRowsPerTile : want_rows;
+            rows_per_tile = want_rows;
             tile_elems = (unsigned)rows_per_tile * row_elems;
             def = Shape{ 0, 6, 5, 2, 1, 1 };
         } else if (!any_coded && !any_rot) def = Shape{ 0, 4, 8, 0, 1 };
@@ -569,11 +701,9 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     int ctas_per_sm = ctx->tuning.ctas_per_sm > 0 ? ctx->tuning.ctas_per_sm : def.ctas_per_sm;
     int stages = ctx->tuning.stages > 0 ? ctx->tuning.stages : def.stages;
     const size_t smem_limit = (size_t)ctx->env.smem_optin;
-    // more than four rows per tile, and dense ops run as rows, go to the kernels built for that
-    const bool wide = rows_per_tile > kMaxRowsPerTile || !as_rows.empty();
-    kdn_status fit = fit_stages(stages, groups, lag, ctx->tuning.stages <= 0, stage_bytes, ctas_per_sm, smem_limit, rows_per_tile, wide);
+    kdn_status fit = fit_stages(stages, groups, lag, ctx->tuning.stages <= 0, stage_bytes, ctas_per_sm, smem_limit, rows_per_tile);
     if (fit != KDN_OK) return fit;
-    const size_t smem = smem_bytes(stages, stage_bytes, rows_per_tile, wide);
+    const size_t smem = smem_bytes(stages, stage_bytes, rows_per_tile);
 
     // Few ops travel as kernel parameters; otherwise through a ring slot (pinned staging + device copy).  A ring
     // slot is also what owns the rotation table.
@@ -653,38 +783,8 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     lp.rows_per_tile = rows_per_tile;
 
     if (kc_groups > 0) {
-        // key planes of the per-channel key codecs: one CTA per (64-token group, layer, op)
-        // channels per CTA: at most 256 (36 KiB of shared memory, six CTAs per SM), a multiple of eight that divides the row
-        unsigned n_split = 1;
-        while (row_elems / n_split > kKcCols && row_elems % (n_split * 2u * 8u) == 0u) n_split *= 2u;
-        const unsigned cols = row_elems / n_split;
-        const size_t kc_smem = kc_smem_bytes(cols);
-        if (kc_smem > smem_limit) return KDN_E_UNSUPPORTED;
-        unsigned kc_threads = (cols / 8u + 7u) / 8u * 32u;       // a warp per 64 channels
-        if (kc_threads > 512u) kc_threads = 512u;
-        if (kc_threads < 64u) kc_threads = 64u;
-        KcLaunch kp{};
-        kp.one = 1.0f;
-        kp.wait_limit_ns = ctx->wait_limit_ns;
-        kp.cols = cols;
-        kp.n_split = n_split;
-        kp.ops = inl ? nullptr : slot->d_ops;
-        kp.n_ops = n;
-        kp.k_layers = pool.d_k;
-        kp.n_blocks = pool.nb;
-        kp.bs = pool.bs;
-        kp.row_elems = row_elems;
-        kp.status = ctx->d_status;
-        if (inl) std::memcpy(kp.inline_ops, lp.inline_ops, sizeof(DevOp) * (size_t)n);
-        {
-            int per_sm = 0;                                  // first sight of the kernel raises its shared-memory limit
-            kdn_status r = ctx->env.resident(kdn_store_kc_kernel, (int)kc_threads, kc_smem, &per_sm);
-            if (r != KDN_OK) return r;
-            if (per_sm < 1) return KDN_E_UNSUPPORTED;
-        }
-        kdn_store_kc_kernel<<<dim3((unsigned)kc_groups * n_split, (unsigned)kc_layers, (unsigned)n), kc_threads, kc_smem, stream>>>(kp);
-        KDN_CUDA(cudaGetLastError());
-        ctx->launches++;
+        kdn_status r = launch_key_planes(ctx, pool, inl ? lp.inline_ops : nullptr, inl ? nullptr : slot->d_ops, n, kc_groups, kc_layers, stream);
+        if (r != KDN_OK) return r;
     }
 
     unsigned long long want = (unsigned long long)ctx->env.sm_count * (unsigned)ctas_per_sm;
@@ -693,7 +793,7 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     // Every launch of the pipeline is a programmatic dependent launch.  After the rotation-table kernel only the warps
     // that read the table wait for it; otherwise every thread waits for the kernel before it, whatever that was.
     lp.wait_all = (OP == OP_COMPOSE && n_rope > 0) ? 0 : 1;
-    kdn_status st = launch_tiles(ctx->env, OP, groups, gw, grid, smem, stream, lp, true, wide);
+    kdn_status st = launch_tiles(ctx->env, OP, groups, gw, grid, smem, stream, lp, true);
     if (st != KDN_OK) return st;
     ctx->launches++;
     ctx->last.op = OP;
@@ -707,7 +807,7 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     ctx->last.smem_bytes = (int32_t)smem;
     ctx->last.n_tiles = (uint32_t)tiles;
     ctx->last.rows_per_tile = rows_per_tile;
-    ctx->last.rows_kernel = wide ? 1 : 0;
+    ctx->last.rows_kernel = 0;
     if (slot) {
         KDN_CUDA(cudaEventRecord(slot->done, stream));
         slot->used = true;

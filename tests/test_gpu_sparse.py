@@ -254,3 +254,51 @@ def test_keep_lists_over_short_rows_take_up_to_16_rows_per_tile(codec, heads, he
         assert np.array_equal(dev.pool_np(), ref)
     finally:
         dev.close()
+
+
+@pytest.mark.parametrize("codec", [RAW, INT8, INT4])
+@pytest.mark.parametrize("heads,head_dim", [(1, 64), (2, 128), (5, 64), (1, 16), (1, 24)])
+def test_rows_moved_one_by_one_at_the_edges_of_a_cta(codec, heads, head_dim):
+    """Keep-lists on the kernels that move token rows one by one: list lengths around the rows a CTA takes (128 and 256 rows of
+    64 elements, ...), rows of one vector, rows no vector divides (these stay in the tile pipeline), enough planes that a CTA goes
+    through several of them, raw and coded ops in one call.  Bit-exact."""
+    if codec != RAW and head_dim % 64:
+        pytest.skip("coded chunks need head_dim % 64 == 0")
+    shape = synth.TOY.with_(n_layers=24, n_kv_heads=heads, head_dim=head_dim, block_size=8, n_blocks=128)
+    dev = Device(shape, seed=91)
+    try:
+        K = dev.K
+        rng = np.random.default_rng(heads * 100 + codec)
+        host = dev.pool_np()
+        tab = rng.permutation(128)[:60].astype(np.int32)
+        rest = np.setdiff1d(np.arange(128), tab).astype(np.int32)
+        lists = [np.sort(rng.choice(480, n, replace=False)) for n in (1, 15, 63, 64, 65, 127, 128, 129, 255, 256, 257, 300)]
+        wants = [oracle.store(host, tab, 0, len(k), codec, keep=k) for k in lists]
+        raw_want = oracle.store(host, tab, 0, len(lists[4]), RAW, keep=lists[4])
+        ops, keeps, expect = [], [], []
+        for i in range(36):                                              # several planes a CTA
+            k, w = lists[i % 12], wants[i % 12]
+            buf = dev.chunk_buf(len(k), codec)
+            ops.append(dev.op(dev.table(tab), 0, buf, len(k), codec))
+            keeps.append(dev_list(dev, k).data_ptr())
+            expect.append((buf, w))
+        raw_buf = dev.chunk_buf(65, RAW)
+        raw_op = dev.op(dev.table(tab), 0, raw_buf, 65, RAW)
+        K.kdn_store_sparse(dev.ctx, dev.pool_id, ops + [raw_op], keeps + [keeps[4]], dev.stream.cuda_stream)
+        assert dev.sync() == 0
+        assert ("rows" in K.kdn_last_launch(dev.ctx)["kernel"]) == (heads * head_dim % 16 == 0)
+        for buf, w in expect + [(raw_buf, raw_want)]:
+            assert np.array_equal(to_np(buf), w)
+        dtab = rng.permutation(rest)[:60].astype(np.int32)
+        for i in range(12):                                              # codes only, then with a raw op beside them
+            ref = dev.pool_np()
+            extra = [dev.op(dev.table(tab), 0, raw_buf, 65, RAW)] if i == 11 else []
+            K.kdn_retrieve_sparse(dev.ctx, dev.pool_id, [dev.op(dev.table(dtab), 0, expect[i][0], len(lists[i]), codec)] + extra,
+                                  [keeps[i]] + [keeps[4]] * len(extra), dev.stream.cuda_stream)
+            assert dev.sync() == 0
+            oracle.retrieve(ref, dtab, 0, len(lists[i]), codec, wants[i], keep=lists[i])
+            if extra:
+                oracle.retrieve(ref, tab, 0, 65, RAW, raw_want, keep=lists[4])
+            assert np.array_equal(dev.pool_np(), ref), i
+    finally:
+        dev.close()
