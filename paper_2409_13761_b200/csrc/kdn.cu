@@ -37,7 +37,6 @@ constexpr int kMaxOpsPerLaunch = 4096;
 constexpr unsigned kMaxTilesPerLaunch = 0x7fff0000u;
 constexpr size_t kDefaultSlabBytes = (size_t)256 << 20;
 constexpr unsigned kTdCols = 128;           // channels per CTA of the token-delta kernels
-constexpr unsigned kKcCols = 256;           // channels per CTA of the key-plane store of the per-channel key codecs
 
 struct Pool {
     int L, H, D, bs;
@@ -420,20 +419,15 @@ kdn_status ensure_table(RingSlot *slot, int n_rope, int half)
 kdn_status launch_key_planes(kdn_ctx *ctx, const Pool &pool, const DevOp *inl, const DevOp *d_ops, int n, int groups, int layers, cudaStream_t stream)
 {
     const unsigned row_elems = (unsigned)pool.H * (unsigned)pool.D;
-    // channels per CTA: at most 256 (36 KiB of shared memory, six CTAs per SM), a multiple of eight that divides the row
-    unsigned n_split = 1;
-    while (row_elems / n_split > kKcCols && row_elems % (n_split * 2u * 8u) == 0u) n_split *= 2u;
-    const unsigned cols = row_elems / n_split;
-    const size_t kc_smem = kc_smem_bytes(cols);
-    if (kc_smem > (size_t)ctx->env.smem_optin) return KDN_E_UNSUPPORTED;
-    unsigned kc_threads = (cols / 8u + 7u) / 8u * 32u;       // a warp per 64 channels
-    if (kc_threads > 512u) kc_threads = 512u;
-    if (kc_threads < 64u) kc_threads = 64u;
+    // channels per CTA: a multiple of 64 that divides the row, as many as the kernel takes if that can be
+    unsigned cols = row_elems < kKcCols ? row_elems : kKcCols;
+    while (row_elems % cols) cols -= 64u;
     KcLaunch kp{};
     kp.one = 1.0f;
-    kp.wait_limit_ns = ctx->wait_limit_ns;
     kp.cols = cols;
-    kp.n_split = n_split;
+    kp.n_split = row_elems / cols;
+    kp.bs_shift = -1;
+    for (int b = 0; b < 31; ++b) if (pool.bs == 1 << b) kp.bs_shift = b;
     kp.ops = d_ops;
     kp.n_ops = n;
     kp.k_layers = pool.d_k;
@@ -442,11 +436,7 @@ kdn_status launch_key_planes(kdn_ctx *ctx, const Pool &pool, const DevOp *inl, c
     kp.row_elems = row_elems;
     kp.status = ctx->d_status;
     if (inl) std::memcpy(kp.inline_ops, inl, sizeof(DevOp) * (size_t)n);
-    int per_sm = 0;                                          // first sight of the kernel raises its shared-memory limit
-    kdn_status r = ctx->env.resident(kdn_store_kc_kernel, (int)kc_threads, kc_smem, &per_sm);
-    if (r != KDN_OK) return r;
-    if (per_sm < 1) return KDN_E_UNSUPPORTED;
-    kdn_store_kc_kernel<<<dim3((unsigned)groups * n_split, (unsigned)layers, (unsigned)n), kc_threads, kc_smem, stream>>>(kp);
+    kdn_store_kc_kernel<<<dim3((unsigned)groups * kp.n_split, (unsigned)layers, (unsigned)n), cols / 2u, 0, stream>>>(kp);
     KDN_CUDA(cudaGetLastError());
     ctx->launches++;
     return KDN_OK;
@@ -792,7 +782,7 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     const int gw = ctx->tuning.group_warps > 0 ? ctx->tuning.group_warps : def.gw;
     // Every launch of the pipeline is a programmatic dependent launch.  After the rotation-table kernel only the warps
     // that read the table wait for it; otherwise every thread waits for the kernel before it, whatever that was.
-    lp.wait_all = (OP == OP_COMPOSE && n_rope > 0) ? 0 : 1;
+    lp.wait_all = (OP == OP_COMPOSE && n_rope > 0) ? 0 : kc_groups > 0 ? 2 : 1;
     kdn_status st = launch_tiles(ctx->env, OP, groups, gw, grid, smem, stream, lp, true);
     if (st != KDN_OK) return st;
     ctx->launches++;

@@ -112,8 +112,10 @@ struct Launch {
     unsigned long long wait_limit_ns;   // a pipeline wait gives up after this long (the drain waits keep kWaitLimitNs)
     int rows_per_tile;        // keep-list ops: listed token rows per tile (1: one row per tile)
     int wait_all;             // the launch may start while the kernel before it in the stream still runs (programmatic
-                              // dependent launch): every thread waits for that kernel before it touches global memory.
-                              // 0: only the warps that read the rotation table wait (the kernel before is the table kernel)
+                              // dependent launch).  1: every thread waits for that kernel before it touches global memory.
+                              // 0: only the warps that read the rotation table wait (the kernel before is the table kernel).
+                              // 2: they wait before they leave (the kernel before, itself an ordinary launch, stores the key
+                              // planes of the same chunks: the two may overlap, and what comes behind this one waits for both)
     float one;                // 1.0f, as a launch parameter: the coding loops form "product + constant" as
                               // fma(product, one, constant), and with a multiplier the assembler cannot see there
                               // is nothing it could contract with the multiply before it (the codecs round twice)
@@ -867,7 +869,7 @@ __device__ __forceinline__ void tile_pipeline(const Launch &P)
         fence_async_smem();
     }
     __syncthreads();
-    if (P.wait_all) dependency_wait();                      // returns at once when the launch was an ordinary one
+    if (P.wait_all == 1) dependency_wait();                 // returns at once when the launch was an ordinary one
 
     const unsigned grid = gridDim.x, bid = blockIdx.x;
     const unsigned n_my = P.n_tiles > bid ? (P.n_tiles - bid + grid - 1u) / grid : 0u;
@@ -1093,6 +1095,7 @@ __device__ __forceinline__ void tile_pipeline(const Launch &P)
             if (st >= (unsigned)S) { st -= (unsigned)S; ph ^= 1u; }
         }
     }
+    if (P.wait_all == 2) dependency_wait();
     __syncthreads();
 }
 
@@ -1130,155 +1133,78 @@ __device__ __forceinline__ long long group_row_pos(const DevOp &op, unsigned g, 
 
 // Storing the key planes of a per-channel key codec needs, for every channel, the largest magnitude over 64 tokens
 // before the first code can be formed, so it does not fit the streaming tile pipeline.  One CTA takes one
-// (op, layer, 64-token group, slice of `cols` channels): the slice of the group's token rows is brought into shared
-// memory with bulk copies (one per token row; one per pool block when the slice is the whole row); pass 1 reduces
-// |x| per channel over four token slices; one thread per channel combines them, forms scale and reciprocal
-// (two IEEE divides) and writes the scale; pass 2 codes each element with its channel's reciprocal
-// and writes the codes straight to the chunk.  Several CTAs share an SM (the host picks `cols` so that they fit), so
-// one CTA's loads overlap the arithmetic of the others.
-// The host guarantees: block_size divides 64, the op's token offset is a multiple of block_size, row_elems % 64 == 0,
-// cols % 8 == 0 and cols divides row_elems.
-// Shared memory: 64 * cols * 2 (rows) + 4 * cols * 2 (slice maxima) + cols * 4 (reciprocals) + 16.
+// (op, layer, 64-token group, slice of `cols` channels), a warp 64 of the channels for all 64 tokens: lane (j, q) octet j in token
+// quarter q, sixteen 16-byte loads straight into registers (no shared tile: every value is used by one thread only).  The group's largest
+// magnitudes meet through two shuffles, each lane forms the scale and the reciprocal of two of its octet's channels, and
+// four more shuffles hand every lane the reciprocals of all eight; then it codes its tokens and writes them straight to the chunk.
+// Bound by memory and by the latency of a CTA's two phases (20 warps an SM at 96 registers).  8B shape, 16 chunks of 512 tokens, int8: the
+// whole store 295 us with a tile in shared memory filled by 64 bulk copies, 274 us this way; int4 276 -> 246 us.  (128 or 256 channels a CTA:
+// the same; 64 or 512: 2-4 % slower; six CTAs an SM spill: 289.)
+// The host guarantees: row_elems % 64 == 0, cols % 64 == 0 and cols divides row_elems; for dense ops block_size divides 64 and the op's
+// token offset is a multiple of block_size.
 struct KcLaunch {
     const DevOp *ops;         // device array, or nullptr: inline_ops
     int n_ops;
     void *const *k_layers;
     long long n_blocks;
     int bs;
+    int bs_shift;             // log2(bs), -1 where bs is not a power of two
     unsigned row_elems;
     unsigned cols;            // channels per CTA
     unsigned n_split;         // row_elems / cols
     int *status;
     float one;                // 1.0f (see Launch::one)
-    unsigned long long wait_limit_ns;   // the wait for the tile gives up after this long
     DevOp inline_ops[kInlineOps];
 };
 
-constexpr unsigned kKcSlices = 4;                          // token slices in pass 1 and pass 2
-constexpr unsigned kKcTok = 64u / kKcSlices;              // tokens per slice
-__host__ __device__ inline size_t kc_smem_bytes(unsigned cols)
-{
-    return (size_t)64 * cols * 2u + 16u;                   // the tile, the barrier and the abort word
-}
+constexpr unsigned kKcTok = 16u;                          // tokens of a lane
+constexpr unsigned kKcCols = 256u;                        // channels per CTA at most, a warp per 64
 
-__global__ void __launch_bounds__(512) kdn_store_kc_kernel(const __grid_constant__ KcLaunch P)
+__global__ void __launch_bounds__(kKcCols / 2u, 5) kdn_store_kc_kernel(const __grid_constant__ KcLaunch P)
 {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ unsigned long long rows[64];                 // pool addresses of the group's token rows (slice start)
+    release_dependents();                                   // the value planes' kernel shares nothing with this one: it may start as this one drains
     const DevOp *ops = P.ops ? P.ops : P.inline_ops;
-    const DevOp op = ops[blockIdx.z];
-    if (op.codec < 3) return;
+    const DevOp &op = ops[blockIdx.z];
+    if (op.codec != 3 && op.codec != 4) return;
     const unsigned g = blockIdx.x / P.n_split, part = blockIdx.x - g * P.n_split, li = blockIdx.y;
-    const unsigned n_groups = ((unsigned)op.T + 63u) >> 6;
+    const unsigned T = (unsigned)op.T, n_groups = (T + 63u) >> 6;
     if (g >= n_groups || li >= (unsigned)op.nl) return;
     const bool int4 = op.codec == 4;
     const float qmax = int4 ? 7.0f : 127.0f;
-    const unsigned RE = P.row_elems, C = P.cols, c0 = part * C;
-    const unsigned t0 = g << 6;
-    const unsigned n_tok = (unsigned)op.T - t0 < 64u ? (unsigned)op.T - t0 : 64u;
-
-    unsigned char *X = smem_raw;                                             // [n_tok][C] bf16
-    unsigned long long *bar_mem = reinterpret_cast<unsigned long long *>(X + (size_t)64 * C * 2u);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(bar_mem + 1);
-    const uint32_t bar = smem_u32(bar_mem);
-    const int tid = (int)threadIdx.x;
-
-    if (tid == 0) {
-        mbar_init(bar, 1u);
-        *abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        fence_async_smem();
+    const unsigned RE = P.row_elems, c0 = part * P.cols, t0 = g << 6;
+    const unsigned n_tok = T - t0 < 64u ? T - t0 : 64u, tid = threadIdx.x;
+    bool bad = false;
+    const unsigned char *base = reinterpret_cast<const unsigned char *>(P.k_layers[op.l0 + (int)li]);
+    for (unsigned t = tid; t < n_tok; t += blockDim.x) {
+        const long long pos = group_row_pos(op, g, t);
+        const long long blk = P.bs_shift >= 0 ? pos >> P.bs_shift : pos / P.bs;
+        const long long id = pos < 0 ? -1 : (long long)__ldg(op.table + blk);
+        if (id < 0 || id >= P.n_blocks) bad = true;
+        else rows[t] = (unsigned long long)(base + ((unsigned long long)(id * P.bs + (pos - blk * P.bs)) * RE + c0) * 2ull);
     }
-    __syncthreads();
-    if (tid < 32) {
-        // warp 0 brings the rows in: lane r takes token rows r and r + 32, each found through its own table entry
-        const unsigned char *base = reinterpret_cast<const unsigned char *>(P.k_layers[op.l0 + (int)li]);
-        long long id[2] = { 0, 0 }, pos[2] = { 0, 0 };
-        bool bad = false;
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const unsigned t = (unsigned)tid + 32u * (unsigned)k;
-            if (t < n_tok) {
-                pos[k] = group_row_pos(op, g, t);
-                if (pos[k] < 0) { bad = true; continue; }
-                id[k] = __ldg(op.table + pos[k] / P.bs);
-                if (id[k] < 0 || id[k] >= P.n_blocks) bad = true;
-            }
-        }
-        if (__any_sync(0xffffffffu, bad)) {
-            if (tid == 0) {
-                atomicCAS(P.status, 0, kStatusRange);
-                *abort_flag = 1;                                              // nothing is loaded, nothing is written
-            }
-        } else {
-            if (tid == 0) mbar_arrive_expect_tx(bar, n_tok * C * 2u);
-            __syncwarp();
-            if (P.n_split == 1u && op.list_mode == 0) {
-                // the whole row: a block's tokens are contiguous in the pool, one copy per block (pieces <= 32 KiB)
-                if (tid == 0) {
-                    const long long first_block = (op.off + (long long)t0) / P.bs;
-                    for (unsigned t = 0; t < n_tok; t += (unsigned)P.bs) {
-                        const unsigned k = n_tok - t < (unsigned)P.bs ? n_tok - t : (unsigned)P.bs;
-                        const long long b = __ldg(op.table + first_block + t / (unsigned)P.bs);
-                        const unsigned char *src = base + (unsigned long long)b * P.bs * RE * 2ull;
-                        const unsigned bytes = k * RE * 2u;
-                        for (unsigned o = 0; o < bytes; o += 32768u)
-                            bulk_g2s(smem_u32(X + (size_t)t * RE * 2u + o), src + o, bytes - o < 32768u ? bytes - o : 32768u, bar);
-                    }
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    const unsigned t = (unsigned)tid + 32u * (unsigned)k;
-                    if (t < n_tok) {
-                        const unsigned slot = (unsigned)(pos[k] % P.bs);
-                        const unsigned char *src = base + (((unsigned long long)id[k] * P.bs + slot) * RE + c0) * 2ull;
-                        bulk_g2s(smem_u32(X + (size_t)t * C * 2u), src, C * 2u, bar);
-                    }
-                }
-            }
-        }
-    }
-    __syncthreads();
-    if (*abort_flag) return;
-    const bool landed = mbar_wait(bar, 0u, abort_flag, P.wait_limit_ns);
-    if (!__syncthreads_and(landed)) {                                         // all threads leave together
-        if (tid == 0) {
-            atomicCAS(P.status, 0, kStatusTimeout);
-            // one more bounded wait, so that the CTA does not leave while a copy into its shared memory is in flight
-            const unsigned long long t0 = global_timer_ns();
-            while (!mbar_try_wait(bar, 0u))
-                if (global_timer_ns() - t0 > kWaitLimitNs) break;
-        }
+    if (__syncthreads_or(bad)) {                            // nothing is loaded, nothing is written
+        if (tid == 0) atomicCAS(P.status, 0, kStatusRange);
         return;
     }
-
-    // From here on the warps do not meet again: a warp owns 64 channels (eight octets) for all 64 tokens, lane (j, q)
-    // takes octet j of them in token quarter q.  The group's largest magnitudes meet through two shuffles, each lane
-    // forms the scale and the reciprocal of two of its octet's channels, and four more shuffles hand every lane the
-    // reciprocals of all eight.
-    const unsigned octets = C >> 3;
-    const unsigned lane = (unsigned)tid & 31u, j = lane & 7u, q = lane >> 3;
-    const unsigned o = ((unsigned)tid >> 5) * 8u + j;
-    const bool act = o < octets;
-    const unsigned ta = q * kKcTok, tb = ta + kKcTok < n_tok ? ta + kKcTok : n_tok;
-    const unsigned char *Xo = X + (size_t)o * 16u;
-    // pass 1: the largest magnitudes of the lane's octet over its tokens, as packed bf16 pairs
-    uint32_t m0 = 0u, m1 = 0u, m2 = 0u, m3 = 0u;
-    if (act) {
-        if (n_tok == 64u) {                                                   // a full group: a fixed trip count, loads batched
+    const unsigned lane = tid & 31u, j = lane & 7u, q = lane >> 3;
+    const unsigned o = (tid >> 5) * 8u + j;                  // octet of the slice (whole warps have channels: cols % 64 == 0)
+    const unsigned ta = q * kKcTok;
+    const bool full = n_tok == 64u;
+    uint4 x[kKcTok];
+    if (full) {
 #pragma unroll
-            for (unsigned i = 0; i < kKcTok; ++i) {
-                const uint4 x = lds128(Xo + (size_t)(ta + i) * C * 2u);
-                m0 = maxabs_bf16x2(m0, x.x); m1 = maxabs_bf16x2(m1, x.y);
-                m2 = maxabs_bf16x2(m2, x.z); m3 = maxabs_bf16x2(m3, x.w);
-            }
-        } else {
-            for (unsigned t = ta; t < tb; ++t) {
-                const uint4 x = lds128(Xo + (size_t)t * C * 2u);
-                m0 = maxabs_bf16x2(m0, x.x); m1 = maxabs_bf16x2(m1, x.y);
-                m2 = maxabs_bf16x2(m2, x.z); m3 = maxabs_bf16x2(m3, x.w);
-            }
-        }
+        for (unsigned i = 0; i < kKcTok; ++i) x[i] = __ldg(reinterpret_cast<const uint4 *>(rows[ta + i]) + o);
+    } else {
+#pragma unroll
+        for (unsigned i = 0; i < kKcTok; ++i)
+            x[i] = ta + i < n_tok ? __ldg(reinterpret_cast<const uint4 *>(rows[ta + i]) + o) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    uint32_t m0 = 0u, m1 = 0u, m2 = 0u, m3 = 0u;
+#pragma unroll
+    for (unsigned i = 0; i < kKcTok; ++i) {
+        m0 = maxabs_bf16x2(m0, x[i].x); m1 = maxabs_bf16x2(m1, x[i].y);
+        m2 = maxabs_bf16x2(m2, x[i].z); m3 = maxabs_bf16x2(m3, x[i].w);
     }
 #pragma unroll
     for (int d = 8; d <= 16; d <<= 1) {
@@ -1292,7 +1218,7 @@ __global__ void __launch_bounds__(512) kdn_store_kc_kernel(const __grid_constant
     const float sc_lo = __fdiv_rn(a_lo, qmax), sc_hi = __fdiv_rn(a_hi, qmax);
     const bool ok_lo = sc_lo >= 1.17549435e-38f, ok_hi = sc_hi >= 1.17549435e-38f;   // smallest normal fp32; false for NaN too
     const float inv_lo = ok_lo ? __fdiv_rn(qmax, a_lo) : 0.0f, inv_hi = ok_hi ? __fdiv_rn(qmax, a_hi) : 0.0f;
-    if (act) {
+    {
         const unsigned long long per_layer = (unsigned long long)n_groups * RE + (((unsigned long long)op.T * RE) >> 6);
         float *g_scales = reinterpret_cast<float *>(op.scales) + (unsigned long long)li * per_layer + (unsigned long long)g * RE + c0 + o * 8u + q * 2u;
         g_scales[0] = ok_lo ? sc_lo : 0.0f;
@@ -1302,32 +1228,25 @@ __global__ void __launch_bounds__(512) kdn_store_kc_kernel(const __grid_constant
     const f32x2 i1 = pack2(__shfl_sync(0xffffffffu, inv_lo, (int)j + 8), __shfl_sync(0xffffffffu, inv_hi, (int)j + 8));
     const f32x2 i2 = pack2(__shfl_sync(0xffffffffu, inv_lo, (int)j + 16), __shfl_sync(0xffffffffu, inv_hi, (int)j + 16));
     const f32x2 i3 = pack2(__shfl_sync(0xffffffffu, inv_lo, (int)j + 24), __shfl_sync(0xffffffffu, inv_hi, (int)j + 24));
-    if (!act) return;
-    // pass 2: codes
     const float magic = 12582912.0f + (int4 ? 8.0f : 128.0f);
     const f32x2 magic2 = pack2(magic, magic);
     const f32x2 minus_m2 = pack2(-12582912.0f, -12582912.0f);
     const f32x2 k256 = pack2(256.0f, 256.0f);
     const f32x2 one2 = pack2(P.one, P.one);
-    const unsigned long long plane_elem = ((unsigned long long)li * 2ull * (unsigned long long)op.T + t0) * RE + c0 + o * 8u;   // K plane, token t0
-    auto code_row = [&](unsigned t) {
-        const uint4 x = lds128(Xo + (size_t)t * C * 2u);
-        const f32x2 r01 = add2_unfused(mul2(bf16x2_widen(x.x), i0), magic2, one2);
-        const f32x2 r23 = add2_unfused(mul2(bf16x2_widen(x.y), i1), magic2, one2);
-        const f32x2 r45 = add2_unfused(mul2(bf16x2_widen(x.z), i2), magic2, one2);
-        const f32x2 r67 = add2_unfused(mul2(bf16x2_widen(x.w), i3), magic2, one2);
+    const unsigned long long e0 = ((unsigned long long)li * 2ull * (unsigned long long)op.T + t0 + ta) * RE + c0 + o * 8u;   // K plane, the lane's first token
+    unsigned char *dst = op.data + (int4 ? e0 >> 1 : e0);
+    const unsigned step = int4 ? RE >> 1 : RE;
+#pragma unroll
+    for (unsigned i = 0; i < kKcTok; ++i) {
+        if (!full && ta + i >= n_tok) break;
+        const f32x2 r01 = add2_unfused(mul2(bf16x2_widen(x[i].x), i0), magic2, one2);
+        const f32x2 r23 = add2_unfused(mul2(bf16x2_widen(x[i].y), i1), magic2, one2);
+        const f32x2 r45 = add2_unfused(mul2(bf16x2_widen(x[i].z), i2), magic2, one2);
+        const f32x2 r67 = add2_unfused(mul2(bf16x2_widen(x[i].w), i3), magic2, one2);
         const f32x2 ga = gather2(r01, r23, minus_m2, k256), gb = gather2(r45, r67, minus_m2, k256);
-        const unsigned long long e = plane_elem + (unsigned long long)t * RE;
-        if (int4)
-            *reinterpret_cast<uint32_t *>(op.data + (e >> 1)) = __byte_perm(nibbles4_from(ga), nibbles4_from(gb), 0x5410) ^ 0x88888888u;
-        else
-            *reinterpret_cast<uint2 *>(op.data + e) = make_uint2(codes4_from(ga), codes4_from(gb));
-    };
-    if (n_tok == 64u) {
-#pragma unroll 4
-        for (unsigned i = 0; i < kKcTok; ++i) code_row(ta + i);
-    } else {
-        for (unsigned t = ta; t < tb; ++t) code_row(t);
+        if (int4) *reinterpret_cast<uint32_t *>(dst) = __byte_perm(nibbles4_from(ga), nibbles4_from(gb), 0x5410) ^ 0x88888888u;
+        else *reinterpret_cast<uint2 *>(dst) = make_uint2(codes4_from(ga), codes4_from(gb));
+        dst += step;
     }
 }
 
