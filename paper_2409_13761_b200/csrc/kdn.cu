@@ -36,6 +36,7 @@ constexpr int kRing = 8;                   // launches that may be queued before
 constexpr int kMaxOpsPerLaunch = 4096;
 constexpr unsigned kMaxTilesPerLaunch = 0x7fff0000u;
 constexpr size_t kDefaultSlabBytes = (size_t)256 << 20;
+constexpr size_t kOwnTableBytes = 16384;    // of a rotation table that every CTA makes for itself, at most
 constexpr unsigned kTdCols = 128;           // channels per CTA of the token-delta kernels
 
 struct Pool {
@@ -693,20 +694,36 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     const size_t smem_limit = (size_t)ctx->env.smem_optin;
     kdn_status fit = fit_stages(stages, groups, lag, ctx->tuning.stages <= 0, stage_bytes, ctas_per_sm, smem_limit, rows_per_tile);
     if (fit != KDN_OK) return fit;
-    const size_t smem = smem_bytes(stages, stage_bytes, rows_per_tile);
+    size_t smem = smem_bytes(stages, stage_bytes, rows_per_tile);
+    // A few rotations: every CTA makes its own table in shared memory, if that leaves the launch its CTAs -- no table kernel in front, no ring
+    // slot, and back-to-back calls overlap.  One 128-token chunk re-rotated: 12.8 -> 6.9 us (8B shape; one head: 12.4 -> 4.2); ten rows of a 1 GiB
+    // request cost what the table kernel did (418 -> 417 us).
+    int n_rotations = 0;
+    bool one_theta = true;
+    double theta = 0.0;
+    for (int i = 0; i < n; ++i)
+        if (hops[i].rotate) {
+            if (n_rotations++ == 0) theta = hops[i].rp.theta;
+            one_theta &= hops[i].rp.theta == theta;
+        }
+    const size_t table_bytes = (size_t)(n_rotations + 1) * (size_t)(pool.D / 2) * sizeof(float2);      // (and the frequencies)
+    const size_t off_rope = (smem + 15u) & ~(size_t)15u;
+    const bool own_table = OP == OP_COMPOSE && n_rotations > 0 && one_theta && n <= kInlineOps && table_bytes <= kOwnTableBytes &&
+                           (off_rope + table_bytes) * (size_t)ctas_per_sm <= smem_limit - 1024u * (size_t)ctas_per_sm;
+    if (own_table) smem = off_rope + table_bytes;
 
     // Few ops travel as kernel parameters; otherwise through a ring slot (pinned staging + device copy).  A ring
     // slot is also what owns the rotation table.
     const bool inl = n <= kInlineOps;
     RingSlot *slot = nullptr;
-    if (!inl || any_rot) {
+    if (!inl || (any_rot && !own_table)) {
         slot = &ctx->ring[ctx->ring_next++ % kRing];
         if (slot->used) KDN_CUDA(cudaEventSynchronize(slot->done));
     }
     Launch lp{};
     RopeInline rope_inl{};
     DevOp *h_ops = inl ? lp.inline_ops : slot->h_ops;
-    RopeParam *h_rope = inl ? rope_inl.p : (slot ? slot->h_rope : nullptr);
+    RopeParam *h_rope = own_table ? lp.inline_rope : inl ? rope_inl.p : slot ? slot->h_rope : nullptr;
 
     unsigned long long tiles = 0;
     int n_rope = 0;
@@ -736,7 +753,7 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
 
     if (!inl) KDN_CUDA(cudaMemcpyAsync(slot->d_ops, slot->h_ops, sizeof(DevOp) * (size_t)n, cudaMemcpyHostToDevice, stream));
     const int half = pool.D / 2;
-    if (n_rope) {
+    if (n_rope && !own_table) {
         {
             kdn_status r = ensure_table(slot, n_rope, half);
             if (r != KDN_OK) return r;
@@ -761,6 +778,7 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     lp.tile_elems = tile_elems;
     lp.tpb = tpb;
     lp.rope = slot ? slot->d_table : nullptr;
+    if (own_table) { lp.off_rope = (unsigned)off_rope; lp.n_rope = n_rope; }
     lp.status = ctx->d_status;
     lp.stages = stages;
     lp.stage_bytes = stage_bytes;
@@ -782,7 +800,7 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     const int gw = ctx->tuning.group_warps > 0 ? ctx->tuning.group_warps : def.gw;
     // Every launch of the pipeline is a programmatic dependent launch.  After the rotation-table kernel only the warps
     // that read the table wait for it; otherwise every thread waits for the kernel before it, whatever that was.
-    lp.wait_all = (OP == OP_COMPOSE && n_rope > 0) ? 0 : kc_groups > 0 ? 2 : 1;
+    lp.wait_all = (OP == OP_COMPOSE && n_rope > 0 && !own_table) ? 0 : kc_groups > 0 ? 2 : 1;
     kdn_status st = launch_tiles(ctx->env, OP, groups, gw, grid, smem, stream, lp, true);
     if (st != KDN_OK) return st;
     ctx->launches++;

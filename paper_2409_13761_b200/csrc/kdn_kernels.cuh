@@ -119,6 +119,9 @@ struct Launch {
     float one;                // 1.0f, as a launch parameter: the coding loops form "product + constant" as
                               // fma(product, one, constant), and with a multiplier the assembler cannot see there
                               // is nothing it could contract with the multiply before it (the codecs round twice)
+    unsigned off_rope;        // compose: not 0: the CTA makes its own rotation table, at this offset of shared memory, from inline_rope
+    int n_rope;               // rows of it
+    RopeParam inline_rope[kInlineOps];
     DevOp inline_ops[kInlineOps];
 };
 
@@ -560,6 +563,29 @@ __device__ __forceinline__ void dequantise_kc_tile(const unsigned char *B, const
     }
 }
 
+// Rotation table: row r, frequency i -> (cos, sin) of delta_r * theta_r^(-2i/D), evaluated in fp64 and
+// rounded once to fp32 (an fp32 angle would lose more than half a bf16 ulp at large position shifts).
+__device__ __forceinline__ double rope_freq(double theta, int i, int D) { return pow(theta, -2.0 * (double)i / (double)D); }
+__device__ __forceinline__ float2 rope_entry(long long delta, double inv_freq)
+{
+    double s, c;
+    sincos((double)delta * inv_freq, &s, &c);
+    return make_float2((float)c, (float)s);
+}
+// A CTA's own table, by the `n` threads that will read it: the frequencies first (one theta for all rows), then the rows.
+// (Not inlined: its registers are not the pipeline's.)
+__device__ __noinline__ void rope_fill(const Launch &P, double *freq, float2 *table, int t, int n)
+{
+    const int half = P.D >> 1;
+    for (int i = t; i < half; i += n) freq[i] = rope_freq(P.inline_rope[0].theta, i, P.D);
+    asm volatile("bar.sync 9, %0;" ::"r"(n) : "memory");
+    for (int idx = t; idx < P.n_rope * half; idx += n) {
+        const int r = idx / half;
+        table[idx] = rope_entry(P.inline_rope[r].delta, freq[idx - r * half]);
+    }
+    asm volatile("bar.sync 9, %0;" ::"r"(n) : "memory");
+}
+
 // Rotation coefficients a thread keeps in registers: (cos, sin, -sin) for 8 consecutive frequencies,
 // as four packed pairs each.
 struct RotCoef {
@@ -574,7 +600,7 @@ __device__ __forceinline__ void load_coef(RotCoef &rc, const float2 *table, int 
     const float4 *p = reinterpret_cast<const float4 *>(table + (size_t)rope * half + col);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const float4 v = __ldg(p + k);                     // (cos, sin) of frequencies 2k and 2k + 1
+        const float4 v = p[k];                             // (cos, sin) of frequencies 2k and 2k + 1
         rc.c[k] = pack2(v.x, v.z);
         rc.s[k] = pack2(v.y, v.w);
         rc.ns[k] = pack2(-v.y, -v.w);
@@ -869,7 +895,8 @@ __device__ __forceinline__ void tile_pipeline(const Launch &P)
         fence_async_smem();
     }
     __syncthreads();
-    if (P.wait_all == 1) dependency_wait();                 // returns at once when the launch was an ordinary one
+    if (P.wait_all == 1 && !(OP == OP_COMPOSE && warp != kLoaderWarp && warp != 1 + kGroups * kGW))
+        dependency_wait();                                  // (the compute warps of compose wait below) returns at once when the launch was an ordinary one
 
     const unsigned grid = gridDim.x, bid = blockIdx.x;
     const unsigned n_my = P.n_tiles > bid ? (P.n_tiles - bid + grid - 1u) / grid : 0u;
@@ -1027,8 +1054,18 @@ __device__ __forceinline__ void tile_pipeline(const Launch &P)
         const int ct = (tid - 32) % (int)kGT;
         RotCoef rc;
         rc.rope = -1; rc.col = 0xffffffffu;
-        // the rotation table is written by the kernel launched just before this one; only these warps read it
-        if (OP == OP_COMPOSE) dependency_wait();
+        const float2 *rope_table = P.rope;
+        if (OP == OP_COMPOSE) {
+            // a table of the CTA's own needs nothing from the kernel before; one in memory is written by the kernel launched
+            // just before this one, and only these warps read it
+            if (P.off_rope) {
+                double *freq = reinterpret_cast<double *>(smem_raw + P.off_rope);
+                float2 *own = reinterpret_cast<float2 *>(freq + (P.D >> 1));
+                rope_fill(P, freq, own, tid - 32, kGroups * (int)kGT);
+                rope_table = own;
+            }
+            dependency_wait();
+        }
         unsigned st = (unsigned)group;                        // S is a multiple of kGroups: st wraps exactly at S
         uint32_t ph = 0;
         for (unsigned slot = (unsigned)group; slot < n_my; slot += (unsigned)kGroups) {
@@ -1063,16 +1100,16 @@ __device__ __forceinline__ void tile_pipeline(const Launch &P)
                     }
                     if (flags & TF_KCHAN) {
                         if (OP == OP_COMPOSE && (flags & TF_ROTATE)) {
-                            if (flags & TF_INT4) rotate_tile<2, true>(A, B, Sc, n, (unsigned)P.D, P.rope, sm.desc[st].rope, rc, ct, kGT, P.row_elems);
-                            else rotate_tile<1, true>(A, B, Sc, n, (unsigned)P.D, P.rope, sm.desc[st].rope, rc, ct, kGT, P.row_elems);
+                            if (flags & TF_INT4) rotate_tile<2, true>(A, B, Sc, n, (unsigned)P.D, rope_table, sm.desc[st].rope, rc, ct, kGT, P.row_elems);
+                            else rotate_tile<1, true>(A, B, Sc, n, (unsigned)P.D, rope_table, sm.desc[st].rope, rc, ct, kGT, P.row_elems);
                         } else if (flags & TF_INT4) {
                             dequantise_kc_tile<true, OP != OP_COMPOSE>(B, Sc, A, n, P.row_elems, ct, kGT);
                         } else {
                             dequantise_kc_tile<false, OP != OP_COMPOSE>(B, Sc, A, n, P.row_elems, ct, kGT);
                         }
                     } else if (OP == OP_COMPOSE && (flags & TF_ROTATE)) {
-                        if (flags & TF_INT4) rotate_tile<2>(A, B, Sc, n, (unsigned)P.D, P.rope, sm.desc[st].rope, rc, ct, kGT);
-                        else rotate_tile<1>(A, B, Sc, n, (unsigned)P.D, P.rope, sm.desc[st].rope, rc, ct, kGT);
+                        if (flags & TF_INT4) rotate_tile<2>(A, B, Sc, n, (unsigned)P.D, rope_table, sm.desc[st].rope, rc, ct, kGT);
+                        else rotate_tile<1>(A, B, Sc, n, (unsigned)P.D, rope_table, sm.desc[st].rope, rc, ct, kGT);
                     } else if (flags & TF_INT4) {
                         if (n == kGT * 32u) dequantise4_tile(B, Sc, A, kGT * 32u, ct, kGT);
                         else dequantise4_tile(B, Sc, A, n, ct, kGT);
@@ -1082,7 +1119,7 @@ __device__ __forceinline__ void tile_pipeline(const Launch &P)
                     }
                     computed = true;
                 } else if (OP == OP_COMPOSE && (flags & TF_ROTATE)) {
-                    rotate_tile<0>(A, nullptr, nullptr, n, (unsigned)P.D, P.rope, sm.desc[st].rope, rc, ct, kGT);
+                    rotate_tile<0>(A, nullptr, nullptr, n, (unsigned)P.D, rope_table, sm.desc[st].rope, rc, ct, kGT);
                     computed = true;
                 }
             }
@@ -1250,24 +1287,19 @@ __global__ void __launch_bounds__(kKcCols / 2u, 5) kdn_store_kc_kernel(const __g
     }
 }
 
-// Rotation table: row r, frequency i -> (cos, sin) of delta_r * theta_r^(-2i/D), evaluated in fp64 and
-// rounded once to fp32 (an fp32 angle would lose more than half a bf16 ulp at large position shifts).
+// Few rows: passed as kernel parameters; more: params.
 struct RopeInline { RopeParam p[kInlineOps]; };
 
 __global__ void kdn_rope_table_kernel(const RopeParam *params, const __grid_constant__ RopeInline inl, int n_rows, int D,
                                       float2 *table)
 {
     release_dependents();                                  // the compose kernel may set up and start its loads now
-    if (!params) params = inl.p;                           // few rows: passed as kernel parameters
+    if (!params) params = inl.p;
     const int half = D >> 1;
     const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (long long)n_rows * half) return;
     const int r = (int)(idx / half), i = (int)(idx - (long long)r * half);
-    const double inv_freq = pow(params[r].theta, -2.0 * (double)i / (double)D);
-    const double phi = (double)params[r].delta * inv_freq;
-    double s, c;
-    sincos(phi, &s, &c);
-    table[idx] = make_float2((float)c, (float)s);
+    table[idx] = rope_entry(params[r].delta, rope_freq(params[r].theta, i, D));
 }
 
 }  // namespace kdn
