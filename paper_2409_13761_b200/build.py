@@ -5,11 +5,14 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libkdn.so")
+NATIVE = os.path.join(HERE, "_kdn_native.so")            # argument marshalling for kdn.py
+NATIVE_SOURCE = os.path.join(CSRC, "kdn_py.c")
 SOURCES = [os.path.join(CSRC, "kdn.cu"), os.path.join(CSRC, "kdn_shell.cu")]
 DEPS = SOURCES + [os.path.join(CSRC, "kdn_kernels.cuh"), os.path.join(CSRC, "kdn_rows.cuh"), os.path.join(CSRC, "kdn_td.cuh"), os.path.join(ROOT, "include", "kdn.h")]
 
@@ -28,7 +31,27 @@ def up_to_date() -> bool:
     return all(os.path.getmtime(d) <= t for d in DEPS)
 
 
+def native_up_to_date() -> bool:
+    return os.path.exists(NATIVE) and all(os.path.getmtime(d) <= os.path.getmtime(NATIVE)
+                                          for d in (NATIVE_SOURCE, os.path.join(ROOT, "include", "kdn.h")))
+
+
+def build_native(force: bool = False) -> str:
+    """Compile the extension module with the Python-side marshalling (needs a C compiler and Python's headers)."""
+    if not force and native_up_to_date():
+        return NATIVE
+    cc = shutil.which("gcc") or shutil.which("cc")
+    if not cc:
+        raise RuntimeError("no C compiler found")
+    tmp = NATIVE + ".%d.tmp" % os.getpid()
+    subprocess.run([cc, "-O2", "-Wall", "-shared", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"],
+                    NATIVE_SOURCE, "-o", tmp], check=True)
+    os.replace(tmp, NATIVE)
+    return NATIVE
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_native(force)
     if not force and up_to_date():
         return LIB
     tmp = LIB + ".%d.tmp" % os.getpid()

@@ -173,6 +173,30 @@ def _load() -> C.CDLL:
 lib = _load()
 
 
+def _load_native():
+    """The native marshalling of the per-request calls; None where it cannot be had (ctypes then does the same, slower)."""
+    try:
+        _build.build_native()
+    except Exception:                                 # no C compiler or no Python headers; a module built elsewhere may be there
+        pass
+    try:
+        from . import _kdn_native
+    except ImportError:
+        return None
+    return _kdn_native
+
+
+_native = _load_native()
+
+
+def _entry(name: str) -> int:
+    return C.cast(getattr(lib, name), C.c_void_p).value
+
+
+_STORE, _RETRIEVE, _COMPOSE, _STORE_SPARSE, _RETRIEVE_SPARSE = (
+    _entry(n) for n in ("kdn_store", "kdn_retrieve", "kdn_compose", "kdn_store_sparse", "kdn_retrieve_sparse"))
+
+
 class KdnError(RuntimeError):
     def __init__(self, status: int, where: str):
         self.status = int(status)
@@ -293,10 +317,14 @@ def kdn_validate_compose(desc: kdn_pool_desc, reqs: Sequence[ComposeReq]) -> int
 
 
 def kdn_store(ctx, pool_id: int, ops: Sequence[XferOp], stream: int = 0, side_stream: int = 0) -> None:
+    if _native is not None:
+        return _check(_native.call_xfer(_STORE, ctx, pool_id, ops, stream, side_stream), "kdn_store")
     _check(lib.kdn_store(ctx, pool_id, xfer_array(ops), len(ops), stream, side_stream), "kdn_store")
 
 
 def kdn_retrieve(ctx, pool_id: int, ops: Sequence[XferOp], stream: int = 0, side_stream: int = 0) -> None:
+    if _native is not None:
+        return _check(_native.call_xfer(_RETRIEVE, ctx, pool_id, ops, stream, side_stream), "kdn_retrieve")
     _check(lib.kdn_retrieve(ctx, pool_id, xfer_array(ops), len(ops), stream, side_stream), "kdn_retrieve")
 
 
@@ -319,10 +347,14 @@ def sparse_array(ops: Sequence[XferOp], keeps: Sequence[int]):
 
 def kdn_store_sparse(ctx, pool_id: int, ops: Sequence[XferOp], keeps: Sequence[int], stream: int = 0, side_stream: int = 0) -> None:
     """keeps[i]: device address of the int32 keep-list of ops[i] (ops[i].chunk.n_tokens entries)."""
+    if _native is not None:
+        return _check(_native.call_sparse(_STORE_SPARSE, ctx, pool_id, ops, keeps, stream, side_stream), "kdn_store_sparse")
     _check(lib.kdn_store_sparse(ctx, pool_id, sparse_array(ops, keeps), len(ops), stream, side_stream), "kdn_store_sparse")
 
 
 def kdn_retrieve_sparse(ctx, pool_id: int, ops: Sequence[XferOp], keeps: Sequence[int], stream: int = 0, side_stream: int = 0) -> None:
+    if _native is not None:
+        return _check(_native.call_sparse(_RETRIEVE_SPARSE, ctx, pool_id, ops, keeps, stream, side_stream), "kdn_retrieve_sparse")
     _check(lib.kdn_retrieve_sparse(ctx, pool_id, sparse_array(ops, keeps), len(ops), stream, side_stream), "kdn_retrieve_sparse")
 
 
@@ -358,6 +390,8 @@ def kdn_compose_select(ctx, pool_id: int, reqs: Sequence[ComposeReq], selects, s
 
 
 def kdn_compose(ctx, pool_id: int, reqs: Sequence[ComposeReq], stream: int = 0, side_stream: int = 0) -> None:
+    if _native is not None:
+        return _check(_native.call_compose(_COMPOSE, ctx, pool_id, reqs, stream, side_stream), "kdn_compose")
     _check(lib.kdn_compose(ctx, pool_id, compose_array(reqs), len(reqs), stream, side_stream), "kdn_compose")
 
 
