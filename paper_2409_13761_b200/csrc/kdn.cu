@@ -872,10 +872,9 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
         tp.n_split = n_split;
         while ((1u << tp.split_shift) < n_split) ++tp.split_shift;
         tp.word_row = cols * 4u;
-        tp.one = 1;
         tp.fone = 1.0f;
         for (unsigned i = 0; i < 12u; ++i) tp.pow2[i] = 1u << i;
-        tp.minus_two = -2;
+        tp.minus_one = -1;
         tp.bs_shift = -1;
         for (int b = 0; b < 31; ++b) if (pool.bs == 1 << b) tp.bs_shift = b;
         tp.status = ctx->d_status;

@@ -54,7 +54,7 @@ struct TdLaunch {
     unsigned split_shift;     // log2(n_split)
     unsigned words;           // decode: 32-bit words kept per sub-stream (the longest of the launch's codecs, and one more)
     int bs_shift;             // log2(bs), -1 where bs is not a power of two
-    int one, minus_two;       // 1 and -2 as launch parameters: see TdStream
+    int minus_one;            // -1 as a launch parameter: see TdStream
     float fone;               // 1.0f (see Launch::one)
     unsigned pow2[12];        // 1 << i: multiply-adds by these stay on the multiplier's pipe (as literals they become shifts)
     unsigned word_row;        // decode: bytes of one row of interleaved words (4 * cols), for the same reason
@@ -735,17 +735,17 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 14 : 1) kdn
 // One sub-stream on its way through the decoder.  Everything is kept in the form that takes the fewest operations of the
 // pipe that shifts, compares and logic share (it issues every other cycle and is what bounds this kernel):
 //  * the words hold the complement of the stream, so the ones of the unary part are leading zeros.  With h the next 32
-//    bits, n = clz(h), z = (h << n) >> (31 - k) = 2^(k+1) - 1 - rem, and v = z - n 2^k = c - u with c = 2^(k+1) - 1, the
-//    symbol u never appears itself;
-//  * 2 e (e = the signed code or code difference) is u for even u and -(u + 1) for odd u, i.e. with s = v & 1
-//    2 e = s (2 c + 1 - 2 v) + v - c - 1: multiply-adds, which run on the other integer pipe (their small constant factors
-//    arrive as launch parameters: known ones would be turned back into shifts and adds);
+//    bits, n = clz(h) and len = n + k + 1, z = h >> (32 - len) = 2^(k+1) - 1 - rem, and v = z - n 2^k = c - u with
+//    c = 2^(k+1) - 1, the symbol u never appears itself;
+//  * 2 e (e = the signed code or code difference) is u for even u and -(u + 1) for odd u, i.e. v - c - 1, or, where v is odd,
+//    2 c + 1 - v - c - 1: one predicated multiply-add (it runs on the other integer pipe; its constant factors arrive as launch
+//    parameters: known ones would be turned back into shifts and adds);
 //  * the running code is kept as the bits of the fp32 number 2^22 + 512 + q, whose unit in the last place is 1/2: adding
 //    2 e to the bits adds e to the number, and one subtraction gives q exactly.
 struct TdStream {
     uint32_t col;          // shared address of word 0 of the sub-stream
     unsigned bp;           // bits consumed
-    unsigned k1, sh;       // k + 1, 31 - k
+    unsigned nk1;          // -(k + 1)
     int kneg;              // -2^k
     int c21;               // 2 c + 1
     int d, c2;             // next = acc * d + c2 + ...: d = 1 in delta mode, else 0 and c2 holds the fresh start
@@ -760,20 +760,12 @@ __device__ __forceinline__ void td_stream_init(TdStream &s, uint32_t col, unsign
     const int c = (int)((2u << k) - 1u);
     s.col = col;
     s.bp = 0u;
-    s.k1 = k + 1u;
-    s.sh = 31u - k;
+    s.nk1 = 0u - (k + 1u);
     s.kneg = -(int)(1u << k);
     s.c21 = 2 * c + 1;
     s.d = (param & 8u) ? 1 : 0;
     s.c2 = -(c + 1) + ((param & 8u) ? 0 : kTdCodeBits);
     s.acc = kTdCodeBits;
-}
-// (PTX shifts by 32 and more give 0: a window of ones only)
-__device__ __forceinline__ uint32_t td_shl(uint32_t x, unsigned n)
-{
-    uint32_t r;
-    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(n));
-    return r;
 }
 template <unsigned kCols>
 __device__ __forceinline__ uint32_t td_window(const TdStream &s, unsigned row_b)
@@ -785,26 +777,24 @@ __device__ __forceinline__ uint32_t td_window(const TdStream &s, unsigned row_b)
     return __funnelshift_l(w1, w0, s.bp);
 }
 // The next symbol out of the window h, taken not to be an escape; returns the length of its unary part (15 and more: it was one)
-// and, in len, the length of the code word.
-__device__ __forceinline__ unsigned td_symbol(const TdLaunch &P, TdStream &s, uint32_t h, unsigned &len)
+// and, in nlen, minus the length of the code word (shifts take their count modulo 32: by nlen means by 32 - len).
+__device__ __forceinline__ unsigned td_symbol(const TdLaunch &P, TdStream &s, uint32_t h, unsigned &nlen)
 {
     unsigned n;
     asm("bfind.shiftamt.u32 %0, %1;" : "=r"(n) : "r"(h));
-    const int z = (int)(td_shl(h, n) >> s.sh);
-    const int v = (int)n * s.kneg + z;
-    len = n + s.k1;
-    s.bp += len;
-    const int a = v * P.minus_two + s.c21;
-    const int r = v * P.one + (s.acc * s.d + s.c2);
-    s.acc = (v & 1) * a + r;
+    nlen = s.nk1 - n;
+    int v = (int)n * s.kneg + (int)__funnelshift_r(h, 0u, nlen);
+    s.bp -= nlen;
+    asm("{ .reg .pred p; .reg .b32 t; and.b32 t, %0, 1; setp.ne.s32 p, t, 0; @p mad.lo.s32 %0, %0, %1, %2; }" : "+r"(v) : "r"(P.minus_one), "r"(s.c21));
+    s.acc = v + (s.acc * s.d + s.c2);
     return n;
 }
 // The same with escapes.
 __device__ __forceinline__ void td_symbol_any(const TdLaunch &P, TdStream &s, uint32_t h, unsigned raw_bits)
 {
     if ((h >> 17) != 0u) {                                  // fewer than fifteen ones
-        unsigned len;
-        td_symbol(P, s, h, len);
+        unsigned nlen;
+        td_symbol(P, s, h, nlen);
         return;
     }
     const int u = (int)((~h << 15) >> (32u - raw_bits));
@@ -815,7 +805,7 @@ __device__ __forceinline__ void td_symbol_any(const TdLaunch &P, TdStream &s, ui
 constexpr unsigned kTdStep = 4;                             // symbols of a stream between two looks for escapes
 // kTdStep symbols of two streams side by side, kWin of them out of one 32-bit window (code words of 4-bit codes are short:
 // four in a window; of 8-bit codes: two).  Taken to be no escapes and to fit their windows; where that was wrong, once more
-// with care.  (8B shape, 32 chunks of 512 tokens, 4-bit codes: a window a symbol 965 us, two 908, four 867.)
+// with care.  (8B shape, 32 chunks of 512 tokens, 4-bit codes, an earlier form: a window a symbol 965 us, two 908, four 867.)
 template <unsigned kCols, unsigned kWin>
 __device__ __forceinline__ void td_step(const TdLaunch &P, TdStream &x, TdStream &y, unsigned row_b, unsigned max_bits, unsigned raw_bits,
                                         int (&vx)[kTdStep], int (&vy)[kTdStep])
@@ -834,8 +824,8 @@ __device__ __forceinline__ void td_step(const TdLaunch &P, TdStream &x, TdStream
             unsigned lx, ly;
             const unsigned nx = td_symbol(P, x, hx, lx), ny = td_symbol(P, y, hy, ly);
             longest = max(longest, max(nx, ny));
-            hx = td_shl(hx, lx);
-            hy = td_shl(hy, ly);
+            hx = __funnelshift_r(0u, hx, lx);               // hx << length
+            hy = __funnelshift_r(0u, hy, ly);
             vx[i + j] = x.acc; vy[i + j] = y.acc;
         }
         most = max(most, max(x.bp - from_x, y.bp - from_y));
@@ -851,17 +841,18 @@ __device__ __forceinline__ void td_step(const TdLaunch &P, TdStream &x, TdStream
     }
 }
 
-// Bound by the integer pipes (8B shape, 4-bit codes: ALU pipe about 70 %, issue slots 80 %, DRAM 30 %); what was done
-// about it is at TdStream and td_step.  A thread decodes two channels side by side -- neighbours, whose bf16 values make one
-// word, or, where keys are re-rotated, the two channels of a rotation pair -- so that one stream's chain of dependent
-// operations hides the other's, and writes finished values into the rows: no pass over codes.  Half of the rows at a time
-// keeps a CTA of 64 threads at 16 KiB of shared memory, fourteen (8-bit codes: ten) to an SM.  The rows leave with 128-bit
-// stores, sixteen lanes to a 256-byte piece of a token row.  8B shape, 32 chunks of 512 tokens, 4-bit codes: 1727 -> 867 us
-// against one thread per channel, a code tile and a separate pass that multiplied.
+// Bound by instruction issue and the integer pipes (8B shape, 4-bit codes: issue slots 83 %, multiply-add pipe 67 %, logic 55 %, DRAM 45 %;
+// 18 instructions a symbol); what was done about it is at TdStream and td_step.  A thread decodes two channels side by side --
+// neighbours, whose bf16 values make one word, or, where keys are re-rotated, the two channels of a rotation pair -- so that one
+// stream's chain of dependent operations hides the other's, and writes finished values into the rows: no pass over codes.  Half
+// of the rows at a time keeps a CTA of 64 threads at 16 KiB of shared memory, twelve (8-bit codes: ten) to an SM; all rows at a time
+// are 15 % slower.  The rows leave with 128-bit stores, sixteen lanes to a 256-byte piece of a token row.  8B shape, 32 chunks of 512
+// tokens, 4-bit codes: 1728 us with one thread per channel, a code tile and a separate pass that multiplied, 730 us this way; 8-bit
+// codes 1765 -> 900 us.
 // kCols: channels per CTA when known at compile time (the usual slice; every stride in the decoding loop is then an
 // immediate), 0: taken from the launch record.
 template <bool kCompose, unsigned kCols>
-__global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 14 : 1) kdn_td_decode_kernel(const __grid_constant__ TdLaunch P)
+__global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 12 : 1) kdn_td_decode_kernel(const __grid_constant__ TdLaunch P)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const TdSlice s = td_slice(P);
@@ -1057,11 +1048,21 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 14 : 1) kdn
             }
         }
         __syncthreads();
-        // rows -> pool blocks
-        for (unsigned v = tid; v < nt * vecs; v += nthreads) {
-            const unsigned t = v / vecs, c = v - t * vecs;
-            const unsigned long long d = rows[t0 + t];
-            if (d) *reinterpret_cast<uint4 *>(d + 16ull * c) = lds128(A + (size_t)v * 16u);
+        // rows -> pool blocks, sixteen bytes a lane
+        if (kCols && nt == kTdHalf) {
+            constexpr unsigned kLanes = kCols ? kCols / 8u : 1u, kStep = kCols ? kCols / 2u / kLanes : 1u;      // lanes a row, rows a pass
+            const unsigned c = tid & (kLanes - 1u), r = tid / kLanes;
+#pragma unroll
+            for (unsigned i = 0; i < kTdHalf; i += kStep) {
+                const unsigned long long d = rows[t0 + i + r];
+                if (d) *reinterpret_cast<uint4 *>(d + 16ull * c) = lds128(A + (size_t)((i + r) * kLanes + c) * 16u);
+            }
+        } else {
+            for (unsigned v = tid; v < nt * vecs; v += nthreads) {
+                const unsigned t = v / vecs, c = v - t * vecs;
+                const unsigned long long d = rows[t0 + t];
+                if (d) *reinterpret_cast<uint4 *>(d + 16ull * c) = lds128(A + (size_t)v * 16u);
+            }
         }
         __syncthreads();
     }
