@@ -65,7 +65,7 @@ struct TdLaunch {
     DevOp inline_ops[kInlineOps];
 };
 
-// Shared memory of the encoder: the rows' addresses, a little scratch, the stream staging area.
+// Shared memory of the encoder: the rows' addresses, a little scratch, the stream staging area, a word per channel.
 // Behind the encoder's staging area: room for the longest thing a channel could write from the last planned byte on (64
 // appends, a word each, and the last word), so that a sub-stream that came out longer than planned -- the pool changed under the store --
 // garbles the chunk's bytes, which the caller has then forfeited, but never leaves the area.
@@ -78,10 +78,8 @@ constexpr unsigned kTdEncodeHead = 66u * 8u + 32u * 4u + 112u;      // a multipl
 // then still inside the CTA's memory, and garbage either way.
 constexpr unsigned kTdHalf = 32;                            // rows between two write-outs
 __host__ __device__ inline unsigned td_words(int codec) { return td_max_len(codec) / 4u + 1u; }   // the longest sub-stream, and the word after
-__host__ __device__ inline size_t td_encode_smem_bytes(unsigned cols, unsigned words)
-{
-    return kTdEncodeHead + (size_t)cols * (words - 1u) * 4u + 32u + kTdStageSlack;
-}
+__host__ __device__ inline size_t td_stage_bytes(unsigned cols, unsigned words) { return (size_t)cols * (words - 1u) * 4u + 32u + kTdStageSlack; }
+__host__ __device__ inline size_t td_encode_smem_bytes(unsigned cols, unsigned words) { return kTdEncodeHead + td_stage_bytes(cols, words) + 4u * cols; }
 __host__ __device__ inline size_t td_decode_words_bytes(unsigned cols, unsigned words) { return (size_t)words * cols * 4u; }
 __host__ __device__ inline size_t td_decode_rows_bytes(unsigned cols, unsigned words)
 {
@@ -509,45 +507,48 @@ __global__ void __launch_bounds__(kTdScanThreads) kdn_td_scan_kernel(const __gri
 struct TdOut {
     uint32_t acc;          // the bits not yet written, in the low (bits mod 32) bits; garbage above them
     unsigned bits;         // bits so far, those of the first word that are not the sub-stream's own included
-    uint32_t wp;           // shared address of the word being filled
-    unsigned k, len0;      // Rice parameter; k + 1 - (bits of 2^23 >> k)
+    uint32_t wp, next;     // shared address the word being filled goes to, and the one after it
+    unsigned k, nlen0;     // Rice parameter; (bits of 2^23 >> k) - (k + 1)
     uint32_t kmask, kbit;  // 2^k - 1, 2^k
-    unsigned limit;        // k + 16: code words this long are escapes
+    int limit;             // -(k + 16): code words this long are escapes
 };
 constexpr unsigned kTdLoad = 8;                              // tokens loaded ahead
 constexpr uint32_t kTdUZero = 0x4B000000u;                   // bits of 2^23
 
-__device__ __forceinline__ void td_out_init(TdOut &o, uint32_t addr, unsigned param)
+// addr: where the sub-stream goes in the staging area; aside: a word of the thread's own, for the first word until the end
+__device__ __forceinline__ void td_out_init(TdOut &o, uint32_t addr, uint32_t aside, unsigned param)
 {
     o.k = param & 7u;
     o.kbit = 1u << o.k;
     o.kmask = o.kbit - 1u;
-    o.len0 = o.k + 1u - (kTdUZero >> o.k);
-    o.limit = o.k + 16u;
+    o.nlen0 = (kTdUZero >> o.k) - (o.k + 1u);
+    o.limit = -(int)(o.k + 16u);
     o.acc = 0u;
     o.bits = (addr & 3u) * 8u;
-    o.wp = addr & ~3u;
+    o.wp = aside;
+    o.next = (addr & ~3u) + 4u;
 }
-// Append the low `len` bits of w (1 <= len <= 32, nothing above them).  A word that is full is OR-ed into the staging area: the
-// first and the last word of a sub-stream also hold bits of its neighbours.  (The shifts take their count modulo 32.)
-__device__ __forceinline__ void td_append(TdOut &o, uint32_t w, unsigned len)
+// Append the low `len` bits of w (1 <= len <= 32, nothing above them; nlen = -len).  (Shifts take their count modulo 32.)  Words go
+// out with plain predicated stores, since all but the first and the last are the sub-stream's own: the first, which its neighbour's last
+// bits share, is kept aside.  (An OR into the staging area for every word cost a
+// branch round the instruction: store of 16 chunks 923 -> 898 us.)
+__device__ __forceinline__ void td_append(TdOut &o, uint32_t w, unsigned nlen)
 {
-    const uint32_t left = __funnelshift_l(0u, w, 0u - len);                 // left-aligned
+    const uint32_t left = __funnelshift_l(0u, w, nlen);                     // left-aligned
     const uint32_t word = __funnelshift_r(left, o.acc, o.bits);
-    const unsigned bits = o.bits + len;
-    o.acc = __funnelshift_r(left, o.acc, 0u - len);
-    // (predicated by hand: a branch around two instructions costs more than they do)
-    asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p red.shared.or.b32 [%0], %1; @p add.u32 %0, %0, 4; }"
-                 : "+r"(o.wp) : "r"(word), "r"((o.bits ^ bits) & ~31u) : "memory");
+    const unsigned bits = o.bits - nlen;
+    o.acc = __funnelshift_r(left, o.acc, nlen);
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %3, 0; @p st.shared.u32 [%0], %2; @p mov.b32 %0, %1; @p add.u32 %1, %1, 4; }"
+                 : "+r"(o.wp), "+r"(o.next) : "r"(word), "r"((o.bits ^ bits) & ~31u) : "memory");
     o.bits = bits;
 }
 // One symbol, escapes included; ub: bits of 2^23 + u.
 __device__ __forceinline__ void td_append_any(TdOut &o, uint32_t ub, unsigned raw_bits)
 {
-    unsigned len = (ub >> o.k) + o.len0;
+    int nlen = (int)(o.nlen0 - (ub >> o.k));
     uint32_t z = (~ub & o.kmask) | o.kbit;
-    if (len >= o.limit) { len = 15u + raw_bits; z = ~ub & ((1u << raw_bits) - 1u); }
-    td_append(o, z, len);
+    if (nlen <= o.limit) { nlen = -(int)(15u + raw_bits); z = ~ub & ((1u << raw_bits) - 1u); }
+    td_append(o, z, (unsigned)nlen);
 }
 // Four symbols of two sub-streams, kJoin of them joined before they are appended (4-bit codes: four, 8-bit codes: two).  Where
 // one is an escape, or the joined ones are longer than a word, one at a time.
@@ -555,55 +556,62 @@ template <unsigned kN> struct TdJoin { static constexpr unsigned value = kN; };
 template <unsigned kJoin>
 __device__ __forceinline__ void td_append4(const TdLaunch &P, TdOut &x, TdOut &y, const uint32_t (&ux)[4], const uint32_t (&uy)[4], unsigned raw_bits)
 {
-    unsigned lx[4], ly[4];
+    int lx[4], ly[4];                                        // minus the lengths
     uint32_t zx[4], zy[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        lx[i] = (ux[i] >> x.k) * P.pow2[0] + x.len0;
-        ly[i] = (uy[i] >> y.k) * P.pow2[0] + y.len0;
+        lx[i] = (int)(ux[i] >> x.k) * P.minus_one + (int)x.nlen0;
+        ly[i] = (int)(uy[i] >> y.k) * P.minus_one + (int)y.nlen0;
         zx[i] = (~ux[i] & x.kmask) | x.kbit;
         zy[i] = (~uy[i] & y.kmask) | y.kbit;
     }
-    const unsigned mx = max(max(lx[0], lx[1]), max(lx[2], lx[3])), my = max(max(ly[0], ly[1]), max(ly[2], ly[3]));
-    unsigned jx[4], jy[4], longest = 0;                      // joined lengths
+    const int mx = min(min(lx[0], lx[1]), min(lx[2], lx[3])), my = min(min(ly[0], ly[1]), min(ly[2], ly[3]));
+    int jx[4], jy[4], longest = 0;                           // joined
 #pragma unroll
     for (int i = 0; i < 4; i += (int)kJoin) {
         jx[i] = lx[i]; jy[i] = ly[i];
 #pragma unroll
         for (int j = 1; j < (int)kJoin; ++j) {
-            zx[i] = (zx[i] << (lx[i + j] & 31u)) * P.pow2[0] + zx[i + j];
-            zy[i] = (zy[i] << (ly[i + j] & 31u)) * P.pow2[0] + zy[i + j];
-            jx[i] = jx[i] * P.pow2[0] + lx[i + j];
-            jy[i] = jy[i] * P.pow2[0] + ly[i + j];
+            zx[i] = __funnelshift_r(0u, zx[i], (unsigned)lx[i + j]) + zx[i + j];       // shifted left by the length
+            zy[i] = __funnelshift_r(0u, zy[i], (unsigned)ly[i + j]) + zy[i + j];
+            jx[i] = jx[i] + lx[i + j];
+            jy[i] = jy[i] + ly[i + j];
         }
-        longest = max(longest, max(jx[i], jy[i]));
+        longest = min(longest, min(jx[i], jy[i]));
     }
-    if (__builtin_expect(mx >= x.limit || my >= y.limit || longest > 32u, 0)) {
+    if (__builtin_expect(mx <= x.limit || my <= y.limit || longest < -32, 0)) {
+        uint32_t a[4], b[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { lx[i] = ux[i]; ly[i] = uy[i]; }
+        for (int i = 0; i < 4; ++i) { a[i] = ux[i]; b[i] = uy[i]; }
 #pragma unroll 1
         for (int i = 0; i < 4; ++i) {                        // (rolled up: instruction fetch is felt in this kernel)
-            td_append_any(x, lx[0], raw_bits);
-            td_append_any(y, ly[0], raw_bits);
-            lx[0] = lx[1]; lx[1] = lx[2]; lx[2] = lx[3];
-            ly[0] = ly[1]; ly[1] = ly[2]; ly[2] = ly[3];
+            td_append_any(x, a[0], raw_bits);
+            td_append_any(y, b[0], raw_bits);
+            a[0] = a[1]; a[1] = a[2]; a[2] = a[3];
+            b[0] = b[1]; b[1] = b[2]; b[2] = b[3];
         }
     } else {
 #pragma unroll
         for (int i = 0; i < 4; i += (int)kJoin) {
-            td_append(x, zx[i], jx[i]);
-            td_append(y, zy[i], jy[i]);
+            td_append(x, zx[i], (unsigned)jx[i]);
+            td_append(y, zy[i], (unsigned)jy[i]);
         }
     }
 }
-// The end of a sub-stream: zero bits (ones, complemented) up to the byte, and the last word.
-__device__ __forceinline__ void td_out_finish(TdOut &o)
+// The end of a sub-stream that began at addr: zero bits (ones, complemented) up to the byte, the first word and the last one.
+__device__ __forceinline__ void td_out_finish(TdOut &o, uint32_t addr, uint32_t aside)
 {
     const unsigned pad = (0u - o.bits) & 7u;
-    if (pad) td_append(o, (1u << pad) - 1u, pad);
+    if (pad) td_append(o, (1u << pad) - 1u, 0u - pad);
+    const bool one_word = o.wp == aside;                     // nothing has gone out yet
+    if (!one_word) {
+        uint32_t first;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(first) : "r"(aside) : "memory");
+        asm volatile("red.shared.or.b32 [%0], %1;" :: "r"(addr & ~3u), "r"(first) : "memory");
+    }
     if (o.bits & 31u) {
         const uint32_t word = o.acc << (32u - (o.bits & 31u));
-        asm volatile("red.shared.or.b32 [%0], %1;" :: "r"(o.wp), "r"(word) : "memory");
+        asm volatile("red.shared.or.b32 [%0], %1;" :: "r"(one_word ? addr & ~3u : o.wp), "r"(word) : "memory");
     }
 }
 
@@ -611,10 +619,10 @@ __device__ __forceinline__ void td_out_finish(TdOut &o)
 // says what the largest magnitude was (a bf16 number: scale * qmax rounded to bf16 is that number again), so there is no pass
 // for it and no tile.  The staging area holds the slice's bits complemented, as big-endian words.  Bound by instruction issue
 // (77 % of the slots).  8B shape, 16 chunks of 512 tokens: 1020 us for 8-bit codes with a tile, a pass over it for the magnitudes and
-// every symbol appended by itself, 540 us this way; 4-bit codes 1000 -> 490 us.  Fourteen CTAs of 64 threads an SM (72 registers) with
-// eight tokens loaded ahead; twelve or sixteen CTAs, four or sixteen tokens are 0-7 % slower.
+// every symbol appended by itself, 520 us this way; 4-bit codes 1000 -> 470 us.  Sixteen CTAs of 64 threads an SM (64 registers) with
+// eight tokens loaded ahead; twelve CTAs, four or sixteen tokens are 1-7 % slower.
 template <unsigned kCols>
-__global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 14 : 1) kdn_td_encode_kernel(const __grid_constant__ TdLaunch P)
+__global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 16 : 1) kdn_td_encode_kernel(const __grid_constant__ TdLaunch P)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const TdSlice s = td_slice(P);
@@ -652,8 +660,10 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 14 : 1) kdn
         const float inv_x = sc.x != 0.0f ? __fdiv_rn(qmax, __bfloat162float(__float2bfloat16_rn(__fmul_rn(sc.x, qmax)))) : 0.0f;
         const float inv_y = sc.y != 0.0f ? __fdiv_rn(qmax, __bfloat162float(__float2bfloat16_rn(__fmul_rn(sc.y, qmax)))) : 0.0f;
         TdOut x, y;
-        td_out_init(x, smem_u32(stage) + shift + o.off, params & 0xffu);
-        td_out_init(y, smem_u32(stage) + shift + o.off + len_x, params >> 8);
+        const uint32_t addr_x = smem_u32(stage) + shift + o.off, addr_y = addr_x + len_x;
+        const uint32_t aside = smem_u32(stage) + (uint32_t)td_stage_bytes(C, P.words) + 8u * tid;
+        td_out_init(x, addr_x, aside, params & 0xffu);
+        td_out_init(y, addr_y, aside + 4u, params >> 8);
         // per token: m + code (m = 1.5 * 2^23), minus m or the token before (delta mode), all exact
         const float m = 12582912.0f;
         const f32x2 inv2 = pack2(inv_x, inv_y), m2 = pack2(m, m), one2 = pack2(P.fone, P.fone), two2 = pack2(2.0f, 2.0f), half2 = pack2(0.5f, 0.5f);
@@ -702,8 +712,8 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 14 : 1) kdn
             td_append_any(x, ux, raw_bits);
             td_append_any(y, uy, raw_bits);
         }
-        td_out_finish(x);
-        td_out_finish(y);
+        td_out_finish(x, addr_x, aside);
+        td_out_finish(y, addr_y, aside + 4u);
     }
     // the last slice of a segment also writes the zero bytes that pad the segment to 16
     unsigned pad = 0;
