@@ -823,6 +823,24 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     return KDN_OK;
 }
 
+// An ordinary grid that may be set up while the kernel before it in the stream drains (it waits for that kernel itself).
+template <typename K, typename L>
+kdn_status launch_behind(K kernel, dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, const L &lp)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    KDN_CUDA(cudaLaunchKernelEx(&cfg, kernel, lp));
+    return KDN_OK;
+}
+
 // Ops whose chunk is in a token-delta Rice codec: at most kInlineOps per launch, their records travel as kernel
 // parameters.  Store is three launches (plan, scan, encode), retrieve and compose one (plus the rotation table).
 kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops, int n, cudaStream_t stream)
@@ -889,14 +907,13 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
             if (r != KDN_OK) return r;
             if (per_sm < 1) return KDN_E_UNSUPPORTED;
             const unsigned plan_threads = (cols + 31u) & ~31u;           // a warp takes 32 channels
-            if (plan_threads == 128u) kdn_td_plan_kernel<128><<<grid, 128, 0, stream>>>(tp);
-            else kdn_td_plan_kernel<512><<<grid, plan_threads, 0, stream>>>(tp);
-            KDN_CUDA(cudaGetLastError());
-            kdn_td_scan_kernel<<<(unsigned)m, kTdScanThreads, 0, stream>>>(tp);
-            KDN_CUDA(cudaGetLastError());
-            if (cols == kTdCols) kdn_td_encode_kernel<kTdCols><<<grid, enc_threads, smem_enc, stream>>>(tp);
-            else kdn_td_encode_kernel<0><<<grid, enc_threads, smem_enc, stream>>>(tp);
-            KDN_CUDA(cudaGetLastError());
+            if (plan_threads == 128u) r = launch_behind(kdn_td_plan_kernel<128>, grid, 128u, 0, stream, tp);
+            else r = launch_behind(kdn_td_plan_kernel<512>, grid, plan_threads, 0, stream, tp);
+            if (r == KDN_OK) r = launch_behind(kdn_td_scan_kernel, dim3((unsigned)m), kTdScanThreads, 0, stream, tp);
+            if (r != KDN_OK) return r;
+            if (cols == kTdCols) r = launch_behind(kdn_td_encode_kernel<kTdCols>, grid, enc_threads, smem_enc, stream, tp);
+            else r = launch_behind(kdn_td_encode_kernel<0>, grid, enc_threads, smem_enc, stream, tp);
+            if (r != KDN_OK) return r;
             ctx->launches += 3;
         } else {
             const size_t smem = td_decode_smem_bytes(cols, tp.words);
@@ -920,7 +937,8 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
                 r = ctx->env.resident(kdn_td_decode_kernel<COMPOSE, COLS>, (int)dec_threads, smem, &per_sm); \
                 if (r != KDN_OK) return r;                                                                  \
                 if (per_sm < 1) return KDN_E_UNSUPPORTED;                                                   \
-                kdn_td_decode_kernel<COMPOSE, COLS><<<grid, dec_threads, smem, stream>>>(tp);               \
+                r = launch_behind(kdn_td_decode_kernel<COMPOSE, COLS>, grid, dec_threads, smem, stream, tp); \
+                if (r != KDN_OK) return r;                                                                  \
             }
             if (cols == kTdCols) {
                 if (OP == OP_COMPOSE) KDN_TD_DECODE(true, kTdCols) else KDN_TD_DECODE(false, kTdCols)

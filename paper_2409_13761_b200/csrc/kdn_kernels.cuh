@@ -1162,7 +1162,7 @@ __device__ __forceinline__ long long group_row_pos(const DevOp &op, unsigned g, 
 {
     const unsigned i = (g << 6) + t;
     if (op.list_mode != 1) return op.off + (long long)i;      // (a select-list chooses among the chunk's tokens, it does not move them)
-    const long long rel = __ldg(op.list + i);
+    const long long rel = op.list[i];
     const long long p = op.off + rel;
     return (rel < 0 || p >= op.pos_end) ? -1ll : p;
 }

@@ -130,7 +130,7 @@ __device__ __forceinline__ unsigned td_lower_bound(const int32_t *list, unsigned
     unsigned lo = 0, hi = n;
     while (lo < hi) {
         const unsigned mid = (lo + hi) >> 1;
-        if ((long long)__ldg(list + mid) < key) lo = mid + 1u; else hi = mid;
+        if ((long long)list[mid] < key) lo = mid + 1u; else hi = mid;
     }
     return lo;
 }
@@ -199,19 +199,19 @@ __device__ __forceinline__ TdOffsets td_offsets(const unsigned char *lens, unsig
     return o;
 }
 
-// Pool addresses of the slice in the token rows of the group, row t at rows[t + t / 32] (0 for rows past the chunk's end).  All
-// threads of the block call this; true when one of the thread's rows lies outside the pool or the table.
-__device__ __forceinline__ bool td_row_addresses(const TdLaunch &P, const TdSlice &s, unsigned long long *rows)
+// Pool addresses of the slice in the token rows of the group, row t at rows[t + t / 32] (0 for rows past the chunk's end).  Threads
+// t = first, first + step, ... of those who fill one table call this; true when one of the thread's rows lies outside the pool or the table.
+__device__ __forceinline__ bool td_row_addresses(const TdLaunch &P, const TdSlice &s, unsigned long long *rows, unsigned first, unsigned step)
 {
     const unsigned char *base = reinterpret_cast<const unsigned char *>((s.kv ? P.v_layers : P.k_layers)[s.op.l0 + (int)s.li]);
     bool bad = false;
-    for (unsigned t = threadIdx.x; t < 64u; t += blockDim.x) {
+    for (unsigned t = first; t < 64u; t += step) {
         unsigned long long a = 0ull;
         if (t < s.n_tok) {
             const long long pos = group_row_pos(s.op, s.g, t);
             long long id = -1;
             const long long blk = P.bs_shift >= 0 ? pos >> P.bs_shift : pos / P.bs;
-            if (pos >= 0) id = __ldg(s.op.table + blk);
+            if (pos >= 0) id = s.op.table[blk];
             if (id < 0 || id >= P.n_blocks) bad = true;
             else a = (unsigned long long)(base + ((unsigned long long)(id * P.bs + (pos - blk * P.bs)) * P.row_elems + s.c0) * 2ull);
         }
@@ -391,33 +391,38 @@ __device__ __forceinline__ unsigned td_plan_channel(const TdLaunch &P, const uin
 // A warp takes 32 channels: lanes l and l + 16 hold the same two channels, tokens 0-31 and 32-63, straight from the pool in
 // registers (no shared tile: every value is used once, and a thread has 32 loads in flight).  Bound by the pipe of logic and shifts
 // (two thirds busy).  8B shape, 16 chunks of 512 tokens, 8-bit codes: 1100 us with a table of code-word lengths looked up per
-// symbol, 345 us this way; 4-bit codes 1080 -> 230 us.  Seven CTAs of 128 threads an SM (72 registers): 345 us, eight 365.
+// symbol, 330 us this way; 4-bit codes 1080 -> 220 us.  Six CTAs of 128 threads an SM (80 registers); seven or eight spill and are 2 % slower.
 // kThreads: 128 is the usual slice of 128 channels, 512 stands for any other.
 template <unsigned kThreads>
-__global__ void __launch_bounds__(kThreads, kThreads == 128u ? 7 : 1) kdn_td_plan_kernel(const __grid_constant__ TdLaunch P)
+__global__ void __launch_bounds__(kThreads, kThreads == 128u ? 6 : 1) kdn_td_plan_kernel(const __grid_constant__ TdLaunch P)
 {
-    __shared__ unsigned long long rows[66];                 // pool addresses of the group's token rows (0: past the chunk's end), ...
-    __shared__ unsigned warp_bytes[16];                     // ... row t at index t + t / 32: the two that a warp reads at once in different banks
+    // pool addresses of the group's token rows (0: past the chunk's end), row t at index t + t / 32: the two that a warp reads at once in
+    // different banks.  A table a warp: no barrier in this kernel, a warp computes while others load.
+    __shared__ unsigned long long all_rows[kThreads / 32u][66];
+    dependency_wait();
+    release_dependents();
     const TdSlice s = td_slice(P);
     if (!s.valid) return;
     const unsigned C = P.cols, RE = P.row_elems, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const int codec = s.op.codec;
     const TdLayout &lay = P.layout[blockIdx.z];
     const unsigned long long row = (unsigned long long)s.seg * RE + s.c0;
-    const bool bad = td_row_addresses(P, s, rows);
+    unsigned long long *rows = all_rows[warp];
+    const bool bad = td_row_addresses(P, s, rows, lane, 32u);
+    __syncwarp();
     const unsigned half = lane >> 4, pair = warp * 16u + (lane & 15u), ch = 2u * pair + half;      // ch: the channel the thread answers for
     const bool act = 2u * pair < C;                         // (C is a multiple of 16)
-    unsigned *slice_bytes = reinterpret_cast<unsigned *>(s.op.data + lay.streams) + (size_t)s.seg * P.n_split + s.part;
-    if (__syncthreads_or(bad)) {
-        // a slice that is given up leaves lengths of zero behind: the scan and the encoder then see a consistent, if
+    unsigned *warp_bytes = reinterpret_cast<unsigned *>(s.op.data + lay.streams) + ((size_t)s.seg * P.n_split + s.part) * ((C + 31u) >> 5) + warp;
+    if (__any_sync(0xffffffffu, bad)) {
+        // channels that are given up leave lengths of zero behind: the scan and the encoder then see a consistent, if
         // incomplete, chunk instead of whatever the buffer held before
         if (act) {
             s.op.data[lay.lens + row + ch] = 0;
             s.op.data[lay.params + row + ch] = 0;
         }
-        if (tid == 0) {
+        if (lane == 0) {
             atomicCAS(P.status, 0, kStatusRange);
-            *slice_bytes = 0u;
+            *warp_bytes = 0u;
         }
         return;
     }
@@ -427,10 +432,10 @@ __global__ void __launch_bounds__(kThreads, kThreads == 128u ? 7 : 1) kdn_td_pla
     const unsigned n_mine = !act ? 0u : s.n_tok < 32u * half ? 0u : s.n_tok - 32u * half;
     if (full && act) {
 #pragma unroll
-        for (int t = 0; t < 32; ++t) x[t] = __ldg(reinterpret_cast<const uint32_t *>(my_rows[t] + (unsigned long long)(2u * pair) * P.pow2[1]));
+        for (int t = 0; t < 32; ++t) x[t] = __ldcg(reinterpret_cast<const uint32_t *>(my_rows[t] + (unsigned long long)(2u * pair) * P.pow2[1]));
     } else {
 #pragma unroll
-        for (int t = 0; t < 32; ++t) x[t] = (unsigned)t < n_mine ? __ldg(reinterpret_cast<const uint32_t *>(my_rows[t]) + pair) : 0u;
+        for (int t = 0; t < 32; ++t) x[t] = (unsigned)t < n_mine ? __ldcg(reinterpret_cast<const uint32_t *>(my_rows[t]) + pair) : 0u;
     }
     uint32_t m0 = maxabs_bf16x2(x[0], x[1]), m1 = maxabs_bf16x2(x[2], x[3]);
 #pragma unroll
@@ -454,33 +459,29 @@ __global__ void __launch_bounds__(kThreads, kThreads == 128u ? 7 : 1) kdn_td_pla
         s.op.data[lay.lens + row + ch] = (unsigned char)len;
         s.op.data[lay.params + row + ch] = (unsigned char)(best & 15u);
     }
-    // The slice's bytes are left for the scan at the start of the streams, four bytes a slice: the encoder overwrites them, as
+    // The warp's bytes are left for the scan at the start of the streams, four bytes a warp: the encoder overwrites them, as
     // every sub-stream takes at least a byte.
     const unsigned sum = __reduce_add_sync(0xffffffffu, len);
-    if (lane == 0) warp_bytes[warp] = sum;
-    __syncthreads();
-    if (tid == 0) {
-        unsigned total = 0;
-        for (unsigned w = 0; w < (blockDim.x >> 5); ++w) total += warp_bytes[w];
-        *slice_bytes = total;
-    }
+    if (lane == 0) *warp_bytes = sum;
 }
 
 // ------------------------------------------------------------------------------------------ store: scan --
 
 // One CTA per op: seg_off[s + 1] = seg_off[s] + the segment's sub-stream bytes rounded up to 16, 1024 segments at a time.
 // Latency is all that counts here: 512 tokens at the 8B shape took 58 us when the lengths were added up here, and take 5 now
-// that the planner leaves one sum per slice.
+// that the planner leaves sums behind.
 constexpr unsigned kTdScanThreads = 1024;
 __global__ void __launch_bounds__(kTdScanThreads) kdn_td_scan_kernel(const __grid_constant__ TdLaunch P)
 {
     __shared__ unsigned scratch[33];
+    dependency_wait();
+    release_dependents();
     const DevOp op = P.inline_ops[blockIdx.x];
     if (op.codec < 5 || op.T <= 0) return;
     const TdLayout &lay = P.layout[blockIdx.x];
     unsigned long long *seg_off = reinterpret_cast<unsigned long long *>(op.data);
-    const unsigned *slice_bytes = reinterpret_cast<const unsigned *>(op.data + lay.streams);
-    const unsigned tid = threadIdx.x;
+    const unsigned *warp_bytes = reinterpret_cast<const unsigned *>(op.data + lay.streams);
+    const unsigned tid = threadIdx.x, per_seg = P.n_split * ((P.cols + 31u) >> 5);
     unsigned long long run = lay.streams;
     if (tid == 0) {
         seg_off[0] = run;
@@ -489,8 +490,18 @@ __global__ void __launch_bounds__(kTdScanThreads) kdn_td_scan_kernel(const __gri
     for (unsigned long long base = 0; base < lay.S; base += kTdScanThreads) {
         const unsigned long long sidx = base + tid;
         unsigned size = 0;
-        if (sidx < lay.S)
-            for (unsigned p = 0; p < P.n_split; ++p) size += slice_bytes[sidx * P.n_split + p];
+        if (sidx < lay.S) {
+            if ((per_seg & 3u) == 0u) {
+                const uint4 *mine = reinterpret_cast<const uint4 *>(warp_bytes + sidx * per_seg);
+#pragma unroll 8
+                for (unsigned p = 0; p < (per_seg >> 2); ++p) {
+                    const uint4 v = mine[p];
+                    size += v.x + v.y + v.z + v.w;
+                }
+            } else {
+                for (unsigned p = 0; p < per_seg; ++p) size += warp_bytes[sidx * per_seg + p];
+            }
+        }
         size = (size + 15u) & ~15u;
         unsigned total;
         const unsigned before = td_block_scan(size, scratch, &total);
@@ -637,7 +648,10 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 16 : 1) kdn
     const TdLayout &lay = P.layout[blockIdx.z];
     const unsigned long long row = (unsigned long long)s.seg * RE;
     const bool act = 2u * tid < C;
-    const bool bad = td_row_addresses(P, s, rows);
+    // (this kernel may start as soon as the scan's CTAs have seen the planner end: the row addresses are what it can have ready)
+    const bool bad = td_row_addresses(P, s, rows, tid, nthreads);
+    dependency_wait();
+    release_dependents();
     const TdOffsets o = td_offsets(s.op.data + lay.lens + row, s.c0, C, nthreads, scratch);
     const unsigned long long seg_begin = reinterpret_cast<const unsigned long long *>(s.op.data)[s.seg];
     unsigned char *dst = s.op.data + seg_begin + o.before;
@@ -683,7 +697,7 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 16 : 1) kdn
         auto load = [&](unsigned t0, uint32_t (&v)[kTdLoad]) {
             const unsigned long long *r = rows + t0 + (t0 >> 5);
 #pragma unroll
-            for (int i = 0; i < (int)kTdLoad; ++i) v[i] = __ldg(reinterpret_cast<const uint32_t *>(r[i] + (unsigned long long)(2u * tid) * P.pow2[1]));
+            for (int i = 0; i < (int)kTdLoad; ++i) v[i] = __ldcg(reinterpret_cast<const uint32_t *>(r[i] + (unsigned long long)(2u * tid) * P.pow2[1]));
         };
         auto code = [&](auto join) -> unsigned {
             unsigned t0 = 0;
@@ -708,7 +722,7 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 16 : 1) kdn
 #pragma unroll 1
         for (; t0 < s.n_tok; ++t0) {
             uint32_t ux, uy;
-            symbol(__ldg(reinterpret_cast<const uint32_t *>(rows[t0 + (t0 >> 5)]) + tid), ux, uy);
+            symbol(__ldcg(reinterpret_cast<const uint32_t *>(rows[t0 + (t0 >> 5)]) + tid), ux, uy);
             td_append_any(x, ux, raw_bits);
             td_append_any(y, uy, raw_bits);
         }
@@ -865,6 +879,8 @@ template <bool kCompose, unsigned kCols>
 __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 12 : 1) kdn_td_decode_kernel(const __grid_constant__ TdLaunch P)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
+    dependency_wait();
+    release_dependents();
     const TdSlice s = td_slice(P);
     if (!s.valid) return;
     const unsigned C = kCols ? kCols : P.cols, RE = P.row_elems;
@@ -948,7 +964,7 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 12 : 1) kdn
             bool bad = false;
             unsigned r = i;
             if (selecting) {
-                const long long c = (long long)__ldg(s.op.list + i) - ((long long)s.g << 6);
+                const long long c = (long long)s.op.list[i] - ((long long)s.g << 6);
                 bad = c < 0 || c >= (long long)s.n_tok;                   // (a list that is not increasing)
                 r = (unsigned)c;
             }
@@ -957,7 +973,7 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 12 : 1) kdn
                 bad = pos < 0;
                 if (!bad) {
                     const long long blk = P.bs_shift >= 0 ? pos >> P.bs_shift : pos / P.bs;
-                    const long long id = __ldg(s.op.table + blk);
+                    const long long id = s.op.table[blk];
                     bad = id < 0 || id >= P.n_blocks;
                     if (!bad) rows[r] = (unsigned long long)(base + ((unsigned long long)(id * P.bs + (pos - blk * P.bs)) * RE + s.c0) * 2ull);
                 }
@@ -1016,7 +1032,7 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 12 : 1) kdn
     const f32x2 sc2 = pack2(sc_a, sc_b), zero2 = pack2(-kTdCodeZero, -kTdCodeZero);
     f32x2 cc = 0ull, ss = 0ull;
     if (rotating && act) {
-        const float2 cs = __ldg(P.rope + (size_t)s.op.rope * half + (tid - head * half));
+        const float2 cs = *(P.rope + (size_t)s.op.rope * half + (tid - head * half));
         cc = pack2(cs.x, cs.x);
         ss = pack2(-cs.y, cs.y);
     }
