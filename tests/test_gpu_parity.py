@@ -591,3 +591,42 @@ def test_coded_ops_on_pool_blocks_of_2_kib_or_less_run_as_token_rows(codec, bs, 
         assert np.array_equal(dev.pool_np(), ref)
     finally:
         dev.close()
+
+
+@pytest.mark.parametrize("codec", [RAW, INT8])
+def test_every_step_of_a_layerwise_call_comes_after_what_filled_the_host_chunk(codec):
+    """The side stream is ordered behind the caller's stream once per layer-wise call: a page-locked chunk that a copy queued on the
+    caller's stream fills late is whole when its last layers cross, slabs are reused by later steps only when they have been read, and the
+    caller's work queued behind the call sees every layer."""
+    shape = synth.TOY.with_(n_layers=9, n_kv_heads=4, head_dim=64, block_size=16, n_blocks=128)
+    dev = Device(shape, seed=41)
+    try:
+        K = dev.K
+        K.kdn_set_staging_bytes(dev.ctx, 512 * 1024)            # one layer of 400 tokens is 400 KiB raw: a slab a step
+        host = dev.pool_np()
+        perm = np.random.default_rng(12).permutation(128).astype(np.int32)
+        T = 400
+        want = oracle.store(host, perm[:26], 9, T, codec)
+        ballast = torch.empty(1 << 28, dtype=torch.uint8, device=dev.dev)
+        hbuf = dev.chunk_buf(T, codec, pinned=True, fill=0)
+        staged = torch.from_numpy(want).to(dev.dev)
+        side = torch.cuda.Stream(device=dev.dev)
+        ref = host.copy()
+        oracle.retrieve(ref, perm[40:66], 3, T, codec, want)
+        for step, own_side in ((1, 0), (2, side.cuda_stream), (4, 0)):
+            hbuf.zero_()
+            torch.cuda.synchronize()
+            with torch.cuda.stream(dev.stream):
+                for _ in range(8):
+                    ballast.fill_(2)
+                hbuf.copy_(staged, non_blocking=True)
+            K.kdn_retrieve_layerwise(dev.ctx, dev.pool_id, [dev.op(dev.table(perm[40:66]), 3, hbuf, T, codec)], step, dev.stream.cuda_stream, own_side)
+            assert dev.sync() == 0
+            assert np.array_equal(dev.pool_np(), ref), step
+            for t in dev.k + dev.v:
+                t[torch.from_numpy(perm[40:66].astype(np.int64)).to(dev.dev)] = 0
+            ref2 = dev.pool_np()
+            oracle.retrieve(ref2, perm[40:66], 3, T, codec, want)
+            ref = ref2
+    finally:
+        dev.close()
