@@ -647,6 +647,15 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
         // per-channel key chunks on small pool blocks (2 / 1 KV heads of the 8B shape: retrieve 4.7 / 2.9 -> 6.3 / 5.8 TB/s)
         def = tile_elems * 2u <= 4096u ? Shape{ 0, 8, 8, 2, 1, 1 } : Shape{ 0, 4, 4, 1, 1 };
     }
+    if (!any_list && !kc_decode && any_coded && !any_rot && tile_elems * 2u == 8192u && ctx->tuning.tile_bytes <= 0) {
+        // A small coded launch, 8 to 32 tiles an SM, is pipeline fill and drain: four slots in four CTAs of one group each start sooner than six in
+        // three CTAs of two (8B shape, 77 tokens int8: store 6.4 -> 6.1 us, retrieve 6.0 -> 5.7; 200 tokens 9.5 -> 9.1 and 8.8 -> 8.6;
+        // 512 tokens, 55 tiles an SM: store 20.6 -> 20.4 but retrieve 20.4 -> 20.6 and int4 18.1 -> 18.5; 6 tiles an SM: 4.9 -> 5.0)
+        unsigned long long tiles_ahead = 0;
+        for (int i = 0; i < n; ++i) tiles_ahead += (unsigned long long)hops[i].op.nl * (OP == OP_STORE && is_kc(hops[i].op.codec) ? 1ull : 2ull) * (unsigned)hops[i].op.nblk * tpb;
+        const unsigned long long sms = (unsigned long long)ctx->env.sm_count;
+        if (tiles_ahead >= 8ull * sms && tiles_ahead < 32ull * sms) def = Shape{ 8192, 4, 4, 1, 1 };
+    }
     if (!any_list && !kc_decode && ctx->tuning.tile_bytes <= 0) {
         // A pool block smaller than the tile the shape was tuned for (few KV heads per GPU under tensor parallelism, or
         // a small block_size) caps the tile at the block.  From sweeps on the 8B shape with 4, 2 and 1 KV heads:
