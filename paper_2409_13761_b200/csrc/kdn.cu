@@ -444,23 +444,56 @@ kdn_status launch_key_planes(kdn_ctx *ctx, const Pool &pool, const DevOp *inl, c
     return KDN_OK;
 }
 
-// Whether a launch goes to the kernels that move token rows one by one (kdn_rows.cuh): keep-lists over rows of up to 1024 elements --
-// the tile pipeline issues a copy a row -- and coded dense ops on pool blocks of 2 KiB or less, where a coding tile that stops at the
-// end of its block is far too small.  Half of the tokens kept, us in the tile pipeline / here (8B shape, 16 x 1024 tokens): two heads (rows of
-// 256) retrieve int8 114 / 79, int4 115 / 70, store int8 117 / 77, int4 117 / 66; one head raw (32 x 1024) 125 / 93; eight heads (rows of
-// 1024, 16 x 512) retrieve int8 146 / 144, int4 142 / 127, store int8 143 / 140, raw 172 / 171.  Only the retrieve of long rows with a scale per channel
-// (eight heads: 185 / 327) stays, since it would read the scales of every row anew.
-bool rows_apply(const kdn_ctx *ctx, const Pool &pool, int OP, bool any_coded, bool any_rot, bool any_list, bool any_kc, const HostOp *hops, int n)
+// Vectors of a rows launch's thread (see kdn_rows.cuh) and what follows from it.
+struct RowsShape { unsigned vec, vpr, unit, rows; unsigned long long ctas; };     // ctas: with one plane each
+RowsShape rows_shape(const Pool &pool, int OP, const HostOp *hops, int n)
+{
+    RowsShape r{};
+    const unsigned row_elems = (unsigned)pool.H * (unsigned)pool.D;
+    bool all_coded = true;
+    for (int i = 0; i < n; ++i) all_coded &= hops[i].op.codec != KDN_CODEC_RAW_BF16;
+    r.vec = OP == OP_STORE || all_coded ? 16u : 8u;
+    r.vpr = row_elems / r.vec;
+    r.unit = row_elems < 2048u ? 2048u / row_elems : 1u;
+    if (r.unit > 16u) r.unit = 16u;
+    r.rows = (OP == OP_STORE ? kRowsVectors / 2u : (unsigned)kRowsVectors) * kRowsThreads / r.vpr;
+    if (r.rows > kRowsPerCta) r.rows = kRowsPerCta;
+    if (r.rows > r.unit) r.rows = r.rows / r.unit * r.unit;
+    if (r.rows)
+        for (int i = 0; i < n; ++i) {
+            const unsigned rows = (unsigned)(hops[i].op.list_mode ? hops[i].op.n_list : hops[i].op.T);
+            r.ctas += (unsigned long long)((rows + r.rows - 1u) / r.rows) * (unsigned)hops[i].op.nl * 2ull;
+        }
+    return r;
+}
+
+// Whether a launch goes to the kernels that move token rows one by one (kdn_rows.cuh).
+// Keep-lists over rows of up to 1024 elements: the tile pipeline issues a copy a row.  Half of the tokens kept, us in the tile pipeline / here
+// (8B shape, 16 x 1024 tokens): two heads (rows of 256) retrieve int8 114 / 76, int4 115 / 69, store int8 117 / 78, int4 117 / 66; one head raw
+// (32 x 1024) 125 / 92; eight heads (rows of 1024, 16 x 512) retrieve int8 146 / 144, int4 142 / 122, store int8 143 / 140, raw 172 / 171.  Only the
+// retrieve of long rows with a scale per channel (eight heads: 185 / 327) stays, since it would read the scales of every row anew.
+// Coded dense ops on pool blocks of 2 KiB or less: a coding tile that stops at the end of its block is far too small (int8, blocks of four tokens
+// of one head: 135 / 76).  On blocks of 4 KiB it depends on the size (one head, int8): one chunk of 512 tokens store 5.8 / 5.3, retrieve 5.5 / 5.1; 64 chunks
+// 157 / 152 and 152 / 149; in between, where these kernels' CTAs make a few uneven waves, the pipeline is ahead (8 x 300 tokens 15.7 / 17).
+// Large retrieves of 4-bit codes (eight heads): 32 chunks 454 / 446, 4 chunks 66.8 / 64, four of 1500 tokens of 80 layers 426 / 407; one chunk 18.0 / 18.8.
+bool rows_apply(const kdn_ctx *ctx, const Pool &pool, int OP, bool any_coded, bool any_rot, bool any_list, bool any_kc, bool all_int4, const HostOp *hops, int n)
 {
     const unsigned row_elems = (unsigned)pool.H * (unsigned)pool.D;
     const kdn_tuning &t = ctx->tuning;
     // a caller-set launch shape is one of the tile pipeline
     if (t.tile_bytes > 0 || t.stages > 0 || t.ctas_per_sm > 0 || t.compute_groups > 0 || t.store_lag > 0 || t.group_warps > 0) return false;
     if ((OP != OP_STORE && OP != OP_RETRIEVE) || any_rot || row_elems % 16u) return false;
-    if (!any_list) return any_coded && !any_kc && (unsigned long long)pool.bs * row_elems * 2ull <= 2048ull;
-    for (int i = 0; i < n; ++i)
-        if (hops[i].op.list_mode != 1) return false;
-    return row_elems < 512u || (row_elems <= 1024u && !(any_kc && OP == OP_RETRIEVE));
+    if (any_list) {
+        for (int i = 0; i < n; ++i)
+            if (hops[i].op.list_mode != 1) return false;
+        return row_elems < 512u || (row_elems <= 1024u && !(any_kc && OP == OP_RETRIEVE));
+    }
+    if (!any_coded || any_kc) return false;
+    const unsigned long long block_bytes = (unsigned long long)pool.bs * row_elems * 2ull;
+    if (block_bytes <= 2048ull) return true;
+    if (row_elems > 1024u || (block_bytes > 4096ull && !(all_int4 && OP == OP_RETRIEVE))) return false;
+    const unsigned long long ctas = rows_shape(pool, OP, hops, n).ctas, wave = 4ull * (unsigned)ctx->env.sm_count;
+    return ctas >= 12ull * wave || (block_bytes <= 4096ull && ctas <= wave);
 }
 
 kdn_status launch_rows(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops, int n, cudaStream_t stream)
@@ -473,27 +506,21 @@ kdn_status launch_rows(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hop
         if (slot->used) KDN_CUDA(cudaEventSynchronize(slot->done));
     }
     DevOp *h_ops = inl ? lp.inline_ops : slot->h_ops;
-    bool all_coded = true;
-    for (int i = 0; i < n; ++i) all_coded &= hops[i].op.codec != KDN_CODEC_RAW_BF16;
     constexpr int kj = kRowsVectors;
-    const unsigned vec = OP == OP_STORE || all_coded ? 16u : 8u;
-    const unsigned vectors = OP == OP_STORE ? kj / 2u : kj;    // a thread
+    const RowsShape shape = rows_shape(pool, OP, hops, n);
+    const unsigned vec = shape.vec;
     lp.row_elems = (unsigned)pool.H * (unsigned)pool.D;
-    lp.vpr = lp.row_elems / vec;
-    lp.unit = lp.row_elems < 2048u ? 2048u / lp.row_elems : 1u;
-    if (lp.unit > 16u) lp.unit = 16u;
-    lp.rows = vectors * kRowsThreads / lp.vpr;
-    if (lp.rows > kRowsPerCta) lp.rows = kRowsPerCta;
-    if (lp.rows > lp.unit) lp.rows = lp.rows / lp.unit * lp.unit;
+    lp.vpr = shape.vpr;
+    lp.unit = shape.unit;
+    lp.rows = shape.rows;
     lp.vpr_magic = lp.rows > 1u && lp.vpr > 1u ? 0xffffffffu / lp.vpr + 1u : 0u;
-    unsigned long long ctas = 0;                             // with one plane each
-    for (int i = 0; i < n; ++i) {
-        const unsigned rows = (unsigned)(hops[i].op.list_mode ? hops[i].op.n_list : hops[i].op.T);
-        ctas += (unsigned long long)((rows + lp.rows - 1u) / lp.rows) * (unsigned)hops[i].op.nl * 2ull;
-    }
-    // planes a CTA goes through: enough to pay for the look-ups and the pipeline's start, few enough to leave some waves of CTAs
-    lp.planes = 1u;
-    while (lp.planes < 16u && ctas / (lp.planes * 2u) >= 6ull * (unsigned)ctx->env.sm_count) lp.planes *= 2u;
+    // Planes a CTA goes through: enough to pay for the look-ups and the pipeline's start, few enough to leave 2.5 waves of CTAs (a store,
+    // whose CTAs do more work each: 1.7), or one wave instead of two uneven ones.  Two heads, half of 16 x 1024 tokens kept, int8, 1 / 2 / 4 / 8 / 16
+    // planes: retrieve 88 / 75 / 76 / 78 / 85 us, store 125 / 91 / 81 / 78 / 78; of 4 x 500 tokens retrieve 13.6 / 11.9 / 13.1 / 16.8.
+    const unsigned long long wave = 4ull * (unsigned)ctx->env.sm_count, want = OP == OP_STORE ? wave * 17ull / 10ull : wave * 5ull / 2ull;
+    lp.planes = 16u;
+    while (lp.planes > 1u && shape.ctas / lp.planes < want) --lp.planes;
+    if (lp.planes == 1u && shape.ctas > wave && shape.ctas <= 2ull * wave) lp.planes = 2u;
     int kc_layers = 0, kc_groups = 0;
     unsigned long long tiles = 0;
     for (int i = 0; i < n; ++i) {
@@ -582,7 +609,7 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     }
     const bool compute = any_coded || any_rot;
     const unsigned row_elems = (unsigned)pool.H * (unsigned)pool.D;
-    if (rows_apply(ctx, pool, OP, any_coded, any_rot, any_list, any_kc, hops, n)) return launch_rows(ctx, pool, OP, hops, n, stream);
+    if (rows_apply(ctx, pool, OP, any_coded, any_rot, any_list, any_kc, all_int4, hops, n)) return launch_rows(ctx, pool, OP, hops, n, stream);
 
     // tile size: whole 16-byte units; whole 64-element groups with int8 / int4; whole head rows with rotation
     unsigned unit = 8;

@@ -9,7 +9,7 @@
 // slots that only this thread uses -- a deeper queue than registers would hold -- kStages planes ahead, counted on an mbarrier
 // per stage (bounded waits, as in the tile pipeline); nothing else is synchronised.  On the chunk side a CTA's vectors are
 // contiguous whatever the rows do; on the pool side a row is.  Bound by memory and, when coding, by the latency of a plane: 8B shape with
-// two heads, half of 16 x 1024 tokens kept, int8: retrieve 79 us (5.2 TB/s), store 77 us (5.3 TB/s).  Loads into registers instead of
+// two heads, half of 16 x 1024 tokens kept, int8: retrieve 76 us (5.4 TB/s), store 78 us (5.3 TB/s).  Loads into registers instead of
 // slots: 92 and 87 us.
 #pragma once
 

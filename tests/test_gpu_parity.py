@@ -630,3 +630,64 @@ def test_every_step_of_a_layerwise_call_comes_after_what_filled_the_host_chunk(c
             ref = ref2
     finally:
         dev.close()
+
+
+@pytest.mark.parametrize("codec", [INT8, INT4])
+def test_dense_ops_on_one_head_blocks_of_4_kib_move_row_by_row(codec):
+    """Blocks of 4 KiB (one head, sixteen tokens): a call that is one wave of CTAs or less goes to the kernels that move token rows one by one;
+    offsets and lengths that are no multiple of anything.  Bit-exact."""
+    shape = synth.TOY.with_(n_layers=3, n_kv_heads=1, head_dim=128, block_size=16, n_blocks=128)
+    dev = Device(shape, seed=51)
+    try:
+        K = dev.K
+        host = dev.pool_np()
+        perm = np.random.default_rng(codec).permutation(128).astype(np.int32)
+        for T, off in ((1, 0), (77, 11), (128, 0), (300, 5)):
+            nb = -(-(off + T) // 16)
+            want = oracle.store(host, perm[:nb], off, T, codec)
+            buf = dev.chunk_buf(T, codec)
+            dev.store([dev.op(dev.table(perm[:nb]), off, buf, T, codec)])
+            assert dev.sync() == 0
+            assert "rows" in K.kdn_last_launch(dev.ctx)["kernel"]
+            assert np.array_equal(to_np(buf), want)
+            ref = dev.pool_np()
+            dev.retrieve([dev.op(dev.table(perm[40:40 + nb]), off, buf, T, codec)])
+            assert dev.sync() == 0
+            assert "rows" in K.kdn_last_launch(dev.ctx)["kernel"]
+            oracle.retrieve(ref, perm[40:40 + nb], off, T, codec, want)
+            assert np.array_equal(dev.pool_np(), ref)
+    finally:
+        dev.close()
+
+
+def test_large_retrieves_of_4_bit_codes_move_row_by_row():
+    """Retrieves of 4-bit codes with many waves of CTAs go to the kernels that move token rows one by one, whatever the block size; the
+    same call with an int8 chunk in it does not.  Bit-exact."""
+    shape = synth.TOY.with_(n_layers=24, n_kv_heads=8, head_dim=128, block_size=8, n_blocks=256)
+    dev = Device(shape, seed=53)
+    try:
+        K = dev.K
+        rng = np.random.default_rng(5)
+        host = dev.pool_np()
+        perm = rng.permutation(256).astype(np.int32)
+        Ts = [1 + i % 8 for i in range(8)]
+        bufs, wants, codecs = [], [], [INT4] * 7 + [INT8]
+        for i, T in enumerate(Ts):
+            bufs.append(dev.chunk_buf(T, codecs[i]))
+            wants.append(oracle.store(host, perm[2 * i:2 * i + 2], i, T, codecs[i]))
+        dev.store([dev.op(dev.table(perm[2 * i:2 * i + 2]), i, bufs[i], T, codecs[i]) for i, T in enumerate(Ts)])
+        assert dev.sync() == 0
+        for last in (7, 8):
+            ref = dev.pool_np()
+            ops = []
+            for k in range(160):
+                i = k % last
+                tab = perm[20 + k:21 + k]
+                ops.append(dev.op(dev.table(tab), 0, bufs[i], Ts[i], codecs[i]))
+                oracle.retrieve(ref, tab, 0, Ts[i], codecs[i], wants[i])
+            dev.retrieve(ops)
+            assert dev.sync() == 0
+            assert ("rows" in K.kdn_last_launch(dev.ctx)["kernel"]) == (last == 7)
+            assert np.array_equal(dev.pool_np(), ref)
+    finally:
+        dev.close()
