@@ -114,8 +114,9 @@ struct Launch {
     int wait_all;             // the launch may start while the kernel before it in the stream still runs (programmatic
                               // dependent launch).  1: every thread waits for that kernel before it touches global memory.
                               // 0: only the warps that read the rotation table wait (the kernel before is the table kernel).
-                              // 2: they wait before they leave (the kernel before, itself an ordinary launch, stores the key
-                              // planes of the same chunks: the two may overlap, and what comes behind this one waits for both)
+                              // 2: they wait before they leave (the kernel before stores the key planes of the same chunks and lets
+                              // this one start only when it has itself waited: the two may overlap, and what comes behind this
+                              // one waits for both)
     float one;                // 1.0f, as a launch parameter: the coding loops form "product + constant" as
                               // fma(product, one, constant), and with a multiplier the assembler cannot see there
                               // is nothing it could contract with the multiply before it (the codecs round twice)
@@ -1200,7 +1201,10 @@ constexpr unsigned kKcCols = 256u;                        // channels per CTA at
 __global__ void __launch_bounds__(kKcCols / 2u, 5) kdn_store_kc_kernel(const __grid_constant__ KcLaunch P)
 {
     __shared__ unsigned long long rows[64];                 // pool addresses of the group's token rows (slice start)
-    release_dependents();                                   // the value planes' kernel shares nothing with this one: it may start as this one drains
+    // the value planes' kernel shares nothing with this one: it may start as this one drains (which, as this one lets it only after
+    // having waited itself, is after the kernel before this one)
+    dependency_wait();
+    release_dependents();
     const DevOp *ops = P.ops ? P.ops : P.inline_ops;
     const DevOp &op = ops[blockIdx.z];
     if (op.codec != 3 && op.codec != 4) return;
@@ -1216,7 +1220,7 @@ __global__ void __launch_bounds__(kKcCols / 2u, 5) kdn_store_kc_kernel(const __g
     for (unsigned t = tid; t < n_tok; t += blockDim.x) {
         const long long pos = group_row_pos(op, g, t);
         const long long blk = P.bs_shift >= 0 ? pos >> P.bs_shift : pos / P.bs;
-        const long long id = pos < 0 ? -1 : (long long)__ldg(op.table + blk);
+        const long long id = pos < 0 ? -1 : (long long)op.table[blk];
         if (id < 0 || id >= P.n_blocks) bad = true;
         else rows[t] = (unsigned long long)(base + ((unsigned long long)(id * P.bs + (pos - blk * P.bs)) * RE + c0) * 2ull);
     }
@@ -1231,11 +1235,11 @@ __global__ void __launch_bounds__(kKcCols / 2u, 5) kdn_store_kc_kernel(const __g
     uint4 x[kKcTok];
     if (full) {
 #pragma unroll
-        for (unsigned i = 0; i < kKcTok; ++i) x[i] = __ldg(reinterpret_cast<const uint4 *>(rows[ta + i]) + o);
+        for (unsigned i = 0; i < kKcTok; ++i) x[i] = __ldcg(reinterpret_cast<const uint4 *>(rows[ta + i]) + o);
     } else {
 #pragma unroll
         for (unsigned i = 0; i < kKcTok; ++i)
-            x[i] = ta + i < n_tok ? __ldg(reinterpret_cast<const uint4 *>(rows[ta + i]) + o) : make_uint4(0u, 0u, 0u, 0u);
+            x[i] = ta + i < n_tok ? __ldcg(reinterpret_cast<const uint4 *>(rows[ta + i]) + o) : make_uint4(0u, 0u, 0u, 0u);
     }
     uint32_t m0 = 0u, m1 = 0u, m2 = 0u, m3 = 0u;
 #pragma unroll

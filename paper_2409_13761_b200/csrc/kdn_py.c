@@ -177,18 +177,55 @@ static int get_req(PyObject *q, kdn_compose_req *out, kdn_chunk *parts, int64_t 
     Py_XDECREF(ds); Py_XDECREF(ps); Py_XDECREF(do_); Py_XDECREF(po);
     return bad ? -1 : 0;
 }
-static PyObject *call_compose(PyObject *self, PyObject *const *a, Py_ssize_t n_args)
+/* selects[r]: a sequence with an entry per part of reqs[r], false (every token) or (address, count). */
+static int get_select(PyObject *sel, kdn_select *out, const int32_t **ptrs, int32_t *counts, Py_ssize_t parts)
 {
-    (void)self;
+    PyObject *seq = PySequence_Fast(sel, "a request's selects are a sequence");
+    if (!seq) return -1;
+    int bad = PySequence_Fast_GET_SIZE(seq) != parts;
+    if (bad) PyErr_SetString(PyExc_ValueError, "selects have to have an entry per part");
+    for (Py_ssize_t j = 0; !bad && j < parts; ++j) {
+        PyObject *e = PySequence_Fast_GET_ITEM(seq, j);
+        const int given = PyObject_IsTrue(e);
+        ptrs[j] = NULL;
+        counts[j] = 0;
+        if (given < 0) { bad = 1; break; }
+        if (!given) continue;
+        PyObject *address = PySequence_GetItem(e, 0), *count = address ? PySequence_GetItem(e, 1) : NULL;
+        void *p = NULL;
+        bad = !count || as_address(address, &p) != 0;
+        if (!bad) {
+            const long long c = PyLong_AsLongLong(count);
+            bad = c == -1 && PyErr_Occurred() != NULL;
+            ptrs[j] = (const int32_t *)p;
+            counts[j] = (int32_t)c;
+        }
+        Py_XDECREF(count);
+        Py_XDECREF(address);
+    }
+    Py_DECREF(seq);
+    out->part_select = ptrs;
+    out->part_n_select = counts;
+    return bad ? -1 : 0;
+}
+
+typedef kdn_status (*select_fn)(kdn_ctx *, int, const kdn_compose_req *, const kdn_select *, int, void *, void *);
+static PyObject *compose(PyObject *entry, PyObject *ctx_, PyObject *pool_, PyObject *reqs_, PyObject *selects_, PyObject *stream_, PyObject *side_)
+{
     void *fn, *ctx, *stream, *side;
-    if (n_args != 6) { PyErr_SetString(PyExc_TypeError, "six arguments"); return NULL; }
-    const long pool = PyLong_AsLong(a[2]);
-    if ((pool == -1 && PyErr_Occurred()) || as_address(a[0], &fn) || as_address(a[1], &ctx) || as_address(a[4], &stream) || as_address(a[5], &side)) return NULL;
-    PyObject *seq = PySequence_Fast(a[3], "reqs is a sequence");
+    const long pool = PyLong_AsLong(pool_);
+    if ((pool == -1 && PyErr_Occurred()) || as_address(entry, &fn) || as_address(ctx_, &ctx) || as_address(stream_, &stream) || as_address(side_, &side)) return NULL;
+    PyObject *seq = PySequence_Fast(reqs_, "reqs is a sequence");
     if (!seq) return NULL;
+    PyObject *sels = selects_ ? PySequence_Fast(selects_, "selects is a sequence") : NULL;
+    if (selects_ && !sels) { Py_DECREF(seq); return NULL; }
     const Py_ssize_t n = PySequence_Fast_GET_SIZE(seq);
     Py_ssize_t total = 0;
     int bad = 0;
+    if (sels && PySequence_Fast_GET_SIZE(sels) != n) {
+        PyErr_SetString(PyExc_ValueError, "selects have to have an entry per request");
+        bad = 1;
+    }
     for (Py_ssize_t i = 0; !bad && i < n; ++i) {
         PyObject *p = PyObject_GetAttr(PySequence_Fast_GET_ITEM(seq, i), s_parts);
         const Py_ssize_t k = p ? PySequence_Size(p) : -1;
@@ -198,29 +235,53 @@ static PyObject *call_compose(PyObject *self, PyObject *const *a, Py_ssize_t n_a
     kdn_compose_req few[FEW], *reqs = n <= FEW ? few : malloc(sizeof *reqs * (size_t)n);
     kdn_chunk few_parts[FEW], *parts = total <= FEW ? few_parts : malloc(sizeof *parts * (size_t)total);
     int64_t few_pos[FEW], *pos = total <= FEW ? few_pos : malloc(sizeof *pos * (size_t)total);
-    if (!bad && (!reqs || !parts || !pos)) { PyErr_NoMemory(); bad = 1; }
+    kdn_select few_sel[FEW], *sel = n <= FEW ? few_sel : malloc(sizeof *sel * (size_t)n);
+    const int32_t *few_ptr[FEW], **ptr = total <= FEW ? few_ptr : malloc(sizeof *ptr * (size_t)total);
+    int32_t few_cnt[FEW], *cnt = total <= FEW ? few_cnt : malloc(sizeof *cnt * (size_t)total);
+    if (!bad && (!reqs || !parts || !pos || !sel || !ptr || !cnt)) { PyErr_NoMemory(); bad = 1; }
     Py_ssize_t used = 0;
     for (Py_ssize_t i = 0; !bad && i < n; ++i) {
         bad = get_req(PySequence_Fast_GET_ITEM(seq, i), &reqs[i], parts + used, pos + used, total - used) != 0;
+        if (!bad && sels) bad = get_select(PySequence_Fast_GET_ITEM(sels, i), &sel[i], ptr + used, cnt + used, reqs[i].n_parts) != 0;
         if (!bad) used += reqs[i].n_parts;
     }
     kdn_status st = KDN_OK;
     if (!bad) {
         Py_BEGIN_ALLOW_THREADS
-        st = ((compose_fn)fn)((kdn_ctx *)ctx, (int)pool, reqs, (int)n, stream, side);
+        st = sels ? ((select_fn)fn)((kdn_ctx *)ctx, (int)pool, reqs, sel, (int)n, stream, side) : ((compose_fn)fn)((kdn_ctx *)ctx, (int)pool, reqs, (int)n, stream, side);
         Py_END_ALLOW_THREADS
     }
+    if (cnt != few_cnt) free(cnt);
+    if (ptr != few_ptr) free(ptr);
+    if (sel != few_sel) free(sel);
     if (pos != few_pos) free(pos);
     if (parts != few_parts) free(parts);
     if (reqs != few) free(reqs);
+    Py_XDECREF(sels);
     Py_DECREF(seq);
     return bad ? NULL : PyLong_FromLong((long)st);
+}
+/* call_compose(entry, ctx, pool_id, reqs, stream, side_stream) -> status */
+static PyObject *call_compose(PyObject *self, PyObject *const *a, Py_ssize_t n_args)
+{
+    (void)self;
+    if (n_args != 6) { PyErr_SetString(PyExc_TypeError, "six arguments"); return NULL; }
+    return compose(a[0], a[1], a[2], a[3], NULL, a[4], a[5]);
+}
+/* call_compose_select(entry, ctx, pool_id, reqs, selects, stream, side_stream) -> status */
+static PyObject *call_compose_select(PyObject *self, PyObject *const *a, Py_ssize_t n_args)
+{
+    (void)self;
+    if (n_args != 7) { PyErr_SetString(PyExc_TypeError, "seven arguments"); return NULL; }
+    return compose(a[0], a[1], a[2], a[3], a[4], a[5], a[6]);
 }
 
 static PyMethodDef methods[] = {
     { "call_xfer", (PyCFunction)(void (*)(void))call_xfer, METH_FASTCALL, "call_xfer(entry, ctx, pool_id, ops, stream, side_stream) -> status" },
     { "call_sparse", (PyCFunction)(void (*)(void))call_sparse, METH_FASTCALL, "call_sparse(entry, ctx, pool_id, ops, keeps, stream, side_stream) -> status" },
     { "call_compose", (PyCFunction)(void (*)(void))call_compose, METH_FASTCALL, "call_compose(entry, ctx, pool_id, reqs, stream, side_stream) -> status" },
+    { "call_compose_select", (PyCFunction)(void (*)(void))call_compose_select, METH_FASTCALL,
+      "call_compose_select(entry, ctx, pool_id, reqs, selects, stream, side_stream) -> status" },
     { NULL, NULL, 0, NULL }
 };
 static struct PyModuleDef module = { PyModuleDef_HEAD_INIT, "_kdn_native", "Native argument marshalling for kdn.py.", -1, methods, NULL, NULL, NULL, NULL };

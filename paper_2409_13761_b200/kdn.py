@@ -193,8 +193,8 @@ def _entry(name: str) -> int:
     return C.cast(getattr(lib, name), C.c_void_p).value
 
 
-_STORE, _RETRIEVE, _COMPOSE, _STORE_SPARSE, _RETRIEVE_SPARSE = (
-    _entry(n) for n in ("kdn_store", "kdn_retrieve", "kdn_compose", "kdn_store_sparse", "kdn_retrieve_sparse"))
+_STORE, _RETRIEVE, _COMPOSE, _STORE_SPARSE, _RETRIEVE_SPARSE, _COMPOSE_SELECT = (
+    _entry(n) for n in ("kdn_store", "kdn_retrieve", "kdn_compose", "kdn_store_sparse", "kdn_retrieve_sparse", "kdn_compose_select"))
 
 
 class KdnError(RuntimeError):
@@ -378,6 +378,8 @@ def kdn_retrieve_file(ctx, pool_id: int, ops: Sequence[XferOp], fds: Sequence[in
 
 def kdn_compose_select(ctx, pool_id: int, reqs: Sequence[ComposeReq], selects, stream: int = 0, side_stream: int = 0) -> None:
     """selects[r]: list with one entry per part of reqs[r]: None (every token) or (device address, count)."""
+    if _native is not None:
+        return _check(_native.call_compose_select(_COMPOSE_SELECT, ctx, pool_id, reqs, selects, stream, side_stream), "kdn_compose_select")
     arr = (kdn_select * max(1, len(reqs)))()
     keep = []
     for r, sel in enumerate(selects):

@@ -60,6 +60,24 @@ def test_requests(n, parts):
     assert kdn._native.call_compose(C.cast(entry, C.c_void_p).value, 8, 0, reqs, 0, 0) == 0
 
 
+def test_selects():
+    reqs = [kdn.ComposeReq(64, 9, [o.chunk for o in records(k)], list(range(k)), 1e4) for k in (3, 0, 20)]
+    selects = [[None, (0x5000, 7), None], [], [(0x6000 + j, j) if j % 2 else None for j in range(20)]]
+
+    @C.CFUNCTYPE(C.c_int, C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_int, C.c_void_p, C.c_void_p)
+    def entry(ctx, pool, p, sel, count, stream, side):
+        got = C.cast(sel, C.POINTER(kdn.kdn_select))
+        assert count == 3 and (ctx, pool, stream, side) == (8, 1, 2, 3)
+        for r, want in enumerate(selects):
+            for j, w in enumerate(want):
+                assert (got[r].part_select[j], got[r].part_n_select[j]) == (w if w else (None, 0))
+        return 0
+
+    assert kdn._native.call_compose_select(C.cast(entry, C.c_void_p).value, 8, 1, reqs, selects, 2, 3) == 0
+    with pytest.raises(ValueError):
+        kdn._native.call_compose_select(0, 8, 1, reqs, selects[:2], 2, 3)
+
+
 def test_bad_arguments_raise_and_do_not_call():
     with pytest.raises(AttributeError):
         kdn._native.call_xfer(0, 0, 0, [object()], 0, 0)
