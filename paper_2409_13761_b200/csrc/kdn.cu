@@ -115,7 +115,6 @@ struct kdn_ctx {
     LaunchEnv env;                          // SM count, shared-memory limit, per-kernel occupancy cache
     std::vector<Pool> pools;
     RingSlot ring[kRing];
-    unsigned char *h_ring = nullptr, *d_ring = nullptr; // what the slots' records live in (page-locked, device)
     unsigned ring_next = 0;
     int *d_status = nullptr;
     int *h_status = nullptr;                // pinned
@@ -1524,16 +1523,12 @@ kdn_status kdn_create(kdn_ctx **out, int device)
     if (cudaMalloc((void **)&ctx->d_status, sizeof(int)) != cudaSuccess) return fail(KDN_E_NOMEM);
     if (cudaMemset(ctx->d_status, 0, sizeof(int)) != cudaSuccess) return fail(KDN_E_CUDA);
     if (cudaMallocHost((void **)&ctx->h_status, sizeof(int)) != cudaSuccess) return fail(KDN_E_NOMEM);
-    // the descriptor ring: one page-locked and one device block, cut into slots
-    constexpr size_t kOps = sizeof(DevOp) * kMaxOpsPerLaunch, kRope = sizeof(RopeParam) * kMaxOpsPerLaunch;
-    if (cudaMallocHost((void **)&ctx->h_ring, kRing * (kOps + kRope)) != cudaSuccess) return fail(KDN_E_NOMEM);
-    if (cudaMalloc((void **)&ctx->d_ring, kRing * (kOps + kRope)) != cudaSuccess) return fail(KDN_E_NOMEM);
     for (int i = 0; i < kRing; ++i) {
         RingSlot &s = ctx->ring[i];
-        s.h_ops = reinterpret_cast<DevOp *>(ctx->h_ring + i * (kOps + kRope));
-        s.d_ops = reinterpret_cast<DevOp *>(ctx->d_ring + i * (kOps + kRope));
-        s.h_rope = reinterpret_cast<RopeParam *>(ctx->h_ring + i * (kOps + kRope) + kOps);
-        s.d_rope = reinterpret_cast<RopeParam *>(ctx->d_ring + i * (kOps + kRope) + kOps);
+        if (cudaMallocHost((void **)&s.h_ops, sizeof(DevOp) * kMaxOpsPerLaunch) != cudaSuccess) return fail(KDN_E_NOMEM);
+        if (cudaMalloc((void **)&s.d_ops, sizeof(DevOp) * kMaxOpsPerLaunch) != cudaSuccess) return fail(KDN_E_NOMEM);
+        if (cudaMallocHost((void **)&s.h_rope, sizeof(RopeParam) * kMaxOpsPerLaunch) != cudaSuccess) return fail(KDN_E_NOMEM);
+        if (cudaMalloc((void **)&s.d_rope, sizeof(RopeParam) * kMaxOpsPerLaunch) != cudaSuccess) return fail(KDN_E_NOMEM);
         if (cudaEventCreateWithFlags(&s.done, cudaEventDisableTiming) != cudaSuccess) return fail(KDN_E_CUDA);
     }
     *out = ctx;
@@ -1547,6 +1542,10 @@ void kdn_destroy(kdn_ctx *ctx)
     cudaDeviceSynchronize();
     for (int i = 0; i < kRing; ++i) {
         RingSlot &s = ctx->ring[i];
+        if (s.h_ops) cudaFreeHost(s.h_ops);
+        if (s.d_ops) cudaFree(s.d_ops);
+        if (s.h_rope) cudaFreeHost(s.h_rope);
+        if (s.d_rope) cudaFree(s.d_rope);
         if (s.d_table) cudaFree(s.d_table);
         if (s.done) cudaEventDestroy(s.done);
     }
@@ -1563,8 +1562,6 @@ void kdn_destroy(kdn_ctx *ctx)
         if (ctx->bounce[i]) cudaFreeHost(ctx->bounce[i]);
         if (ctx->bounce_done[i]) cudaEventDestroy(ctx->bounce_done[i]);
     }
-    if (ctx->h_ring) cudaFreeHost(ctx->h_ring);
-    if (ctx->d_ring) cudaFree(ctx->d_ring);
     if (ctx->fork) cudaEventDestroy(ctx->fork);
     if (ctx->own_side) cudaStreamDestroy(ctx->own_side);
     if (ctx->d_status) cudaFree(ctx->d_status);
