@@ -385,8 +385,8 @@ kdn_status kdn_set_tuning(kdn_ctx *ctx, const kdn_tuning *tuning);
  * on first use).  Takes effect at the next pinned-host call; frees slabs already allocated. */
 kdn_status kdn_set_staging_bytes(kdn_ctx *ctx, size_t bytes_per_slab);
 
-/* Limit, in nanoseconds, after which a wait inside the tile pipeline (and the wait of a key-plane or token-delta CTA for
- * its rows or bytes) gives up and the launch reports KDN_E_TIMEOUT
+/* Limit, in nanoseconds, after which a wait inside the tile pipeline or the rows kernels (and the wait of a token-delta
+ * decoder for its bytes) gives up and the launch reports KDN_E_TIMEOUT
  * (default, and ns = 0: two seconds).  The waits that let a CTA's own copies finish before it leaves always keep the
  * default.  Meant for exercising the error path: with a limit shorter than a memory access the next launches give up
  * almost at once, write little or nothing, and kdn_status_sync returns KDN_E_TIMEOUT; nothing faults or hangs, and
@@ -398,9 +398,9 @@ uint64_t kdn_launch_count(const kdn_ctx *ctx);
 
 /* Shape of the context's most recent launch of the tile pipeline, for reports: op 0 store / 1 retrieve / 2 compose
  * (the kernel is kdn_store_kernel / kdn_retrieve_kernel / kdn_compose_kernel<compute_groups, group_warps>, or, with
- * rows_kernel = 1, kdn_store_rows_kernel / kdn_retrieve_rows_kernel: tiles of up to 16 token rows, which keep-lists over
- * short rows and dense coded ops on pool blocks of 2 KiB or less are given); rows_per_tile: token rows per tile of a
- * keep-list launch (1 otherwise); grid is what was asked for (the launch itself never exceeds the CTAs resident at once). */
+ * rows_kernel = 1, kdn_store_rows_kernel / kdn_retrieve_rows_kernel, which move token rows one by one: compute_groups is then
+ * the slots a thread fills and group_warps the elements of its vectors); rows_per_tile: token rows per tile of a
+ * keep-list launch (1 otherwise); grid is what was asked for (a launch of the pipeline never exceeds the CTAs resident at once). */
 typedef struct {
     int32_t  op, compute_groups, group_warps, tile_bytes, stages, ctas_per_sm, store_lag, grid, smem_bytes;
     uint32_t n_tiles;
