@@ -433,6 +433,21 @@ kdn_status launch_behind(K kernel, dim3 grid, unsigned threads, size_t smem, cud
     return KDN_OK;
 }
 
+// The records of a launch to its ring slot: from `put` (n <= kPutOps), or from the slot's page-locked side.
+kdn_status send_ops(kdn_ctx *ctx, RingSlot *slot, PutLaunch *put, int n, cudaStream_t stream)
+{
+    if (!put) {
+        KDN_CUDA(cudaMemcpyAsync(slot->d_ops, slot->h_ops, sizeof(DevOp) * (size_t)n, cudaMemcpyHostToDevice, stream));
+        return KDN_OK;
+    }
+    put->dst = slot->d_ops;
+    put->n = n;
+    kdn_status r = launch_behind(kdn_put_ops_kernel, dim3(1), kPutThreads, 0, stream, *put);
+    if (r != KDN_OK) return r;
+    ctx->launches++;
+    return KDN_OK;
+}
+
 // Key planes of the per-channel key codecs, store: one CTA per (64-token group, slice of channels, layer, op).  The ops' records are
 // inl[0 .. n) (kernel parameters) or at d_ops.
 kdn_status launch_key_planes(kdn_ctx *ctx, const Pool &pool, const DevOp *inl, const DevOp *d_ops, int n, int groups, int layers, cudaStream_t stream)
@@ -519,13 +534,14 @@ bool rows_apply(const kdn_ctx *ctx, const Pool &pool, int OP, bool any_coded, bo
 kdn_status launch_rows(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops, int n, cudaStream_t stream)
 {
     RowsLaunch lp{};
-    const bool inl = n <= kInlineOps;
+    const bool inl = n <= kInlineOps, put = !inl && n <= kPutOps;
     RingSlot *slot = nullptr;
     if (!inl) {
         slot = &ctx->ring[ctx->ring_next++ % kRing];
         if (slot->used) KDN_CUDA(cudaEventSynchronize(slot->done));
     }
-    DevOp *h_ops = inl ? lp.inline_ops : slot->h_ops;
+    PutLaunch by_kernel;
+    DevOp *h_ops = inl ? lp.inline_ops : put ? by_kernel.ops : slot->h_ops;
     constexpr int kj = kRowsVectors;
     const RowsShape shape = rows_shape(pool, OP, hops, n);
     const unsigned vec = shape.vec;
@@ -557,7 +573,10 @@ kdn_status launch_rows(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hop
         if (tiles > kMaxTilesPerLaunch) return KDN_E_UNSUPPORTED;
     }
     if (tiles == 0) return KDN_OK;
-    if (!inl) KDN_CUDA(cudaMemcpyAsync(slot->d_ops, slot->h_ops, sizeof(DevOp) * (size_t)n, cudaMemcpyHostToDevice, stream));
+    if (!inl) {
+        kdn_status r = send_ops(ctx, slot, put ? &by_kernel : nullptr, n, stream);
+        if (r != KDN_OK) return r;
+    }
     lp.ops = inl ? nullptr : slot->d_ops;
     lp.n_ops = n;
     lp.k_layers = pool.d_k;
@@ -769,9 +788,9 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
                            (off_rope + table_bytes) * (size_t)ctas_per_sm <= smem_limit - 1024u * (size_t)ctas_per_sm;
     if (own_table) smem = off_rope + table_bytes;
 
-    // Few ops travel as kernel parameters; otherwise through a ring slot (pinned staging + device copy).  A ring
+    // Few ops travel as kernel parameters (a few more as those of a kernel in front); otherwise through a ring slot (pinned staging + device copy).  A ring
     // slot is also what owns the rotation table.
-    const bool inl = n <= kInlineOps;
+    const bool inl = n <= kInlineOps, put = !inl && n <= kPutOps;
     RingSlot *slot = nullptr;
     if (!inl || (any_rot && !own_table)) {
         slot = &ctx->ring[ctx->ring_next++ % kRing];
@@ -779,8 +798,9 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     }
     Launch lp{};
     RopeInline rope_inl{};
-    DevOp *h_ops = inl ? lp.inline_ops : slot->h_ops;
-    RopeParam *h_rope = own_table ? lp.inline_rope : inl ? rope_inl.p : slot ? slot->h_rope : nullptr;
+    PutLaunch by_kernel;
+    DevOp *h_ops = inl ? lp.inline_ops : put ? by_kernel.ops : slot->h_ops;
+    RopeParam *h_rope = own_table ? lp.inline_rope : inl || put ? rope_inl.p : slot ? slot->h_rope : nullptr;
 
     unsigned long long tiles = 0;
     int n_rope = 0;
@@ -808,16 +828,19 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     }
     if (tiles == 0) return KDN_OK;
 
-    if (!inl) KDN_CUDA(cudaMemcpyAsync(slot->d_ops, slot->h_ops, sizeof(DevOp) * (size_t)n, cudaMemcpyHostToDevice, stream));
+    if (!inl) {
+        kdn_status r = send_ops(ctx, slot, put ? &by_kernel : nullptr, n, stream);
+        if (r != KDN_OK) return r;
+    }
     const int half = pool.D / 2;
     if (n_rope && !own_table) {
         {
             kdn_status r = ensure_table(slot, n_rope, half);
             if (r != KDN_OK) return r;
         }
-        if (!inl) KDN_CUDA(cudaMemcpyAsync(slot->d_rope, slot->h_rope, sizeof(RopeParam) * (size_t)n_rope, cudaMemcpyHostToDevice, stream));
+        if (!inl && !put) KDN_CUDA(cudaMemcpyAsync(slot->d_rope, slot->h_rope, sizeof(RopeParam) * (size_t)n_rope, cudaMemcpyHostToDevice, stream));
         const long long total = (long long)n_rope * half;
-        kdn_rope_table_kernel<<<(unsigned)((total + 127) / 128), 128, 0, stream>>>(inl ? nullptr : slot->d_rope, rope_inl, n_rope,
+        kdn_rope_table_kernel<<<(unsigned)((total + 127) / 128), 128, 0, stream>>>(inl || put ? nullptr : slot->d_rope, rope_inl, n_rope,
                                                                               pool.D, slot->d_table);
         KDN_CUDA(cudaGetLastError());
         ctx->launches++;

@@ -1291,8 +1291,30 @@ __global__ void __launch_bounds__(kKcCols / 2u, 5) kdn_store_kc_kernel(const __g
     }
 }
 
+// Records of a launch of more than kInlineOps and up to kPutOps ops: a small kernel's parameters, which it writes to the ring slot that the
+// launch reads them from.  A copy of the same bytes goes through a copy engine, and the hand-over to the engine and back, 6-10 us, stands
+// between two kernels; this one is set up as the kernel before drains, as is the launch behind it.  us through a copy / this kernel: 33 retrieves
+// of half of 100 tokens, two heads, int8 36.1 / 26.5; 33 stores of 117 tokens, two heads, int8 49.4 / 40.5; raw retrieves of 100 tokens of eight
+// heads, 33 of them 149 / 142, 64: 274 / 269, 128: 537 / 531.  Letting the launch start before the records are written costs 2-9 us of that.
+constexpr int kPutOps = 128;
+constexpr int kPutThreads = 256;
+struct PutLaunch {
+    DevOp *dst;
+    int n;
+    DevOp ops[kPutOps];
+};
+__global__ void __launch_bounds__(kPutThreads) kdn_put_ops_kernel(const __grid_constant__ PutLaunch P)
+{
+    static_assert(sizeof(DevOp) % 8 == 0, "records are copied as 8-byte words");
+    dependency_wait();                                     // what may still read the slot ended with, or before, the kernel before this one
+    const unsigned long long *src = reinterpret_cast<const unsigned long long *>(P.ops);
+    unsigned long long *dst = reinterpret_cast<unsigned long long *>(P.dst);
+    for (unsigned i = threadIdx.x; i < (unsigned)P.n * (unsigned)(sizeof(DevOp) / 8u); i += kPutThreads) dst[i] = src[i];
+    release_dependents();                                  // (not before: CTAs of the launch would be placed round this one, unevenly)
+}
+
 // Few rows: passed as kernel parameters; more: params.
-struct RopeInline { RopeParam p[kInlineOps]; };
+struct RopeInline { RopeParam p[kPutOps]; };
 
 __global__ void kdn_rope_table_kernel(const RopeParam *params, const __grid_constant__ RopeInline inl, int n_rows, int D,
                                       float2 *table)

@@ -691,3 +691,63 @@ def test_large_retrieves_of_4_bit_codes_move_row_by_row():
             assert np.array_equal(dev.pool_np(), ref)
     finally:
         dev.close()
+
+
+@pytest.mark.parametrize("n", [32, 33, 128, 129])
+def test_records_reach_the_kernels_whichever_way_they_travel(n):
+    """Calls of so many ops that their records travel as the launch's parameters, as those of a kernel in front of it, or through a copy:
+    store (a per-channel key codec among them), store and retrieve by keep-lists, retrieve, and a composed request of n re-rotated parts, call
+    after call into the same ring of records."""
+    shape = synth.TOY.with_(n_blocks=640)
+    dev = Device(shape, seed=77)
+    try:
+        K, bs, stream = dev.K, shape.block_size, dev.stream.cuda_stream
+        host = dev.pool_np()
+        ref = host.copy()
+        perm = np.random.default_rng(n).permutation(shape.n_blocks).astype(np.int32)
+        codecs = (RAW, INT8, INT4, oracle.INT8_KC64)
+        keep = np.array([0, 1, 3, 7, 8, 13], dtype=np.int32)
+        d_keep = dev.table(keep)
+        stored, kept = [], []
+        for i in range(n):
+            tab, T, codec = perm[2 * i:2 * i + 2], 1 + (7 * i) % 17, codecs[i % 4]
+            stored.append((tab, T, codec, dev.chunk_buf(T, codec), dev.chunk_buf(len(keep), codecs[i % 3])))
+        tabs = [dev.table(s[0]) for s in stored]
+        for _ in range(2):
+            dev.store([dev.op(t, 0, s[3], s[1], s[2]) for t, s in zip(tabs, stored)])
+            K.kdn_store_sparse(dev.ctx, dev.pool_id, [dev.op(t, 0, s[4], len(keep), codecs[i % 3]) for i, (t, s) in enumerate(zip(tabs, stored))],
+                               [d_keep.data_ptr()] * n, stream)
+        assert dev.sync() == 0
+        for i, (tab, T, codec, buf, kbuf) in enumerate(stored):
+            assert np.array_equal(to_np(buf), oracle.store(host, tab, 0, T, codec)), i
+            kept.append(oracle.store(host, tab, 0, len(keep), codecs[i % 3], keep=keep))
+            assert np.array_equal(to_np(kbuf), kept[-1]), i
+        # back into other blocks: chunks into two blocks each, the listed tokens over the first of them
+        dst = [perm[2 * n + 2 * i:2 * n + 2 * i + 2] for i in range(n)]
+        d_dst = [dev.table(d) for d in dst]
+        dev.retrieve([dev.op(t, 0, s[3], s[1], s[2]) for t, s in zip(d_dst, stored)])
+        K.kdn_retrieve_sparse(dev.ctx, dev.pool_id, [dev.op(t, 0, s[4], len(keep), codecs[i % 3]) for i, (t, s) in enumerate(zip(d_dst, stored))],
+                              [d_keep.data_ptr()] * n, stream)
+        assert dev.sync() == 0
+        for i, (tab, T, codec, buf, kbuf) in enumerate(stored):
+            oracle.retrieve(ref, dst[i], 0, T, codec, to_np(buf))
+            oracle.retrieve(ref, dst[i], 0, len(keep), codecs[i % 3], kept[i], keep=keep)
+        assert np.array_equal(dev.pool_np(), ref)
+        # one request of n parts behind one another, all but the first re-rotated
+        req = perm[4 * n:4 * n + 120] if 4 * n + 120 <= shape.n_blocks else perm[:120]
+        parts = [s for s in stored if s[2] != oracle.INT8_KC64] * 2
+        parts = (parts + parts)[:n]
+        places = np.concatenate([[0], np.cumsum([p[1] for p in parts])])
+        assert places[-1] <= 120 * bs
+        dev.compose([K.ComposeReq(dev.table(req).data_ptr(), len(req), [dev.chunk(p[3], p[1], p[2], 0) for p in parts],
+                                  [int(x) for x in places[:-1]], shape.rope_theta)])
+        assert dev.sync() == 0
+        kref, kmag = oracle.compose(ref, req, [(to_np(p[3]), p[1], p[2], 0, int(x)) for p, x in zip(parts, places)], shape.rope_theta, want_ref=True)
+        got = dev.pool_np()
+        rot = np.zeros(got.shape, dtype=bool)
+        pos = np.arange(int(places[1]), int(places[-1]))
+        rot[:, 0, req[pos // bs], pos % bs] = True
+        assert np.array_equal(got[~rot], ref[~rot])
+        check_rotated_keys(gather_positions(got, req, pos)[:, 0], kref[:, pos], kmag[:, pos], gather_positions(ref, req, pos)[:, 0])
+    finally:
+        dev.close()
