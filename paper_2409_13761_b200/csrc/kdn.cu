@@ -505,8 +505,9 @@ RowsShape rows_shape(const Pool &pool, int OP, const HostOp *hops, int n)
 // Whether a launch goes to the kernels that move token rows one by one (kdn_rows.cuh).
 // Keep-lists over rows of up to 1024 elements: the tile pipeline issues a copy a row.  Half of the tokens kept, us in the tile pipeline / here
 // (8B shape, 16 x 1024 tokens): two heads (rows of 256) retrieve int8 114 / 76, int4 115 / 69, store int8 117 / 78, int4 117 / 66; one head raw
-// (32 x 1024) 125 / 92; eight heads (rows of 1024, 16 x 512) retrieve int8 146 / 144, int4 142 / 122, store int8 143 / 140, raw 172 / 171.  Only the
-// retrieve of long rows with a scale per channel (eight heads: 185 / 327) stays, since it would read the scales of every row anew.
+// (32 x 1024) 125 / 92; eight heads (rows of 1024, 16 x 512) retrieve int8 146 / 144, int4 142 / 122, store int8 143 / 140, raw 172 / 171.  The
+// retrieve of long rows with a scale per channel (eight heads: 185 / 327) stays, since it would read the scales of every row anew; so does that of long
+// raw rows, which a copy a row moves as well without the uneven waves of these CTAs (eight heads, half of 3 x 165 tokens 9.8 / 14.1; four heads 9.1 / 6.8).
 // Coded dense ops on pool blocks of 2 KiB or less: a coding tile that stops at the end of its block is far too small (int8, blocks of four tokens
 // of one head: 135 / 76).  On blocks of 4 KiB it depends on the size (one head, int8): one chunk of 512 tokens store 5.8 / 5.3, retrieve 5.5 / 5.1; 64 chunks
 // 157 / 152 and 152 / 149; in between, where these kernels' CTAs make a few uneven waves, the pipeline is ahead (8 x 300 tokens 15.7 / 17).
@@ -521,7 +522,7 @@ bool rows_apply(const kdn_ctx *ctx, const Pool &pool, int OP, bool any_coded, bo
     if (any_list) {
         for (int i = 0; i < n; ++i)
             if (hops[i].op.list_mode != 1) return false;
-        return row_elems < 512u || (row_elems <= 1024u && !(any_kc && OP == OP_RETRIEVE));
+        return row_elems < 512u || (row_elems <= 1024u && !(OP == OP_RETRIEVE && (any_kc || (!any_coded && row_elems > 512u))));
     }
     if (!any_coded || any_kc) return false;
     const unsigned long long block_bytes = (unsigned long long)pool.bs * row_elems * 2ull;
