@@ -718,10 +718,19 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
         // A small coded launch, 8 to 32 tiles an SM, is pipeline fill and drain: four slots in four CTAs of one group each start sooner than six in
         // three CTAs of two (8B shape, 77 tokens int8: store 6.4 -> 6.1 us, retrieve 6.0 -> 5.7; 200 tokens 9.5 -> 9.1 and 8.8 -> 8.6;
         // 512 tokens, 55 tiles an SM: store 20.6 -> 20.4 but retrieve 20.4 -> 20.6 and int4 18.1 -> 18.5; 6 tiles an SM: 4.9 -> 5.0)
+        // Not where a CTA meets only one or two places of a plane, its stride being a multiple of half a plane's tiles, and some places hold no
+        // token: CTAs there would have nothing to do (80 layers, 193 tokens of two heads in blocks of 64, int8 store: 7.8 us, with four CTAs 8.5).
         unsigned long long tiles_ahead = 0;
-        for (int i = 0; i < n; ++i) tiles_ahead += (unsigned long long)hops[i].op.nl * (OP == OP_STORE && is_kc(hops[i].op.codec) ? 1ull : 2ull) * (unsigned)hops[i].op.nblk * tpb;
         const unsigned long long sms = (unsigned long long)ctx->env.sm_count;
-        if (tiles_ahead >= 8ull * sms && tiles_ahead < 32ull * sms) def = Shape{ 8192, 4, 4, 1, 1 };
+        bool uneven = false;
+        for (int i = 0; i < n; ++i) {
+            const DevOp &op = hops[i].op;
+            const unsigned long long plane = (unsigned long long)(unsigned)op.nblk * tpb;
+            tiles_ahead += (unsigned long long)op.nl * (OP == OP_STORE && is_kc(op.codec) ? 1ull : 2ull) * plane;
+            const unsigned long long tokens = plane * tile_elems / row_elems;      // of a plane's tiles
+            uneven |= plane && (2ull * 4ull * sms) % plane == 0ull && tokens >= (unsigned)op.T + tile_elems / row_elems;
+        }
+        if (tiles_ahead >= 8ull * sms && tiles_ahead < 32ull * sms && !uneven) def = Shape{ 8192, 4, 4, 1, 1 };
     }
     if (!any_list && !kc_decode && ctx->tuning.tile_bytes <= 0) {
         // A pool block smaller than the tile the shape was tuned for (few KV heads per GPU under tensor parallelism, or
