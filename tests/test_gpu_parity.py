@@ -751,3 +751,28 @@ def test_records_reach_the_kernels_whichever_way_they_travel(n):
         check_rotated_keys(gather_positions(got, req, pos)[:, 0], kref[:, pos], kmag[:, pos], gather_positions(ref, req, pos)[:, 0])
     finally:
         dev.close()
+
+
+@pytest.mark.parametrize("T,four", [(193, False), (241, True), (256, True)])
+@pytest.mark.parametrize("codec", [INT8, INT4])
+def test_small_coded_launches_take_four_ctas_an_sm_unless_some_would_idle(T, four, codec):
+    """A plane of 16 tiles, which the stride of four CTAs an SM is a multiple of: without a token in the last tiles another shape runs, with
+    one in every tile that one.  Bit-exact both ways."""
+    shape = synth.TOY.with_(n_layers=40, n_kv_heads=2, head_dim=128, block_size=64, n_blocks=8)
+    dev = Device(shape, seed=31)
+    try:
+        K = dev.K
+        ref = dev.pool_np()
+        perm = np.random.default_rng(3).permutation(8).astype(np.int32)
+        buf = dev.chunk_buf(T, codec)
+        dev.store([dev.op(dev.table(perm[:4]), 0, buf, T, codec)])
+        assert dev.sync() == 0
+        assert (K.kdn_last_launch(dev.ctx)["ctas_per_sm"] == 4) == four
+        want = oracle.store(ref, perm[:4], 0, T, codec)
+        assert np.array_equal(to_np(buf), want)
+        dev.retrieve([dev.op(dev.table(perm[4:]), 0, buf, T, codec)])
+        assert dev.sync() == 0
+        oracle.retrieve(ref, perm[4:], 0, T, codec, want)
+        assert np.array_equal(dev.pool_np(), ref)
+    finally:
+        dev.close()
