@@ -51,7 +51,17 @@ def build_native(force: bool = False) -> str:
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    build_native(force)
+    """The library, and the extension module where that can be had (without it kdn.py marshals through ctypes)."""
+    lib = build_library(force, verbose)
+    try:
+        build_native(force)
+    except Exception as exc:                                 # no C compiler, or no Python headers
+        print("%s was not built, ctypes does its work: %s" % (os.path.basename(NATIVE), exc), file=sys.stderr)
+    return lib
+
+
+def build_library(force: bool = False, verbose: bool = False) -> str:
+    """Compile libkdn.so (needs nvcc, nothing of Python's)."""
     if not force and up_to_date():
         return LIB
     tmp = LIB + ".%d.tmp" % os.getpid()
@@ -72,7 +82,7 @@ def cuda_home() -> str:
 
 def build_example(name: str, out_dir: str) -> str:
     """Compile examples/<name>.c (plain C99 against include/kdn.h) and link it with libkdn.so; returns the executable."""
-    build()
+    build_library()
     src = os.path.join(HERE, "examples", name + ".c")
     exe = os.path.join(out_dir, name)
     cc = shutil.which("gcc") or shutil.which("cc")

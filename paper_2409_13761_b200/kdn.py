@@ -93,7 +93,7 @@ def _load() -> C.CDLL:
     path = _build.LIB
     if not _build.up_to_date():
         try:
-            _build.build()
+            _build.build_library()
         except Exception as exc:                      # no nvcc, or the compile failed
             if not os.path.exists(path):
                 raise ImportError("libkdn.so is missing and could not be built: %s" % exc) from exc
