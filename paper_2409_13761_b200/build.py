@@ -1,6 +1,7 @@
 """Build libkdn.so (CUDA, sm_100a only) in-tree with nvcc.  ``python -m paper_2409_13761_b200.build``."""
 from __future__ import annotations
 
+import hashlib
 import os
 import shutil
 import subprocess
@@ -11,8 +12,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libkdn.so")
-NATIVE = os.path.join(HERE, "_kdn_native.so")            # argument marshalling for kdn.py
-NATIVE_SOURCE = os.path.join(CSRC, "kdn_py.c")
+NATIVE = os.path.join(HERE, "_kdn_native" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))      # argument marshalling for kdn.py; of one interpreter
+NATIVE_DEPS = [os.path.join(CSRC, "kdn_py.c"), os.path.join(ROOT, "include", "kdn.h")]
 SOURCES = [os.path.join(CSRC, "kdn.cu"), os.path.join(CSRC, "kdn_shell.cu")]
 DEPS = SOURCES + [os.path.join(CSRC, "kdn_kernels.cuh"), os.path.join(CSRC, "kdn_rows.cuh"), os.path.join(CSRC, "kdn_td.cuh"), os.path.join(ROOT, "include", "kdn.h")]
 
@@ -31,9 +32,20 @@ def up_to_date() -> bool:
     return all(os.path.getmtime(d) <= t for d in DEPS)
 
 
+def native_stamp() -> str:
+    """What the extension module was made from: it fills the header's records, so one made from another header must never be used."""
+    h = hashlib.sha256()
+    for d in NATIVE_DEPS:
+        with open(d, "rb") as f:
+            h.update(f.read())
+    return "kdn-native-" + h.hexdigest()
+
+
 def native_up_to_date() -> bool:
-    return os.path.exists(NATIVE) and all(os.path.getmtime(d) <= os.path.getmtime(NATIVE)
-                                          for d in (NATIVE_SOURCE, os.path.join(ROOT, "include", "kdn.h")))
+    if not os.path.exists(NATIVE):
+        return False
+    with open(NATIVE, "rb") as f:
+        return native_stamp().encode() in f.read()
 
 
 def build_native(force: bool = False) -> str:
@@ -45,7 +57,7 @@ def build_native(force: bool = False) -> str:
         raise RuntimeError("no C compiler found")
     tmp = NATIVE + ".%d.tmp" % os.getpid()
     subprocess.run([cc, "-O2", "-Wall", "-shared", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"],
-                    NATIVE_SOURCE, "-o", tmp], check=True)
+                    '-DKDN_STAMP="%s"' % native_stamp(), NATIVE_DEPS[0], "-o", tmp], check=True)
     os.replace(tmp, NATIVE)
     return NATIVE
 

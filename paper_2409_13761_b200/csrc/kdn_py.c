@@ -294,5 +294,7 @@ PyMODINIT_FUNC PyInit__kdn_native(void)
         { &s_base_pos, "base_pos" }, { &s_parts, "parts" }, { &s_part_dst_pos, "part_dst_pos" }, { &s_rope_theta, "rope_theta" }, { &s_rope_style, "rope_style" } };
     for (size_t i = 0; i < sizeof names / sizeof *names; ++i)
         if (!(*names[i].to = PyUnicode_InternFromString(names[i].text))) return NULL;
-    return PyModule_Create(&module);
+    PyObject *m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "stamp", KDN_STAMP)) { Py_DECREF(m); return NULL; }      /* (build.py looks for it in the file) */
+    return m;
 }

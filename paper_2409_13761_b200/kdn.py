@@ -7,6 +7,7 @@ if libkdn.so is absent and cannot be built.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 from dataclasses import dataclass
 from typing import List, Optional, Sequence
@@ -179,11 +180,15 @@ def _load_native():
         _build.build_native()
     except Exception:                                 # no C compiler or no Python headers; a module built elsewhere may be there
         pass
+    if not _build.native_up_to_date():                # ... but one made from another header has the records laid out differently
+        return None
     try:
-        from . import _kdn_native
+        spec = importlib.util.spec_from_file_location(__package__ + "._kdn_native", _build.NATIVE)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
     except ImportError:
         return None
-    return _kdn_native
+    return module
 
 
 _native = _load_native()

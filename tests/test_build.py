@@ -1,9 +1,10 @@
 """What is built without what: the library needs nvcc alone, the extension module a C compiler and Python's headers."""
 import os
+import sysconfig
 
 import pytest
 
-from paper_2409_13761_b200 import build
+from paper_2409_13761_b200 import build, kdn
 
 
 @pytest.fixture
@@ -42,3 +43,26 @@ def test_a_library_that_cannot_be_built_is_an_error(commands, monkeypatch):
 def test_the_library_alone_needs_no_c_compiler(commands):
     assert build.build_library() == build.LIB
     assert [os.path.basename(c[0]) for c in commands] == ["nvcc"]
+
+
+@pytest.mark.skipif(kdn._native is None, reason="no C compiler or no Python headers")
+def test_a_module_made_from_another_header_or_for_another_interpreter_is_not_used(monkeypatch, tmp_path):
+    assert build.NATIVE.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    assert kdn._native.stamp == build.native_stamp()
+
+    def fails(force=False):
+        raise RuntimeError("no C compiler found")
+
+    monkeypatch.setattr(build, "build_native", fails)
+    with open(build.NATIVE, "rb") as f:
+        module = f.read()
+    other = tmp_path / os.path.basename(build.NATIVE)
+    monkeypatch.setattr(build, "NATIVE", str(other))
+    assert kdn._load_native() is None                        # there is none for this interpreter
+    other.write_bytes(module)
+    assert kdn._load_native().stamp == build.native_stamp()
+    other.unlink()
+    stamp = build.native_stamp().encode()
+    other.write_bytes(module.replace(stamp, stamp[:-1] + (b"0" if stamp[-1:] != b"0" else b"1")))
+    os.utime(other, (4e9, 4e9))                              # newer than its source
+    assert not build.native_up_to_date() and kdn._load_native() is None
