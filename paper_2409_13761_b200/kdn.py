@@ -246,6 +246,10 @@ class ComposeReq:
     rope_style: int = 0
 
 
+if _native is not None:
+    _native.set_types(Chunk, C.c_void_p)
+
+
 def pool_desc(n_layers: int, n_kv_heads: int, head_dim: int, block_size: int, n_blocks: int,
               k_layers: Optional[Sequence[int]] = None, v_layers: Optional[Sequence[int]] = None) -> kdn_pool_desc:
     """Build a kdn_pool_desc; the pointer arrays are kept alive on the returned object."""
@@ -323,13 +327,23 @@ def kdn_validate_compose(desc: kdn_pool_desc, reqs: Sequence[ComposeReq]) -> int
 
 def kdn_store(ctx, pool_id: int, ops: Sequence[XferOp], stream: int = 0, side_stream: int = 0) -> None:
     if _native is not None:
-        return _check(_native.call_xfer(_STORE, ctx, pool_id, ops, stream, side_stream), "kdn_store")
+        try:
+            status = _native.call_xfer(_STORE, ctx, pool_id, ops, stream, side_stream)
+        except Exception:                             # not a plain form: nothing was called, ctypes decides
+            pass
+        else:
+            return _check(status, "kdn_store")
     _check(lib.kdn_store(ctx, pool_id, xfer_array(ops), len(ops), stream, side_stream), "kdn_store")
 
 
 def kdn_retrieve(ctx, pool_id: int, ops: Sequence[XferOp], stream: int = 0, side_stream: int = 0) -> None:
     if _native is not None:
-        return _check(_native.call_xfer(_RETRIEVE, ctx, pool_id, ops, stream, side_stream), "kdn_retrieve")
+        try:
+            status = _native.call_xfer(_RETRIEVE, ctx, pool_id, ops, stream, side_stream)
+        except Exception:                             # not a plain form: nothing was called, ctypes decides
+            pass
+        else:
+            return _check(status, "kdn_retrieve")
     _check(lib.kdn_retrieve(ctx, pool_id, xfer_array(ops), len(ops), stream, side_stream), "kdn_retrieve")
 
 
@@ -353,13 +367,23 @@ def sparse_array(ops: Sequence[XferOp], keeps: Sequence[int]):
 def kdn_store_sparse(ctx, pool_id: int, ops: Sequence[XferOp], keeps: Sequence[int], stream: int = 0, side_stream: int = 0) -> None:
     """keeps[i]: device address of the int32 keep-list of ops[i] (ops[i].chunk.n_tokens entries)."""
     if _native is not None:
-        return _check(_native.call_sparse(_STORE_SPARSE, ctx, pool_id, ops, keeps, stream, side_stream), "kdn_store_sparse")
+        try:
+            status = _native.call_sparse(_STORE_SPARSE, ctx, pool_id, ops, keeps, stream, side_stream)
+        except Exception:                             # not a plain form: nothing was called, ctypes decides
+            pass
+        else:
+            return _check(status, "kdn_store_sparse")
     _check(lib.kdn_store_sparse(ctx, pool_id, sparse_array(ops, keeps), len(ops), stream, side_stream), "kdn_store_sparse")
 
 
 def kdn_retrieve_sparse(ctx, pool_id: int, ops: Sequence[XferOp], keeps: Sequence[int], stream: int = 0, side_stream: int = 0) -> None:
     if _native is not None:
-        return _check(_native.call_sparse(_RETRIEVE_SPARSE, ctx, pool_id, ops, keeps, stream, side_stream), "kdn_retrieve_sparse")
+        try:
+            status = _native.call_sparse(_RETRIEVE_SPARSE, ctx, pool_id, ops, keeps, stream, side_stream)
+        except Exception:                             # not a plain form: nothing was called, ctypes decides
+            pass
+        else:
+            return _check(status, "kdn_retrieve_sparse")
     _check(lib.kdn_retrieve_sparse(ctx, pool_id, sparse_array(ops, keeps), len(ops), stream, side_stream), "kdn_retrieve_sparse")
 
 
@@ -384,11 +408,18 @@ def kdn_retrieve_file(ctx, pool_id: int, ops: Sequence[XferOp], fds: Sequence[in
 def kdn_compose_select(ctx, pool_id: int, reqs: Sequence[ComposeReq], selects, stream: int = 0, side_stream: int = 0) -> None:
     """selects[r]: list with one entry per part of reqs[r]: None (every token) or (device address, count)."""
     if _native is not None:
-        return _check(_native.call_compose_select(_COMPOSE_SELECT, ctx, pool_id, reqs, selects, stream, side_stream), "kdn_compose_select")
+        try:
+            status = _native.call_compose_select(_COMPOSE_SELECT, ctx, pool_id, reqs, selects, stream, side_stream)
+        except Exception:                             # not a plain form: nothing was called, ctypes decides
+            pass
+        else:
+            return _check(status, "kdn_compose_select")
     arr = (kdn_select * max(1, len(reqs)))()
     keep = []
     for r, sel in enumerate(selects):
         n = len(sel)
+        if r < len(reqs) and n < len(reqs[r].parts):
+            raise ValueError("selects have to have an entry per part")
         ptrs = (C.c_void_p * max(1, n))(*[(x[0] if x else None) for x in sel])
         cnts = (C.c_int32 * max(1, n))(*[(x[1] if x else 0) for x in sel])
         keep.append((ptrs, cnts))
@@ -398,7 +429,12 @@ def kdn_compose_select(ctx, pool_id: int, reqs: Sequence[ComposeReq], selects, s
 
 def kdn_compose(ctx, pool_id: int, reqs: Sequence[ComposeReq], stream: int = 0, side_stream: int = 0) -> None:
     if _native is not None:
-        return _check(_native.call_compose(_COMPOSE, ctx, pool_id, reqs, stream, side_stream), "kdn_compose")
+        try:
+            status = _native.call_compose(_COMPOSE, ctx, pool_id, reqs, stream, side_stream)
+        except Exception:                             # not a plain form: nothing was called, ctypes decides
+            pass
+        else:
+            return _check(status, "kdn_compose")
     _check(lib.kdn_compose(ctx, pool_id, compose_array(reqs), len(reqs), stream, side_stream), "kdn_compose")
 
 
