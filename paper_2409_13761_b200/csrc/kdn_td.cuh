@@ -95,30 +95,30 @@ __host__ __device__ inline size_t td_decode_smem_bytes(unsigned cols, unsigned w
 __device__ __forceinline__ uint32_t td_be(uint32_t w) { return __byte_perm(w, 0u, 0x0123); }
 
 // Exclusive prefix sum of one value per thread over the block (blockDim.x a multiple of 32, at most 1024);
-// *total receives the sum.  `scratch` is 33 words of shared memory.
-__device__ __forceinline__ unsigned td_block_scan(unsigned v, unsigned *scratch, unsigned *total)
+// *total receives the sum.  `scratch` is 33 words of shared memory.  (64 bits: the segments that a step adds up may take more than 4 GiB.)
+__device__ __forceinline__ unsigned long long td_block_scan(unsigned long long v, unsigned long long *scratch, unsigned long long *total)
 {
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    unsigned inc = v;
+    unsigned long long inc = v;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-        const unsigned o = __shfl_up_sync(0xffffffffu, inc, d);
+        const unsigned long long o = __shfl_up_sync(0xffffffffu, inc, d);
         if (lane >= (unsigned)d) inc += o;
     }
     if (lane == 31u) scratch[warp] = inc;
     __syncthreads();
     if (warp == 0) {
-        unsigned w = lane < nwarps ? scratch[lane] : 0u, winc = w;
+        unsigned long long w = lane < nwarps ? scratch[lane] : 0ull, winc = w;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            const unsigned o = __shfl_up_sync(0xffffffffu, winc, d);
+            const unsigned long long o = __shfl_up_sync(0xffffffffu, winc, d);
             if (lane >= (unsigned)d) winc += o;
         }
         scratch[lane] = winc - w;
         if (lane == 31u) scratch[32] = winc;
     }
     __syncthreads();
-    const unsigned r = scratch[warp] + inc - v;
+    const unsigned long long r = scratch[warp] + inc - v;
     *total = scratch[32];
     __syncthreads();
     return r;
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == 128u ? 6 : 1) kdn_td_pla
 constexpr unsigned kTdScanThreads = 1024;
 __global__ void __launch_bounds__(kTdScanThreads) kdn_td_scan_kernel(const __grid_constant__ TdLaunch P)
 {
-    __shared__ unsigned scratch[33];
+    __shared__ unsigned long long scratch[33];
     dependency_wait();
     release_dependents();
     const DevOp op = P.inline_ops[blockIdx.x];
@@ -502,9 +502,9 @@ __global__ void __launch_bounds__(kTdScanThreads) kdn_td_scan_kernel(const __gri
                 for (unsigned p = 0; p < per_seg; ++p) size += warp_bytes[sidx * per_seg + p];
             }
         }
-        size = (size + 15u) & ~15u;
-        unsigned total;
-        const unsigned before = td_block_scan(size, scratch, &total);
+        size = (size + 15u) & ~15u;                          // (of one segment: at most 72 bytes for each of 2^24 channels)
+        unsigned long long total;
+        const unsigned long long before = td_block_scan(size, scratch, &total);
         if (sidx < lay.S) seg_off[sidx + 1ull] = run + before + size;
         run += total;
     }

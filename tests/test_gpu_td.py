@@ -508,3 +508,46 @@ def test_a_block_id_outside_the_pool_in_a_store_is_reported_and_nothing_leaves_t
         assert np.array_equal(to_np(buf)[:used], want[:used])
     finally:
         dev.close()
+
+
+def test_segment_offsets_beyond_32_bits():
+    """1024 segments of 65536 channels at about 69 bytes each add up to more than 4 GiB: every segment's place is the sum of the
+    sizes before it.  All layers, groups and K and V read one and the same block, so all segments are alike."""
+    shape = synth.TOY.with_(n_layers=8, n_kv_heads=512, head_dim=128, block_size=64, n_blocks=2)
+    one = shape.with_(n_layers=1)
+    T, G, codec = 64 * 64, 64, TD8
+    host = np.empty((1, 2, 2, 64, 512, 128), dtype=np.uint16)
+    host[:] = bf16_bits(np.random.default_rng(5).uniform(-1.0, 1.0, host.shape[2:]))     # (uniform: the longest sub-streams)
+    dev = Device(one, pool_np=host)
+    K = dev.K
+    try:
+        desc = K.pool_desc(8, 512, 128, 64, 2, [dev.k[0].data_ptr()] * 8, [dev.k[0].data_ptr()] * 8)
+        pool_id = K.kdn_pool_register(dev.ctx, desc)
+        lay = K.kdn_td_layout(desc, T, codec)
+        S = lay["segments"]
+        assert S == 1024
+        want = oracle.store(host, np.zeros(1, dtype=np.int32), 0, 64, codec)                # two segments of the same kind
+        lw = oracle.td_layout(1, 512, 128, 64, codec)
+        off_w = want[:24].view(np.uint64).astype(np.int64)
+        size = int(off_w[1] - off_w[0])
+        assert S * size > 1 << 32
+        buf = torch.empty(lay["capacity"], dtype=torch.uint8, device=dev.dev)
+        table = dev.table(np.zeros(G, dtype=np.int32))
+        K.kdn_store(dev.ctx, pool_id, [K.XferOp(table.data_ptr(), G, 0, K.Chunk(buf.data_ptr(), buf.numel(), T, codec))], dev.stream.cuda_stream)
+        assert dev.sync() == 0
+        off = buf[:8 * (S + 1)].view(torch.int64).cpu().numpy()
+        assert np.array_equal(off, lay["streams_offset"] + size * np.arange(S + 1, dtype=np.int64))
+        first = buf[off[0]:off[1]]
+        assert np.array_equal(to_np(first), want[off_w[0]:off_w[1]])
+        assert np.array_equal(to_np(buf[lay["lens_offset"]:lay["lens_offset"] + 65536]), want[lw["lens"]:lw["lens"] + 65536])
+        for s in range(1, S):
+            assert torch.equal(buf[off[s]:off[s + 1]], first), s
+        # and back, into the other block
+        table1 = dev.table(np.ones(G, dtype=np.int32))
+        K.kdn_retrieve(dev.ctx, pool_id, [K.XferOp(table1.data_ptr(), G, 0, K.Chunk(buf.data_ptr(), buf.numel(), T, codec))], dev.stream.cuda_stream)
+        assert dev.sync() == 0
+        ref = host.copy()
+        oracle.retrieve(ref, np.ones(1, dtype=np.int32), 0, 64, codec, want)
+        assert np.array_equal(dev.pool_np()[0, 0], ref[0, 0])
+    finally:
+        dev.close()
