@@ -77,6 +77,9 @@
  *   chunk whose bytes in use exceed a staging slab, or whose offset table no store can have written, is refused).
  *   kdn_retrieve_file takes them the same way (the offset table is read from the file first, then the bytes in use,
  *   so only those need be in the file); kdn_store_file does not, for the reason kdn_store does not write host chunks.
+ * Coded values have to be finite.  A NaN or an infinity is not kept: what it decodes to, and what the rest of its group of 64 does, is
+ *   not specified (key planes of the per-channel key codecs: also its token's values in the channels next to it); every other group is
+ *   coded as without it.  Raw chunks keep every bit.
  * Key re-rotation in kdn_compose: the stored keys of a part carry rotary
  *   position embedding for positions base_pos + t; placing the part at
  *   dst_pos rotates each pair (k[i], k[i + D/2]) of every head by

@@ -343,6 +343,14 @@ __device__ __forceinline__ uint32_t maxabs_bf16x2(uint32_t a, uint32_t b)
     return d;
 }
 
+// The same, a NaN where either is one.
+__device__ __forceinline__ uint32_t maxabs_nan_bf16x2(uint32_t a, uint32_t b)
+{
+    uint32_t d;
+    asm("max.NaN.xorsign.abs.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+
 // Rounding trick used by quantise_tile: round_half_even(x * inv) sits in the low mantissa bits of the fp32 sum of the
 // (already rounded) product with 1.5 * 2^23 + bias.  For |x * inv| < 2^22 the adder itself rounds the sum to an
 // integer, ties to even (the bias is even, so ties fall the same way), and the mantissa holds code + bias.  The

@@ -94,6 +94,15 @@ __host__ __device__ inline size_t td_decode_smem_bytes(unsigned cols, unsigned w
 // Big-endian view of a little-endian word: the stream's first byte in the top bits.
 __device__ __forceinline__ uint32_t td_be(uint32_t w) { return __byte_perm(w, 0u, 0x0123); }
 
+// The code of one bf16 value, given its channel's reciprocal: round_half_even(x * inv), formed as two separately rounded fp32 operations.
+// What is not finite (a NaN; an infinity, whose channel's reciprocal is zero) has the code -1: the planner and the encoder, which work
+// on several values at once, put it in where they meet one, so that it spoils no more than its own channel.
+__device__ __forceinline__ int td_code(uint32_t x_bf16, float inv)
+{
+    const float p = __fmul_rn(__uint_as_float(x_bf16 << 16), inv);
+    return p == p ? (int)(signed char)(__float_as_uint(__fadd_rn(p, 12582912.0f)) & 0xffu) : -1;
+}
+
 // Exclusive prefix sum of one value per thread over the block (blockDim.x a multiple of 32, at most 1024);
 // *total receives the sum.  `scratch` is 33 words of shared memory.  (64 bits: the segments that a step adds up may take more than 4 GiB.)
 __device__ __forceinline__ unsigned long long td_block_scan(unsigned long long v, unsigned long long *scratch, unsigned long long *total)
@@ -311,9 +320,10 @@ __device__ __forceinline__ unsigned td_plan_mode(const TdLaunch &P, unsigned bes
 
 // Two channels of 32 tokens (x: bf16 pairs) -> bits * 16 + parameters of the one channel this thread answers for (lane 16 + l
 // has tokens 32-63 of the channels lane l has 0-31 of; lane l answers for the first of the two).  n: tokens of the group.
-// kFull: n = 64, known when the code is made.
+// kFull: n = 64, known when the code is made.  odd (one value for the warp): some of the tokens are not finite, those of the masks odd_a and odd_b.
 template <bool kInt4, bool kFull>
-__device__ __forceinline__ unsigned td_plan_channel(const TdLaunch &P, const uint32_t (&x)[32], float inv_a, float inv_b, unsigned n, bool act)
+__device__ __forceinline__ unsigned td_plan_channel(const TdLaunch &P, const uint32_t (&x)[32], float inv_a, float inv_b, unsigned n, bool act,
+                                                    bool odd, uint32_t odd_a, uint32_t odd_b)
 {
     constexpr int kW = kInt4 ? 4 : 8;                       // words per channel before, planes after transposing
     const f32x2 inv2 = pack2(inv_a, inv_b), one2 = pack2(P.fone, P.fone);
@@ -345,6 +355,13 @@ __device__ __forceinline__ unsigned td_plan_channel(const TdLaunch &P, const uin
     }
     td_transpose<kW>(P, wa);
     td_transpose<kW>(P, wb);
+    if (__builtin_expect(odd, 0)) {
+#pragma unroll
+        for (int i = 0; i < kW; ++i) {                       // bias - 1: ones below the top plane
+            wa[i] = i < kW - 1 ? wa[i] | odd_a : wa[i] & ~odd_a;
+            wb[i] = i < kW - 1 ? wb[i] | odd_b : wb[i] & ~odd_b;
+        }
+    }
     // each of the two lanes that share a pair of channels takes one of them over whole
     const bool upper = (threadIdx.x & 16u) != 0u;
     uint32_t lo[kW], hi[kW];
@@ -437,11 +454,25 @@ __global__ void __launch_bounds__(kThreads, kThreads == 128u ? 6 : 1) kdn_td_pla
 #pragma unroll
         for (int t = 0; t < 32; ++t) x[t] = (unsigned)t < n_mine ? __ldcg(reinterpret_cast<const uint32_t *>(my_rows[t]) + pair) : 0u;
     }
-    uint32_t m0 = maxabs_bf16x2(x[0], x[1]), m1 = maxabs_bf16x2(x[2], x[3]);
+    uint32_t m0 = maxabs_nan_bf16x2(x[0], x[1]), m1 = maxabs_nan_bf16x2(x[2], x[3]);
 #pragma unroll
-    for (int t = 4; t < 32; t += 2) { m0 = maxabs_bf16x2(m0, x[t]); m1 = maxabs_bf16x2(m1, x[t + 1]); }
-    m0 = maxabs_bf16x2(m0, m1);
-    m0 = maxabs_bf16x2(m0, __shfl_xor_sync(0xffffffffu, m0, 16));
+    for (int t = 4; t < 32; t += 2) { m0 = maxabs_nan_bf16x2(m0, x[t]); m1 = maxabs_nan_bf16x2(m1, x[t + 1]); }
+    m0 = maxabs_nan_bf16x2(m0, m1);
+    m0 = maxabs_nan_bf16x2(m0, __shfl_xor_sync(0xffffffffu, m0, 16));
+    // Values that are not finite would spoil the codes of the tokens that share a word with theirs: noted, and zeroed.  A channel's
+    // largest magnitude is that of its numbers, infinities included.
+    const bool odd = __any_sync(0xffffffffu, (m0 & 0x7f80u) == 0x7f80u || (m0 & 0x7f800000u) == 0x7f800000u);
+    uint32_t odd_a = 0u, odd_b = 0u;
+    if (__builtin_expect(odd, 0)) {
+        m0 = 0u;
+#pragma unroll
+        for (int t = 0; t < 32; ++t) {
+            m0 = maxabs_bf16x2(m0, x[t]);
+            if ((x[t] & 0x7f80u) == 0x7f80u) { odd_a |= 1u << t; x[t] &= 0xffff0000u; }
+            if ((x[t] & 0x7f800000u) == 0x7f800000u) { odd_b |= 1u << t; x[t] &= 0x0000ffffu; }
+        }
+        m0 = maxabs_bf16x2(m0, __shfl_xor_sync(0xffffffffu, m0, 16));
+    }
     // scale and reciprocal of the thread's own channel, the other channel's reciprocal from its partner
     const float qmax = (float)td_qmax(codec);
     const float a = __uint_as_float(half ? m0 & 0x7fff0000u : (m0 & 0x7fffu) << 16);
@@ -451,8 +482,8 @@ __global__ void __launch_bounds__(kThreads, kThreads == 128u ? 6 : 1) kdn_td_pla
     const float other = __shfl_xor_sync(0xffffffffu, inv, 16);
     const float inv_a = half ? other : inv, inv_b = half ? inv : other;
     unsigned best;
-    if (codec == 5) best = full ? td_plan_channel<false, true>(P, x, inv_a, inv_b, 64u, act) : td_plan_channel<false, false>(P, x, inv_a, inv_b, s.n_tok, act);
-    else best = full ? td_plan_channel<true, true>(P, x, inv_a, inv_b, 64u, act) : td_plan_channel<true, false>(P, x, inv_a, inv_b, s.n_tok, act);
+    if (codec == 5) best = full ? td_plan_channel<false, true>(P, x, inv_a, inv_b, 64u, act, odd, odd_a, odd_b) : td_plan_channel<false, false>(P, x, inv_a, inv_b, s.n_tok, act, odd, odd_a, odd_b);
+    else best = full ? td_plan_channel<true, true>(P, x, inv_a, inv_b, 64u, act, odd, odd_a, odd_b) : td_plan_channel<true, false>(P, x, inv_a, inv_b, s.n_tok, act, odd, odd_a, odd_b);
     const unsigned len = act ? (best + 7u * 16u) >> 7 : 0u;                   // bytes of the sub-stream
     if (act) {
         reinterpret_cast<float *>(s.op.data + lay.scales)[row + ch] = ok ? sc : 0.0f;
@@ -562,10 +593,12 @@ __device__ __forceinline__ void td_append_any(TdOut &o, uint32_t ub, unsigned ra
     td_append(o, z, (unsigned)nlen);
 }
 // Four symbols of two sub-streams, kJoin of them joined before they are appended (4-bit codes: four, 8-bit codes: two).  Where
-// one is an escape, or the joined ones are longer than a word, one at a time.
+// one is an escape, or the joined ones are longer than a word, one at a time.  A NaN looks like a very long escape: again(i, a, b) then
+// forms symbol i of both sub-streams with care, and leaves behind what the next one needs.
 template <unsigned kN> struct TdJoin { static constexpr unsigned value = kN; };
-template <unsigned kJoin>
-__device__ __forceinline__ void td_append4(const TdLaunch &P, TdOut &x, TdOut &y, const uint32_t (&ux)[4], const uint32_t (&uy)[4], unsigned raw_bits)
+template <unsigned kJoin, typename Again>
+__device__ __forceinline__ void td_append4(const TdLaunch &P, TdOut &x, TdOut &y, const uint32_t (&ux)[4], const uint32_t (&uy)[4], unsigned raw_bits,
+                                           Again again)
 {
     int lx[4], ly[4];                                        // minus the lengths
     uint32_t zx[4], zy[4];
@@ -594,6 +627,14 @@ __device__ __forceinline__ void td_append4(const TdLaunch &P, TdOut &x, TdOut &y
         uint32_t a[4], b[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) { a[i] = ux[i]; b[i] = uy[i]; }
+        if (__builtin_expect(min(mx, my) < -4096, 0)) {      // (of a number: -516 or more)
+#pragma unroll 1
+            for (int i = 0; i < 4; ++i) {
+                a[0] = a[1]; a[1] = a[2]; a[2] = a[3];
+                b[0] = b[1]; b[1] = b[2]; b[2] = b[3];
+                again((unsigned)i, a[3], b[3]);
+            }
+        }
 #pragma unroll 1
         for (int i = 0; i < 4; ++i) {                        // (rolled up: instruction fetch is felt in this kernel)
             td_append_any(x, a[0], raw_bits);
@@ -693,6 +734,16 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 16 : 1) kdn
             a = __float_as_uint(__fadd_rn(fabsf(fa), 8388607.5f));
             b = __float_as_uint(__fadd_rn(fabsf(fb), 8388607.5f));
         };
+        // the same of token t, whatever it is (one that is not finite also spoils `base`)
+        auto again = [&](unsigned t, uint32_t &a, uint32_t &b) {
+            const uint32_t v = __ldcg(reinterpret_cast<const uint32_t *>(rows[t + (t >> 5)]) + tid);
+            const uint32_t u = t ? __ldcg(reinterpret_cast<const uint32_t *>(rows[t - 1u + ((t - 1u) >> 5)]) + tid) : 0u;
+            const int qx = td_code(v & 0xffffu, inv_x), qy = td_code(v >> 16, inv_y);
+            const int ex = dx ? qx - td_code(u & 0xffffu, inv_x) : qx, ey = dy ? qy - td_code(u >> 16, inv_y) : qy;
+            a = kTdUZero + (unsigned)((ex << 1) ^ (ex >> 31));
+            b = kTdUZero + (unsigned)((ey << 1) ^ (ey >> 31));
+            base = fma2(pack2(m + (float)qx, m + (float)qy), nd2, nc2);
+        };
         // kTdLoad tokens at a time, the next ones already on their way
         auto load = [&](unsigned t0, uint32_t (&v)[kTdLoad]) {
             const unsigned long long *r = rows + t0 + (t0 >> 5);
@@ -713,7 +764,7 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 16 : 1) kdn
                     uint32_t ux[4], uy[4];
 #pragma unroll
                     for (int j = 0; j < 4; ++j) symbol(v[i + j], ux[j], uy[j]);
-                    td_append4<decltype(join)::value>(P, x, y, ux, uy, raw_bits);
+                    td_append4<decltype(join)::value>(P, x, y, ux, uy, raw_bits, [&](unsigned j, uint32_t &a, uint32_t &b) { again(t0 + (unsigned)i + j, a, b); });
                 }
             }
             return t0;
@@ -723,6 +774,7 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 16 : 1) kdn
         for (; t0 < s.n_tok; ++t0) {
             uint32_t ux, uy;
             symbol(__ldcg(reinterpret_cast<const uint32_t *>(rows[t0 + (t0 >> 5)]) + tid), ux, uy);
+            if (max(ux, uy) > 0x7f800000u) again(t0, ux, uy);
             td_append_any(x, ux, raw_bits);
             td_append_any(y, uy, raw_bits);
         }

@@ -551,3 +551,88 @@ def test_segment_offsets_beyond_32_bits():
         assert np.array_equal(dev.pool_np()[0, 0], ref[0, 0])
     finally:
         dev.close()
+
+
+def encode_bits(bits, T, codec):
+    """Chunk of bf16 bit patterns [L][2][T][R]: as the oracle codes finite values; a NaN or an infinity has the code -1 and only an
+    infinity takes part in the group's largest magnitude (its scale is then infinite and every finite value's code 0)."""
+    L, R = bits.shape[0], bits.shape[3]
+    qmax = 127 if codec == TD8 else 7
+    lay = oracle.td_layout(L, R // 64, 64, T, codec)
+    chunk = np.zeros(lay["capacity"], dtype=np.uint8)
+    off, at, seg = [lay["streams"]], lay["streams"], 0
+    scales = chunk[lay["scales"]:lay["lens"]].view(np.float32)
+    for l in range(L):
+        for kv in range(2):
+            for t0 in range(0, T, 64):
+                with np.errstate(all="ignore"):
+                    x = (bits[l, kv, t0:t0 + 64].astype(np.uint32) << 16).view(np.float32)
+                    a = np.where(np.isnan(x), np.float32(0), np.abs(x)).max(axis=0)
+                    sc = a / np.float32(qmax)
+                    ok = sc >= np.finfo(np.float32).tiny
+                    p = x * np.where(ok, np.float32(qmax) / a, np.float32(0))
+                    q = np.where(np.isfinite(p), np.rint(p), -1).astype(np.int8)
+                scales[seg * R:(seg + 1) * R] = np.where(ok, sc, np.float32(0))
+                for c in range(R):
+                    data, param = oracle.td_encode_channel(q[:, c], qmax)
+                    chunk[lay["lens"] + seg * R + c], chunk[lay["params"] + seg * R + c] = data.size, param
+                    chunk[at:at + data.size] = data
+                    at += data.size
+                at = -(-at // 16) * 16
+                off.append(at)
+                seg += 1
+    chunk[:8 * len(off)] = np.array(off, dtype=np.uint64).view(np.uint8)
+    return chunk
+
+
+@pytest.mark.parametrize("codec", [TD8, TD4], ids=["int8td", "int4td"])
+@pytest.mark.parametrize("rho", [0.0, 0.99])
+def test_a_value_that_is_not_finite_stays_in_its_channel(codec, rho):
+    """NaNs and infinities at the ends of groups, in the remainder of a short group, in either and in both channels of a pair: the
+    planner and the encoder agree on their code, so every other channel's sub-stream is untouched."""
+    shape = synth.TOY.with_(n_layers=1, n_kv_heads=2, head_dim=128, block_size=16, n_blocks=64)
+    T, R = 170, 256                                                       # groups of 64, 64 and 42 tokens; two slices
+    perm = np.random.default_rng(3).permutation(64).astype(np.int32)
+    src, dst = perm[:11], perm[11:22]
+    x = synth.correlated_tokens(shape, T, rho, seed=21).view(torch.int16).numpy().view(np.uint16).reshape(1, 2, T, R).copy()
+    k, v = synth.make_pool(shape, "cpu", seed=22)
+
+    def pool_of(bits):
+        synth.place_tokens(k, v, src, 0, torch.from_numpy(bits.reshape(1, 2, T, 2, 128).view(np.int16)).view(torch.bfloat16))
+        return synth.pool_to_numpy(k, v)
+
+    clean = pool_of(x)
+    want = oracle.store(clean, src, 0, T, codec)
+    used = oracle.td_used_bytes(want, 1, 2, 128, T, codec)
+    assert np.array_equal(encode_bits(x, T, codec)[:used], want[:used])
+    bad = [(0, 0, 0x7fc0), (1, 63, 0xffc1), (6, 64, 0x7f81), (7, 64, 0xffff), (9, 5, 0x7f80), (12, 5, 0xff80), (13, 70, 0x7fc0),
+           (37, 131, 0x7f80), (100, 168, 0x7fc0), (103, 169, 0xff80), (126, 127, 0x7fff), (127, 31, 0x7fc0), (128, 32, 0x7fc0),
+           (255, 100, 0x7fc0), (255, 101, 0x7f80), (254, 169, 0xffc0)]
+    for c, t, b in bad:
+        x[0, c & 1 ^ 1, t, c] = b
+        x[0, 1, t, c] = b
+    x[0, 0, :64, 50] = 0x7fc0                                             # nothing else in a group
+    x[0, 0, 1::3, 200] = 0x7fc0
+    x[0, 1, 2::5, 201] = 0xff80
+    with np.errstate(all="ignore"):
+        healthy = np.isfinite((x.astype(np.uint32) << 16).view(np.float32)).all(axis=2)        # [1][2][R]
+    host = pool_of(x)
+    dev = Device(shape, pool_np=host)
+    try:
+        want = encode_bits(x, T, codec)
+        used = oracle.td_used_bytes(want, 1, 2, 128, T, codec)
+        buf = dev.chunk_buf(T, codec)
+        dev.store([dev.op(dev.table(src), 0, buf, T, codec)])
+        assert dev.sync() == 0
+        got = to_np(buf)
+        assert used_bytes(dev.K, dev.desc, buf, T, codec)[0] == used
+        assert np.array_equal(got[:used], want[:used])
+        assert np.all(got[used:] == 0xA5)
+        dev.retrieve([dev.op(dev.table(dst), 0, buf, T, codec)])
+        assert dev.sync() == 0
+        ref = host.copy()
+        oracle.retrieve(ref, dst, 0, T, codec, want)
+        g, r = dev.pool_np()[:, :, dst].reshape(1, 2, -1, R)[:, :, :T], ref[:, :, dst].reshape(1, 2, -1, R)[:, :, :T]
+        assert np.array_equal(np.moveaxis(g, 2, 3)[healthy], np.moveaxis(r, 2, 3)[healthy])
+    finally:
+        dev.close()
