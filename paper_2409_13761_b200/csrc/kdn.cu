@@ -890,7 +890,7 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     const int gw = ctx->tuning.group_warps > 0 ? ctx->tuning.group_warps : def.gw;
     // Every launch of the pipeline is a programmatic dependent launch.  After the rotation-table kernel only the warps
     // that read the table wait for it; otherwise every thread waits for the kernel before it, whatever that was.
-    lp.wait_all = (OP == OP_COMPOSE && n_rope > 0 && !own_table) ? 0 : kc_groups > 0 ? 2 : 1;
+    lp.wait_all = (OP == OP_COMPOSE && n_rope > 0 && !own_table) ? 0 : kc_groups > 0 && inl ? 2 : 1;
     kdn_status st = launch_tiles(ctx->env, OP, groups, gw, grid, smem, stream, lp, true);
     if (st != KDN_OK) return st;
     ctx->launches++;

@@ -116,7 +116,8 @@ struct Launch {
                               // 0: only the warps that read the rotation table wait (the kernel before is the table kernel).
                               // 2: they wait before they leave (the kernel before stores the key planes of the same chunks and lets
                               // this one start only when it has itself waited: the two may overlap, and what comes behind this
-                              // one waits for both)
+                              // one waits for both).  Until then nothing is read but the launch's parameters (the ops' records are
+                              // among them), the layers' addresses, tables and lists (by ld_ahead) and the pool (by bulk copies)
     float one;                // 1.0f, as a launch parameter: the coding loops form "product + constant" as
                               // fma(product, one, constant), and with a multiplier the assembler cannot see there
                               // is nothing it could contract with the multiply before it (the codecs round twice)
@@ -260,6 +261,16 @@ __device__ __forceinline__ void group_bar_sync(int group, unsigned gthreads)
 // kernel start early.
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void release_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A load ahead of dependency_wait(), of a table or list that a kernel before the one in front may have written.  The kernel in front let this one
+// start only after its own wait: by then those writes have been performed for the whole device.  They are documented to be visible to the grid
+// that waited, which may not have had a CTA on this SM, so this load must not be served from what the SM has cached: it is a strong
+// one at the device's scope.  (Bulk copies read through the L2 anyway.)
+__device__ __forceinline__ int32_t ld_ahead(const int32_t *p)
+{
+    int32_t v;
+    asm("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
 
 __device__ __forceinline__ uint4 lds128(const void *p) { return *reinterpret_cast<const uint4 *>(p); }
 __device__ __forceinline__ uint2 lds64(const void *p) { return *reinterpret_cast<const uint2 *>(p); }
@@ -710,6 +721,7 @@ __device__ __forceinline__ void decode_tile(const Launch &P, unsigned g, TileDes
         if (ops[mid].tile_begin <= g) lo = mid; else hi = mid - 1;
     }
     const DevOp op = ops[lo];
+    auto entry = [](const int32_t *p) { return OP == OP_STORE ? ld_ahead(p) : __ldg(p); };      // (a store may not have waited yet: wait_all = 2)
     const unsigned gl = g - op.tile_begin;
     unsigned plane, n;
     long long id_index;                                     // block-table entry of the tile
@@ -730,11 +742,11 @@ __device__ __forceinline__ void decode_tile(const Launch &P, unsigned g, TileDes
         for (int r = 0; r < kMaxRowsPerTile; ++r) {
             rows[r] = 0u;
             if ((unsigned)r < nr) {
-                const long long rel = __ldg(op.list + i0 + (unsigned)r);
+                const long long rel = entry(op.list + i0 + (unsigned)r);
                 const long long p = op.off + rel;
                 if (rel < 0 || p >= op.pos_end || (long long)(i0 + (unsigned)r) >= op.T) { bad = true; continue; }
                 const long long bi = p / P.bs;
-                const long long id = __ldg(op.table + bi);
+                const long long id = entry(op.table + bi);
                 if (id < 0 || id >= P.n_blocks) { bad = true; continue; }
                 rows[r] = (unsigned)(id * P.bs + (p - bi * P.bs));
             }
@@ -767,7 +779,7 @@ __device__ __forceinline__ void decode_tile(const Launch &P, unsigned g, TileDes
         // one listed token (one row of H * D elements) per tile
         plane = gl / (unsigned)op.n_list;
         const unsigned i = gl - plane * (unsigned)op.n_list;
-        const long long rel = __ldg(op.list + i);
+        const long long rel = entry(op.list + i);
         const long long c = op.list_mode == 2 ? rel : (long long)i;      // chunk token
         const long long p = op.off + rel;
         if (rel < 0 || p >= op.pos_end || c >= op.T) { atomicCAS(P.status, 0, kStatusRange); return; }
@@ -801,7 +813,7 @@ __device__ __forceinline__ void decode_tile(const Launch &P, unsigned g, TileDes
     if (many_rows) {
         d.g_pool = (unsigned long long)base;
     } else {
-        const long long id = __ldg(op.table + id_index);
+        const long long id = entry(op.table + id_index);
         if (id < 0 || id >= P.n_blocks) { atomicCAS(P.status, 0, kStatusRange); d.flags = 0; return; }
         d.g_pool = (unsigned long long)(base + ((unsigned long long)id * P.bs * P.row_elems + pool_elem) * 2ull);
     }
@@ -1166,12 +1178,13 @@ kdn_compose_kernel(const __grid_constant__ Launch P) { tile_pipeline<OP_COMPOSE,
 // ------------------------------------------------ keys of the per-channel key codecs --
 
 // Request position of row t of group g of an op: off + 64 g + t, or, for a keep-list op, off + list[64 g + t].
-// Returns -1 for a list entry that is negative or points past the block table.
+// Returns -1 for a list entry that is negative or points past the block table.  kAhead: see ld_ahead.
+template <bool kAhead = false>
 __device__ __forceinline__ long long group_row_pos(const DevOp &op, unsigned g, unsigned t)
 {
     const unsigned i = (g << 6) + t;
     if (op.list_mode != 1) return op.off + (long long)i;      // (a select-list chooses among the chunk's tokens, it does not move them)
-    const long long rel = op.list[i];
+    const long long rel = kAhead ? ld_ahead(op.list + i) : op.list[i];
     const long long p = op.off + rel;
     return (rel < 0 || p >= op.pos_end) ? -1ll : p;
 }

@@ -210,6 +210,8 @@ __device__ __forceinline__ TdOffsets td_offsets(const unsigned char *lens, unsig
 
 // Pool addresses of the slice in the token rows of the group, row t at rows[t + t / 32] (0 for rows past the chunk's end).  Threads
 // t = first, first + step, ... of those who fill one table call this; true when one of the thread's rows lies outside the pool or the table.
+// kAhead: before the wait for the kernel in front (see ld_ahead).
+template <bool kAhead>
 __device__ __forceinline__ bool td_row_addresses(const TdLaunch &P, const TdSlice &s, unsigned long long *rows, unsigned first, unsigned step)
 {
     const unsigned char *base = reinterpret_cast<const unsigned char *>((s.kv ? P.v_layers : P.k_layers)[s.op.l0 + (int)s.li]);
@@ -217,10 +219,10 @@ __device__ __forceinline__ bool td_row_addresses(const TdLaunch &P, const TdSlic
     for (unsigned t = first; t < 64u; t += step) {
         unsigned long long a = 0ull;
         if (t < s.n_tok) {
-            const long long pos = group_row_pos(s.op, s.g, t);
+            const long long pos = group_row_pos<kAhead>(s.op, s.g, t);
             long long id = -1;
             const long long blk = P.bs_shift >= 0 ? pos >> P.bs_shift : pos / P.bs;
-            if (pos >= 0) id = s.op.table[blk];
+            if (pos >= 0) id = kAhead ? ld_ahead(s.op.table + blk) : s.op.table[blk];
             if (id < 0 || id >= P.n_blocks) bad = true;
             else a = (unsigned long long)(base + ((unsigned long long)(id * P.bs + (pos - blk * P.bs)) * P.row_elems + s.c0) * 2ull);
         }
@@ -425,7 +427,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == 128u ? 6 : 1) kdn_td_pla
     const TdLayout &lay = P.layout[blockIdx.z];
     const unsigned long long row = (unsigned long long)s.seg * RE + s.c0;
     unsigned long long *rows = all_rows[warp];
-    const bool bad = td_row_addresses(P, s, rows, lane, 32u);
+    const bool bad = td_row_addresses<false>(P, s, rows, lane, 32u);
     __syncwarp();
     const unsigned half = lane >> 4, pair = warp * 16u + (lane & 15u), ch = 2u * pair + half;      // ch: the channel the thread answers for
     const bool act = 2u * pair < C;                         // (C is a multiple of 16)
@@ -689,8 +691,8 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 16 : 1) kdn
     const TdLayout &lay = P.layout[blockIdx.z];
     const unsigned long long row = (unsigned long long)s.seg * RE;
     const bool act = 2u * tid < C;
-    // (this kernel may start as soon as the scan's CTAs have seen the planner end: the row addresses are what it can have ready)
-    const bool bad = td_row_addresses(P, s, rows, tid, nthreads);
+    // this kernel may start as soon as the scan's CTAs have seen the planner end: the row addresses are what it can have ready
+    const bool bad = td_row_addresses<true>(P, s, rows, tid, nthreads);
     dependency_wait();
     release_dependents();
     const TdOffsets o = td_offsets(s.op.data + lay.lens + row, s.c0, C, nthreads, scratch);

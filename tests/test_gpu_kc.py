@@ -292,3 +292,40 @@ def test_a_wait_that_runs_out_in_the_key_plane_store(codec):
         assert np.array_equal(to_np(buf), oracle.store(host, tab, 0, T, codec))
     finally:
         dev.close()
+
+
+@pytest.mark.parametrize("codec", KC + [oracle.INT8_TD64], ids=["int8kc", "int4kc", "int8td"])
+@pytest.mark.parametrize("n", [1, 40])
+@pytest.mark.parametrize("listed", [False, True], ids=["dense", "keep"])
+def test_tables_and_lists_rewritten_just_before_a_store(codec, n, listed):
+    """The kernels of these stores overlap, and some look up tables and lists before they wait for the kernel in front: what a kernel of
+    the caller's has written to them last is what counts.  Stores back to back, the one table and the one list rewritten before each."""
+    shape = synth.TOY.with_(n_layers=2, n_kv_heads=4, head_dim=64, block_size=16, n_blocks=96)
+    dev = Device(shape, seed=12)
+    try:
+        K = dev.K
+        rng = np.random.default_rng(8)
+        host, rounds, T, span = dev.pool_np(), 8, 70, 160
+        tabs = [rng.permutation(96)[:10].astype(np.int32) for _ in range(rounds)]
+        lists = [np.sort(rng.permutation(span)[:T]).astype(np.int32) for _ in range(rounds)]
+        d_tabs, d_lists = [dev.table(t) for t in tabs], [dev.table(x) for x in lists]
+        table, keep = dev.table(tabs[0]), dev.table(lists[0])
+        bufs = [[dev.chunk_buf(T, codec) for _ in range(n)] for _ in range(rounds)]
+        torch.cuda.synchronize()
+        with torch.cuda.stream(dev.stream):
+            for r in range(rounds):
+                torch.add(d_tabs[r], 0, out=table)
+                torch.add(d_lists[r], 0, out=keep)
+                ops = [dev.op(table, 0, b, T, codec) for b in bufs[r]]
+                if listed:
+                    K.kdn_store_sparse(dev.ctx, dev.pool_id, ops, [keep.data_ptr()] * n, dev.stream.cuda_stream)
+                else:
+                    K.kdn_store(dev.ctx, dev.pool_id, ops, dev.stream.cuda_stream)
+        assert dev.sync() == 0
+        for r in range(rounds):
+            want = oracle.store(host, tabs[r], 0, T, codec, keep=lists[r] if listed else None)
+            used = want.size if codec != oracle.INT8_TD64 else oracle.td_used_bytes(want, shape.n_layers, 4, 64, T, codec)
+            for b in bufs[r]:
+                assert np.array_equal(to_np(b)[:used], want[:used])
+    finally:
+        dev.close()
