@@ -721,7 +721,10 @@ __device__ __forceinline__ void decode_tile(const Launch &P, unsigned g, TileDes
         if (ops[mid].tile_begin <= g) lo = mid; else hi = mid - 1;
     }
     const DevOp op = ops[lo];
-    auto entry = [](const int32_t *p) { return OP == OP_STORE ? ld_ahead(p) : __ldg(p); };      // (a store may not have waited yet: wait_all = 2)
+    // A store may not have waited yet (wait_all = 2).  Keep-lists and their tables are read anew for every plane, from the SM's cache where they may
+    // (half of 16 x 512 tokens, rows of 1024 elements, int8: store 149 us, 152 with strong loads); a dense op looks up once a tile.
+    const bool ahead = OP == OP_STORE && (op.list_mode == 0 || P.wait_all == 2);
+    auto entry = [ahead](const int32_t *p) { return ahead ? ld_ahead(p) : __ldg(p); };
     const unsigned gl = g - op.tile_begin;
     unsigned plane, n;
     long long id_index;                                     // block-table entry of the tile
