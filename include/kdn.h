@@ -223,7 +223,9 @@ typedef struct {
  * CTAs per SM; compute_groups: groups of four compute warps per CTA in launches that code, decode or
  * rotate; group_warps: warps per group, 4 (groups 1, 2, 3, 4 or 6) or 1 (groups 2, 4 or 8); store_lag: how many shared-to-global copies may still be draining before
  * the storer waits (1..16).  stages is raised to store_lag + 2 and rounded down to a multiple of
- * compute_groups.  Settings that do not fit in shared memory are rejected with KDN_E_UNSUPPORTED. */
+ * compute_groups.  Settings that do not fit in shared memory are rejected with KDN_E_UNSUPPORTED.  Launches whose tiles would take more
+ * than four token rows (keep-lists over short rows), and dense coded ops on pool blocks of 2 KiB or less with no tile_bytes set, have
+ * kernels of their own, to which none of this applies, unless compute_groups or group_warps is set. */
 typedef struct {
     int32_t tile_bytes;
     int32_t stages;

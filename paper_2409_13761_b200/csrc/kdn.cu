@@ -516,8 +516,16 @@ bool rows_apply(const kdn_ctx *ctx, const Pool &pool, int OP, bool any_coded, bo
 {
     const unsigned row_elems = (unsigned)pool.H * (unsigned)pool.D;
     const kdn_tuning &t = ctx->tuning;
-    // a caller-set launch shape is one of the tile pipeline
-    if (t.tile_bytes > 0 || t.stages > 0 || t.ctas_per_sm > 0 || t.compute_groups > 0 || t.store_lag > 0 || t.group_warps > 0) return false;
+    const unsigned long long block_bytes = (unsigned long long)pool.bs * row_elems * 2ull;
+    // A caller-set launch shape is one of the tile pipeline and asks for it, save where its tiles would take more than four rows, which the
+    // pipeline does not do, or end with blocks of 2 KiB or less, and nothing is said of groups or, there, of tiles.  Slots, CTAs an SM and copies
+    // in flight, set for other launches, are no reason to give these up (two heads, half of 16 x 1024 tokens kept, int8 retrieve, eight
+    // slots set: 145 us in the pipeline, 76 here; 32 x 1024 tokens of one head in blocks of four: 474 / 141).
+    if (t.compute_groups > 0 || t.group_warps > 0) return false;
+    if (t.tile_bytes > 0 || t.stages > 0 || t.ctas_per_sm > 0 || t.store_lag > 0) {
+        const unsigned tile_rows = (t.tile_bytes > 0 ? (unsigned)t.tile_bytes / 2u : 2048u) / row_elems;
+        if (any_list ? tile_rows <= (unsigned)kMaxRowsPerTile : t.tile_bytes > 0 || block_bytes > 2048ull) return false;
+    }
     if ((OP != OP_STORE && OP != OP_RETRIEVE) || any_rot || row_elems % 16u) return false;
     if (any_list) {
         for (int i = 0; i < n; ++i)
@@ -525,7 +533,6 @@ bool rows_apply(const kdn_ctx *ctx, const Pool &pool, int OP, bool any_coded, bo
         return row_elems < 512u || (row_elems <= 1024u && !(OP == OP_RETRIEVE && (any_kc || (!any_coded && row_elems > 512u))));
     }
     if (!any_coded || any_kc) return false;
-    const unsigned long long block_bytes = (unsigned long long)pool.bs * row_elems * 2ull;
     if (block_bytes <= 2048ull) return true;
     if (row_elems > 1024u || (block_bytes > 4096ull && !(all_int4 && OP == OP_RETRIEVE))) return false;
     const unsigned long long ctas = rows_shape(pool, OP, hops, n).ctas, wave = 4ull * (unsigned)ctx->env.sm_count;

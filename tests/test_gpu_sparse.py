@@ -302,3 +302,46 @@ def test_rows_moved_one_by_one_at_the_edges_of_a_cta(codec, heads, head_dim):
             assert np.array_equal(dev.pool_np(), ref), i
     finally:
         dev.close()
+
+
+@pytest.mark.parametrize("tuning", [dict(stages=8), dict(ctas_per_sm=4), dict(store_lag=2), dict(tile_bytes=8192), dict(compute_groups=2, group_warps=1)],
+                         ids=lambda t: next(iter(t)))
+@pytest.mark.parametrize("codec", [RAW, INT8], ids=["raw", "int8"])
+def test_a_launch_shape_set_for_other_calls_leaves_short_rows_where_they_are_fast(codec, tuning):
+    """Slots, CTAs and copies in flight, or a tile of many rows, do not take keep-lists over short rows and dense coded ops on tiny blocks out of the
+    kernels that move rows one by one; groups do, and so does a tile size for dense ops.  The results are the same."""
+    groups = "compute_groups" in tuning
+    rng = np.random.default_rng(13)
+    for heads, bs in ((2, 16), (1, 4)):
+        shape = synth.TOY.with_(n_layers=2, n_kv_heads=heads, head_dim=128, block_size=bs, n_blocks=1600 // bs)
+        dev = Device(shape, seed=14)
+        try:
+            K = dev.K
+            K.kdn_set_tuning(dev.ctx, **tuning)
+            host, T, nb = dev.pool_np(), 150, -(-300 // bs)
+            tab, dst = rng.permutation(shape.n_blocks)[:2 * nb].astype(np.int32).reshape(2, nb)
+            keep = np.sort(rng.permutation(300)[:T]).astype(np.int32)
+            ref = host.copy()
+            for kept in (keep, None):
+                buf = dev.chunk_buf(T, codec)
+                ops, back = [dev.op(dev.table(tab), 0, buf, T, codec)], [dev.op(dev.table(dst), 0, buf, T, codec)]
+                rows = not groups and (kept is not None or (codec == INT8 and bs == 4 and "tile_bytes" not in tuning))
+                lists = [dev_list(dev, keep).data_ptr()]
+                if kept is not None:
+                    K.kdn_store_sparse(dev.ctx, dev.pool_id, ops, lists, dev.stream.cuda_stream)
+                else:
+                    dev.store(ops)
+                assert dev.sync() == 0
+                assert ("rows" in K.kdn_last_launch(dev.ctx)["kernel"]) == rows
+                want = oracle.store(host, tab, 0, T, codec, keep=kept)
+                assert np.array_equal(to_np(buf), want)
+                if kept is not None:
+                    K.kdn_retrieve_sparse(dev.ctx, dev.pool_id, back, lists, dev.stream.cuda_stream)
+                else:
+                    dev.retrieve(back)
+                assert dev.sync() == 0
+                assert ("rows" in K.kdn_last_launch(dev.ctx)["kernel"]) == rows
+                oracle.retrieve(ref, dst, 0, T, codec, want, keep=kept)
+                assert np.array_equal(dev.pool_np(), ref)
+        finally:
+            dev.close()
