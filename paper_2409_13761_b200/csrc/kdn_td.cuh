@@ -675,8 +675,9 @@ __device__ __forceinline__ void td_out_finish(TdOut &o, uint32_t addr, uint32_t 
 // (77 % of the slots).  8B shape, 16 chunks of 512 tokens: 1020 us for 8-bit codes with a tile, a pass over it for the magnitudes and
 // every symbol appended by itself, 520 us this way; 4-bit codes 1000 -> 470 us.  Sixteen CTAs of 64 threads an SM (64 registers) with
 // eight tokens loaded ahead; twelve CTAs, four or sixteen tokens are 1-7 % slower.
+// (Other slices: at most 256 threads, 96 registers; at 104 a slice of 192 channels loses a CTA an SM and 10 %.)
 template <unsigned kCols>
-__global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 16 : 1) kdn_td_encode_kernel(const __grid_constant__ TdLaunch P)
+__global__ void __launch_bounds__(kCols ? kCols / 2u : 320u, kCols ? 16 : 2) kdn_td_encode_kernel(const __grid_constant__ TdLaunch P)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const TdSlice s = td_slice(P);
