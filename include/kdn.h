@@ -404,7 +404,8 @@ uint64_t kdn_launch_count(const kdn_ctx *ctx);
 /* Shape of the context's most recent launch of the tile pipeline, for reports: op 0 store / 1 retrieve / 2 compose
  * (the kernel is kdn_store_kernel / kdn_retrieve_kernel / kdn_compose_kernel<compute_groups, group_warps>, or, with
  * rows_kernel = 1, kdn_store_rows_kernel / kdn_retrieve_rows_kernel, which move token rows one by one: compute_groups is then
- * the slots a thread fills and group_warps the elements of its vectors); rows_per_tile: token rows per tile of a
+ * the slots a thread fills and group_warps the elements of its vectors, or, with rows_kernel = 2, kdn_compose_own_kernel, whose CTAs each
+ * make the rotation table for themselves); rows_per_tile: token rows per tile of a
  * keep-list launch (1 otherwise); grid is what was asked for (a launch of the pipeline never exceeds the CTAs resident at once). */
 typedef struct {
     int32_t  op, compute_groups, group_warps, tile_bytes, stages, ctas_per_sm, store_lag, grid, smem_bytes;

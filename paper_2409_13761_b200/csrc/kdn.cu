@@ -395,6 +395,13 @@ kdn_status launch_tiles(LaunchEnv &env, int OP, int groups, int gw, unsigned gri
         if (OP == OP_RETRIEVE) return launch_kernel(env, kdn_retrieve_kernel<G, W>, threads_for(G, W), grid, smem, stream, lp, overlap); \
         return launch_kernel(env, kdn_compose_kernel<G, W>, threads_for(G, W), grid, smem, stream, lp, overlap);               \
     }
+    if (lp.off_rope) {
+#define KDN_OWN_CASE(G, W) if (groups == G && gw == W) return launch_kernel(env, kdn_compose_own_kernel<G, W>, threads_for(G, W), grid, smem, stream, lp, overlap);
+        KDN_OWN_CASE(1, 4) KDN_OWN_CASE(2, 4) KDN_OWN_CASE(3, 4) KDN_OWN_CASE(4, 4) KDN_OWN_CASE(6, 4)
+        KDN_OWN_CASE(2, 1) KDN_OWN_CASE(4, 1) KDN_OWN_CASE(8, 1)
+#undef KDN_OWN_CASE
+        return KDN_E_UNSUPPORTED;
+    }
     KDN_CASE(0, 4) KDN_CASE(1, 4) KDN_CASE(2, 4) KDN_CASE(3, 4) KDN_CASE(4, 4) KDN_CASE(6, 4)
     KDN_CASE(2, 1) KDN_CASE(4, 1) KDN_CASE(8, 1)
 #undef KDN_CASE
@@ -789,20 +796,31 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     if (fit != KDN_OK) return fit;
     size_t smem = smem_bytes(stages, stage_bytes, rows_per_tile);
     // A few rotations: every CTA makes its own table in shared memory, if that leaves the launch its CTAs -- no table kernel in front, no ring
-    // slot, and back-to-back calls overlap.  One 128-token chunk re-rotated: 12.8 -> 6.9 us (8B shape; one head: 12.4 -> 4.2); ten rows of a 1 GiB
-    // request cost what the table kernel did (418 -> 417 us).
+    // slot, and back-to-back calls overlap.  One 128-token chunk re-rotated: 10.2 -> 6.6 us (8B shape; one head: 8.2 -> 4.7); ten rows of a 1 GiB
+    // request cost what the table kernel did (418 -> 417 us).  Not where many tiles of less than 4 KiB keep the loader busy, in whose loop the
+    // kernel with the table's code is slower (blocks of one token, 8 heads, int8, us with the table kernel / without: 2 x 256 tokens
+    // 37.1 / 37.4, 4 x 256 67.6 / 71.3, 8 x 1024 475 / 520; blocks of 4 KiB: the same); listed tokens gain at every size (16 x 2048,
+    // half of them: 776 / 711).  A stream that is being captured takes no launch with a ring slot, so there it stays.
     int n_rotations = 0;
     bool one_theta = true;
     double theta = 0.0;
-    for (int i = 0; i < n; ++i)
+    unsigned long long tiles_ahead = 0;
+    for (int i = 0; i < n; ++i) {
+        tiles_ahead += 2ull * (unsigned)hops[i].op.nl * (unsigned)hops[i].op.nblk * tpb;
         if (hops[i].rotate) {
             if (n_rotations++ == 0) theta = hops[i].rp.theta;
             one_theta &= hops[i].rp.theta == theta;
         }
+    }
     const size_t table_bytes = (size_t)(n_rotations + 1) * (size_t)(pool.D / 2) * sizeof(float2);      // (and the frequencies)
     const size_t off_rope = (smem + 15u) & ~(size_t)15u;
-    const bool own_table = OP == OP_COMPOSE && n_rotations > 0 && one_theta && n <= kInlineOps && table_bytes <= kOwnTableBytes &&
-                           (off_rope + table_bytes) * (size_t)ctas_per_sm <= smem_limit - 1024u * (size_t)ctas_per_sm;
+    bool own_table = OP == OP_COMPOSE && n_rotations > 0 && one_theta && n <= kInlineOps && table_bytes <= kOwnTableBytes &&
+                     (off_rope + table_bytes) * (size_t)ctas_per_sm <= smem_limit - 1024u * (size_t)ctas_per_sm;
+    if (own_table && !any_list && tile_elems * 2u < 4096u && tiles_ahead > 64ull * (unsigned)ctx->env.sm_count * (unsigned)ctas_per_sm) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        KDN_CUDA(cudaStreamIsCapturing(stream, &capture));
+        own_table = capture != cudaStreamCaptureStatusNone;
+    }
     if (own_table) smem = off_rope + table_bytes;
 
     // Few ops travel as kernel parameters (a few more as those of a kernel in front); otherwise through a ring slot (pinned staging + device copy).  A ring
@@ -895,8 +913,9 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     unsigned long long want = (unsigned long long)ctx->env.sm_count * (unsigned)ctas_per_sm;
     const unsigned grid = (unsigned)(tiles < want ? tiles : want);
     const int gw = ctx->tuning.group_warps > 0 ? ctx->tuning.group_warps : def.gw;
-    // Every launch of the pipeline is a programmatic dependent launch.  After the rotation-table kernel only the warps
-    // that read the table wait for it; otherwise every thread waits for the kernel before it, whatever that was.
+    // Every launch of the pipeline is a programmatic dependent launch.  After the rotation-table kernel only the warps that read the table wait for
+    // it; behind the key planes of the same chunks every thread does before it leaves, if the ops' records came as parameters; otherwise
+    // every thread waits for the kernel before it, whatever that was.
     lp.wait_all = (OP == OP_COMPOSE && n_rope > 0 && !own_table) ? 0 : kc_groups > 0 && inl ? 2 : 1;
     kdn_status st = launch_tiles(ctx->env, OP, groups, gw, grid, smem, stream, lp, true);
     if (st != KDN_OK) return st;
@@ -912,7 +931,7 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     ctx->last.smem_bytes = (int32_t)smem;
     ctx->last.n_tiles = (uint32_t)tiles;
     ctx->last.rows_per_tile = rows_per_tile;
-    ctx->last.rows_kernel = 0;
+    ctx->last.rows_kernel = own_table ? 2 : 0;
     if (slot) {
         KDN_CUDA(cudaEventRecord(slot->done, stream));
         slot->used = true;

@@ -121,7 +121,7 @@ struct Launch {
     float one;                // 1.0f, as a launch parameter: the coding loops form "product + constant" as
                               // fma(product, one, constant), and with a multiplier the assembler cannot see there
                               // is nothing it could contract with the multiply before it (the codecs round twice)
-    unsigned off_rope;        // compose: not 0: the CTA makes its own rotation table, at this offset of shared memory, from inline_rope
+    unsigned off_rope;        // kdn_compose_own_kernel: where in shared memory the CTA makes its rotation table, from inline_rope; others: 0
     int n_rope;               // rows of it
     RopeParam inline_rope[kInlineOps];
     DevOp inline_ops[kInlineOps];
@@ -593,7 +593,7 @@ __device__ __forceinline__ float2 rope_entry(long long delta, double inv_freq)
     return make_float2((float)c, (float)s);
 }
 // A CTA's own table, by the `n` threads that will read it: the frequencies first (one theta for all rows), then the rows.
-// (Not inlined: its registers are not the pipeline's.)
+// (Not inlined: its registers would be the pipeline's.)
 __device__ __noinline__ void rope_fill(const Launch &P, double *freq, float2 *table, int t, int n)
 {
     const int half = P.D >> 1;
@@ -614,13 +614,14 @@ struct RotCoef {
     unsigned col;  // first frequency index
 };
 
+template <bool kOwn>      // whether the table lies in the CTA's shared memory
 __device__ __forceinline__ void load_coef(RotCoef &rc, const float2 *table, int rope, unsigned col, unsigned half)
 {
     if (rc.rope == rope && rc.col == col) return;
     const float4 *p = reinterpret_cast<const float4 *>(table + (size_t)rope * half + col);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const float4 v = p[k];                             // (cos, sin) of frequencies 2k and 2k + 1
+        const float4 v = kOwn ? p[k] : __ldg(p + k);       // (cos, sin) of frequencies 2k and 2k + 1
         rc.c[k] = pack2(v.x, v.z);
         rc.s[k] = pack2(v.y, v.w);
         rc.ns[k] = pack2(-v.y, -v.w);
@@ -646,7 +647,7 @@ __device__ __forceinline__ void rotate8(const f32x2 *u, const f32x2 *w, const Ro
 // frequencies of one head row: elements [col, col+8) and [D/2 + col, D/2 + col + 8).
 // kCodec = 0: bf16 at A, in place.  kCodec = 1 / 2: int8 / int4 codes at B and scales at S -> bf16 at A.
 // kChan: the codes carry one scale per channel (S[channel], row_elems of them) instead of one per 64 elements.
-template <int kCodec, bool kChan = false>
+template <int kCodec, bool kOwn, bool kChan = false>
 __device__ __forceinline__ void rotate_tile(unsigned char *A, const unsigned char *B, const float *S, unsigned n,
                                             unsigned D, const float2 *table, int rope, RotCoef &rc, int ct, unsigned gthreads,
                                             unsigned row_elems = 0)
@@ -660,7 +661,7 @@ __device__ __forceinline__ void rotate_tile(unsigned char *A, const unsigned cha
     for (unsigned it = (unsigned)ct; it < items; it += gthreads) {
         const unsigned r = pow2 ? it >> shift : it / per_row;
         const unsigned col = (it - r * per_row) << 3;
-        load_coef(rc, table, rope, col, half);
+        load_coef<kOwn>(rc, table, rope, col, half);
         const unsigned e_lo = r * D + col, e_hi = e_lo + half;
         f32x2 u[4], w[4];
         if (kCodec != 0) {
@@ -892,7 +893,8 @@ __host__ __device__ inline size_t smem_bytes(int stages, unsigned stage_bytes, i
            (rows_per_tile > 1 ? 16u * (size_t)stages + 16u * 64u : 0u);
 }
 
-template <int OP, int kGroups, int kGW>
+// kOwn (compose): the CTA makes its own rotation table, at P.off_rope.
+template <int OP, int kGroups, int kGW, bool kOwn = false>
 __device__ __forceinline__ void tile_pipeline(const Launch &P)
 {
     constexpr bool kCompute = kGroups > 0;
@@ -919,8 +921,8 @@ __device__ __forceinline__ void tile_pipeline(const Launch &P)
         fence_async_smem();
     }
     __syncthreads();
-    if (P.wait_all == 1 && !(OP == OP_COMPOSE && warp != kLoaderWarp && warp != 1 + kGroups * kGW))
-        dependency_wait();                                  // (the compute warps of compose wait below) returns at once when the launch was an ordinary one
+    if (P.wait_all == 1 && !(kOwn && warp != kLoaderWarp && warp != 1 + kGroups * kGW))
+        dependency_wait();                                  // (compute warps with a table to make wait below) returns at once when the launch was an ordinary one
 
     const unsigned grid = gridDim.x, bid = blockIdx.x;
     const unsigned n_my = P.n_tiles > bid ? (P.n_tiles - bid + grid - 1u) / grid : 0u;
@@ -1079,17 +1081,14 @@ __device__ __forceinline__ void tile_pipeline(const Launch &P)
         RotCoef rc;
         rc.rope = -1; rc.col = 0xffffffffu;
         const float2 *rope_table = P.rope;
-        if (OP == OP_COMPOSE) {
-            // a table of the CTA's own needs nothing from the kernel before; one in memory is written by the kernel launched
-            // just before this one, and only these warps read it
-            if (P.off_rope) {
-                double *freq = reinterpret_cast<double *>(smem_raw + P.off_rope);
-                float2 *own = reinterpret_cast<float2 *>(freq + (P.D >> 1));
-                rope_fill(P, freq, own, tid - 32, kGroups * (int)kGT);
-                rope_table = own;
-            }
-            dependency_wait();
+        if constexpr (kOwn) {                                 // needs nothing from the kernel before
+            double *freq = reinterpret_cast<double *>(smem_raw + P.off_rope);
+            float2 *own = reinterpret_cast<float2 *>(freq + (P.D >> 1));
+            rope_fill(P, freq, own, tid - 32, kGroups * (int)kGT);
+            rope_table = own;
         }
+        // (one in memory is written by the kernel launched just before this one, and only these warps read it)
+        if (OP == OP_COMPOSE) dependency_wait();
         unsigned st = (unsigned)group;                        // S is a multiple of kGroups: st wraps exactly at S
         uint32_t ph = 0;
         for (unsigned slot = (unsigned)group; slot < n_my; slot += (unsigned)kGroups) {
@@ -1124,16 +1123,16 @@ __device__ __forceinline__ void tile_pipeline(const Launch &P)
                     }
                     if (flags & TF_KCHAN) {
                         if (OP == OP_COMPOSE && (flags & TF_ROTATE)) {
-                            if (flags & TF_INT4) rotate_tile<2, true>(A, B, Sc, n, (unsigned)P.D, rope_table, sm.desc[st].rope, rc, ct, kGT, P.row_elems);
-                            else rotate_tile<1, true>(A, B, Sc, n, (unsigned)P.D, rope_table, sm.desc[st].rope, rc, ct, kGT, P.row_elems);
+                            if (flags & TF_INT4) rotate_tile<2, kOwn, true>(A, B, Sc, n, (unsigned)P.D, rope_table, sm.desc[st].rope, rc, ct, kGT, P.row_elems);
+                            else rotate_tile<1, kOwn, true>(A, B, Sc, n, (unsigned)P.D, rope_table, sm.desc[st].rope, rc, ct, kGT, P.row_elems);
                         } else if (flags & TF_INT4) {
                             dequantise_kc_tile<true, OP != OP_COMPOSE>(B, Sc, A, n, P.row_elems, ct, kGT);
                         } else {
                             dequantise_kc_tile<false, OP != OP_COMPOSE>(B, Sc, A, n, P.row_elems, ct, kGT);
                         }
                     } else if (OP == OP_COMPOSE && (flags & TF_ROTATE)) {
-                        if (flags & TF_INT4) rotate_tile<2>(A, B, Sc, n, (unsigned)P.D, rope_table, sm.desc[st].rope, rc, ct, kGT);
-                        else rotate_tile<1>(A, B, Sc, n, (unsigned)P.D, rope_table, sm.desc[st].rope, rc, ct, kGT);
+                        if (flags & TF_INT4) rotate_tile<2, kOwn>(A, B, Sc, n, (unsigned)P.D, rope_table, sm.desc[st].rope, rc, ct, kGT);
+                        else rotate_tile<1, kOwn>(A, B, Sc, n, (unsigned)P.D, rope_table, sm.desc[st].rope, rc, ct, kGT);
                     } else if (flags & TF_INT4) {
                         if (n == kGT * 32u) dequantise4_tile(B, Sc, A, kGT * 32u, ct, kGT);
                         else dequantise4_tile(B, Sc, A, n, ct, kGT);
@@ -1143,7 +1142,7 @@ __device__ __forceinline__ void tile_pipeline(const Launch &P)
                     }
                     computed = true;
                 } else if (OP == OP_COMPOSE && (flags & TF_ROTATE)) {
-                    rotate_tile<0>(A, nullptr, nullptr, n, (unsigned)P.D, rope_table, sm.desc[st].rope, rc, ct, kGT);
+                    rotate_tile<0, kOwn>(A, nullptr, nullptr, n, (unsigned)P.D, rope_table, sm.desc[st].rope, rc, ct, kGT);
                     computed = true;
                 }
             }
@@ -1177,6 +1176,13 @@ kdn_retrieve_kernel(const __grid_constant__ Launch P) { tile_pipeline<OP_RETRIEV
 template <int kGroups, int kGW>
 __global__ void __launch_bounds__(threads_for(kGroups, kGW), min_ctas_for_compose(kGroups, kGW))
 kdn_compose_kernel(const __grid_constant__ Launch P) { tile_pipeline<OP_COMPOSE, kGroups, kGW>(P); }
+
+// The same where every CTA makes its own rotation table.  Apart, since a call in a kernel costs registers, which the loader's loop feels where
+// there are few of them and many small tiles: single-warp groups, 8 x 1024 tokens of 8 heads in blocks of one, int8, 475 us, 526 with
+// the call in the kernel.
+template <int kGroups, int kGW>
+__global__ void __launch_bounds__(threads_for(kGroups, kGW), min_ctas_for_compose(kGroups, kGW))
+kdn_compose_own_kernel(const __grid_constant__ Launch P) { tile_pipeline<OP_COMPOSE, kGroups, kGW, true>(P); }
 
 // ------------------------------------------------ keys of the per-channel key codecs --
 

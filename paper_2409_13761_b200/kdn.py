@@ -473,7 +473,7 @@ def kdn_last_launch(ctx) -> dict:
     info = kdn_launch_info()
     _check(lib.kdn_last_launch(ctx, C.byref(info)), "kdn_last_launch")
     d = {name: int(getattr(info, name)) for name, _ in kdn_launch_info._fields_}
-    d["kernel"] = "kdn_%s%s_kernel<%d, %d>" % (("store", "retrieve", "compose")[d["op"]], "_rows" if d["rows_kernel"] else "",
+    d["kernel"] = "kdn_%s%s_kernel<%d, %d>" % (("store", "retrieve", "compose")[d["op"]], ("", "_rows", "_own")[d["rows_kernel"]],
                                                d["compute_groups"], d["group_warps"])
     return d
 

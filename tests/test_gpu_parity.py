@@ -776,3 +776,34 @@ def test_small_coded_launches_take_four_ctas_an_sm_unless_some_would_idle(T, fou
         assert np.array_equal(dev.pool_np(), ref)
     finally:
         dev.close()
+
+
+@pytest.mark.parametrize("T", [910, 980])
+def test_many_tiny_tiles_take_their_rotation_table_from_memory(T):
+    """Blocks of one token of 256 bytes: up to 64 tiles a CTA make their own table, more are given one by the table kernel."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    shape = synth.TOY.with_(n_layers=40, n_kv_heads=1, head_dim=128, block_size=1, n_blocks=2 * T)
+    dev = Device(shape, seed=62)
+    try:
+        K = dev.K
+        host = dev.pool_np()
+        perm = np.random.default_rng(5).permutation(2 * T).astype(np.int32)
+        buf = dev.chunk_buf(T, INT8)
+        dev.store([dev.op(dev.table(perm[:T]), 0, buf, T, INT8)])
+        assert dev.sync() == 0
+        want = oracle.store(host, perm[:T], 0, T, INT8)
+        dev.compose([K.ComposeReq(dev.table(perm[T:]).data_ptr(), T, [dev.chunk(buf, T, INT8, 9)], [0], 5e5)])
+        assert dev.sync() == 0
+        info = K.kdn_last_launch(dev.ctx)
+        assert info["n_tiles"] == 80 * T
+        assert ("own" in info["kernel"]) == (info["n_tiles"] <= 64 * sms * info["ctas_per_sm"])
+        if sms == 148 and info["ctas_per_sm"] == 8:
+            assert ("own" in info["kernel"]) == (T == 910)
+        ref = host.copy()
+        kref, kmag = oracle.compose(ref, perm[T:], [(want, T, INT8, 9, 0)], 5e5, want_ref=True)
+        got = dev.pool_np()
+        p = np.arange(T)
+        assert np.array_equal(got[:, 1], ref[:, 1])
+        check_rotated_keys(gather_positions(got, perm[T:], p)[:, 0], kref, kmag, gather_positions(ref, perm[T:], p)[:, 0])
+    finally:
+        dev.close()
