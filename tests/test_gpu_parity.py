@@ -778,6 +778,43 @@ def test_small_coded_launches_take_four_ctas_an_sm_unless_some_would_idle(T, fou
         dev.close()
 
 
+@pytest.mark.parametrize("codec", [RAW, INT8], ids=["raw", "int8"])
+def test_requests_of_two_rope_thetas_in_one_call(codec):
+    """One theta: every CTA makes its own rotation table; two in one call: the table kernel does.  Same chunks, both ways, against the oracle."""
+    shape = synth.TOY.with_(n_layers=2, n_kv_heads=2, head_dim=64, block_size=16, n_blocks=128)
+    dev = Device(shape, seed=61)
+    try:
+        K = dev.K
+        host = dev.pool_np()
+        perm = np.random.default_rng(4).permutation(128).astype(np.int32)
+        T = 100
+        bufs = [dev.chunk_buf(T, codec) for _ in range(2)]
+        dev.store([dev.op(dev.table(perm[7 * i:7 * i + 7]), 0, bufs[i], T, codec) for i in range(2)])
+        assert dev.sync() == 0
+        wants = [oracle.store(host, perm[7 * i:7 * i + 7], 0, T, codec) for i in range(2)]
+        for thetas in ((1e4, 5e5), (1e4, 1e4), (5e5, 5e5)):
+            ref = dev.pool_np()
+            tabs = [perm[20 + 20 * r:40 + 20 * r] for r in range(2)]
+            before = K.kdn_launch_count(dev.ctx)
+            dev.compose([K.ComposeReq(dev.table(tabs[r]).data_ptr(), 20, [dev.chunk(b, T, codec, 3 + r) for b in bufs], [50, 150], thetas[r]) for r in range(2)])
+            assert dev.sync() == 0
+            own = thetas[0] == thetas[1]
+            assert ("own" in K.kdn_last_launch(dev.ctx)["kernel"]) == own and K.kdn_launch_count(dev.ctx) - before == (1 if own else 2)
+            got = dev.pool_np()
+            rot = np.zeros(got.shape, dtype=bool)
+            checks = []
+            for r in range(2):
+                kref, kmag = oracle.compose(ref, tabs[r], [(wants[j], T, codec, 3 + r, (50, 150)[j]) for j in range(2)], thetas[r], want_ref=True)
+                p = 50 + np.arange(2 * T)
+                rot[:, 0, tabs[r][p // 16], p % 16] = True
+                checks.append((p, tabs[r], kref, kmag))
+            assert np.array_equal(got[~rot], ref[~rot])
+            for p, tab, kref, kmag in checks:
+                check_rotated_keys(gather_positions(got, tab, p)[:, 0], kref[:, p], kmag[:, p], gather_positions(ref, tab, p)[:, 0])
+    finally:
+        dev.close()
+
+
 @pytest.mark.parametrize("T", [910, 980])
 def test_many_tiny_tiles_take_their_rotation_table_from_memory(T):
     """Blocks of one token of 256 bytes: up to 64 tiles a CTA make their own table, more are given one by the table kernel."""
