@@ -566,12 +566,13 @@ kdn_status launch_rows(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hop
     lp.rows = shape.rows;
     lp.vpr_magic = lp.rows > 1u && lp.vpr > 1u ? 0xffffffffu / lp.vpr + 1u : 0u;
     // Planes a CTA goes through: enough to pay for the look-ups and the pipeline's start, few enough to leave 2.5 waves of CTAs (a store,
-    // whose CTAs do more work each: 1.7), or one wave instead of two uneven ones.  Two heads, half of 16 x 1024 tokens kept, int8, 1 / 2 / 4 / 8 / 16
+    // whose CTAs do more work each: 1.7), but two where one would make more than a wave (one plane / two, us: half of 1000 tokens of four heads, raw
+    // retrieve, 3.5 waves 13.2 / 10.6; of 1500 of two, int8 store, 2.6 waves 11.5 / 9.9; of 2200, raw, 3.8 waves 14.4 / 11.2).  Two heads, half of 16 x 1024 tokens kept, int8, 1 / 2 / 4 / 8 / 16
     // planes: retrieve 88 / 75 / 76 / 78 / 85 us, store 125 / 91 / 81 / 78 / 78; of 4 x 500 tokens retrieve 13.6 / 11.9 / 13.1 / 16.8.
     const unsigned long long wave = 4ull * (unsigned)ctx->env.sm_count, want = OP == OP_STORE ? wave * 17ull / 10ull : wave * 5ull / 2ull;
     lp.planes = 16u;
     while (lp.planes > 1u && shape.ctas / lp.planes < want) --lp.planes;
-    if (lp.planes == 1u && shape.ctas > wave && shape.ctas <= 2ull * wave) lp.planes = 2u;
+    if (lp.planes == 1u && shape.ctas > wave) lp.planes = 2u;
     int kc_layers = 0, kc_groups = 0;
     unsigned long long tiles = 0;
     for (int i = 0; i < n; ++i) {
@@ -912,12 +913,26 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
 
     unsigned long long want = (unsigned long long)ctx->env.sm_count * (unsigned)ctas_per_sm;
     const unsigned grid = (unsigned)(tiles < want ? tiles : want);
+    // CTAs that are placed while the kernel in front still holds some SMs gather on the others, where more of them fit than the shape means, and stay
+    // there.  Small tiles are bound by what a CTA does, so the crowded SMs finish last.
+    bool early = true;
+    if (kc_groups > 0 && tile_elems * 2u < 4096u) {
+        // room for no more than the shape's CTAs keeps them even (blocks of one token, per-channel keys, us without / with: 16 x 512 tokens of 8 heads
+        // 451 / 371, and 375 when the launch waits for the key planes; 512 tokens 32.3 / 29.2; tiles of 4 KiB and more: the same)
+        const size_t least = ((smem_limit + 1024u) / ((size_t)ctas_per_sm + 1u) - 1024u + 255u) & ~(size_t)127u;
+        if (smem < least && least <= smem_limit) smem = least;
+    } else if (put && !compute && tile_elems * 2u <= 256u && tiles > 64ull * grid) {
+        // behind the kernel that writes the records, the copy form loses by the smaller L1 that goes with it, and waits instead (79 raw stores of 1652
+        // tokens of one head of 64, blocks of one: 2469 us early, 2390 with less room, 2286 after; 40 of 100 tokens of one of 128 107.9 / 102.2
+        // / 103.4, 64 of 512 762 / 796 / 765)
+        early = false;
+    }
     const int gw = ctx->tuning.group_warps > 0 ? ctx->tuning.group_warps : def.gw;
-    // Every launch of the pipeline is a programmatic dependent launch.  After the rotation-table kernel only the warps that read the table wait for
+    // Otherwise every launch of the pipeline is a programmatic dependent launch.  After the rotation-table kernel only the warps that read the table wait for
     // it; behind the key planes of the same chunks every thread does before it leaves, if the ops' records came as parameters; otherwise
     // every thread waits for the kernel before it, whatever that was.
     lp.wait_all = (OP == OP_COMPOSE && n_rope > 0 && !own_table) ? 0 : kc_groups > 0 && inl ? 2 : 1;
-    kdn_status st = launch_tiles(ctx->env, OP, groups, gw, grid, smem, stream, lp, true);
+    kdn_status st = launch_tiles(ctx->env, OP, groups, gw, grid, smem, stream, lp, early);
     if (st != KDN_OK) return st;
     ctx->launches++;
     ctx->last.op = OP;

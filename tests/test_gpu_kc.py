@@ -329,3 +329,26 @@ def test_tables_and_lists_rewritten_just_before_a_store(codec, n, listed):
                 assert np.array_equal(to_np(b)[:used], want[:used])
     finally:
         dev.close()
+
+
+@pytest.mark.parametrize("n", [1, 40])
+@pytest.mark.parametrize("codec", KC, ids=["int8kc", "int4kc"])
+def test_value_planes_of_tiny_blocks_fill_the_sms_evenly(codec, n):
+    """Behind the key planes' kernel, tiles of less than 4 KiB take so much shared memory that an SM has room for the shape's CTAs and no more."""
+    shape = synth.TOY.with_(n_layers=3, n_kv_heads=5, head_dim=64, block_size=1, n_blocks=700)
+    dev = Device(shape, seed=17)
+    try:
+        K = dev.K
+        host, T = dev.pool_np(), 130
+        tabs = [np.random.default_rng(i).permutation(700)[:T].astype(np.int32) for i in range(n)]
+        bufs = [dev.chunk_buf(T, codec) for _ in range(n)]
+        dev.store([dev.op(dev.table(t), 0, b, T, codec) for t, b in zip(tabs, bufs)])
+        assert dev.sync() == 0
+        info = K.kdn_last_launch(dev.ctx)
+        per_sm = torch.cuda.get_device_properties(0).shared_memory_per_multiprocessor
+        assert info["tile_bytes"] == 640
+        assert info["ctas_per_sm"] * (info["smem_bytes"] + 1024) <= per_sm < (info["ctas_per_sm"] + 1) * (info["smem_bytes"] + 1024)
+        for t, b in zip(tabs, bufs):
+            assert np.array_equal(to_np(b), oracle.store(host, t, 0, T, codec))
+    finally:
+        dev.close()
