@@ -345,3 +345,33 @@ def test_a_launch_shape_set_for_other_calls_leaves_short_rows_where_they_are_fas
                 assert np.array_equal(dev.pool_np(), ref)
         finally:
             dev.close()
+
+
+@pytest.mark.parametrize("n_keep,planes", [(288, 1), (289, 2), (600, 2), (1470, 2), (2209, 3)])
+def test_planes_that_a_cta_of_the_row_kernels_goes_through(n_keep, planes):
+    """One plane a CTA where that makes no more than a wave of CTAs (four an SM), two up to seven and a half waves.  Rows of 512 elements, 16 to a CTA, raw retrieve;
+    32 planes."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("sizes of a card with 148 SMs")
+    shape = synth.TOY.with_(n_layers=16, n_kv_heads=4, head_dim=128, block_size=16, n_blocks=320)
+    dev = Device(shape, seed=18)
+    try:
+        K = dev.K
+        rng = np.random.default_rng(2)
+        perm = rng.permutation(320).astype(np.int32)
+        src, dst = perm[:160], perm[160:]
+        keep = np.sort(rng.permutation(2560)[:n_keep]).astype(np.int32)
+        host = dev.pool_np()
+        buf, lists = dev.chunk_buf(n_keep, RAW), [dev_list(dev, keep).data_ptr()]
+        K.kdn_store_sparse(dev.ctx, dev.pool_id, [dev.op(dev.table(src), 0, buf, n_keep, RAW)], lists, dev.stream.cuda_stream)
+        K.kdn_retrieve_sparse(dev.ctx, dev.pool_id, [dev.op(dev.table(dst), 0, buf, n_keep, RAW)], lists, dev.stream.cuda_stream)
+        assert dev.sync() == 0
+        info = K.kdn_last_launch(dev.ctx)
+        assert info["grid"] == -(-n_keep // 16) * -(-32 // planes) and "rows" in info["kernel"]
+        want = oracle.store(host, src, 0, n_keep, RAW, keep=keep)
+        assert np.array_equal(to_np(buf), want)
+        ref = host.copy()
+        oracle.retrieve(ref, dst, 0, n_keep, RAW, want, keep=keep)
+        assert np.array_equal(dev.pool_np(), ref)
+    finally:
+        dev.close()
