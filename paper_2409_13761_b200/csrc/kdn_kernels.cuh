@@ -722,9 +722,9 @@ __device__ __forceinline__ void decode_tile(const Launch &P, unsigned g, TileDes
         if (ops[mid].tile_begin <= g) lo = mid; else hi = mid - 1;
     }
     const DevOp op = ops[lo];
-    // A store may not have waited yet (wait_all = 2).  Keep-lists and their tables are read anew for every plane, from the SM's cache where they may
-    // (half of 16 x 512 tokens, rows of 1024 elements, int8: store 149 us, 152 with strong loads); a dense op looks up once a tile.
-    const bool ahead = OP == OP_STORE && (op.list_mode == 0 || P.wait_all == 2);
+    // A store may not have waited yet (wait_all = 2).  One that has takes tables and lists from the SM's cache where it can: keep-lists are read
+    // anew for every plane (half of 16 x 512 tokens, rows of 1024 elements, int8: 149 us, 152 with strong loads), tables of tiny blocks for every row.
+    const bool ahead = OP == OP_STORE && P.wait_all == 2;
     auto entry = [ahead](const int32_t *p) { return ahead ? ld_ahead(p) : __ldg(p); };
     const unsigned gl = g - op.tile_begin;
     unsigned plane, n;
