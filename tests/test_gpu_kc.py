@@ -267,8 +267,9 @@ def test_keep_list_chunks_against_the_oracle(shape, codec):
 
 @pytest.mark.parametrize("codec", KC, ids=["int8kc", "int4kc"])
 def test_a_wait_that_runs_out_in_the_key_plane_store(codec):
-    """The key-plane kernel's wait for its tile is bounded too: KDN_E_TIMEOUT, no write outside the chunk, the pool
-    untouched, and the context bit-exact again once the default bound is back."""
+    """The key planes' kernel waits for nothing that can run out: with a bound shorter than a memory access their codes and scales are exact,
+    whatever the value planes' pipeline beside it reports; no write outside the chunk, the pool untouched, and the context bit-exact
+    again once the default bound is back."""
     shape = synth.TOY.with_(n_layers=2, n_kv_heads=4, head_dim=64, block_size=16, n_blocks=96)
     dev = Device(shape, seed=9)
     try:
@@ -282,9 +283,15 @@ def test_a_wait_that_runs_out_in_the_key_plane_store(codec):
         buf = arena[guard:guard + n]
         K.kdn_set_wait_limit_ns(dev.ctx, 40)
         dev.store([dev.op(dev.table(tab), 0, buf, T, codec)])
-        assert dev.sync() in (0, K.KDN_E_TIMEOUT)                         # (0: every CTA found its rows landed in time)
+        assert dev.sync() in (0, K.KDN_E_TIMEOUT)                         # (0: every CTA of the value planes found its rows landed in time)
         assert np.array_equal(dev.pool_np(), host)
         a = to_np(arena)
+        want, R = oracle.store(host, tab, 0, T, codec), 256
+        plane = T * R // (2 if codec == KC[1] else 1)                     # bytes of a plane's codes
+        scales = (-(-T // 64) * R + T * R // 64) * 4                      # bytes of a layer's scales, its keys' first
+        for l in range(2):
+            for at, size in ((2 * l * plane, plane), (4 * plane + l * scales, -(-T // 64) * R * 4)):
+                assert np.array_equal(a[guard + at:guard + at + size], want[at:at + size])
         assert np.all(a[:guard] == 0x5C) and np.all(a[-guard:] == 0x5C)
         K.kdn_set_wait_limit_ns(dev.ctx, 0)
         dev.store([dev.op(dev.table(tab), 0, buf, T, codec)])
