@@ -45,6 +45,7 @@ N_CHUNKS, CHUNK_TOKENS = 64, 512
 N_PARTS, PART_TOKENS, SUFFIX_TOKENS = 10, 1024, 256
 RAW, INT8, INT4, INT8KC, INT4KC, INT8TD, INT4TD = 0, 1, 2, 3, 4, 5, 6
 FALLBACK_HBM_GBS = 6650.0
+TD_DECODE_INSTS = {INT8TD: 23.4, INT4TD: 21.0}     # warp instructions per 32 symbols of the token-delta decoder (profiles/ncu_token_delta_kernels_llama3_8b.md)
 
 
 def bytes_per_elem(codec: int) -> float:
@@ -614,11 +615,12 @@ def extras_8b(leg, dev_sets, reps, which=EXTRAS):
                     "retrieve_ms": ms_retr, "retrieve_gbs": moved / (ms_retr * 1e-3) / 1e9, "retrieve_tokens_per_s": n_td * T / (ms_retr * 1e-3),
                     "compose_ms": ms_comp, "compose_gbs": moved / (ms_comp * 1e-3) / 1e9,
                     "retrieve_frac_of_8000": moved / (ms_retr * 1e-3) / 1e9 / 8000.0,
-                    # the decoder is bound by instruction issue, not by HBM: 148 SMs x 4 schedulers x 1.965 GHz x 32 lanes,
-                    # at 23.5 warp instructions per 32 symbols (profiler count)
-                    "retrieve_roofline": {"bound": "issue", "unit": "symbols/s", "achieved": n_td * T * E / (ms_retr * 1e-3),
-                                          "peak": 148 * 4 * 1.965e9 * 32 / 23.5,
-                                          "frac": n_td * T * E / (ms_retr * 1e-3) / (148 * 4 * 1.965e9 * 32 / 23.5)},
+                    "retrieve_roofline": {"bound": "hbm", "unit": "GB/s", "achieved": moved / (ms_retr * 1e-3) / 1e9, "peak": measured_hbm_peak()[0],
+                                          "frac": moved / (ms_retr * 1e-3) / 1e9 / measured_hbm_peak()[0]},
+                    # what keeps it from there is instruction issue: the present decoder's warp instructions (profiler count) as a share of the
+                    # issue slots of 148 SMs x 4 schedulers x 1.965 GHz
+                    "retrieve_issue": {"warp_instructions_per_32_symbols": TD_DECODE_INSTS[codec],
+                                       "share_of_slots": n_td * T * E / 32 * TD_DECODE_INSTS[codec] / (ms_retr * 1e-3) / (148 * 4 * 1.965e9)},
                     "from_host_ms": host_ms, "from_host_link_gbs": used / (host_ms * 1e-3) / 1e9,
                     "from_host_bf16_gbs_delivered": bf16_bytes / (host_ms * 1e-3) / 1e9}
                 del buf

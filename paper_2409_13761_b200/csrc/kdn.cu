@@ -708,15 +708,15 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
             while (want_rows & (want_rows - 1)) want_rows &= want_rows - 1;
         if (want_rows > kMaxRowsPerTile) want_rows = kMaxRowsPerTile;
         if (!any_coded && !any_rot && all_keep && want_rows >= 2 && row_elems < 1024u && (unsigned long long)pool.nb * (unsigned)pool.bs < 0xffffffffull) {
-            // copy form on rows shorter than 2 KiB (few KV heads per GPU): several rows per tile as well
+            // copy form on rows shorter than 2 KiB (retrieves of more than 512 elements, and caller-set shapes): several rows per tile as well
             rows_per_tile = want_rows;
             tile_elems = (unsigned)rows_per_tile * row_elems;
             def = Shape{ 0, 4, 8, 0, 1 };
         } else if (any_coded && !any_rot && all_keep && want_rows >= 2 && (unsigned long long)pool.nb * (unsigned)pool.bs < 0xffffffffull) {
-            // coded keep-list launches: a tile takes several listed rows -- neighbours in the chunk, so its codes and
-            // scales move with one copy each, and rows that are neighbours in the pool share a copy too.  From a sweep on
-            // the 8B shape with half of the tokens kept: two 1024-element rows per tile, five CTAs per SM with two
-            // single-warp groups each, one store in flight (int8 5.1 -> 5.9 TB/s, int4 4.0 -> 4.9)
+            // coded keep-list launches that rows_apply leaves here (retrieves with a scale per channel over rows of 512 to 1024 elements, and
+            // caller-set shapes): a tile takes several listed rows -- neighbours in the chunk, so its codes and scales move with one
+            // copy each, and rows that are neighbours in the pool share a copy too.  From a sweep on the 8B shape with half of the
+            // tokens kept: five CTAs per SM with two single-warp groups each, one store in flight (a row a tile 5.1, so 5.9 TB/s; int4 4.0, 4.9)
             rows_per_tile = want_rows;
             tile_elems = (unsigned)rows_per_tile * row_elems;
             def = Shape{ 0, 6, 5, 2, 1, 1 };

@@ -10,7 +10,7 @@
 // per stage (bounded waits, as in the tile pipeline); nothing else is synchronised.  On the chunk side a CTA's vectors are
 // contiguous whatever the rows do; on the pool side a row is.  Bound by memory and, when coding, by the latency of a plane: 8B shape with
 // two heads, half of 16 x 1024 tokens kept, int8: retrieve 76 us (5.4 TB/s), store 78 us (5.3 TB/s).  Loads into registers instead of
-// slots: 92 and 87 us.
+// slots: 92 and 87 us.  (The retrieve of vectors of sixteen elements spills 24 bytes at the 64 registers that four CTAs an SM leave.)
 #pragma once
 
 #include "kdn_kernels.cuh"

@@ -920,8 +920,8 @@ __device__ __forceinline__ void td_step(const TdLaunch &P, TdStream &x, TdStream
     }
 }
 
-// Bound by instruction issue and the integer pipes (8B shape, 4-bit codes: issue slots 83 %, multiply-add pipe 67 %, logic 55 %, DRAM 45 %;
-// 18 instructions a symbol); what was done about it is at TdStream and td_step.  A thread decodes two channels side by side --
+// Bound by instruction issue and the integer pipes (8B shape, 4-bit codes: issue slots 83 %, logic 55 %, DRAM 37 %, 21 warp instructions per 32
+// symbols; 8-bit codes 76 %, 48 %, 38 %, 23.4); what was done about it is at TdStream and td_step.  A thread decodes two channels side by side --
 // neighbours, whose bf16 values make one word, or, where keys are re-rotated, the two channels of a rotation pair -- so that one
 // stream's chain of dependent operations hides the other's, and writes finished values into the rows: no pass over codes.  Half
 // of the rows at a time keeps a CTA of 64 threads at 16 KiB of shared memory, twelve (8-bit codes: ten) to an SM; all rows at a time
