@@ -635,3 +635,36 @@ def test_a_value_that_is_not_finite_stays_in_its_channel(codec, rho):
         assert np.array_equal(np.moveaxis(g, 2, 3)[healthy], np.moveaxis(r, 2, 3)[healthy])
     finally:
         dev.close()
+
+
+@pytest.mark.parametrize("T", [64, 93])
+@pytest.mark.parametrize("codec", [TD8, TD4], ids=["int8td", "int4td"])
+def test_the_cheapest_parameters_are_found_whatever_the_tails(codec, T):
+    """The planner leaves a parameter out where a bound says that it cannot win: channels whose bulk is 2^-j of their largest value, with none to
+    many large values, so that every k wins somewhere, ties occur, and symbols sit on both sides of an escape.  Bit-exact."""
+    shape = synth.TOY.with_(n_layers=2, n_kv_heads=4, head_dim=64, block_size=16, n_blocks=24)
+    rng = np.random.default_rng(77 + T)
+    nb = -(-T // 16)
+    tab = rng.permutation(24)[:nb].astype(np.int32)
+    x = rng.standard_normal((2, 2, nb * 16, 4, 64)).astype(np.float32)
+    c = np.arange(256).reshape(4, 64)
+    x *= 2.0 ** -(c % 9)                                                       # the bulk
+    large = rng.random(x.shape) < ((c // 9) % 7) * 0.03                        # the tail, of one or two sizes
+    x = np.where(large, np.sign(x) * np.where(c & 1, 1.0, rng.choice([0.12, 0.5, 1.0], x.shape)), np.clip(x, -1.0, 1.0)).astype(np.float32)
+    x[0, :, 1:] += x[0, :, :-1] * 0.9                                          # (one layer with neighbours alike)
+    pool = np.zeros((2, 2, 24, 16, 4, 64), dtype=np.uint16)
+    t = np.arange(nb * 16)
+    pool[:, :, tab[t // 16], t % 16] = bf16_bits(x)
+    dev = Device(shape, pool_np=pool)
+    try:
+        want = oracle.store(pool, tab, 0, T, codec)
+        used = oracle.td_used_bytes(want, 2, 4, 64, T, codec)
+        lay = dev.K.kdn_td_layout(dev.desc, T, codec)
+        params = want[lay["params_offset"]:lay["streams_offset"]]
+        assert len(np.unique(params & 7)) >= (7 if codec == TD8 else 4) and len(np.unique(params >> 3)) == 2
+        buf = dev.chunk_buf(T, codec)
+        dev.store([dev.op(dev.table(tab), 0, buf, T, codec)])
+        assert dev.sync() == 0
+        assert np.array_equal(to_np(buf)[:used], want[:used])
+    finally:
+        dev.close()
