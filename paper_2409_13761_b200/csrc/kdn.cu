@@ -958,6 +958,20 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
 // parameters.  Store is three launches (plan, scan, encode), retrieve and compose one (plus the rotation table).
 kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops, int n, cudaStream_t stream)
 {
+    // a launch of the decoder has chunks of one codec
+    if (OP != OP_STORE) {
+        bool mixed = false;
+        for (int i = 1; i < n; ++i) mixed |= hops[i].op.codec != hops[0].op.codec;
+        if (mixed) {
+            for (const bool int4 : {false, true}) {
+                std::vector<HostOp> part;
+                for (int i = 0; i < n; ++i) if ((hops[i].op.codec == KDN_CODEC_INT4_TD64) == int4) part.push_back(hops[i]);
+                const kdn_status r = launch_td(ctx, pool, OP, part.data(), (int)part.size(), stream);
+                if (r != KDN_OK) return r;
+            }
+            return KDN_OK;
+        }
+    }
     const unsigned row_elems = (unsigned)pool.H * (unsigned)pool.D;
     // channels per CTA: a multiple of 16 that divides the row, whole heads when keys are re-rotated, kTdCols if possible
     // (small slices: many CTAs share an SM, and each one's loads, decoding and stores overlap the others')
@@ -1045,19 +1059,22 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
             }
             kdn_status r = KDN_OK;
             const unsigned dec_threads = (cols / 2u + 31u) & ~31u;       // a thread decodes two channels
-#define KDN_TD_DECODE(COMPOSE, COLS)                                                                        \
+#define KDN_TD_DECODE(COMPOSE, COLS, INT4)                                                                  \
             {                                                                                               \
-                r = ctx->env.resident(kdn_td_decode_kernel<COMPOSE, COLS>, (int)dec_threads, smem, &per_sm); \
+                r = ctx->env.resident(kdn_td_decode_kernel<COMPOSE, COLS, INT4>, (int)dec_threads, smem, &per_sm); \
                 if (r != KDN_OK) return r;                                                                  \
                 if (per_sm < 1) return KDN_E_UNSUPPORTED;                                                   \
-                r = launch_behind(kdn_td_decode_kernel<COMPOSE, COLS>, grid, dec_threads, smem, stream, tp); \
+                r = launch_behind(kdn_td_decode_kernel<COMPOSE, COLS, INT4>, grid, dec_threads, smem, stream, tp); \
                 if (r != KDN_OK) return r;                                                                  \
             }
+#define KDN_TD_DECODE_OP(COLS, INT4) if (OP == OP_COMPOSE) KDN_TD_DECODE(true, COLS, INT4) else KDN_TD_DECODE(false, COLS, INT4)
+            const bool int4 = hops[first].op.codec == KDN_CODEC_INT4_TD64;
             if (cols == kTdCols) {
-                if (OP == OP_COMPOSE) KDN_TD_DECODE(true, kTdCols) else KDN_TD_DECODE(false, kTdCols)
+                if (int4) KDN_TD_DECODE_OP(kTdCols, true) else KDN_TD_DECODE_OP(kTdCols, false)
             } else {
-                if (OP == OP_COMPOSE) KDN_TD_DECODE(true, 0) else KDN_TD_DECODE(false, 0)
+                if (int4) KDN_TD_DECODE_OP(0, true) else KDN_TD_DECODE_OP(0, false)
             }
+#undef KDN_TD_DECODE_OP
 #undef KDN_TD_DECODE
             KDN_CUDA(cudaGetLastError());
             ctx->launches++;

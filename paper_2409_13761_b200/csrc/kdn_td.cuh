@@ -895,7 +895,6 @@ __device__ __forceinline__ unsigned td_symbol(const TdLaunch &P, TdStream &s, ui
     asm("bfind.shiftamt.u32 %0, %1;" : "=r"(n) : "r"(h));
     nlen = s.nk1 - n;
     int v = (int)n * s.kneg + (int)__funnelshift_r(h, 0u, nlen);
-    s.bp -= nlen;
     asm("{ .reg .pred p; .reg .b32 t; and.b32 t, %0, 1; setp.ne.s32 p, t, 0; @p mad.lo.s32 %0, %0, %1, %2; }" : "+r"(v) : "r"(P.minus_one), "r"(s.c21));
     s.acc = v + (s.acc * s.d + s.c2);
     return n;
@@ -906,6 +905,7 @@ __device__ __forceinline__ void td_symbol_any(const TdLaunch &P, TdStream &s, ui
     if ((h >> 17) != 0u) {                                  // fewer than fifteen ones
         unsigned nlen;
         td_symbol(P, s, h, nlen);
+        s.bp -= nlen;
         return;
     }
     const int u = (int)((~h << 15) >> (32u - raw_bits));
@@ -913,13 +913,13 @@ __device__ __forceinline__ void td_symbol_any(const TdLaunch &P, TdStream &s, ui
     s.acc = (u ^ -(u & 1)) + (s.d ? s.acc : kTdCodeBits);
 }
 
-constexpr unsigned kTdStep = 4;                             // symbols of a stream between two looks for escapes
-// kTdStep symbols of two streams side by side, kWin of them out of one 32-bit window (code words of 4-bit codes are short:
-// four in a window; of 8-bit codes: two).  Taken to be no escapes and to fit their windows; where that was wrong, once more
-// with care.  (8B shape, 32 chunks of 512 tokens, 4-bit codes, an earlier form: a window a symbol 965 us, two 908, four 867.)
-template <unsigned kCols, unsigned kWin>
+// kStep symbols of two streams side by side, kWin of them out of one 32-bit window (code words of 4-bit codes are short:
+// four in a window, eight a step; of 8-bit codes three and six).  Taken to be no escapes and to fit their windows; where that was wrong, once more
+// with care.  (8B shape, 32 chunks of 512 tokens, 4-bit codes, an earlier form: a window a symbol 965 us, two 908, four 867.  Now, correlation 0.9:
+// steps of four in one kernel for both codecs 724, of eight in a kernel of their own 710; 8-bit codes, pairs 892, triples 864.)
+template <unsigned kCols, unsigned kWin, unsigned kStep>
 __device__ __forceinline__ void td_step(const TdLaunch &P, TdStream &x, TdStream &y, unsigned row_b, unsigned max_bits, unsigned raw_bits,
-                                        int (&vx)[kTdStep], int (&vy)[kTdStep])
+                                        int (&vx)[kStep], int (&vy)[kStep])
 {
     x.bp = x.bp < max_bits ? x.bp : max_bits;               // (a damaged stream cannot run off the area)
     y.bp = y.bp < max_bits ? y.bp : max_bits;
@@ -927,24 +927,26 @@ __device__ __forceinline__ void td_step(const TdLaunch &P, TdStream &x, TdStream
     const int acc_x = x.acc, acc_y = y.acc;
     unsigned longest = 0, most = 0;
 #pragma unroll
-    for (unsigned i = 0; i < kTdStep; i += kWin) {
+    for (unsigned i = 0; i < kStep; i += kWin) {
         uint32_t hx = td_window<kCols>(x, row_b), hy = td_window<kCols>(y, row_b);
-        const unsigned from_x = x.bp, from_y = y.bp;
+        unsigned bx = 0u, by = 0u;                          // minus the bits taken out of the window
 #pragma unroll
         for (unsigned j = 0; j < kWin; ++j) {
             unsigned lx, ly;
             const unsigned nx = td_symbol(P, x, hx, lx), ny = td_symbol(P, y, hy, ly);
-            longest = max(longest, max(nx, ny));
+            longest = __vimax3_u32(longest, nx, ny);
+            bx += lx; by += ly;
             hx = __funnelshift_r(0u, hx, lx);               // hx << length
             hy = __funnelshift_r(0u, hy, ly);
             vx[i + j] = x.acc; vy[i + j] = y.acc;
         }
-        most = max(most, max(x.bp - from_x, y.bp - from_y));
+        x.bp -= bx; y.bp -= by;
+        most = __vimax3_u32(most, 0u - bx, 0u - by);
     }
     if (__builtin_expect(longest >= 15u || most > 32u, 0)) {
         x.bp = bp_x; y.bp = bp_y; x.acc = acc_x; y.acc = acc_y;
 #pragma unroll
-        for (unsigned i = 0; i < kTdStep; ++i) {
+        for (unsigned i = 0; i < kStep; ++i) {
             td_symbol_any(P, x, td_window<kCols>(x, row_b), raw_bits);
             td_symbol_any(P, y, td_window<kCols>(y, row_b), raw_bits);
             vx[i] = x.acc; vy[i] = y.acc;
@@ -962,22 +964,23 @@ __device__ __forceinline__ void td_step(const TdLaunch &P, TdStream &x, TdStream
 // codes 1765 -> 900 us.
 // kCols: channels per CTA when known at compile time (the usual slice; every stride in the decoding loop is then an
 // immediate), 0: taken from the launch record.
-template <bool kCompose, unsigned kCols>
+template <bool kCompose, unsigned kCols, bool kInt4>
 __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 12 : 1) kdn_td_decode_kernel(const __grid_constant__ TdLaunch P)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     dependency_wait();
     release_dependents();
+    constexpr int codec = kInt4 ? 6 : 5;
+    constexpr unsigned kWords = kInt4 ? 11u : 19u;                       // td_words(codec)
     const TdSlice s = td_slice(P);
-    if (!s.valid) return;
+    if (!s.valid || s.op.codec != codec) return;
     const unsigned C = kCols ? kCols : P.cols, RE = P.row_elems;
-    const int codec = s.op.codec;
-    const unsigned raw_bits = (unsigned)td_raw_bits(codec);
+    constexpr unsigned raw_bits = kInt4 ? 5u : 9u;
     const unsigned nthreads = kCols ? kCols / 2u : blockDim.x;
 
     uint32_t *I = reinterpret_cast<uint32_t *>(smem_raw);                // interleaved sub-streams [word][C]
-    unsigned char *A = smem_raw + td_decode_words_bytes(C, P.words);     // the slice's stream bytes, then bf16 rows [kTdHalf][C]
-    unsigned *offs = reinterpret_cast<unsigned *>(A + td_decode_rows_bytes(C, P.words));   // where each channel's sub-stream starts
+    unsigned char *A = smem_raw + td_decode_words_bytes(C, kWords);     // the slice's stream bytes, then bf16 rows [kTdHalf][C]
+    unsigned *offs = reinterpret_cast<unsigned *>(A + td_decode_rows_bytes(C, kWords));   // where each channel's sub-stream starts
     unsigned long long *rows = reinterpret_cast<unsigned long long *>(offs + C);     // pool address of each token row's slice, 0: not written
     unsigned *scratch = reinterpret_cast<unsigned *>(rows + 64);         // 64 words
     unsigned long long *bar_mem = reinterpret_cast<unsigned long long *>(reinterpret_cast<unsigned char *>(scratch) + 256u);
@@ -1114,8 +1117,7 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 12 : 1) kdn
         td_stream_init(y, smem_u32(col_b), param_b);
     }
     __syncthreads();                                                      // stream bytes no longer read: the rows may be written
-    const unsigned row_b = P.word_row, max_bits = (P.words - 1u) * 32u;   // a sub-stream's last symbol starts before that bit
-    const bool short_codes = codec == 6;
+    const unsigned row_b = P.word_row, max_bits = (kWords - 1u) * 32u;   // a sub-stream's last symbol starts before that bit
     const f32x2 sc2 = pack2(sc_a, sc_b), zero2 = pack2(-kTdCodeZero, -kTdCodeZero);
     f32x2 cc = 0ull, ss = 0ull;
     if (rotating && act) {
@@ -1143,13 +1145,21 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 12 : 1) kdn
         const unsigned nt = s.n_tok - t0 < kTdHalf ? s.n_tok - t0 : kTdHalf;
         if (act) {
             unsigned t = 0;
+            auto steps = [&](auto win, auto step) {
+                constexpr unsigned kStep = (unsigned)decltype(step)::value;
 #pragma unroll 1
-            for (; t + kTdStep <= nt; t += kTdStep) {
-                int vx[kTdStep], vy[kTdStep];
-                if (short_codes) td_step<kCols, 4>(P, x, y, row_b, max_bits, raw_bits, vx, vy);
-                else td_step<kCols, 2>(P, x, y, row_b, max_bits, raw_bits, vx, vy);
+                for (; t + kStep <= nt; t += kStep) {
+                    int vx[kStep], vy[kStep];
+                    td_step<kCols, (unsigned)decltype(win)::value, kStep>(P, x, y, row_b, max_bits, raw_bits, vx, vy);
 #pragma unroll
-                for (unsigned i = 0; i < kTdStep; ++i) put(t + i, vx[i], vy[i]);
+                    for (unsigned i = 0; i < kStep; ++i) put(t + i, vx[i], vy[i]);
+                }
+            };
+            if (kInt4) {
+                steps(TdConst<4>(), TdConst<8>());
+            } else {
+                steps(TdConst<3>(), TdConst<6>());
+                steps(TdConst<2>(), TdConst<2>());
             }
 #pragma unroll 1
             for (; t < nt; ++t) {

@@ -668,3 +668,10 @@ def test_the_cheapest_parameters_are_found_whatever_the_tails(codec, T):
         assert np.array_equal(to_np(buf)[:used], want[:used])
     finally:
         dev.close()
+
+
+@pytest.mark.parametrize("T", [2, 6, 7, 8, 9, 14, 38, 47, 62])
+@pytest.mark.parametrize("codec", [TD8, TD4], ids=["int8td", "int4td"])
+def test_lengths_around_the_decoder_steps(codec, T):
+    """Steps of six symbols, three to a window, then of two (8-bit codes), or of eight, four to a window (4-bit codes), and what is left one by one."""
+    test_group_tails_and_escapes_at_every_place(SHAPES[0], codec, T)
