@@ -65,7 +65,7 @@ struct TdLaunch {
     DevOp inline_ops[kInlineOps];
 };
 
-// Shared memory of the encoder: the rows' addresses, a little scratch, the stream staging area, a word per channel.
+// Shared memory of the encoder: the rows' addresses, a little scratch, the stream staging area.
 // Behind the encoder's staging area: room for the longest thing a channel could write from the last planned byte on (64
 // appends, a word each, and the last word), so that a sub-stream that came out longer than planned -- the pool changed under the store --
 // garbles the chunk's bytes, which the caller has then forfeited, but never leaves the area.
@@ -79,7 +79,7 @@ constexpr unsigned kTdEncodeHead = 66u * 8u + 32u * 4u + 112u;      // a multipl
 constexpr unsigned kTdHalf = 32;                            // rows between two write-outs
 __host__ __device__ inline unsigned td_words(int codec) { return td_max_len(codec) / 4u + 1u; }   // the longest sub-stream, and the word after
 __host__ __device__ inline size_t td_stage_bytes(unsigned cols, unsigned words) { return (size_t)cols * (words - 1u) * 4u + 32u + kTdStageSlack; }
-__host__ __device__ inline size_t td_encode_smem_bytes(unsigned cols, unsigned words) { return kTdEncodeHead + td_stage_bytes(cols, words) + 4u * cols; }
+__host__ __device__ inline size_t td_encode_smem_bytes(unsigned cols, unsigned words) { return kTdEncodeHead + td_stage_bytes(cols, words); }
 __host__ __device__ inline size_t td_decode_words_bytes(unsigned cols, unsigned words) { return (size_t)words * cols * 4u; }
 __host__ __device__ inline size_t td_decode_rows_bytes(unsigned cols, unsigned words)
 {
@@ -208,10 +208,10 @@ __device__ __forceinline__ TdOffsets td_offsets(const unsigned char *lens, unsig
     return o;
 }
 
-// Pool addresses of the slice in the token rows of the group, row t at rows[t + t / 32] (0 for rows past the chunk's end).  Threads
+// Pool addresses of the slice in the token rows of the group, row t at rows[t + t / 32], or, without kGap, rows[t] (0 for rows past the chunk's end).  Threads
 // t = first, first + step, ... of those who fill one table call this; true when one of the thread's rows lies outside the pool or the table.
 // kAhead: before the wait for the kernel in front (see ld_ahead).
-template <bool kAhead>
+template <bool kAhead, bool kGap>
 __device__ __forceinline__ bool td_row_addresses(const TdLaunch &P, const TdSlice &s, unsigned long long *rows, unsigned first, unsigned step)
 {
     const unsigned char *base = reinterpret_cast<const unsigned char *>((s.kv ? P.v_layers : P.k_layers)[s.op.l0 + (int)s.li]);
@@ -226,7 +226,7 @@ __device__ __forceinline__ bool td_row_addresses(const TdLaunch &P, const TdSlic
             if (id < 0 || id >= P.n_blocks) bad = true;
             else a = (unsigned long long)(base + ((unsigned long long)(id * P.bs + (pos - blk * P.bs)) * P.row_elems + s.c0) * 2ull);
         }
-        rows[t + (t >> 5)] = a;
+        rows[kGap ? t + (t >> 5) : t] = a;
     }
     return bad;
 }
@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(kThreads, kThreads == 128u ? 6 : 1) kdn_td_pla
     const TdLayout &lay = P.layout[blockIdx.z];
     const unsigned long long row = (unsigned long long)s.seg * RE + s.c0;
     unsigned long long *rows = all_rows[warp];
-    const bool bad = td_row_addresses<false>(P, s, rows, lane, 32u);
+    const bool bad = td_row_addresses<false, true>(P, s, rows, lane, 32u);
     __syncwarp();
     const unsigned half = lane >> 4, pair = warp * 16u + (lane & 15u), ch = 2u * pair + half;      // ch: the channel the thread answers for
     const bool act = 2u * pair < C;                         // (C is a multiple of 16)
@@ -579,89 +579,98 @@ __global__ void __launch_bounds__(kTdScanThreads) kdn_td_scan_kernel(const __gri
 
 // One sub-stream on its way out.  As in the decoder the bits are kept complemented, so that unary parts are zeros: a symbol u
 // is the number 2^(k+1) - 1 - (u mod 2^k) in (u >> k) + k + 1 bits.  u itself comes out of the floating-point pipe as
-// |2 e + 1/2| - 1/2 (2 e for e >= 0, else -2 e - 1), in the low bits of 2^23 + u.
+// |2 e + 1/2| - 1/2 (2 e for e >= 0, else -2 e - 1), in the low bits of 2^23 + u; and from there the length, for two channels at once: a
+// multiply-add by -2^-k that rounds up gives kTdLenZero - (u >> k) - (k + 1), minus the length in the low bits of its representation.  (k = 0: the
+// summand would take 25 bits, so u - 1 stands for u, whose low bits are of no interest then.)
 struct TdOut {
     uint32_t acc;          // the bits not yet written, in the low (bits mod 32) bits; garbage above them
-    unsigned bits;         // bits so far, those of the first word that are not the sub-stream's own included
-    uint32_t wp, next;     // shared address the word being filled goes to, and the one after it
-    unsigned k, nlen0;     // Rice parameter; (bits of 2^23 >> k) - (k + 1)
+    unsigned bits;         // bits so far, those of the first word that are not the sub-stream's own included, modulo 64
+    uint32_t wp;           // shared address of the word being filled
+    unsigned k;            // Rice parameter
     uint32_t kmask, kbit;  // 2^k - 1, 2^k
-    int limit;             // -(k + 16): code words this long are escapes
+    float limit;           // kTdLenZero - (k + 16): code words this long are escapes
 };
 constexpr unsigned kTdLoad = 8;                              // tokens loaded ahead
 constexpr uint32_t kTdUZero = 0x4B000000u;                   // bits of 2^23
+constexpr float kTdLenZero = 12582912.0f;                    // 1.5 * 2^23
+constexpr uint32_t kTdLenBits = 0x4B400000u;                 // its bits, a multiple of 64
 
-// addr: where the sub-stream goes in the staging area; aside: a word of the thread's own, for the first word until the end
-__device__ __forceinline__ void td_out_init(TdOut &o, uint32_t addr, uint32_t aside, unsigned param)
+// addr: where the sub-stream goes in the staging area
+__device__ __forceinline__ void td_out_init(TdOut &o, uint32_t addr, unsigned param)
 {
     o.k = param & 7u;
     o.kbit = 1u << o.k;
     o.kmask = o.kbit - 1u;
-    o.nlen0 = (kTdUZero >> o.k) - (o.k + 1u);
-    o.limit = -(int)(o.k + 16u);
+    o.limit = kTdLenZero - (float)(o.k + 16u);
     o.acc = 0u;
     o.bits = (addr & 3u) * 8u;
-    o.wp = aside;
-    o.next = (addr & ~3u) + 4u;
+    o.wp = addr & ~3u;
 }
-// Append the low `len` bits of w (1 <= len <= 32, nothing above them; nlen = -len).  (Shifts take their count modulo 32.)  Words go
-// out with plain predicated stores, since all but the first and the last are the sub-stream's own: the first, which its neighbour's last
-// bits share, is kept aside.  (An OR into the staging area for every word cost a
-// branch round the instruction: store of 16 chunks 923 -> 898 us.)
+// Append the low `len` bits of w (1 <= len <= 32, nothing above them; nlen = -len, give or take a multiple of 64).  (Shifts take their count modulo 32.)
+// Words go out with plain predicated stores: the first one too, with zeros where its neighbour's last bits belong, which are ORed in at the
+// end.  (An OR into the staging area for every word cost a branch round the instruction: store of 16 chunks 923 -> 898 us.)
 __device__ __forceinline__ void td_append(TdOut &o, uint32_t w, unsigned nlen)
 {
     const uint32_t left = __funnelshift_l(0u, w, nlen);                     // left-aligned
     const uint32_t word = __funnelshift_r(left, o.acc, o.bits);
     const unsigned bits = o.bits - nlen;
     o.acc = __funnelshift_r(left, o.acc, nlen);
-    asm volatile("{ .reg .pred p; setp.ne.u32 p, %3, 0; @p st.shared.u32 [%0], %2; @p mov.b32 %0, %1; @p add.u32 %1, %1, 4; }"
-                 : "+r"(o.wp), "+r"(o.next) : "r"(word), "r"((o.bits ^ bits) & ~31u) : "memory");
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.shared.u32 [%0], %1; @p add.u32 %0, %0, 4; }"
+                 : "+r"(o.wp) : "r"(word), "r"((o.bits ^ bits) & 32u) : "memory");
     o.bits = bits;
 }
-// One symbol, escapes included; ub: bits of 2^23 + u.
+// One symbol, escapes included; ub: bits of 2^23 + u (- 1 for k = 0).
 __device__ __forceinline__ void td_append_any(TdOut &o, uint32_t ub, unsigned raw_bits)
 {
-    int nlen = (int)(o.nlen0 - (ub >> o.k));
-    uint32_t z = (~ub & o.kmask) | o.kbit;
-    if (nlen <= o.limit) { nlen = -(int)(15u + raw_bits); z = ~ub & ((1u << raw_bits) - 1u); }
-    td_append(o, z, (unsigned)nlen);
+    const uint32_t u = (uint32_t)max((int)(ub - kTdUZero) + (o.k ? 0 : 1), 0), q = u >> o.k;       // (2^23 - 1, for k = 0 and u = 0, has bits two below those of 2^23)
+    const bool escape = q >= 15u;
+    td_append(o, escape ? ~u & ((1u << raw_bits) - 1u) : (~u & o.kmask) | o.kbit, 0u - (escape ? 15u + raw_bits : q + o.k + 1u));
 }
-// Four symbols of two sub-streams, kJoin of them joined before they are appended (4-bit codes: four, 8-bit codes: two).  Where
-// one is an escape, or the joined ones are longer than a word, one at a time.  A NaN looks like a very long escape: again(i, a, b) then
-// forms symbol i of both sub-streams with care, and leaves behind what the next one needs.
+__device__ __forceinline__ float td_min3_nan(float a, float b, float c)
+{
+    float d;
+    asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+__device__ __forceinline__ f32x2 td_fma2_up(f32x2 a, f32x2 b, f32x2 c)        // rounded towards +infinity
+{
+    f32x2 d;
+    asm("fma.rp.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+// Four symbols of two sub-streams (ux, uy, and nx, ny: kTdLenZero minus their lengths), kJoin of them joined before they are appended (4-bit codes:
+// four, 8-bit codes: two).  Where one is an escape, or the joined ones are longer than a word, one at a time.  A NaN goes the same way:
+// again(i, a, b) then forms symbol i of both sub-streams with care, and leaves behind what the next one needs.
 template <unsigned kN> struct TdJoin { static constexpr unsigned value = kN; };
 template <unsigned kJoin, typename Again>
-__device__ __forceinline__ void td_append4(const TdLaunch &P, TdOut &x, TdOut &y, const uint32_t (&ux)[4], const uint32_t (&uy)[4], unsigned raw_bits,
-                                           Again again)
+__device__ __forceinline__ void td_append4(TdOut &x, TdOut &y, const uint32_t (&ux)[4], const uint32_t (&uy)[4], const float (&nx)[4], const float (&ny)[4],
+                                           unsigned raw_bits, Again again)
 {
-    int lx[4], ly[4];                                        // minus the lengths
     uint32_t zx[4], zy[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        lx[i] = (int)(ux[i] >> x.k) * P.minus_one + (int)x.nlen0;
-        ly[i] = (int)(uy[i] >> y.k) * P.minus_one + (int)y.nlen0;
         zx[i] = (~ux[i] & x.kmask) | x.kbit;
         zy[i] = (~uy[i] & y.kmask) | y.kbit;
     }
-    const int mx = min(min(lx[0], lx[1]), min(lx[2], lx[3])), my = min(min(ly[0], ly[1]), min(ly[2], ly[3]));
-    int jx[4], jy[4], longest = 0;                           // joined
+    const float mx = td_min3_nan(td_min3_nan(nx[0], nx[1], nx[2]), nx[3], nx[3]), my = td_min3_nan(td_min3_nan(ny[0], ny[1], ny[2]), ny[3], ny[3]);
+    int jx[4], jy[4], longest = 0x7fffffff;                  // joined: minus the lengths, plus kJoin times kTdLenBits
 #pragma unroll
     for (int i = 0; i < 4; i += (int)kJoin) {
-        jx[i] = lx[i]; jy[i] = ly[i];
+        jx[i] = __float_as_int(nx[i]); jy[i] = __float_as_int(ny[i]);
 #pragma unroll
         for (int j = 1; j < (int)kJoin; ++j) {
-            zx[i] = __funnelshift_r(0u, zx[i], (unsigned)lx[i + j]) + zx[i + j];       // shifted left by the length
-            zy[i] = __funnelshift_r(0u, zy[i], (unsigned)ly[i + j]) + zy[i + j];
-            jx[i] = jx[i] + lx[i + j];
-            jy[i] = jy[i] + ly[i + j];
+            zx[i] = __funnelshift_r(0u, zx[i], __float_as_uint(nx[i + j])) + zx[i + j];       // shifted left by the length
+            zy[i] = __funnelshift_r(0u, zy[i], __float_as_uint(ny[i + j])) + zy[i + j];
+            jx[i] = (int)((unsigned)jx[i] + __float_as_uint(nx[i + j]));
+            jy[i] = (int)((unsigned)jy[i] + __float_as_uint(ny[i + j]));
         }
-        longest = min(longest, min(jx[i], jy[i]));
+        longest = __vimin3_s32(longest, jx[i], jy[i]);
     }
-    if (__builtin_expect(mx <= x.limit || my <= y.limit || longest < -32, 0)) {
+    if (__builtin_expect(!(mx > x.limit) || !(my > y.limit) || longest < (int)(kJoin * kTdLenBits - 32u), 0)) {
         uint32_t a[4], b[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) { a[i] = ux[i]; b[i] = uy[i]; }
-        if (__builtin_expect(min(mx, my) < -4096, 0)) {      // (of a number: -516 or more)
+        if (__builtin_expect(mx != mx || my != my, 0)) {
 #pragma unroll 1
             for (int i = 0; i < 4; ++i) {
                 a[0] = a[1]; a[1] = a[2]; a[2] = a[3];
@@ -684,20 +693,18 @@ __device__ __forceinline__ void td_append4(const TdLaunch &P, TdOut &x, TdOut &y
         }
     }
 }
-// The end of a sub-stream that began at addr: zero bits (ones, complemented) up to the byte, the first word and the last one.
-__device__ __forceinline__ void td_out_finish(TdOut &o, uint32_t addr, uint32_t aside)
+// The end of a sub-stream: zero bits (ones, complemented) up to the byte; and, when all of the slice's whole words are out, the bits of its last
+// word, which neighbours may share.
+__device__ __forceinline__ void td_out_pad(TdOut &o)
 {
     const unsigned pad = (0u - o.bits) & 7u;
     if (pad) td_append(o, (1u << pad) - 1u, 0u - pad);
-    const bool one_word = o.wp == aside;                     // nothing has gone out yet
-    if (!one_word) {
-        uint32_t first;
-        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(first) : "r"(aside) : "memory");
-        asm volatile("red.shared.or.b32 [%0], %1;" :: "r"(addr & ~3u), "r"(first) : "memory");
-    }
+}
+__device__ __forceinline__ void td_out_last(const TdOut &o)
+{
     if (o.bits & 31u) {
         const uint32_t word = o.acc << (32u - (o.bits & 31u));
-        asm volatile("red.shared.or.b32 [%0], %1;" :: "r"(one_word ? addr & ~3u : o.wp), "r"(word) : "memory");
+        asm volatile("red.shared.or.b32 [%0], %1;" :: "r"(o.wp), "r"(word) : "memory");
     }
 }
 
@@ -705,7 +712,8 @@ __device__ __forceinline__ void td_out_finish(TdOut &o, uint32_t addr, uint32_t 
 // says what the largest magnitude was (a bf16 number: scale * qmax rounded to bf16 is that number again), so there is no pass
 // for it and no tile.  The staging area holds the slice's bits complemented, as big-endian words.  Bound by instruction issue
 // (77 % of the slots).  8B shape, 16 chunks of 512 tokens: 1020 us for 8-bit codes with a tile, a pass over it for the magnitudes and
-// every symbol appended by itself, 520 us this way; 4-bit codes 1000 -> 470 us.  Sixteen CTAs of 64 threads an SM (64 registers) with
+// every symbol appended by itself, 520 us this way; 4-bit codes 1000 -> 470 us.  Lengths of two channels from one multiply-add, and no word kept
+// aside, took the whole store from 795 to 782 us (uncorrelated), 810 -> 799 (correlation 0.9), 853 -> 851 (0.99), with 4-bit codes 698 -> 692, 693 -> 688, 689 -> 686.  Sixteen CTAs of 64 threads an SM (64 registers) with
 // eight tokens loaded ahead; twelve CTAs, four or sixteen tokens are 1-7 % slower.
 // (Other slices: at most 256 threads, 96 registers; at 104 a slice of 192 channels loses a CTA an SM and 10 %.)
 template <unsigned kCols>
@@ -718,14 +726,14 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 320u, kCols ? 16 : 2) kdn
     const unsigned nthreads = kCols ? kCols / 2u : blockDim.x, tid = threadIdx.x;
     const int codec = s.op.codec;
     const unsigned raw_bits = (unsigned)td_raw_bits(codec);
-    unsigned long long *rows = reinterpret_cast<unsigned long long *>(smem_raw);            // [66]
+    unsigned long long *rows = reinterpret_cast<unsigned long long *>(smem_raw);            // [64], and two to spare
     unsigned *scratch = reinterpret_cast<unsigned *>(rows + 66);                             // 32 words
     unsigned char *stage = smem_raw + kTdEncodeHead;
     const TdLayout &lay = P.layout[blockIdx.z];
     const unsigned long long row = (unsigned long long)s.seg * RE;
     const bool act = 2u * tid < C;
     // this kernel may start as soon as the scan's CTAs have seen the planner end: the row addresses are what it can have ready
-    const bool bad = td_row_addresses<true>(P, s, rows, tid, nthreads);
+    const bool bad = td_row_addresses<true, false>(P, s, rows, tid, nthreads);
     dependency_wait();
     release_dependents();
     const TdOffsets o = td_offsets(s.op.data + lay.lens + row, s.c0, C, nthreads, scratch);
@@ -742,48 +750,57 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 320u, kCols ? 16 : 2) kdn
     }
     const unsigned len_x = o.pair & 0xffu, len_y = o.pair >> 8;
     // (a length of zero: the planner gave this slice up)
-    if (act && len_x != 0u && len_y != 0u && len_x <= td_max_len(codec) && len_y <= td_max_len(codec)) {
+    const bool coding = act && len_x != 0u && len_y != 0u && len_x <= td_max_len(codec) && len_y <= td_max_len(codec);
+    TdOut x, y;
+    if (coding) {
         const unsigned long long at = row + s.c0 + 2u * tid;
         const unsigned params = *reinterpret_cast<const unsigned short *>(s.op.data + lay.params + at);
         const float2 sc = *reinterpret_cast<const float2 *>(s.op.data + lay.scales + 4ull * at);
         const float qmax = (float)td_qmax(codec);
         const float inv_x = sc.x != 0.0f ? __fdiv_rn(qmax, __bfloat162float(__float2bfloat16_rn(__fmul_rn(sc.x, qmax)))) : 0.0f;
         const float inv_y = sc.y != 0.0f ? __fdiv_rn(qmax, __bfloat162float(__float2bfloat16_rn(__fmul_rn(sc.y, qmax)))) : 0.0f;
-        TdOut x, y;
-        const uint32_t addr_x = smem_u32(stage) + shift + o.off, addr_y = addr_x + len_x;
-        const uint32_t aside = smem_u32(stage) + (uint32_t)td_stage_bytes(C, P.words) + 8u * tid;
-        td_out_init(x, addr_x, aside, params & 0xffu);
-        td_out_init(y, addr_y, aside + 4u, params >> 8);
+        const uint32_t addr_x = smem_u32(stage) + shift + o.off;
+        td_out_init(x, addr_x, params & 0xffu);
+        td_out_init(y, addr_x + len_x, params >> 8);
         // per token: m + code (m = 1.5 * 2^23), minus m or the token before (delta mode), all exact
         const float m = 12582912.0f;
         const f32x2 inv2 = pack2(inv_x, inv_y), m2 = pack2(m, m), one2 = pack2(P.fone, P.fone), two2 = pack2(2.0f, 2.0f), half2 = pack2(0.5f, 0.5f);
         const bool dx = (params & 8u) != 0u, dy = (params & 0x800u) != 0u;
         const f32x2 nd2 = pack2(dx ? -1.0f : 0.0f, dy ? -1.0f : 0.0f), nc2 = pack2(dx ? 0.0f : -m, dy ? 0.0f : -m);
         f32x2 base = pack2(-m, -m);
+        const float zero_x = x.k ? 8388607.5f : 8388606.5f, zero_y = y.k ? 8388607.5f : 8388606.5f;
+        auto per_len = [&](unsigned k) { return __uint_as_float((127u - k) << 23); };           // 2^-k
+        const f32x2 per2 = pack2(-per_len(x.k), -per_len(y.k));
+        auto len_zero = [&](unsigned k) { return k ? kTdLenZero + 8388608.0f * per_len(k) - (float)(k + 1u) : kTdLenZero + 8388606.0f; };
+        const f32x2 len2 = pack2(len_zero(x.k), len_zero(y.k));
         auto symbol = [&](uint32_t v, uint32_t &a, uint32_t &b) {
             const f32x2 r = add2_unfused(mul2(bf16x2_widen(v), inv2), m2, one2);
             const f32x2 f = fma2(add2(r, base), two2, half2);
             base = fma2(r, nd2, nc2);
             float fa, fb;
             unpack2(f, fa, fb);
-            a = __float_as_uint(__fadd_rn(fabsf(fa), 8388607.5f));
-            b = __float_as_uint(__fadd_rn(fabsf(fb), 8388607.5f));
+            a = __float_as_uint(__fadd_rn(fabsf(fa), zero_x));
+            b = __float_as_uint(__fadd_rn(fabsf(fb), zero_y));
         };
         // the same of token t, whatever it is (one that is not finite also spoils `base`)
         auto again = [&](unsigned t, uint32_t &a, uint32_t &b) {
-            const uint32_t v = __ldcg(reinterpret_cast<const uint32_t *>(rows[t + (t >> 5)]) + tid);
-            const uint32_t u = t ? __ldcg(reinterpret_cast<const uint32_t *>(rows[t - 1u + ((t - 1u) >> 5)]) + tid) : 0u;
+            const uint32_t v = __ldcg(reinterpret_cast<const uint32_t *>(rows[t]) + tid);
+            const uint32_t u = t ? __ldcg(reinterpret_cast<const uint32_t *>(rows[t - 1u]) + tid) : 0u;
             const int qx = td_code(v & 0xffffu, inv_x), qy = td_code(v >> 16, inv_y);
             const int ex = dx ? qx - td_code(u & 0xffffu, inv_x) : qx, ey = dy ? qy - td_code(u >> 16, inv_y) : qy;
-            a = kTdUZero + (unsigned)((ex << 1) ^ (ex >> 31));
-            b = kTdUZero + (unsigned)((ey << 1) ^ (ey >> 31));
+            a = __float_as_uint((float)((x.k ? 8388608 : 8388607) + ((ex << 1) ^ (ex >> 31))));
+            b = __float_as_uint((float)((y.k ? 8388608 : 8388607) + ((ey << 1) ^ (ey >> 31))));
             base = fma2(pack2(m + (float)qx, m + (float)qy), nd2, nc2);
         };
         // kTdLoad tokens at a time, the next ones already on their way
         auto load = [&](unsigned t0, uint32_t (&v)[kTdLoad]) {
-            const unsigned long long *r = rows + t0 + (t0 >> 5);
+            const ulonglong2 *r = reinterpret_cast<const ulonglong2 *>(rows + t0);
 #pragma unroll
-            for (int i = 0; i < (int)kTdLoad; ++i) v[i] = __ldcg(reinterpret_cast<const uint32_t *>(r[i] + (unsigned long long)(2u * tid) * P.pow2[1]));
+            for (int i = 0; i < (int)kTdLoad; i += 2) {
+                const ulonglong2 d = r[i / 2];
+                v[i] = __ldcg(reinterpret_cast<const uint32_t *>(d.x + (unsigned long long)(2u * tid) * P.pow2[1]));
+                v[i + 1] = __ldcg(reinterpret_cast<const uint32_t *>(d.y + (unsigned long long)(2u * tid) * P.pow2[1]));
+            }
         };
         auto code = [&](auto join) -> unsigned {
             unsigned t0 = 0;
@@ -797,9 +814,13 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 320u, kCols ? 16 : 2) kdn
 #pragma unroll
                 for (int i = 0; i < (int)kTdLoad; i += 4) {
                     uint32_t ux[4], uy[4];
+                    float nx[4], ny[4];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) symbol(v[i + j], ux[j], uy[j]);
-                    td_append4<decltype(join)::value>(P, x, y, ux, uy, raw_bits, [&](unsigned j, uint32_t &a, uint32_t &b) { again(t0 + (unsigned)i + j, a, b); });
+                    for (int j = 0; j < 4; ++j) {
+                        symbol(v[i + j], ux[j], uy[j]);
+                        unpack2(td_fma2_up(pack2_bits(ux[j], uy[j]), per2, len2), nx[j], ny[j]);
+                    }
+                    td_append4<decltype(join)::value>(x, y, ux, uy, nx, ny, raw_bits, [&](unsigned j, uint32_t &a, uint32_t &b) { again(t0 + (unsigned)i + j, a, b); });
                 }
             }
             return t0;
@@ -808,13 +829,18 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 320u, kCols ? 16 : 2) kdn
 #pragma unroll 1
         for (; t0 < s.n_tok; ++t0) {
             uint32_t ux, uy;
-            symbol(__ldcg(reinterpret_cast<const uint32_t *>(rows[t0 + (t0 >> 5)]) + tid), ux, uy);
+            symbol(__ldcg(reinterpret_cast<const uint32_t *>(rows[t0]) + tid), ux, uy);
             if (max(ux, uy) > 0x7f800000u) again(t0, ux, uy);
             td_append_any(x, ux, raw_bits);
             td_append_any(y, uy, raw_bits);
         }
-        td_out_finish(x, addr_x, aside);
-        td_out_finish(y, addr_y, aside + 4u);
+        td_out_pad(x);
+        td_out_pad(y);
+    }
+    __syncthreads();                                         // the whole words of all sub-streams are out
+    if (coding) {
+        td_out_last(x);
+        td_out_last(y);
     }
     // the last slice of a segment also writes the zero bytes that pad the segment to 16
     unsigned pad = 0;
@@ -960,8 +986,8 @@ __device__ __forceinline__ void td_step(const TdLaunch &P, TdStream &x, TdStream
 // stream's chain of dependent operations hides the other's, and writes finished values into the rows: no pass over codes.  Half
 // of the rows at a time keeps a CTA of 64 threads at 16 KiB of shared memory, twelve (8-bit codes: ten) to an SM; all rows at a time
 // are 15 % slower.  The rows leave with 128-bit stores, sixteen lanes to a 256-byte piece of a token row.  8B shape, 32 chunks of 512
-// tokens, 4-bit codes: 1728 us with one thread per channel, a code tile and a separate pass that multiplied, 730 us this way; 8-bit
-// codes 1765 -> 900 us.
+// tokens, 4-bit codes: 1728 us with one thread per channel, a code tile and a separate pass that multiplied, 709 us this way; 8-bit
+// codes 1765 -> 864 us.  (The counters are those of one kernel for both codecs, 724 and 892 us.)
 // kCols: channels per CTA when known at compile time (the usual slice; every stride in the decoding loop is then an
 // immediate), 0: taken from the launch record.
 template <bool kCompose, unsigned kCols, bool kInt4>
