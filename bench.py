@@ -45,7 +45,7 @@ N_CHUNKS, CHUNK_TOKENS = 64, 512
 N_PARTS, PART_TOKENS, SUFFIX_TOKENS = 10, 1024, 256
 RAW, INT8, INT4, INT8KC, INT4KC, INT8TD, INT4TD = 0, 1, 2, 3, 4, 5, 6
 FALLBACK_HBM_GBS = 6650.0
-TD_DECODE_INSTS = {INT8TD: 23.4, INT4TD: 21.0}     # warp instructions per 32 symbols of the token-delta decoder (profiles/ncu_token_delta_kernels_llama3_8b.md)
+TD_DECODE_INSTS = {INT8TD: 23.4, INT4TD: 21.0}     # warp instructions per 32 symbols of the token-delta decoder (profiles/ncu_token_delta_kernels_llama3_8b.md; one kernel for both codecs then)
 
 
 def bytes_per_elem(codec: int) -> float:
