@@ -954,8 +954,32 @@ kdn_status launch_batch(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *ho
     return KDN_OK;
 }
 
+// Slices of a token-delta segment (one CTA each): 0 where a row cannot be cut into slices that the kernels take.  A slice's channels are
+// a multiple of 16 that divides the row, whole heads when keys are re-rotated, kTdCols if possible
+// (small slices: many CTAs share an SM, and each one's loads, decoding and stores overlap the others').
+unsigned td_slices(const Pool &pool, bool any_rot)
+{
+    const unsigned row_elems = (unsigned)pool.H * (unsigned)pool.D, unit = any_rot ? lcm_u(16u, (unsigned)pool.D) : 16u;
+    unsigned n_split = 1;
+    while (row_elems / n_split > kTdCols && row_elems % (n_split * 2u) == 0u && (row_elems / (n_split * 2u)) % unit == 0u) n_split *= 2u;
+    const unsigned cols = row_elems / n_split;
+    return cols % 16u || cols > 512u ? 0u : n_split;
+}
+
+// Whether a call's token-delta ops can run, asked before anything of the call is enqueued: a rotated op needs slices of whole heads, and any of
+// the launches that the call is cut into may be the one that has it.
+kdn_status check_td(const Pool &pool, const std::vector<HostOp> &dev_ops, const std::vector<HostOp> &host_ops)
+{
+    bool any_td = false, any_rot = false;
+    for (const std::vector<HostOp> *ops : { &dev_ops, &host_ops })
+        for (const HostOp &h : *ops)
+            if (is_td(h.op.codec)) { any_td = true; any_rot |= h.rotate; }
+    // (a row that whole heads divide into slices is divided by the narrower unit too)
+    return any_td && !td_slices(pool, any_rot) ? KDN_E_UNSUPPORTED : KDN_OK;
+}
+
 // Ops whose chunk is in a token-delta Rice codec: at most kInlineOps per launch, their records travel as kernel
-// parameters.  Store is three launches (plan, scan, encode), retrieve and compose one (plus the rotation table).
+// parameters.  Store is three launches (plan, scan, encode), retrieve and compose one for each codec (plus the rotation table).
 kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops, int n, cudaStream_t stream)
 {
     // a launch of the decoder has chunks of one codec
@@ -973,15 +997,11 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
         }
     }
     const unsigned row_elems = (unsigned)pool.H * (unsigned)pool.D;
-    // channels per CTA: a multiple of 16 that divides the row, whole heads when keys are re-rotated, kTdCols if possible
-    // (small slices: many CTAs share an SM, and each one's loads, decoding and stores overlap the others')
     bool any_rot = false;
     for (int i = 0; i < n; ++i) any_rot |= hops[i].rotate;
-    const unsigned unit = any_rot ? lcm_u(16u, (unsigned)pool.D) : 16u;
-    unsigned n_split = 1;
-    while (row_elems / n_split > kTdCols && row_elems % (n_split * 2u) == 0u && (row_elems / (n_split * 2u)) % unit == 0u) n_split *= 2u;
+    const unsigned n_split = td_slices(pool, any_rot);
+    if (!n_split) return KDN_E_UNSUPPORTED;
     const unsigned cols = row_elems / n_split;
-    if (cols % 16u || cols > 512u) return KDN_E_UNSUPPORTED;
     const size_t smem_limit = (size_t)ctx->env.smem_optin;
 
     for (int first = 0; first < n; first += kInlineOps) {
@@ -1370,10 +1390,12 @@ kdn_status run_ops(kdn_ctx *ctx, int pool_id, int OP, std::vector<HostOp> &dev_o
 {
     const Pool &pool = ctx->pools[(size_t)pool_id];
     cudaStream_t stream = (cudaStream_t)cuda_stream;
+    kdn_status st = check_td(pool, dev_ops, host_ops);
+    if (st != KDN_OK) return st;
     if (host_ops.empty()) return launch_all(ctx, pool, OP, dev_ops, stream);
     cudaStream_t side = (cudaStream_t)side_stream;
     if (!side) {
-        kdn_status st = ensure_side(ctx);
+        st = ensure_side(ctx);
         if (st != KDN_OK) return st;
         side = ctx->own_side;
     }
@@ -1385,7 +1407,7 @@ kdn_status run_ops(kdn_ctx *ctx, int pool_id, int OP, std::vector<HostOp> &dev_o
     }
     if (!td_host.empty()) {
         if (OP == OP_STORE) return KDN_E_UNSUPPORTED;        // the size of the result is not known before the kernels ran
-        kdn_status st = fork ? fork_side(ctx, stream, side) : KDN_OK;
+        st = fork ? fork_side(ctx, stream, side) : KDN_OK;
         if (st == KDN_OK) st = run_td_host(ctx, pool, OP, td_host, stream, side);
         if (st != KDN_OK) return st;
         if (host_ops.empty()) return launch_all(ctx, pool, OP, dev_ops, stream);
@@ -1415,7 +1437,7 @@ kdn_status run_ops(kdn_ctx *ctx, int pool_id, int OP, std::vector<HostOp> &dev_o
     };
     // Fork: the side stream's copies come after everything already queued on the caller's stream (a copy that filled
     // the pinned chunk, an earlier store into it through another side stream).
-    kdn_status st = fork ? fork_side(ctx, stream, side) : KDN_OK;
+    st = fork ? fork_side(ctx, stream, side) : KDN_OK;
     if (st == KDN_OK) st = run_staged(ctx, pool, OP, host_ops, stream, side, between);
     while (st == KDN_OK && next < dev_ops.size()) st = between();
     // Join: a store's device-to-host copies run on the side stream; the caller's stream waits for them, so that an

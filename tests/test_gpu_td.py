@@ -242,6 +242,38 @@ def test_refusals_and_damaged_chunks():
         dev.close()
 
 
+@pytest.mark.parametrize("still,moved,pinned", [(TD8, TD4, False), (TD4, TD8, False), (TD8, TD8, True), (TD4, TD8, True)])
+def test_a_compose_that_is_refused_writes_nothing(still, moved, pinned):
+    """Rows of five heads of 128 divide into slices, but not into slices of whole heads, which a moved chunk needs: a call that has such a chunk beside
+    one that stays where it was, of the other codec or in host memory, is refused before any of it is enqueued."""
+    shape = synth.TOY.with_(n_layers=1, n_kv_heads=5, head_dim=128, block_size=16, n_blocks=32)
+    dev = Device(shape, seed=9)
+    try:
+        K = dev.K
+        T = 40
+        a, b = dev.chunk_buf(T, still), dev.chunk_buf(T, moved)
+        src = dev.table(np.arange(3, dtype=np.int32))
+        dev.store([dev.op(src, 0, a, T, still), dev.op(src, 0, b, T, moved)])
+        assert dev.sync() == 0
+        if pinned:
+            h = dev.chunk_buf(T, still, pinned=True)
+            h.copy_(a.cpu())
+            a = h
+        before, launches = dev.pool_np(), K.kdn_launch_count(dev.ctx)
+        dst = dev.table(np.arange(8, 16, dtype=np.int32))
+        with pytest.raises(K.KdnError) as e:
+            dev.compose([K.ComposeReq(dst.data_ptr(), 8, [dev.chunk(a, T, still, 0), dev.chunk(b, T, moved, 7)], [0, 64], shape.rope_theta)])
+        assert e.value.status == K.KDN_E_UNSUPPORTED
+        assert dev.sync() == 0
+        assert K.kdn_launch_count(dev.ctx) == launches and np.array_equal(dev.pool_np(), before)
+        # (both where they were: slices of 80 channels do)
+        dev.compose([K.ComposeReq(dst.data_ptr(), 8, [dev.chunk(a, T, still, 0), dev.chunk(b, T, moved, 64)], [0, 64], shape.rope_theta)])
+        assert dev.sync() == 0
+        assert K.kdn_launch_count(dev.ctx) > launches
+    finally:
+        dev.close()
+
+
 @pytest.mark.parametrize("codec", [TD8, TD4], ids=["int8td", "int4td"])
 def test_retrieve_and_compose_from_page_locked_host_chunks(codec):
     """Delivery of compressed chunks (the point of coding them): token-delta chunks kept in page-locked host memory are
