@@ -979,23 +979,9 @@ kdn_status check_td(const Pool &pool, const std::vector<HostOp> &dev_ops, const 
 }
 
 // Ops whose chunk is in a token-delta Rice codec: at most kInlineOps per launch, their records travel as kernel
-// parameters.  Store is three launches (plan, scan, encode), retrieve and compose one for each codec (plus the rotation table).
+// parameters.  Store is three launches (plan, scan, encode), retrieve and compose one (plus the rotation table).
 kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops, int n, cudaStream_t stream)
 {
-    // a launch of the decoder has chunks of one codec
-    if (OP != OP_STORE) {
-        bool mixed = false;
-        for (int i = 1; i < n; ++i) mixed |= hops[i].op.codec != hops[0].op.codec;
-        if (mixed) {
-            for (const bool int4 : {false, true}) {
-                std::vector<HostOp> part;
-                for (int i = 0; i < n; ++i) if ((hops[i].op.codec == KDN_CODEC_INT4_TD64) == int4) part.push_back(hops[i]);
-                const kdn_status r = launch_td(ctx, pool, OP, part.data(), (int)part.size(), stream);
-                if (r != KDN_OK) return r;
-            }
-            return KDN_OK;
-        }
-    }
     const unsigned row_elems = (unsigned)pool.H * (unsigned)pool.D;
     bool any_rot = false;
     for (int i = 0; i < n; ++i) any_rot |= hops[i].rotate;
@@ -1010,6 +996,7 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
         tp.wait_limit_ns = ctx->wait_limit_ns;
         RopeInline rope_inl{};
         int n_rope = 0, max_groups = 0, max_layers = 0;
+        bool any5 = false, any6 = false;
         for (int i = 0; i < m; ++i) {
             DevOp op = hops[first + i].op;
             op.rope = -1;
@@ -1017,6 +1004,7 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
                 rope_inl.p[n_rope] = hops[first + i].rp;
                 op.rope = n_rope++;
             }
+            (op.codec == KDN_CODEC_INT4_TD64 ? any6 : any5) = true;
             tp.inline_ops[i] = op;
             tp.layout[i] = td_layout(pool.L, row_elems, op.T, op.codec);
             if (td_words(op.codec) > tp.words) tp.words = td_words(op.codec);
@@ -1079,21 +1067,19 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
             }
             kdn_status r = KDN_OK;
             const unsigned dec_threads = (cols / 2u + 31u) & ~31u;       // a thread decodes two channels
-#define KDN_TD_DECODE(COMPOSE, COLS, INT4)                                                                  \
+#define KDN_TD_DECODE(COMPOSE, COLS, CODEC)                                                                 \
             {                                                                                               \
-                r = ctx->env.resident(kdn_td_decode_kernel<COMPOSE, COLS, INT4>, (int)dec_threads, smem, &per_sm); \
+                r = ctx->env.resident(kdn_td_decode_kernel<COMPOSE, COLS, CODEC>, (int)dec_threads, smem, &per_sm); \
                 if (r != KDN_OK) return r;                                                                  \
                 if (per_sm < 1) return KDN_E_UNSUPPORTED;                                                   \
-                r = launch_behind(kdn_td_decode_kernel<COMPOSE, COLS, INT4>, grid, dec_threads, smem, stream, tp); \
+                r = launch_behind(kdn_td_decode_kernel<COMPOSE, COLS, CODEC>, grid, dec_threads, smem, stream, tp); \
                 if (r != KDN_OK) return r;                                                                  \
             }
-#define KDN_TD_DECODE_OP(COLS, INT4) if (OP == OP_COMPOSE) KDN_TD_DECODE(true, COLS, INT4) else KDN_TD_DECODE(false, COLS, INT4)
-            const bool int4 = hops[first].op.codec == KDN_CODEC_INT4_TD64;
-            if (cols == kTdCols) {
-                if (int4) KDN_TD_DECODE_OP(kTdCols, true) else KDN_TD_DECODE_OP(kTdCols, false)
-            } else {
-                if (int4) KDN_TD_DECODE_OP(0, true) else KDN_TD_DECODE_OP(0, false)
-            }
+#define KDN_TD_DECODE_COLS(COMPOSE, CODEC) if (cols == kTdCols) KDN_TD_DECODE(COMPOSE, kTdCols, CODEC) else KDN_TD_DECODE(COMPOSE, 0, CODEC)
+#define KDN_TD_DECODE_OP(CODEC) if (OP == OP_COMPOSE) { KDN_TD_DECODE_COLS(true, CODEC) } else { KDN_TD_DECODE_COLS(false, CODEC) }
+            // one launch, whichever codecs its chunks have
+            if (any5 && any6) { KDN_TD_DECODE_OP(0) } else if (any6) { KDN_TD_DECODE_OP(6) } else { KDN_TD_DECODE_OP(5) }
+#undef KDN_TD_DECODE_COLS
 #undef KDN_TD_DECODE_OP
 #undef KDN_TD_DECODE
             KDN_CUDA(cudaGetLastError());

@@ -990,18 +990,21 @@ __device__ __forceinline__ void td_step(const TdLaunch &P, TdStream &x, TdStream
 // codes 1765 -> 864 us.  (The counters are those of one kernel for both codecs, 724 and 892 us.)
 // kCols: channels per CTA when known at compile time (the usual slice; every stride in the decoding loop is then an
 // immediate), 0: taken from the launch record.
-template <bool kCompose, unsigned kCols, bool kInt4>
+// kCodec: the codec of the launch's chunks, 0 where it has chunks of both.  (A kernel per codec takes fewer instructions, but a launch for each
+// half of such a call leaves the SMs to half a call at a time and pays for one more.  8B shape, us a retrieve, two launches / one: a chunk of each codec,
+// 64 tokens 16.2 / 13.5, 512 tokens 65.2 / 59.5, sixteen of each 1064 / 1008; compose, eight of each, 331 tokens, 70B shape with two heads 269 / 252.  Two
+// whole bodies behind one branch were no good: 1145 and 288.)
+template <bool kCompose, unsigned kCols, int kCodec>
 __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 12 : 1) kdn_td_decode_kernel(const __grid_constant__ TdLaunch P)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     dependency_wait();
     release_dependents();
-    constexpr int codec = kInt4 ? 6 : 5;
-    constexpr unsigned kWords = kInt4 ? 11u : 19u;                       // td_words(codec)
     const TdSlice s = td_slice(P);
-    if (!s.valid || s.op.codec != codec) return;
+    if (!s.valid) return;
+    const int codec = kCodec ? kCodec : s.op.codec;
+    const unsigned kWords = td_words(codec), raw_bits = (unsigned)td_raw_bits(codec);
     const unsigned C = kCols ? kCols : P.cols, RE = P.row_elems;
-    constexpr unsigned raw_bits = kInt4 ? 5u : 9u;
     const unsigned nthreads = kCols ? kCols / 2u : blockDim.x;
 
     uint32_t *I = reinterpret_cast<uint32_t *>(smem_raw);                // interleaved sub-streams [word][C]
@@ -1181,11 +1184,11 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 12 : 1) kdn
                     for (unsigned i = 0; i < kStep; ++i) put(t + i, vx[i], vy[i]);
                 }
             };
-            if (kInt4) {
-                steps(TdConst<4>(), TdConst<8>());
+            if (codec == 6) {
+                steps(TdConst<4>(), TdConst<kCodec ? 8 : 4>());
             } else {
-                steps(TdConst<3>(), TdConst<6>());
-                steps(TdConst<2>(), TdConst<2>());
+                steps(TdConst<kCodec ? 3 : 2>(), TdConst<kCodec ? 6 : 4>());
+                if (kCodec) steps(TdConst<2>(), TdConst<2>());
             }
 #pragma unroll 1
             for (; t < nt; ++t) {

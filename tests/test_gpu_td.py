@@ -182,6 +182,51 @@ def test_mixed_batch_and_many_ops():
         dev.close()
 
 
+@pytest.mark.parametrize("shape", [SHAPES[1], SHAPES[3].with_(block_size=16)], ids=["slice128", "slice64"])
+def test_a_call_of_both_codecs_is_one_launch(shape):
+    """Retrieve and compose of chunks of both token-delta codecs: one decoder launch (and the rotation table's), as for chunks of one codec; the
+    decoder takes each slice's codec from its chunk."""
+    dev = Device(shape, seed=53)
+    try:
+        K = dev.K
+        bs, T, n = shape.block_size, 75, 4
+        nb = -(-T // bs)
+        host = dev.pool_np()
+        perm = np.random.default_rng(19).permutation(shape.n_blocks).astype(np.int32)
+        codecs = [TD8, TD4, TD4, TD8]
+        src = perm[:nb]
+        bufs = [dev.chunk_buf(T, c) for c in codecs]
+        dev.store([dev.op(dev.table(src), 0, b, T, c) for b, c in zip(bufs, codecs)])
+        assert dev.sync() == 0
+        wants = [oracle.store(host, src, 0, T, c) for c in codecs]
+        dst = perm[nb:(n + 1) * nb].reshape(n, nb)
+        ops = [dev.op(dev.table(d), 0, b, T, c) for d, b, c in zip(dst, bufs, codecs)]
+        launches = K.kdn_launch_count(dev.ctx)
+        dev.retrieve(ops)
+        assert K.kdn_launch_count(dev.ctx) == launches + 1
+        assert dev.sync() == 0
+        ref = host.copy()
+        for d, w, c in zip(dst, wants, codecs):
+            oracle.retrieve(ref, d, 0, T, c, w)
+        assert np.array_equal(dev.pool_np(), ref)
+        rt = perm[-n * nb:]
+        base = [7, 0, 5, 3 * nb * bs]                                    # three parts are moved, the last stays where it was
+        where = [i * nb * bs for i in range(n)]
+        launches = K.kdn_launch_count(dev.ctx)
+        dev.compose([K.ComposeReq(dev.table(rt).data_ptr(), len(rt), [dev.chunk(b, T, c, p) for b, c, p in zip(bufs, codecs, base)], where, shape.rope_theta)])
+        assert K.kdn_launch_count(dev.ctx) == launches + 2
+        assert dev.sync() == 0
+        kref, kmag = oracle.compose(ref, rt, [(w, T, c, p, d) for w, c, p, d in zip(wants, codecs, base, where)], shape.rope_theta, want_ref=True)
+        got = dev.pool_np()
+        moved = np.concatenate([d + np.arange(T) for b, d in zip(base, where) if b != d])
+        rot = np.zeros(got.shape, dtype=bool)
+        rot[:, 0, rt[moved // bs], moved % bs] = True
+        assert np.array_equal(got[~rot], ref[~rot])
+        check_rotated_keys(got[:, 0, rt[moved // bs], moved % bs], kref[:, moved], kmag[:, moved], ref[:, 0, rt[moved // bs], moved % bs])
+    finally:
+        dev.close()
+
+
 def test_layerwise_retrieve_of_a_token_delta_chunk():
     shape = synth.TOY.with_(n_layers=5, n_kv_heads=2, head_dim=64, block_size=16, n_blocks=64)
     dev = Device(shape, seed=29)
