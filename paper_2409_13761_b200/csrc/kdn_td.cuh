@@ -939,16 +939,12 @@ __device__ __forceinline__ void td_symbol_any(const TdLaunch &P, TdStream &s, ui
     s.acc = (u ^ -(u & 1)) + (s.d ? s.acc : kTdCodeBits);
 }
 
-// kStep symbols of two streams side by side, kWin of them out of one 32-bit window (code words of 4-bit codes are short:
-// four in a window, eight a step; of 8-bit codes three and six).  Taken to be no escapes and to fit their windows; where that was wrong, once more
-// with care.  (8B shape, 32 chunks of 512 tokens, 4-bit codes, an earlier form: a window a symbol 965 us, two 908, four 867.  Now, correlation 0.9:
-// steps of four in one kernel for both codecs 724, of eight in a kernel of their own 710; 8-bit codes, pairs 892, triples 864.)
+// kStep symbols of two streams side by side, kWin of them out of one 32-bit window. Taken to be no escapes and to fit their windows; where that was
+// wrong, once more with care, which takes about three times as long, and one lane's escape holds up its warp: so a step is no longer than
+// it has to be.
 template <unsigned kCols, unsigned kWin, unsigned kStep>
-__device__ __forceinline__ void td_step(const TdLaunch &P, TdStream &x, TdStream &y, unsigned row_b, unsigned max_bits, unsigned raw_bits,
-                                        int (&vx)[kStep], int (&vy)[kStep])
+__device__ __forceinline__ void td_step(const TdLaunch &P, TdStream &x, TdStream &y, unsigned row_b, unsigned raw_bits, int (&vx)[kStep], int (&vy)[kStep])
 {
-    x.bp = x.bp < max_bits ? x.bp : max_bits;               // (a damaged stream cannot run off the area)
-    y.bp = y.bp < max_bits ? y.bp : max_bits;
     const unsigned bp_x = x.bp, bp_y = y.bp;
     const int acc_x = x.acc, acc_y = y.acc;
     unsigned longest = 0, most = 0;
@@ -1174,26 +1170,55 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 512u, kCols ? 12 : 1) kdn
         const unsigned nt = s.n_tok - t0 < kTdHalf ? s.n_tok - t0 : kTdHalf;
         if (act) {
             unsigned t = 0;
-            auto steps = [&](auto win, auto step) {
-                constexpr unsigned kStep = (unsigned)decltype(step)::value;
+            auto clamp = [&]() {                             // (a damaged stream cannot run off the area: at most eight symbols between two of these)
+                x.bp = x.bp < max_bits ? x.bp : max_bits;
+                y.bp = y.bp < max_bits ? y.bp : max_bits;
+            };
+            // steps of step symbols, win to a window, in rounds of times steps; whole: no round that would end past nt
+            auto steps = [&](auto win, auto step, auto times, auto whole) {
+                constexpr unsigned kStep = (unsigned)decltype(step)::value, kTimes = (unsigned)decltype(times)::value;
+                constexpr bool kWhole = decltype(whole)::value != 0;
 #pragma unroll 1
-                for (; t + kStep <= nt; t += kStep) {
-                    int vx[kStep], vy[kStep];
-                    td_step<kCols, (unsigned)decltype(win)::value, kStep>(P, x, y, row_b, max_bits, raw_bits, vx, vy);
+                for (; t + (kWhole ? kTimes * kStep : kStep) <= nt; t += kWhole ? kTimes * kStep : 0u) {
+                    clamp();
 #pragma unroll
-                    for (unsigned i = 0; i < kStep; ++i) put(t + i, vx[i], vy[i]);
+                    for (unsigned i = 0; i < kTimes; ++i) {
+                        if (!kWhole && i && t + kStep > nt) break;
+                        int vx[kStep], vy[kStep];
+                        td_step<kCols, (unsigned)decltype(win)::value, kStep>(P, x, y, row_b, raw_bits, vx, vy);
+#pragma unroll
+                        for (unsigned j = 0; j < kStep; ++j) put(t + (kWhole ? i * kStep : 0u) + j, vx[j], vy[j]);
+                        if (!kWhole) t += kStep;
+                    }
                 }
             };
+            // A look for escapes after every window of 4-bit codes (four to one) and every second one of 8-bit codes, two steps a round, and a last half-round
+            // before single symbols.  Against a look every six or eight symbols and up to seven single ones at the end, 8B shape, us a retrieve: sixteen
+            // chunks of 512 tokens with heavy tails (t distribution, three degrees) 727 -> 659, thirty-two with a jump every 16 tokens 1127 -> 1042 and (4-bit)
+            // 940 -> 817, thirty-two of 7 tokens (4-bit) 33.3 -> 30.2, one of 61 tokens 9.5 -> 7.9, of 29 (4-bit) 6.1 -> 5.25; without any of that the same
+            // (878 -> 874, 700 -> 698).  8-bit codes in compose keep three to a window, which the code of a rotation makes worth while (70B shape, two heads,
+            // 219 -> 216, with jumps 268 -> 240; pairs 226 and 258); in a short launch a window that overflows costs more than that gives, so retrieves take
+            // pairs.  Rounds that may end in the middle share their code with the end of a half: better where a rotation has made the code long (4-bit
+            // codes in compose 184 -> 178, with jumps 227 -> 201), worse elsewhere (698 -> 721).
+            const TdConst<0> part;
+            const TdConst<1> one, whole;
+            const TdConst<2> two;
+            const TdConst<3> three;
+            const TdConst<4> four;
             if (codec == 6) {
-                steps(TdConst<4>(), TdConst<kCodec ? 8 : 4>());
+                if constexpr (!kCompose && kCodec) { steps(four, four, two, whole); steps(four, four, one, whole); }
+                else if constexpr (kCols || !kCodec) steps(four, four, two, part);
+                else steps(four, four, one, whole);
             } else {
-                steps(TdConst<kCodec ? 3 : 2>(), TdConst<kCodec ? 6 : 4>());
-                if (kCodec) steps(TdConst<2>(), TdConst<2>());
+                if constexpr (!kCompose && kCodec) { steps(two, four, two, whole); steps(two, four, one, whole); }
+                else if constexpr (kCompose && kCodec && kCols) { steps(three, three, two, whole); steps(two, two, one, whole); }
+                else if constexpr (!kCompose) steps(two, four, two, part);
+                else if constexpr (!kCodec) steps(two, two, two, part);
+                else steps(two, four, one, whole);
             }
 #pragma unroll 1
             for (; t < nt; ++t) {
-                x.bp = x.bp < max_bits ? x.bp : max_bits;
-                y.bp = y.bp < max_bits ? y.bp : max_bits;
+                clamp();
                 td_symbol_any(P, x, td_window<kCols>(x, row_b), raw_bits);
                 td_symbol_any(P, y, td_window<kCols>(y, row_b), raw_bits);
                 put(t, x.acc, y.acc);

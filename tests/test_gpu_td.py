@@ -49,6 +49,19 @@ def make_pool_np(shape, table, off, T, rho, seed):
     return synth.pool_to_numpy(k, v)
 
 
+def make_escape_pool_np(shape, table, T):
+    """A pool with correlated values at the positions of `table`, and channels with rare large codes among small ones."""
+    bs, n = shape.block_size, len(table) * shape.block_size
+    pool = make_pool_np(shape, table, 0, n, 0.9, seed=T)
+    t = np.arange(n)
+    for c in range(8, 40):
+        x = np.zeros(n, dtype=np.float32)
+        x[(t + c) % (7 + c % 5) == 0] = 2.0 * (1 - 2 * (c & 1))              # escapes at every phase of a step
+        x[(t * 5 + c) % 11 == 0] += 0.07 * (c % 7)                           # among small codes, so that k stays small
+        pool[0, c & 1, table[t // bs], t % bs, 0, c] = bf16_bits(x)
+    return pool
+
+
 def used_bytes(K, desc, buf, T, codec):
     lay = K.kdn_td_layout(desc, T, codec)
     head = to_np(buf[:8 * (lay["segments"] + 1)]).view(np.uint64)
@@ -113,20 +126,14 @@ def test_store_retrieve_compose_against_the_oracle(shape, codec, rho):
 @pytest.mark.parametrize("codec", [TD8, TD4], ids=["int8td", "int4td"])
 @pytest.mark.parametrize("shape", [SHAPES[0], SHAPES[3].with_(block_size=16)], ids=["slice128", "slice64"])
 def test_group_tails_and_escapes_at_every_place(shape, codec, T):
-    """The decoder takes four symbols at a time, several out of one 32-bit window, and half of a group's rows at a time:
+    """The decoder takes two, three or four symbols out of one 32-bit window, rounds of up to eight, and half of a group's rows at a time:
     lengths around those steps, channels whose escapes (rare large codes among zeros) sit at every phase of a step, and
     channels whose code words straddle windows.  Bit-exact."""
     bs = shape.block_size
     rng = np.random.default_rng(1000 + T)
     perm = rng.permutation(shape.n_blocks).astype(np.int32)
     nb = -(-T // bs)
-    pool = make_pool_np(shape, perm[:nb], 0, nb * bs, 0.9, seed=T)
-    t = np.arange(nb * bs)
-    for c in range(8, 40):
-        x = np.zeros(nb * bs, dtype=np.float32)
-        x[(t + c) % (7 + c % 5) == 0] = 2.0 * (1 - 2 * (c & 1))              # escapes at every phase of a step
-        x[(t * 5 + c) % 11 == 0] += 0.07 * (c % 7)                           # among small codes, so that k stays small
-        pool[0, c & 1, perm[t // bs], t % bs, 0, c] = bf16_bits(x)
+    pool = make_escape_pool_np(shape, perm[:nb], T)
     dev = Device(shape, pool_np=pool)
     try:
         want = oracle.store(pool, perm[:nb], 0, T, codec)
@@ -750,5 +757,46 @@ def test_the_cheapest_parameters_are_found_whatever_the_tails(codec, T):
 @pytest.mark.parametrize("T", [2, 6, 7, 8, 9, 14, 38, 47, 62])
 @pytest.mark.parametrize("codec", [TD8, TD4], ids=["int8td", "int4td"])
 def test_lengths_around_the_decoder_steps(codec, T):
-    """Steps of six symbols, three to a window, then of two (8-bit codes), or of eight, four to a window (4-bit codes), and what is left one by one."""
     test_group_tails_and_escapes_at_every_place(SHAPES[0], codec, T)
+
+
+@pytest.mark.parametrize("T", [1, 2, 3, 5, 6, 7, 8, 9, 11, 12, 13, 31, 33, 38, 47, 62, 63, 64])
+@pytest.mark.parametrize("codecs", [(TD8,), (TD4,), (TD8, TD4)], ids=["int8td", "int4td", "both"])
+@pytest.mark.parametrize("shape", [SHAPES[0], SHAPES[3].with_(block_size=16)], ids=["slice128", "slice64"])
+def test_steps_of_every_decoder(shape, codecs, T):
+    """A decoder for each codec and one for calls of both, for retrieve and for compose, for the usual slice and for others, each with steps of its
+    own: lengths around all of them on channels with escapes and straddling code words, keys moved and left where they were."""
+    bs = shape.block_size
+    perm = np.random.default_rng(1000 + T).permutation(shape.n_blocks).astype(np.int32)
+    nb, n = -(-T // bs), 2
+    pool = make_escape_pool_np(shape, perm[:nb], T)
+    dev = Device(shape, pool_np=pool)
+    try:
+        K = dev.K
+        mine = [codecs[i % len(codecs)] for i in range(n)]
+        bufs = [dev.chunk_buf(T, c) for c in mine]
+        dev.store([dev.op(dev.table(perm[:nb]), 0, b, T, c) for b, c in zip(bufs, mine)])
+        wants = [oracle.store(pool, perm[:nb], 0, T, c) for c in mine]
+        dst = perm[nb:3 * nb].reshape(n, nb)
+        dev.retrieve([dev.op(dev.table(d), 0, b, T, c) for d, b, c in zip(dst, bufs, mine)])
+        assert dev.sync() == 0
+        ref = pool.copy()
+        for d, w, c in zip(dst, wants, mine):
+            oracle.retrieve(ref, d, 0, T, c, w)
+        assert np.array_equal(dev.pool_np(), ref)
+        for moved in range(n):                                           # one part is moved, the other one not
+            rt = perm[(3 + 2 * moved) * nb:(5 + 2 * moved) * nb]
+            parts = [(w, T, c, i * nb * bs + (9 if i == moved else 0), i * nb * bs) for i, (w, c) in enumerate(zip(wants, mine))]
+            dev.compose([K.ComposeReq(dev.table(rt).data_ptr(), len(rt), [dev.chunk(b, T, c, p[3]) for b, c, p in zip(bufs, mine, parts)],
+                                      [p[4] for p in parts], shape.rope_theta)])
+            assert dev.sync() == 0
+            kref, kmag = oracle.compose(ref, rt, parts, shape.rope_theta, want_ref=True)
+            got = dev.pool_np()
+            p = moved * nb * bs + np.arange(T)
+            rot = np.zeros(got.shape, dtype=bool)
+            rot[:, 0, rt[p // bs], p % bs] = True
+            assert np.array_equal(got[~rot], ref[~rot])
+            check_rotated_keys(got[:, 0, rt[p // bs], p % bs], kref[:, p], kmag[:, p], ref[:, 0, rt[p // bs], p % bs], min_equal=0.9)
+            ref[:, 0, rt[p // bs], p % bs] = got[:, 0, rt[p // bs], p % bs]
+    finally:
+        dev.close()
