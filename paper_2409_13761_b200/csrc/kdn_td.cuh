@@ -619,12 +619,19 @@ __device__ __forceinline__ void td_append(TdOut &o, uint32_t w, unsigned nlen)
                  : "+r"(o.wp) : "r"(word), "r"((o.bits ^ bits) & 32u) : "memory");
     o.bits = bits;
 }
-// One symbol, escapes included; ub: bits of 2^23 + u (- 1 for k = 0).
-__device__ __forceinline__ void td_append_any(TdOut &o, uint32_t ub, unsigned raw_bits)
+// One symbol, escapes included; ub: bits of 2^23 + u (- 1 for k = 0), n: kTdLenZero minus its length, were it none.  (Length and escape out of the
+// multiply-add that the joined symbols take them from: with integers from u, store of 8 chunks of 512 tokens with 8-bit codes, small values and 2 % large
+// ones: 726 us, this way 674; uncorrelated 420 -> 406, 4-bit codes 355 -> 338.)
+__device__ __forceinline__ void td_append_any(TdOut &o, uint32_t ub, float n, unsigned raw_bits)
 {
-    const uint32_t u = (uint32_t)max((int)(ub - kTdUZero) + (o.k ? 0 : 1), 0), q = u >> o.k;       // (2^23 - 1, for k = 0 and u = 0, has bits two below those of 2^23)
-    const bool escape = q >= 15u;
-    td_append(o, escape ? ~u & ((1u << raw_bits) - 1u) : (~u & o.kmask) | o.kbit, 0u - (escape ? 15u + raw_bits : q + o.k + 1u));
+    const bool escape = n <= o.limit;
+    td_append(o, escape ? ~(ub + (o.kbit & 1u)) & ((1u << raw_bits) - 1u) : (~ub & o.kmask) | o.kbit, escape ? 0u - (15u + raw_bits) : __float_as_uint(n));
+}
+__device__ __forceinline__ float td_fma_up(float a, float b, float c)
+{
+    float d;
+    asm("fma.rp.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
 }
 __device__ __forceinline__ float td_min3_nan(float a, float b, float c)
 {
@@ -644,7 +651,7 @@ __device__ __forceinline__ f32x2 td_fma2_up(f32x2 a, f32x2 b, f32x2 c)        //
 template <unsigned kN> struct TdJoin { static constexpr unsigned value = kN; };
 template <unsigned kJoin, typename Again>
 __device__ __forceinline__ void td_append4(TdOut &x, TdOut &y, const uint32_t (&ux)[4], const uint32_t (&uy)[4], const float (&nx)[4], const float (&ny)[4],
-                                           unsigned raw_bits, Again again)
+                                           float px, float py, float lx, float ly, unsigned raw_bits, Again again)
 {
     uint32_t zx[4], zy[4];
 #pragma unroll
@@ -680,8 +687,8 @@ __device__ __forceinline__ void td_append4(TdOut &x, TdOut &y, const uint32_t (&
         }
 #pragma unroll 1
         for (int i = 0; i < 4; ++i) {                        // (rolled up: instruction fetch is felt in this kernel)
-            td_append_any(x, a[0], raw_bits);
-            td_append_any(y, b[0], raw_bits);
+            td_append_any(x, a[0], td_fma_up(__uint_as_float(a[0]), px, lx), raw_bits);
+            td_append_any(y, b[0], td_fma_up(__uint_as_float(b[0]), py, ly), raw_bits);
             a[0] = a[1]; a[1] = a[2]; a[2] = a[3];
             b[0] = b[1]; b[1] = b[2]; b[2] = b[3];
         }
@@ -773,6 +780,9 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 320u, kCols ? 16 : 2) kdn
         const f32x2 per2 = pack2(-per_len(x.k), -per_len(y.k));
         auto len_zero = [&](unsigned k) { return k ? kTdLenZero + 8388608.0f * per_len(k) - (float)(k + 1u) : kTdLenZero + 8388606.0f; };
         const f32x2 len2 = pack2(len_zero(x.k), len_zero(y.k));
+        float px, py, lx, ly;
+        unpack2(per2, px, py);
+        unpack2(len2, lx, ly);
         auto symbol = [&](uint32_t v, uint32_t &a, uint32_t &b) {
             const f32x2 r = add2_unfused(mul2(bf16x2_widen(v), inv2), m2, one2);
             const f32x2 f = fma2(add2(r, base), two2, half2);
@@ -820,7 +830,7 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 320u, kCols ? 16 : 2) kdn
                         symbol(v[i + j], ux[j], uy[j]);
                         unpack2(td_fma2_up(pack2_bits(ux[j], uy[j]), per2, len2), nx[j], ny[j]);
                     }
-                    td_append4<decltype(join)::value>(x, y, ux, uy, nx, ny, raw_bits, [&](unsigned j, uint32_t &a, uint32_t &b) { again(t0 + (unsigned)i + j, a, b); });
+                    td_append4<decltype(join)::value>(x, y, ux, uy, nx, ny, px, py, lx, ly, raw_bits, [&](unsigned j, uint32_t &a, uint32_t &b) { again(t0 + (unsigned)i + j, a, b); });
                 }
             }
             return t0;
@@ -831,8 +841,8 @@ __global__ void __launch_bounds__(kCols ? kCols / 2u : 320u, kCols ? 16 : 2) kdn
             uint32_t ux, uy;
             symbol(__ldcg(reinterpret_cast<const uint32_t *>(rows[t0]) + tid), ux, uy);
             if (max(ux, uy) > 0x7f800000u) again(t0, ux, uy);
-            td_append_any(x, ux, raw_bits);
-            td_append_any(y, uy, raw_bits);
+            td_append_any(x, ux, td_fma_up(__uint_as_float(ux), px, lx), raw_bits);
+            td_append_any(y, uy, td_fma_up(__uint_as_float(uy), py, ly), raw_bits);
         }
         td_out_pad(x);
         td_out_pad(y);

@@ -800,3 +800,46 @@ def test_steps_of_every_decoder(shape, codecs, T):
             ref[:, 0, rt[p // bs], p % bs] = got[:, 0, rt[p // bs], p % bs]
     finally:
         dev.close()
+
+
+@pytest.mark.parametrize("T", [1, 2, 3, 5, 8, 16, 64, 75])
+@pytest.mark.parametrize("codec", [TD8, TD4], ids=["int8td", "int4td"])
+@pytest.mark.parametrize("shape", [SHAPES[0], SHAPES[3].with_(block_size=16)], ids=["slice128", "slice64"])
+def test_the_encoder_at_every_parameter_and_in_shared_words(shape, codec, T):
+    """Code lengths come from a rounded-up multiply-add in which u - 1 stands for u where k = 0, and first and last words of sub-streams are put together
+    in shared memory: zeros and escapes at k = 0, every other k, both modes, and sub-streams of one byte, four to a word.  Bit-exact."""
+    bs, D = shape.block_size, shape.head_dim
+    rng = np.random.default_rng(T)
+    nb = -(-T // bs)
+    perm = rng.permutation(shape.n_blocks).astype(np.int32)
+    x = rng.standard_normal((shape.n_layers, 2, nb * bs, shape.n_kv_heads, D)).astype(np.float32) * 0.3
+    x[..., 1::2] = np.cumsum(x[..., 1::2], axis=2)                            # (differences are shorter there)
+    c = np.arange(D)
+    x *= 2.0 ** -(c % 9)                                                       # the bulk, so that every k wins somewhere
+    x[:, :, ::16] = np.where(c % 3 == 0, 1.0, x[:, :, ::16])                    # a largest value, an escape where k is small
+    x[:, 0, :, :, :24] = 0.0                                                    # one bit a token: neighbours share words
+    x[:, 1, :, :, 8:24:2] = 0.0
+    x[:, 1, 5::7, :, 24:32] = np.where(np.arange(nb * bs)[5::7, None, None] % 2, 1.0, -1.0)      # zeros and escapes at k = 0
+    x[:, 1, 6::7, :, 24:32] = 0.0
+    pool = np.zeros((shape.n_layers, 2, shape.n_blocks, bs, shape.n_kv_heads, D), dtype=np.uint16)
+    t = np.arange(nb * bs)
+    pool[:, :, perm[t // bs], t % bs] = bf16_bits(x)
+    dev = Device(shape, pool_np=pool)
+    try:
+        want = oracle.store(pool, perm[:nb], 0, T, codec)
+        used = oracle.td_used_bytes(want, shape.n_layers, shape.n_kv_heads, D, T, codec)
+        lay = dev.K.kdn_td_layout(dev.desc, T, codec)
+        lens, params = want[lay["lens_offset"]:lay["params_offset"]], want[lay["params_offset"]:lay["streams_offset"]]
+        if T <= 8:
+            assert np.any((lens[:-3] == 1) & (lens[1:-2] == 1) & (lens[2:-1] == 1) & (lens[3:] == 1))
+        if T == 64:
+            assert len(np.unique(params & 7)) >= (7 if codec == TD8 else 3) and len(np.unique(params >> 3)) == 2
+            raw = 9 if codec == TD8 else 5
+            assert np.any(((params & 7) == 0) & (lens.astype(int) * 8 >= T - 1 + 15 + raw))      # an escape at k = 0
+        buf = dev.chunk_buf(T, codec)
+        dev.store([dev.op(dev.table(perm[:nb]), 0, buf, T, codec)])
+        assert dev.sync() == 0
+        got = to_np(buf)
+        assert np.array_equal(got[:used], want[:used]) and np.all(got[used:] == 0xA5)
+    finally:
+        dev.close()
