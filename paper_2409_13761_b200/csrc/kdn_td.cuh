@@ -255,45 +255,36 @@ template <int kN> __device__ __forceinline__ void td_transpose(const TdLaunch &P
     }
 }
 
-// `sum` plus the sum over 64 symbols of what a code word takes beyond its k + 1 bits, times 16: min(u >> k, ...) for the unary part, or
+// The sum over 64 symbols of what a code word takes beyond its k + 1 bits, times 16, for a k at which a symbol may escape: u >> k for the unary part, or
 // kEsc - 1 - k for an escape (u >> k >= 15).  lo and hi are the planes of u for tokens 0-31 and 32-63; the two halves' numbers are added
 // plane by plane first, which leaves one count per plane of the sum: popc runs at an eighth of the rate of the logic.
 template <int kPlanes, int kMax, int kEsc, int kK>
-__device__ __forceinline__ unsigned td_plan_sum(const TdLaunch &P, unsigned sum, const uint32_t (&lo)[kPlanes], const uint32_t (&hi)[kPlanes])
+__device__ __forceinline__ unsigned td_plan_sum(const TdLaunch &P, const uint32_t (&lo)[kPlanes], const uint32_t (&hi)[kPlanes])
 {
-    constexpr bool kEscapes = (kMax >> kK) >= 15;
-    constexpr int kBits = kEscapes ? 5 : kPlanes - kK;
-    if constexpr (kBits <= 0) {
-        return sum;
-    } else {
-        uint32_t x[2][kBits];
+    constexpr int v = kEsc - 1 - kK;
+    static_assert((kMax >> kK) >= 15, "nothing escapes at this k");
+    static_assert(v >= 16 && v < 32, "the planes of an escape's cost");
+    uint32_t x[2][5];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint32_t (&b)[kPlanes] = h ? hi : lo;
-            if constexpr (kEscapes) {
-                constexpr int v = kEsc - 1 - kK;
-                static_assert(v >= 16 && v < 32, "the planes of an escape's cost");
-                uint32_t over = 0u;                          // bits above the four that a short quotient has
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t (&b)[kPlanes] = h ? hi : lo;
+        uint32_t over = 0u;                                  // bits above the four that a short quotient has
 #pragma unroll
-                for (int i = kK + 4; i < kPlanes; ++i) over |= b[i];
-                const uint32_t esc = (b[kK] & b[kK + 1] & b[kK + 2] & b[kK + 3]) | over;
+        for (int i = kK + 4; i < kPlanes; ++i) over |= b[i];
+        const uint32_t esc = (b[kK] & b[kK + 1] & b[kK + 2] & b[kK + 3]) | over;
 #pragma unroll
-                for (int i = 0; i < 4; ++i) x[h][i] = ((v >> i) & 1) ? b[kK + i] | esc : b[kK + i] & ~esc;
-                x[h][4] = esc;
-            } else {
-#pragma unroll
-                for (int i = 0; i < kBits; ++i) x[h][i] = b[kK + i];
-            }
-        }
-        uint32_t carry = 0u;
-#pragma unroll
-        for (int i = 0; i < kBits; ++i) {
-            const uint32_t p = x[0][i], q = x[1][i];
-            sum += (unsigned)__popc(p ^ q ^ carry) * P.pow2[4 + i];
-            carry = (p & q) | (carry & (p | q));
-        }
-        return sum + (unsigned)__popc(carry) * P.pow2[4 + kBits];
+        for (int i = 0; i < 4; ++i) x[h][i] = ((v >> i) & 1) ? b[kK + i] | esc : b[kK + i] & ~esc;
+        x[h][4] = esc;
     }
+    unsigned sum = 0u;
+    uint32_t carry = 0u;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const uint32_t p = x[0][i], q = x[1][i];
+        sum += (unsigned)__popc(p ^ q ^ carry) * P.pow2[4 + i];
+        carry = (p & q) | (carry & (p | q));
+    }
+    return sum + (unsigned)__popc(carry) * P.pow2[9];
 }
 // The smallest (bits * 16 + mode * 8 + k) over the parameters of one mode, and `best`, for n symbols.  With c_i symbols that have bit i, the sum of
 // u >> k is c_k + 2 c_(k+1) + 4 c_(k+2) + ..: two popc a plane serve every k at which nothing can escape.  Where something can, the
@@ -342,13 +333,15 @@ __device__ __forceinline__ unsigned td_plan_mode(const TdLaunch &P, unsigned bes
         uint32_t esc = (lo[k] & lo[k + 1] & lo[k + 2] & lo[k + 3]) | (hi[k] & hi[k + 1] & hi[k + 2] & hi[k + 3]);
 #pragma unroll
         for (int i = k + 4; i < kPlanes; ++i) esc |= lo[i] | hi[i];
-        const unsigned sum = __any_sync(0xffffffffu, esc != 0u) ? td_plan_sum<kPlanes, kMax, kEsc, k>(P, 0u, lo, hi) : all[k] * 16u;
+        const unsigned sum = __any_sync(0xffffffffu, esc != 0u) ? td_plan_sum<kPlanes, kMax, kEsc, k>(P, lo, hi) : all[k] * 16u;
         best = min(best, sum + n16 * (k + 1u) + (kMode * 8u + k));
     };
-    if constexpr (kFree >= 6) look(TdConst<5>());
-    if constexpr (kFree >= 5) look(TdConst<4>());
-    if constexpr (kFree >= 4) { look(TdConst<3>()); look(TdConst<2>()); look(TdConst<1>()); }
-    if constexpr (kFree >= 1) look(TdConst<0>());
+    if constexpr (kFree > 5) look(TdConst<5>());
+    if constexpr (kFree > 4) look(TdConst<4>());
+    if constexpr (kFree > 3) look(TdConst<3>());
+    if constexpr (kFree > 2) look(TdConst<2>());
+    if constexpr (kFree > 1) look(TdConst<1>());
+    if constexpr (kFree > 0) look(TdConst<0>());
     return best;
 }
 
