@@ -996,6 +996,7 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
         tp.wait_limit_ns = ctx->wait_limit_ns;
         RopeInline rope_inl{};
         int n_rope = 0, max_groups = 0, max_layers = 0;
+        unsigned words = 0;                                          // of the longest sub-stream of the launch's codecs, and one more
         bool any5 = false, any6 = false;
         for (int i = 0; i < m; ++i) {
             DevOp op = hops[first + i].op;
@@ -1007,7 +1008,7 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
             (op.codec == KDN_CODEC_INT4_TD64 ? any6 : any5) = true;
             tp.inline_ops[i] = op;
             tp.layout[i] = td_layout(pool.L, row_elems, op.T, op.codec);
-            if (td_words(op.codec) > tp.words) tp.words = td_words(op.codec);
+            if (td_words(op.codec) > words) words = td_words(op.codec);
             const int g = (op.T + 63) / 64;
             if (g > max_groups) max_groups = g;
             if (op.nl > max_layers) max_layers = op.nl;
@@ -1034,7 +1035,7 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
         const dim3 grid((unsigned)max_groups * n_split, (unsigned)max_layers * 2u, (unsigned)m);
         int per_sm = 0;
         if (OP == OP_STORE) {
-            const size_t smem_enc = td_encode_smem_bytes(cols, tp.words);
+            const size_t smem_enc = td_encode_smem_bytes(cols, words);
             if (smem_enc > smem_limit) return KDN_E_UNSUPPORTED;
             const unsigned enc_threads = (cols / 2u + 31u) & ~31u;       // a thread codes two channels
             kdn_status r = cols == kTdCols ? ctx->env.resident(kdn_td_encode_kernel<kTdCols>, (int)enc_threads, smem_enc, &per_sm)
@@ -1051,7 +1052,7 @@ kdn_status launch_td(kdn_ctx *ctx, const Pool &pool, int OP, const HostOp *hops,
             if (r != KDN_OK) return r;
             ctx->launches += 3;
         } else {
-            const size_t smem = td_decode_smem_bytes(cols, tp.words);
+            const size_t smem = td_decode_smem_bytes(cols, words);
             if (smem > smem_limit) return KDN_E_UNSUPPORTED;
             RingSlot *slot = nullptr;
             if (n_rope) {

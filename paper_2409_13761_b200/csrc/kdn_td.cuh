@@ -52,7 +52,6 @@ struct TdLaunch {
     unsigned cols;            // channels per CTA
     unsigned n_split;         // row_elems / cols, a power of two
     unsigned split_shift;     // log2(n_split)
-    unsigned words;           // decode: 32-bit words kept per sub-stream (the longest of the launch's codecs, and one more)
     int bs_shift;             // log2(bs), -1 where bs is not a power of two
     int minus_one;            // -1 as a launch parameter: see TdStream
     float fone;               // 1.0f (see Launch::one)
