@@ -16,9 +16,11 @@ The same run then times, outside `value`: both ends of the chunk-length sweep (1
 16 and 32, both codecs, fully fragmented tables) and the largest configuration, Llama-3-70B-shaped KV (80 layers,
 library of 16 x 2048-token chunks, 32 requests x 4 chunks filling the 80 GiB pool, four of the retrievals reading
 their chunk from page-locked host memory on a side stream).  `roofline.per_op` lists every op of both workloads as
-[GB/s, fraction of the nominal 8000 GB/s], from the median CUDA-event time of the op over the timed steps.
+[GB/s, fraction of the nominal 8000 GB/s], from the median CUDA-event time of the op over the timed steps (in the longer line; the
+record has the GB/s).
 With --impl reference the CPU oracle is timed instead, on a bounded sample of the same workload.
-The line printed last on stdout is the JSON record.
+The line on stdout is the JSON record; it is kept short (LINE_MOST characters).  Everything that was measured goes to stderr, as one
+longer JSON line.
 """
 from __future__ import annotations
 
@@ -45,7 +47,35 @@ N_CHUNKS, CHUNK_TOKENS = 64, 512
 N_PARTS, PART_TOKENS, SUFFIX_TOKENS = 10, 1024, 256
 RAW, INT8, INT4, INT8KC, INT4KC, INT8TD, INT4TD = 0, 1, 2, 3, 4, 5, 6
 FALLBACK_HBM_GBS = 6650.0
-TD_DECODE_INSTS = {INT8TD: 23.4, INT4TD: 21.0}     # warp instructions per 32 symbols of the token-delta decoder (profiles/ncu_token_delta_kernels_llama3_8b.md; one kernel for both codecs then)
+TD_DECODE_INSTS = {INT8TD: 22.3, INT4TD: 19.8}     # warp instructions per 32 symbols of the token-delta decoders (profiles/ncu_token_delta_kernels_llama3_8b.md)
+LINE_MOST = 2600                                   # a record that is read from the end of a log has to fit there
+
+
+def rounded(x):
+    """Floats to six digits, throughout."""
+    if isinstance(x, dict):
+        return {k: rounded(v) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [rounded(v) for v in x]
+    return float("%.6g" % x) if isinstance(x, float) else x
+
+
+def record_line(rec: dict) -> str:
+    """The record's line: what identifies and judges the run, and per-op figures of both workloads while there is room."""
+    keep = {k: rec[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+                                "dtype", "data", "tokens_per_s_reloaded", "gpu_launches")}
+    keep["config"] = {k: rec["config"][k] for k in ("workload", "l2", "bytes_per_step")}
+    keep["clocks"] = {k: rec["clocks"][k] for k in ("sm_mhz", "sm_max_mhz", "reasons")}
+    keep["e2e"] = {k: rec["e2e"][k] for k in ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "steps", "ms_per_step", "host_link_gbs")}
+    if "cpu_baseline" in rec:
+        keep["cpu_baseline"] = {k: rec["cpu_baseline"][k] for k in ("value", "unit", "cores", "kind", "sample")}
+    keep["roofline"] = {k: rec["roofline"][k] for k in ("bound", "kernel", "op", "achieved", "peak", "peak_kind", "unit", "frac", "traffic")}
+    per_op = rec["roofline"]["per_op"]
+    for name in ("8b", "70b"):
+        line = json.dumps(rounded({**keep, "gbs_" + name: {n: v[0] for n, v in per_op.get(name, {}).items()}}))
+        if name in per_op and len(line) <= LINE_MOST:
+            keep["gbs_" + name] = {n: v[0] for n, v in per_op[name].items()}
+    return json.dumps(rounded(keep))
 
 
 def bytes_per_elem(codec: int) -> float:
@@ -617,8 +647,8 @@ def extras_8b(leg, dev_sets, reps, which=EXTRAS):
                     "retrieve_frac_of_8000": moved / (ms_retr * 1e-3) / 1e9 / 8000.0,
                     "retrieve_roofline": {"bound": "hbm", "unit": "GB/s", "achieved": moved / (ms_retr * 1e-3) / 1e9, "peak": measured_hbm_peak()[0],
                                           "frac": moved / (ms_retr * 1e-3) / 1e9 / measured_hbm_peak()[0]},
-                    # what keeps it from there is instruction issue: the present decoder's warp instructions (profiler count) as a share of the
-                    # issue slots of 148 SMs x 4 schedulers x 1.965 GHz
+                    # what keeps it from there is instruction issue: the decoder's warp instructions (profiler count, correlation 0.9) as a share of
+                    # the issue slots of 148 SMs x 4 schedulers x 1.965 GHz
                     "retrieve_issue": {"warp_instructions_per_32_symbols": TD_DECODE_INSTS[codec],
                                        "share_of_slots": n_td * T * E / 32 * TD_DECODE_INSTS[codec] / (ms_retr * 1e-3) / (148 * 4 * 1.965e9)},
                     "from_host_ms": host_ms, "from_host_link_gbs": used / (host_ms * 1e-3) / 1e9,
@@ -989,7 +1019,8 @@ def run_gpu(args) -> None:
             one = OracleSample(1, 128)                       # the same oracle on one core, on a smaller chunk
             b1, t1, dt1 = one.run_pass()
             rec["cpu_baseline"]["one_core"] = {"value": b1 / dt1 / 1e9, "unit": UNIT, "sample": one.describe(1, b1, dt1)}
-        print(json.dumps(rec))
+        print(json.dumps(rec), file=sys.stderr)
+        print(record_line(rec))
     if dist is not None:
         dist.destroy_process_group()
 
