@@ -432,9 +432,10 @@ __device__ __forceinline__ unsigned td_plan_channel(const TdLaunch &P, const uin
 }
 
 // A warp takes 32 channels: lanes l and l + 16 hold the same two channels, tokens 0-31 and 32-63, straight from the pool in
-// registers (no shared tile: every value is used once, and a thread has 32 loads in flight).  Bound by the pipe of logic and shifts
-// (two thirds busy).  8B shape, 16 chunks of 512 tokens, 8-bit codes: 1100 us with a table of code-word lengths looked up per
-// symbol, 330 us this way; 4-bit codes 1080 -> 220 us.  Six CTAs of 128 threads an SM (80 registers); seven or eight spill and are 2 % slower.
+// registers (no shared tile: every value is used once, and a thread has 32 loads in flight).  Bound by instruction issue, as far as 24 warps an SM, whose
+// loads come in one burst each, can fill it: 71 % of the slots, the pipe of logic and shifts 56 % (4-bit codes 67 and 39 %).  8B shape, 8 chunks of 512
+// tokens, under the profiler: 537 us with a table of code-word lengths looked up per symbol, 168 us this way (uncorrelated; correlation 0.9: 178), 4-bit
+// codes 141.  Six CTAs of 128 threads an SM (78 registers); seven or eight spill and are 2 % slower.
 // kThreads: 128 is the usual slice of 128 channels, 512 stands for any other.
 template <unsigned kThreads>
 __global__ void __launch_bounds__(kThreads, kThreads == 128u ? 6 : 1) kdn_td_plan_kernel(const __grid_constant__ TdLaunch P)
@@ -709,11 +710,11 @@ __device__ __forceinline__ void td_out_last(const TdOut &o)
 
 // A thread quantises and codes two neighbouring channels side by side, token by token, straight from the pool: the planner's scale
 // says what the largest magnitude was (a bf16 number: scale * qmax rounded to bf16 is that number again), so there is no pass
-// for it and no tile.  The staging area holds the slice's bits complemented, as big-endian words.  Bound by instruction issue
-// (77 % of the slots).  8B shape, 16 chunks of 512 tokens: 1020 us for 8-bit codes with a tile, a pass over it for the magnitudes and
-// every symbol appended by itself, 520 us this way; 4-bit codes 1000 -> 470 us.  Lengths of two channels from one multiply-add, and no word kept
-// aside, took the whole store from 795 to 782 us (uncorrelated), 810 -> 799 (correlation 0.9), 853 -> 851 (0.99), with 4-bit codes 698 -> 692, 693 -> 688, 689 -> 686.  Sixteen CTAs of 64 threads an SM (64 registers) with
-// eight tokens loaded ahead; twelve CTAs, four or sixteen tokens are 1-7 % slower.
+// for it and no tile.  The staging area holds the slice's bits complemented, as big-endian words.  Bound by instruction issue and by its loads (73 %
+// of the slots, 31 warps an SM, 21.5 warp instructions per 32 symbols, 4-bit codes 19.1).  8B shape, 8 chunks of 512 tokens, under the profiler: 495 us with a
+// tile, a pass over it for the magnitudes and every symbol appended by itself, 222 us this way; 4-bit codes 196.  The whole store of 16 chunks takes
+// 765 us with 8-bit codes (uncorrelated; correlation 0.9: 780, 0.99: 824), 660, 656 and 654 us with 4-bit ones.  Sixteen CTAs of 64 threads an SM
+// (64 registers) with eight tokens loaded ahead; twelve CTAs, four or sixteen tokens were 1-7 % slower.
 // (Other slices: at most 256 threads, 96 registers; at 104 a slice of 192 channels loses a CTA an SM and 10 %.)
 template <unsigned kCols>
 __global__ void __launch_bounds__(kCols ? kCols / 2u : 320u, kCols ? 16 : 2) kdn_td_encode_kernel(const __grid_constant__ TdLaunch P)
@@ -978,14 +979,14 @@ __device__ __forceinline__ void td_step(const TdLaunch &P, TdStream &x, TdStream
     }
 }
 
-// Bound by instruction issue and the integer pipes (8B shape, 4-bit codes: issue slots 83 %, logic 55 %, DRAM 37 %, 21 warp instructions per 32
-// symbols; 8-bit codes 76 %, 48 %, 38 %, 23.4); what was done about it is at TdStream and td_step.  A thread decodes two channels side by side --
-// neighbours, whose bf16 values make one word, or, where keys are re-rotated, the two channels of a rotation pair -- so that one
-// stream's chain of dependent operations hides the other's, and writes finished values into the rows: no pass over codes.  Half
-// of the rows at a time keeps a CTA of 64 threads at 16 KiB of shared memory, twelve (8-bit codes: ten) to an SM; all rows at a time
-// are 15 % slower.  The rows leave with 128-bit stores, sixteen lanes to a 256-byte piece of a token row.  8B shape, 32 chunks of 512
-// tokens, 4-bit codes: 1728 us with one thread per channel, a code tile and a separate pass that multiplied, 709 us this way; 8-bit
-// codes 1765 -> 864 us.  (The counters are those of one kernel for both codecs, 724 and 892 us.)
+// Bound by instruction issue and the integer pipes (8B shape, 4-bit codes: issue slots 81 %, logic 57 %, DRAM 37 %, 19.8 warp instructions per 32
+// symbols; 8-bit codes 73 %, 49 %, 39 %, 22.3, with ten CTAs an SM where 4-bit codes have fourteen); what was done about it is at TdStream and td_step.  A
+// thread decodes two channels side by side -- neighbours, whose bf16 values make one word, or, where keys are re-rotated, the two channels of a rotation pair --
+// so that one stream's chain of dependent operations hides the other's, and writes finished values into the rows: no pass over codes.  Half
+// of the rows at a time keeps a CTA of 64 threads at 15 KiB of shared memory (8-bit codes: 20); all rows at a time were
+// 15 % slower.  The rows leave with 128-bit stores, sixteen lanes to a 256-byte piece of a token row.  8B shape, 32 chunks of 512
+// tokens, correlation 0.9: 4-bit codes 1728 us with one thread per channel, a code tile and a separate pass that multiplied, 696 us this way; 8-bit
+// codes 1765 -> 873 us.
 // kCols: channels per CTA when known at compile time (the usual slice; every stride in the decoding loop is then an
 // immediate), 0: taken from the launch record.
 // kCodec: the codec of the launch's chunks, 0 where it has chunks of both.  (A kernel per codec takes fewer instructions, but a launch for each
